@@ -123,7 +123,7 @@ attn_encoder_tc_kernel(const AttnEncGroup* __restrict__ groups, int n_groups, in
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    {
       bool ok = true;
       const AttnEncGroup* g_prev = nullptr;
       uint32_t it = 0;
@@ -134,15 +134,15 @@ attn_encoder_tc_kernel(const AttnEncGroup* __restrict__ groups, int n_groups, in
         const int T = g->T, KP = g->KP, d = g->H * 64, n_mt = (T + 127) >> 7;
         const int row0 = r.b * T;
         // Q and K: free once both S = Q K^T of the previous item are complete
-        if (!mbar_wait<false>(bar(B_QK_FREE), (it & 1u) ^ 1u, abort_flag)) { ok = false; atomicExch(status, 11); break; }
-        mbar_expect_tx(bar(B_FULL_QK), (uint32_t)(n_mt * ET_Q_BYTES + KP * 128));
+        if (!mbar_wait<false>(bar(B_QK_FREE), (it & 1u) ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 11); break; }
+        mbar_expect_tx_elect(bar(B_FULL_QK), (uint32_t)(n_mt * ET_Q_BYTES + KP * 128));
         for (int m = 0; m < n_mt; ++m)
-          tma_load_2d(base + ET_OFF_Q + m * ET_Q_BYTES, &g->tmQ, r.h * 64, row0 + m * 128, bar(B_FULL_QK));
-        tma_load_2d(base + ET_OFF_K, &g->tmKV, d + r.h * 64, row0, bar(B_FULL_QK));
+          tma_load_2d_elect(base + ET_OFF_Q + m * ET_Q_BYTES, &g->tmQ, r.h * 64, row0 + m * 128, bar(B_FULL_QK));
+        tma_load_2d_elect(base + ET_OFF_K, &g->tmKV, d + r.h * 64, row0, bar(B_FULL_QK));
         // V: free once the last P V of the previous item is complete
-        if (!mbar_wait<false>(bar(B_V_FREE), (it & 1u) ^ 1u, abort_flag)) { ok = false; atomicExch(status, 12); break; }
-        mbar_expect_tx(bar(B_FULL_V), (uint32_t)(KP * 128));
-        tma_load_2d(base + ET_OFF_V, &g->tmKV, 2 * d + r.h * 64, row0, bar(B_FULL_V));
+        if (!mbar_wait<false>(bar(B_V_FREE), (it & 1u) ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 12); break; }
+        mbar_expect_tx_elect(bar(B_FULL_V), (uint32_t)(KP * 128));
+        tma_load_2d_elect(base + ET_OFF_V, &g->tmKV, 2 * d + r.h * 64, row0, bar(B_FULL_V));
       }
       if (!ok) *abort_flag = 1;
       // copies in flight when a wait gave up: the consumers have left, so nothing reads them; let them land
@@ -158,7 +158,7 @@ attn_encoder_tc_kernel(const AttnEncGroup* __restrict__ groups, int n_groups, in
     // are waiting in TMEM when the softmax warps get there.
     // Barriers of the first query tile complete once per item, those of the second once per item with two
     // tiles: each has its own use counter (items of different models mix).
-    if (lane == 0) {
+    {
       bool ok = true;
       uint32_t cnt_s[2] = {0, 0};               // S = Q K^T issued so far, per tile index
       uint32_t cnt_pv[2] = {0, 0};              // P V issued so far, per tile index
@@ -166,19 +166,19 @@ attn_encoder_tc_kernel(const AttnEncGroup* __restrict__ groups, int n_groups, in
       // Q_m K^T of an item (its Q and K must have landed: caller waited FULL_QK)
       auto issue_s = [&](const AttnEncGroup* g, int m) -> bool {
         // the region still holds O_m of the previous item with this tile until the workers have read it
-        if (!mbar_wait<false>(bar(B_O_EMPTY0 + m), (cnt_s[m] & 1u) ^ 1u, abort_flag)) { atomicExch(status, 14); return false; }
+        if (!mbar_wait<false>(bar(B_O_EMPTY0 + m), (cnt_s[m] & 1u) ^ 1u, abort_flag)) { if (lane == 0) atomicExch(status, 14); return false; }
         tc_fence_after();
         const uint32_t idesc_s = make_idesc(g->KP);
         const uint64_t dq = make_smem_desc(base + ET_OFF_Q + m * ET_Q_BYTES), dk = make_smem_desc(base + ET_OFF_K);
         const uint32_t d_tmem = tmem_base + (uint32_t)(m ? ET_S_COL1 : ET_S_COL0);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) mma_f16(d_tmem, dq + (uint64_t)(k * 2), dk + (uint64_t)(k * 2), idesc_s, k > 0 ? 1u : 0u);
-        mma_commit(bar(B_S_FULL0 + m));
+        for (int k = 0; k < 4; ++k) mma_f16_elect(d_tmem, dq + (uint64_t)(k * 2), dk + (uint64_t)(k * 2), idesc_s, k > 0 ? 1u : 0u);
+        mma_commit_elect(bar(B_S_FULL0 + m));
         ++cnt_s[m];
         return true;
       };
       auto wait_qk = [&]() -> bool {
-        if (!mbar_wait<false>(bar(B_FULL_QK), cnt_qk & 1u, abort_flag)) { atomicExch(status, 13); return false; }
+        if (!mbar_wait<false>(bar(B_FULL_QK), cnt_qk & 1u, abort_flag)) { if (lane == 0) atomicExch(status, 13); return false; }
         tc_fence_after();
         ++cnt_qk;
         return true;
@@ -190,7 +190,7 @@ attn_encoder_tc_kernel(const AttnEncGroup* __restrict__ groups, int n_groups, in
         const int n_mt = (g_next->T + 127) >> 7;
         ok = wait_qk();
         for (int m = 0; m < n_mt && ok; ++m) ok = issue_s(g_next, m);
-        if (ok) mma_commit(bar(B_QK_FREE));     // arrives when every MMA issued so far is complete
+        if (ok) mma_commit_elect(bar(B_QK_FREE));     // arrives when every MMA issued so far is complete
       }
       for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x, ++it) {
         const AttnEncGroup* g = g_next;
@@ -202,7 +202,7 @@ attn_encoder_tc_kernel(const AttnEncGroup* __restrict__ groups, int n_groups, in
           n_mt_next = (g_next->T + 127) >> 7;
         }
         for (int m = 0; m < n_mt && ok; ++m) {
-          if (!mbar_wait<false>(bar(B_P_READY0 + m), cnt_pv[m] & 1u, abort_flag)) { ok = false; atomicExch(status, 16); break; }
+          if (!mbar_wait<false>(bar(B_P_READY0 + m), cnt_pv[m] & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 16); break; }
           tc_fence_after();                     // (P_READY also says that every worker has read S_m out)
           const uint32_t idesc_o = make_idesc(64) | (1u << 16);     // B operand MN-major
           const uint32_t d_tmem = tmem_base + (uint32_t)(m ? ET_S_COL1 : ET_S_COL0);
@@ -210,17 +210,17 @@ attn_encoder_tc_kernel(const AttnEncGroup* __restrict__ groups, int n_groups, in
           for (int k = 0; k < ksteps; ++k) {
             const uint64_t dp = make_smem_desc(base + ET_OFF_P + (k >> 2) * ET_P_BLOCK) + (uint64_t)((k & 3) * 2);
             const uint64_t dv = make_smem_desc_mn(base + ET_OFF_V + k * 2048);   // 16 tokens = two 8-token groups
-            mma_f16(d_tmem, dp, dv, idesc_o, k > 0 ? 1u : 0u);
+            mma_f16_elect(d_tmem, dp, dv, idesc_o, k > 0 ? 1u : 0u);
           }
-          mma_commit(bar(B_O_FULL0 + m));
-          if (m == n_mt - 1) mma_commit(bar(B_V_FREE));     // V may be overwritten once this P V is complete
+          mma_commit_elect(bar(B_O_FULL0 + m));
+          if (m == n_mt - 1) mma_commit_elect(bar(B_V_FREE));     // V may be overwritten once this P V is complete
           ++cnt_pv[m];
         }
         // scores of the next item
         if (ok && has_next) {
           ok = wait_qk();
           for (int m = 0; m < n_mt_next && ok; ++m) ok = issue_s(g_next, m);
-          if (ok) mma_commit(bar(B_QK_FREE));
+          if (ok) mma_commit_elect(bar(B_QK_FREE));
         }
       }
       if (!ok) *abort_flag = 1;

@@ -37,10 +37,7 @@ struct RowDesc {
 };
 
 // C = epi(A W^T + bias).  tmA/tmW are the TMA maps of A [rows, K] and W [N, K] (K innermost,
-// 128-byte swizzle, box 64 x 128 rows for A and 64 x bn rows for W).  The tensor-core kernel cuts
-// the group into tiles_m x tiles_n tiles of 128 x bn and every tile into ksplit ranges of
-// k-blocks; with ksplit > 1 each range leaves an fp32 partial in `partial` and the range that
-// arrives last (counted in `counters`) adds them in range order and runs the epilogue.
+// 128-byte swizzle, 64 columns x the rows a CTA loads of each).
 struct alignas(64) GemmGroup {
   CUtensorMap tmA;
   CUtensorMap tmW;
@@ -56,14 +53,14 @@ struct alignas(64) GemmGroup {
   int epi;
   int tile_start;  // first work item of this group in the launch
   int tiles_m, tiles_n;
-  int bn, ksplit;  // tensor-core kernel only: tile width (128 or 256), k ranges per tile
-  float* partial;  // [ksplit][tiles_m * 128][tiles_n * bn] fp32, ksplit > 1 only
-  int* counters;   // [tiles_m * tiles_n], zero between launches
+  int bn, ksplit;  // tile pairs: bn = tile width; swapped operands: bn = batch rows of a tile, ksplit = k ranges
   int c_rows;      // row extent of tmC (rows at and beyond it are never written)
   int stream;      // 1: at most 16 rows ever, runs in the weight-streaming kernel (16 W rows per block,
-                   // tiles_n = ceil(N / 16), no TMA maps); 0: one-CTA tensor-core tiles; 2: 256-row tiles on
-                   // CTA pairs (tiles_m counts 256-row tiles and tmW's box holds bn / 2 rows)
+                   // tiles_n = ceil(N / 16), no TMA maps); 2: 256-row tiles on CTA pairs (tiles_m counts 256-row
+                   // tiles and tmW's box holds bn / 2 rows); 3: swapped operands (tmA's box holds bn rows, tmW's
+                   // 128); 0: plain CUDA-core comparator
   int pad1, pad2;
+  int pad3[4];
 };
 
 struct GemmLaunch {      // header followed by groups

@@ -30,6 +30,7 @@ namespace {
 constexpr int N_SLOTS = 4;
 constexpr size_t BLOB_BYTES = 4u << 20;
 constexpr int MAX_PROFILE_LAUNCHES = 4096;
+constexpr int PASS_MLP = 11;   // last of a GEMM wave's launches (see epara_step)
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 inline int round_up(int v, int a) { return (v + a - 1) / a * a; }
@@ -132,7 +133,6 @@ struct Model {
   std::deque<Request> q[2];
   int max_chunks;       // decoder
   double kv_bytes_per_token;
-  size_t splitk_bytes = 0, splitk_tiles = 0;   // largest split-k partial buffer / tile count of its GEMMs
 };
 
 // The first BLOB_HEADER bytes of a slot's device blob hold the step's status word; the upload of the blob
@@ -220,8 +220,9 @@ struct Builder {
   }
 };
 
+// one_sum: the whole K of an output element in one accumulator (no k ranges added up afterwards).
 bool add_gemm(Builder& bl, Model* m, const void* A, int lda, long long rows_cap, const void* W, int N, int K,
-              void* C, int ldc, const void* bias, int epi, int rows_per_req) {
+              void* C, int ldc, const void* bias, int epi, int rows_per_req, bool one_sum = false) {
   const int sm_count = bl.sm_count;
   const long long max_rows = (long long)m->max_batch * rows_per_req;   // the most rows this op ever sees
   Op op;
@@ -232,27 +233,24 @@ bool add_gemm(Builder& bl, Model* m, const void* A, int lda, long long rows_cap,
   g.A = (const bf16*)A; g.W = (const bf16*)W; g.C = C; g.bias = (const bf16*)bias;
   g.N = N; g.K = K; g.lda = lda; g.ldw = K; g.ldc = ldc; g.epi = epi | (bias ? EPI_BIAS : 0);
   op.weight_bytes = 2.0 * N * K;
-  gemm_tc_config(rows_cap, N, K, g.epi, sm_count, &g.bn, &g.ksplit);
-  if (max_rows <= GEMM_STREAM_MAX_ROWS && bl.gemm_impl != EPARA_GEMM_SIMT) {
-    g.stream = 1; g.bn = 16; g.ksplit = 1;
-  } else if (max_rows <= GEMM_SWAP_MAX_ROWS && bl.gemm_impl != EPARA_GEMM_SIMT) {
+  g.ksplit = 1;
+  if (bl.gemm_impl == EPARA_GEMM_SIMT) {
+    g.stream = 0;
+  } else if (max_rows <= GEMM_STREAM_MAX_ROWS) {
+    g.stream = 1; g.bn = 16;
+  } else if (!one_sum && gemm_swap_eligible(max_rows, N, K, g.epi, sm_count)) {
     g.stream = 3;                              // W as the MMA's 128-row operand, the batch as its N
-    g.bn = round_up((int)max_rows, 16);
-    g.ksplit = gemm_swap_ksplit(N, K, sm_count);
-  } else if (bl.gemm_impl != EPARA_GEMM_SIMT && gemm_tc_pair_eligible(rows_cap, N, K, g.epi, g.bn, g.ksplit)) {
+    gemm_swap_config(max_rows, N, K, sm_count, &g.bn, &g.ksplit);
+  } else {
     g.stream = 2;                              // 256-row tiles on CTA pairs
-  }
-  if (g.ksplit > 1 && g.stream == 0) {
-    const size_t tiles_m = (size_t)((rows_cap + TC_BM - 1) / TC_BM), tiles_n = (size_t)((N + g.bn - 1) / g.bn);
-    m->splitk_bytes = std::max(m->splitk_bytes, (size_t)g.ksplit * tiles_m * TC_BM * tiles_n * g.bn * 4);
-    m->splitk_tiles = std::max(m->splitk_tiles, tiles_m * tiles_n);
+    gemm_pair_config(max_rows, N, K, g.epi, sm_count, &g.bn);
   }
   if (bl.c && g.stream == 3) {
     if (!make_tmap(&g.tmA, A, rows_cap, K, lda, g.bn)) return false;
     if (!make_tmap(&g.tmW, W, N, K, K, TC_BM)) return false;
-  } else if (bl.c && g.stream != 1) {
+  } else if (bl.c && g.stream == 2) {
     if (!make_tmap(&g.tmA, A, rows_cap, K, lda, TC_BM)) return false;
-    if (!make_tmap(&g.tmW, W, N, K, K, g.stream == 2 ? g.bn / 2 : g.bn)) return false;   // a pair's CTA loads half of the W rows
+    if (!make_tmap(&g.tmW, W, N, K, K, g.bn / 2)) return false;   // a pair's CTA loads half of the W rows
     if (!make_tmap_c(&g.tmC, C, rows_cap, N, ldc, g.epi)) return false;
   }
   g.c_rows = (int)rows_cap;
@@ -412,8 +410,10 @@ int build_model(Builder& bl, Model* m, const epara_config& cfg) {
       if (bl.gemm_impl == EPARA_GEMM_TCGEN05 && gemm_mlp_eligible(Mcap, dm, d.ffn)) {
         if (!add_mlp(bl, m, h, Mcap, w[8], w[9], w[10], w[11], z, dm, d.ffn, T)) return EPARA_E_CUDA;
       } else {
-        if (!add_gemm(bl, m, h, dm, Mcap, w[8], d.ffn, dm, f, d.ffn, w[9], EPI_GELU, T)) return EPARA_E_CUDA;
-        if (!add_gemm(bl, m, f, d.ffn, Mcap, w[10], dm, d.ffn, z, dm, w[11], EPI_RESID_F32, T)) return EPARA_E_CUDA;
+        // (where the fused block exists, its two GEMMs on their own keep its order of summation)
+        const bool one_sum = gemm_mlp_eligible(Mcap, dm, d.ffn);
+        if (!add_gemm(bl, m, h, dm, Mcap, w[8], d.ffn, dm, f, d.ffn, w[9], EPI_GELU, T, one_sum)) return EPARA_E_CUDA;
+        if (!add_gemm(bl, m, f, d.ffn, Mcap, w[10], dm, d.ffn, z, dm, w[11], EPI_RESID_F32, T, one_sum)) return EPARA_E_CUDA;
       }
     }
     const void* const* w = t + 4 + 12 * d.n_layers;
@@ -518,21 +518,6 @@ int build_model(Builder& bl, Model* m, const epara_config& cfg) {
   const size_t n_ops = m->ops.size();
   for (size_t i = 0; i + 3 < n_ops; ++i) m->ops[i].per_token = 1;
   m->ops[n_ops - 3].last_rows = 1;
-  return EPARA_OK;
-}
-
-// Split-k scratch shared by the model's GEMMs (they run one after the other): fp32 partials and
-// per-tile arrival counters (zero between launches).
-int finish_model(Builder& bl, Model* m) {
-  if (m->splitk_bytes == 0) return EPARA_OK;
-  float* partial = (float*)bl.get(m->splitk_bytes);
-  int* counters = (int*)bl.get(m->splitk_tiles * sizeof(int));
-  if (bl.fail) return EPARA_E_RESOURCE;
-  if (bl.c) {
-    if (cudaMemset(counters, 0, m->splitk_tiles * sizeof(int)) != cudaSuccess) return EPARA_E_CUDA;
-    for (Op& op : m->ops)
-      if (op.kind == EPARA_K_GEMM && op.gemm.ksplit > 1 && op.gemm.stream == 0) { op.gemm.partial = partial; op.gemm.counters = counters; }
-  }
   return EPARA_OK;
 }
 
@@ -650,7 +635,6 @@ size_t epara_model_workspace_bytes(const epara_config* cfg, const epara_model_de
   m.max_batch = effective_max_batch(*cfg, *d);
   Builder bl{nullptr, 0, false, device_sm_count(cfg->device), cfg->gemm_impl};
   build_model(bl, &m, *cfg);
-  finish_model(bl, &m);
   return bl.need + 256;
 }
 
@@ -728,7 +712,6 @@ int epara_register_model(epara_ctx* c, const epara_model_desc* d, int* model_id)
   const size_t mark = c->ws_used;
   Builder bl{c, 0, false, c->sm_count, c->cfg.gemm_impl};
   int r = build_model(bl, m, c->cfg);
-  if (r == EPARA_OK) r = finish_model(bl, m);
   if (r != EPARA_OK) {
     c->ws_used = mark;
     delete m;
@@ -945,7 +928,6 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
   static const int sweep[] = {EPARA_K_GATHER, EPARA_K_TRACE, EPARA_K_ASSEMBLE, EPARA_K_NORM, EPARA_K_GEMM, EPARA_K_ROPE,
                               EPARA_K_ATTN_DEC, EPARA_K_ATTN_PREFILL, EPARA_K_ATTN_ENC, EPARA_K_OUTPUT};
   std::vector<Launch> launches;
-  const bool simt = c->cfg.gemm_impl == EPARA_GEMM_SIMT;
   bool more = true;
   while (more && !overflow) {
     more = false;
@@ -967,14 +949,23 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
         }
         continue;
       }
-      // GEMM groups go out in up to three launches: tensor-core tiles (pass 0), the weight-streaming
-      // kernel for groups that never exceed 16 rows (pass 1) and 256-row tiles on CTA pairs for the dense
-      // bf16-output groups (pass 2); encoder attention in two: the tcgen05 kernel (pass 0) and the
+      // GEMM groups go out in one launch per kernel that has a group: CUDA cores (pass 0, comparator
+      // contexts only), the weight-streaming kernel for groups that never exceed 16 rows (pass 1) and
+      // 256-row tiles on CTA pairs (pass 2); encoder attention in two: the tcgen05 kernel (pass 0) and the
       // mma.sync kernel for shapes it does not take (pass 1)
-      // (passes 3 to 6: the swapped-operand kernel with 1, 2, 4 and 8 k ranges per tile)
-      // (pass 7: encoder MLP blocks in the fused kernel)
-      const int n_pass = kind == EPARA_K_GEMM ? 8 : (kind == EPARA_K_ATTN_ENC ? 2 : 1);
+      // (passes 3 to 10: the swapped-operand kernel with 1 to 8 k ranges per tile)
+      // (pass 11: encoder MLP blocks in the fused kernel)
+      const int n_pass = kind == EPARA_K_GEMM ? PASS_MLP + 1 : (kind == EPARA_K_ATTN_ENC ? 2 : 1);
+      unsigned passes = ~0u;                                   // GEMM passes that some model needs
+      if (kind == EPARA_K_GEMM) {
+        passes = 1u << (n_pass - 1);                           // (the last pass also moves the cursors on)
+        for (Active* a : who) {
+          const GemmGroup& g = a->m->ops[a->cursor].gemm;
+          passes |= 1u << (g.stream == 3 ? 2 + g.ksplit : g.stream == 4 ? PASS_MLP : g.stream);
+        }
+      }
       for (int pass = 0; pass < n_pass; ++pass) {
+      if (!((passes >> pass) & 1u)) continue;
       Launch L;
       memset(&L, 0, sizeof(L));
       L.kind = kind;
@@ -1072,12 +1063,9 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
             break;
           }
           case EPARA_K_GEMM: {
-            GemmGroup g = op.gemm;
-            int gpass = g.stream;
-            if (g.stream == 3) gpass = 3 + (g.ksplit >= 8 ? 3 : g.ksplit >= 4 ? 2 : g.ksplit >= 2 ? 1 : 0);
-            if (g.stream == 4) gpass = 7;
+            const int gpass = op.gemm.stream == 3 ? 2 + op.gemm.ksplit : op.gemm.stream == 4 ? PASS_MLP : op.gemm.stream;
             if (gpass != pass) break;                          // another pass takes it
-            if (g.stream == 4) {
+            if (op.gemm.stream == 4) {
               MlpGroup mg = op.mlp;
               mg.M = rows;
               mg.tiles_m = (rows + 2 * TC_BM - 1) / (2 * TC_BM);
@@ -1090,11 +1078,13 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
               if (put(&mg, sizeof(mg), 64) == (size_t)-1) overflow = true;
               break;
             }
+            GemmGroup g = op.gemm;
             g.M = rows;
             if (g.stream == 3) {
-              g.tiles_m = 1; g.tiles_n = gemm_swap_tiles(g.N);
+              g.tiles_m = (rows + g.bn - 1) / g.bn; g.tiles_n = gemm_swap_tiles_n(g.N);
               g.tile_start = total;
-              total += g.tiles_n;
+              total += g.tiles_m * g.tiles_n;
+              L.p3 = std::max(L.p3, g.bn);
             } else if (g.stream == 2) {
               g.tiles_m = (rows + 2 * TC_BM - 1) / (2 * TC_BM); g.tiles_n = (g.N + g.bn - 1) / g.bn;
               g.tile_start = total;
@@ -1105,11 +1095,9 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
               total += g.tiles_n;
               mx = std::max(mx, rows);
             } else {
-              const int tm = simt ? SIMT_TILE : TC_BM, tn = simt ? SIMT_TILE : g.bn;
-              g.tiles_m = (rows + tm - 1) / tm; g.tiles_n = (g.N + tn - 1) / tn;
+              g.tiles_m = (rows + SIMT_TILE - 1) / SIMT_TILE; g.tiles_n = (g.N + SIMT_TILE - 1) / SIMT_TILE;
               g.tile_start = total;
-              total += g.tiles_m * g.tiles_n * (simt ? 1 : g.ksplit);
-              L.p3 = std::max(L.p3, g.bn);
+              total += g.tiles_m * g.tiles_n;
             }
             ++n_put;
             inf.gemm_groups++;
@@ -1196,12 +1184,11 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       case EPARA_K_ASSEMBLE: launch_assemble((const AssembleGroup*)gp, L.n_groups, L.p1, st); break;
       case EPARA_K_NORM: launch_norm((const NormGroup*)gp, L.n_groups, L.p1, st); break;
       case EPARA_K_GEMM:
-        if (L.p2 == 7) err = launch_gemm_mlp_pair((const MlpGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st);
-        else if (L.p2 >= 3) err = launch_gemm_swap((const GemmGroup*)gp, L.n_groups, L.p0, 1 << (L.p2 - 3), dev_status, c->sm_count, st);
+        if (L.p2 == PASS_MLP) err = launch_gemm_mlp_pair((const MlpGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st);
+        else if (L.p2 >= 3) err = launch_gemm_swap((const GemmGroup*)gp, L.n_groups, L.p0, L.p2 - 2, L.p3, dev_status, c->sm_count, st);
         else if (L.p2 == 1) err = launch_gemm_stream((const GemmGroup*)gp, L.n_groups, L.p0, L.p1, st);
         else if (L.p2 == 2) err = launch_gemm_tc_pair((const GemmGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st);
-        else if (simt) launch_gemm_simt((const GemmGroup*)gp, L.n_groups, L.p0, st);
-        else err = launch_gemm_tc((const GemmGroup*)gp, L.n_groups, L.p0, L.p3, dev_status, c->sm_count, st);
+        else launch_gemm_simt((const GemmGroup*)gp, L.n_groups, L.p0, st);
         break;
       case EPARA_K_ROPE: launch_rope_append((const RopeGroup*)gp, L.n_groups, L.p1, st); break;
       case EPARA_K_ATTN_DEC:
@@ -1301,18 +1288,8 @@ int epara_step_profile(epara_ctx* c, float* ms_per_kind, int* launches_per_kind)
 size_t epara_gemm_scratch_bytes(int n) { return (size_t)(n > 0 ? n : 0) * sizeof(GemmGroup) + 256; }
 
 size_t epara_gemm_scratch_bytes_for(int device, const epara_gemm_problem* p, int n) {
-  const int sm_count = device_sm_count(device);
-  size_t bytes = epara_gemm_scratch_bytes(n);
-  for (int i = 0; i < n && p; ++i) {
-    int bn = 128, ks = 1;
-    gemm_tc_config(p[i].M, p[i].N, p[i].K, p[i].epilogue, sm_count, &bn, &ks);
-    if (ks > 1) {
-      const size_t tiles_m = (size_t)(p[i].M + TC_BM - 1) / TC_BM, tiles_n = (size_t)(p[i].N + bn - 1) / bn;
-      bytes = align_up(bytes, 256) + (size_t)ks * tiles_m * TC_BM * tiles_n * bn * 4;
-      bytes = align_up(bytes, 256) + tiles_m * tiles_n * sizeof(int);
-    }
-  }
-  return bytes;
+  (void)device; (void)p;                       // no kernel keeps partial sums in global memory
+  return epara_gemm_scratch_bytes(n);
 }
 
 int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm_problem* p, int n, void* scratch,
@@ -1325,11 +1302,10 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
   cudaStream_t st = (cudaStream_t)cuda_stream;
   const bool simt = impl == EPARA_GEMM_SIMT;
   const int sm_count = device_sm_count(device);
-  std::vector<GemmGroup> gs, gs_stream, gs_pair;   // tensor-core (or CUDA-core) groups; weight-streaming groups (M <= 16); CTA-pair groups
-  std::vector<GemmGroup> gs_swap[4];               // swapped-operand groups (17 to 128 rows) by k ranges per tile: 1, 2, 4, 8
-  int total_swap[4] = {0, 0, 0, 0};
+  std::vector<GemmGroup> gs, gs_stream, gs_pair;   // CUDA-core groups; weight-streaming groups (M <= 16); CTA-pair groups
+  std::vector<GemmGroup> gs_swap[8];               // swapped-operand groups by k ranges per tile (1 to 8)
+  int total_swap[8] = {0}, nb_swap[8] = {0};
   int total = 0, total_stream = 0, max_rows_stream = 0, total_pair = 0;
-  size_t soff = epara_gemm_scratch_bytes(n);
   for (int i = 0; i < n; ++i) {
     const epara_gemm_problem& q = p[i];
     if (!q.A || !q.W || !q.C || q.M < 0 || q.N <= 0 || q.K <= 0) return EPARA_E_INVALID;
@@ -1354,22 +1330,23 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
       gs_stream.push_back(g);
       continue;
     }
-    if (!simt && q.M <= GEMM_SWAP_MAX_ROWS && q.K % 8 == 0) {
+    if (!simt && q.M == 0) continue;
+    if (!simt && gemm_swap_eligible(q.M, q.N, q.K, q.epilogue, sm_count)) {
       g.stream = 3;
-      g.bn = round_up(q.M, 16);
-      g.ksplit = gemm_swap_ksplit(q.N, q.K, sm_count);
-      const int si = g.ksplit >= 8 ? 3 : g.ksplit >= 4 ? 2 : g.ksplit >= 2 ? 1 : 0;
-      g.tiles_m = 1; g.tiles_n = gemm_swap_tiles(q.N);
+      gemm_swap_config(q.M, q.N, q.K, sm_count, &g.bn, &g.ksplit);
+      const int si = g.ksplit - 1;
+      g.tiles_m = (q.M + g.bn - 1) / g.bn; g.tiles_n = gemm_swap_tiles_n(q.N);
       g.tile_start = total_swap[si];
-      total_swap[si] += g.tiles_n;
+      total_swap[si] += g.tiles_m * g.tiles_n;
+      nb_swap[si] = std::max(nb_swap[si], g.bn);
       if (!make_tmap(&g.tmA, q.A, q.M, q.K, q.lda, g.bn)) return EPARA_E_CUDA;
       if (!make_tmap(&g.tmW, q.W, q.N, q.K, q.ldw, TC_BM)) return EPARA_E_CUDA;
       gs_swap[si].push_back(g);
       continue;
     }
-    if (!simt) gemm_tc_config(q.M, q.N, q.K, q.epilogue, sm_count, &g.bn, &g.ksplit);
-    if (!simt && gemm_tc_pair_eligible(q.M, q.N, q.K, q.epilogue, g.bn, g.ksplit)) {
+    if (!simt) {
       g.stream = 2;
+      gemm_pair_config(q.M, q.N, q.K, q.epilogue, sm_count, &g.bn);
       g.tiles_m = (q.M + 2 * TC_BM - 1) / (2 * TC_BM); g.tiles_n = (q.N + g.bn - 1) / g.bn;
       g.tile_start = total_pair;
       total_pair += g.tiles_m * g.tiles_n;
@@ -1379,34 +1356,19 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
       gs_pair.push_back(g);
       continue;
     }
-    const int tm = simt ? SIMT_TILE : TC_BM, tn = simt ? SIMT_TILE : g.bn;
-    g.tiles_m = (q.M + tm - 1) / tm; g.tiles_n = (q.N + tn - 1) / tn;
+    g.tiles_m = (q.M + SIMT_TILE - 1) / SIMT_TILE; g.tiles_n = (q.N + SIMT_TILE - 1) / SIMT_TILE;
     g.tile_start = total;
-    total += g.tiles_m * g.tiles_n * g.ksplit;
-    if (!simt && q.M > 0) {
-      if (!make_tmap(&g.tmA, q.A, q.M, q.K, q.lda, TC_BM)) return EPARA_E_CUDA;
-      if (!make_tmap(&g.tmW, q.W, q.N, q.K, q.ldw, g.bn)) return EPARA_E_CUDA;
-      if (!make_tmap_c(&g.tmC, q.C, q.M, q.N, q.ldc, q.epilogue)) return EPARA_E_CUDA;
-    }
-    if (g.ksplit > 1) {
-      soff = align_up(soff, 256);
-      g.partial = (float*)((unsigned char*)scratch + soff);
-      soff += (size_t)g.ksplit * g.tiles_m * TC_BM * g.tiles_n * g.bn * 4;
-      soff = align_up(soff, 256);
-      g.counters = (int*)((unsigned char*)scratch + soff);
-      if (cudaMemsetAsync(g.counters, 0, (size_t)g.tiles_m * g.tiles_n * sizeof(int), st) != cudaSuccess) return EPARA_E_CUDA;
-      soff += (size_t)g.tiles_m * g.tiles_n * sizeof(int);
-    }
+    total += g.tiles_m * g.tiles_n;
     gs.push_back(g);
   }
   int* status = (int*)scratch;
   GemmGroup* dev_groups = (GemmGroup*)((unsigned char*)scratch + 256);
   GemmGroup* dev_stream = dev_groups + gs.size();
   GemmGroup* dev_pair = dev_stream + gs_stream.size();
-  GemmGroup* dev_swap[4];
+  GemmGroup* dev_swap[8];
   dev_swap[0] = dev_pair + gs_pair.size();
-  for (int i = 1; i < 4; ++i) dev_swap[i] = dev_swap[i - 1] + gs_swap[i - 1].size();
-  for (int i = 0; i < 4; ++i)
+  for (int i = 1; i < 8; ++i) dev_swap[i] = dev_swap[i - 1] + gs_swap[i - 1].size();
+  for (int i = 0; i < 8; ++i)
     if (!gs_swap[i].empty() &&
         cudaMemcpyAsync(dev_swap[i], gs_swap[i].data(), gs_swap[i].size() * sizeof(GemmGroup), cudaMemcpyHostToDevice, st) != cudaSuccess)
       return EPARA_E_CUDA;
@@ -1427,15 +1389,11 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
     err = cudaGetLastError();
   } else {
     const int sm = sm_count;
-    int max_bn = 0;
-    for (const GemmGroup& g : gs) max_bn = std::max(max_bn, g.bn);
-    err = launch_gemm_tc(dev_groups, (int)gs.size(), total, max_bn, status, sm, st);
-    if (err == cudaSuccess)
-      err = launch_gemm_stream(dev_stream, (int)gs_stream.size(), total_stream, max_rows_stream, st);
+    err = launch_gemm_stream(dev_stream, (int)gs_stream.size(), total_stream, max_rows_stream, st);
     if (err == cudaSuccess)
       err = launch_gemm_tc_pair(dev_pair, (int)gs_pair.size(), total_pair, status, sm, st);
-    for (int i = 0; i < 4 && err == cudaSuccess; ++i)
-      err = launch_gemm_swap(dev_swap[i], (int)gs_swap[i].size(), total_swap[i], 1 << i, status, sm, st);
+    for (int i = 0; i < 8 && err == cudaSuccess; ++i)
+      err = launch_gemm_swap(dev_swap[i], (int)gs_swap[i].size(), total_swap[i], i + 1, nb_swap[i], status, sm, st);
   }
   return err == cudaSuccess ? EPARA_OK : EPARA_E_CUDA;
 }

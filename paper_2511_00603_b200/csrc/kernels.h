@@ -17,31 +17,30 @@ void launch_output(const OutputGroup* groups, int n_groups, int max_B, cudaStrea
 constexpr int SIMT_TILE = 64;
 void launch_gemm_simt(const GemmGroup* groups, int n_groups, int total_tiles, cudaStream_t st);
 
-// tcgen05 grouped GEMM, 128 x bn tiles (bn = 128 or 256 per group), persistent.  `status` is a
-// device int the kernel sets non-zero if a bounded wait ran out.  total_items = sum over groups of
-// tiles_m * tiles_n * ksplit.  Returns the cudaError of the launch configuration.
+// tcgen05 grouped GEMM of groups with more than 128 rows (GemmGroup::stream == 2): 256 x bn tiles on CTA pairs,
+// persistent.  `status` is a device int the kernel sets non-zero if a bounded wait ran out.  total_items = sum over
+// groups of tiles_m * tiles_n (tiles_m counts 256-row tiles).  gemm_pair_config() picks bn (128, 192 or 256).
 constexpr int TC_BM = 128;
 constexpr int TC_BN_MAX = 256;
 constexpr int TC_BK = 64;
-void gemm_tc_config(long long rows_cap, int N, int K, int epi, int sm_count, int* bn, int* ksplit);
-bool gemm_tc_pair_eligible(long long rows_cap, int N, int K, int epi, int bn, int ksplit);
+double gemm_pair_config(long long rows_cap, int N, int K, int epi, int sm_count, int* bn);
+cudaError_t launch_gemm_tc_pair(const GemmGroup* groups, int n_groups, int total_items, int* status, int sm_count,
+                                cudaStream_t st);
 bool gemm_mlp_eligible(long long rows_cap, int d, int F);
 cudaError_t launch_gemm_mlp_pair(const MlpGroup* groups, int n_groups, int total_items, int* status, int sm_count,
                                  cudaStream_t st);
-cudaError_t launch_gemm_tc_pair(const GemmGroup* groups, int n_groups, int total_items, int* status, int sm_count,
-                                cudaStream_t st);
-cudaError_t launch_gemm_tc(const GemmGroup* groups, int n_groups, int total_items, int max_bn, int* status,
-                           int sm_count, cudaStream_t st);   // max_bn: widest tile among the groups
 
-// Swapped-operand tensor-core GEMM for groups of 17 to 128 rows (GemmGroup::stream == 3): a cluster of `ksplit`
-// CTAs per tile of 128 output columns; all groups of a launch share ksplit.  GemmGroup::bn holds the row capacity
-// rounded up to 16, tmW the weight map (box 128 rows), tmA the activation map (box bn rows); tile_start counts
-// tiles.  total_items = sum of gemm_swap_tiles(N).
-int gemm_swap_ksplit(int N, int K, int sm_count);
-int gemm_swap_tiles(int N);
-cudaError_t launch_gemm_swap(const GemmGroup* groups, int n_groups, int total_items, int ksplit, int* status, int sm_count,
-                             cudaStream_t st);
-constexpr int GEMM_SWAP_MAX_ROWS = 128;
+// Swapped-operand tensor-core GEMM (GemmGroup::stream == 3): a cluster of `ksplit` CTAs per tile of 128 output
+// columns and bn batch rows; all groups of a launch share ksplit.  gemm_swap_config() picks bn (a multiple of 16, at
+// most GEMM_SWAP_TILE_ROWS) and ksplit from the row capacity; tmW is the weight map (box 128 rows), tmA the activation
+// map (box bn rows); tiles_m = ceil(M / bn), tiles_n = gemm_swap_tiles_n(N), tile_start counts tiles_m * tiles_n.
+// max_nb: widest bn of the launch.
+constexpr int GEMM_SWAP_TILE_ROWS = 256;
+double gemm_swap_config(long long rows_cap, int N, int K, int sm_count, int* nb, int* ksplit);
+bool gemm_swap_eligible(long long rows_cap, int N, int K, int epi, int sm_count);
+int gemm_swap_tiles_n(int N);
+cudaError_t launch_gemm_swap(const GemmGroup* groups, int n_groups, int total_items, int ksplit, int max_nb, int* status,
+                             int sm_count, cudaStream_t st);
 
 // Weight-streaming GEMM for groups that never exceed 16 rows (GemmGroup::stream): one block per 16
 // rows of W over the whole K, mma.sync, no tensor maps.  total_items = sum of gemm_stream_tiles(N).

@@ -233,3 +233,17 @@ def test_gelu_epilogue_sweep_through_identity_gemm(E, rows):
     bad = np.abs(got - ref) > bound
     assert not bad.any(), f"{int(bad.sum())} of {bad.size} outside the bound; worst excess " \
                           f"{float(np.max(np.abs(got - ref) - bound)):.3e} at x = {float(xs[np.unravel_index(np.argmax(np.abs(got - ref) - bound), xs.shape)])}"
+
+
+@pytest.mark.parametrize("rows", [129, 197, 256, 257, 509, 1024])
+def test_grouped_gemm_between_one_tile_and_a_full_chip(E, rows):
+    """Problems of 129 to about a thousand rows: a long K with few output tiles runs with swapped operands in one or
+    more row tiles of up to 256 rows and K split over 2, 4 or 8 CTAs (every owner's share of the rows ragged), the
+    others as tile pairs 128, 192 or 256 wide.  N below and not a multiple of a tile, K not a multiple of a k-block."""
+    cases = [(rows, 768, 3072, ("bias", "resid")), (rows, 2048, 8192, ("resid",)), (rows, 136, 4096, ("bias", "gelu")),
+             (rows, 264, 2056, ("swiglu",)), (rows, 1000, 1544, ("bias",)), (rows, 3072, 512, ()), (rows, 4096, 1024, ("swiglu",))]
+    probs, refs = _run_gemm(E, E.GEMM_TCGEN05, cases, seed=rows)
+    for p, ref, case in zip(probs, refs, cases):
+        assert_close(p["C"][:ref.shape[0], :ref.shape[1]], ref, what=f"gemm {case}")
+    alone, _ = _run_gemm(E, E.GEMM_TCGEN05, cases[:2], seed=rows)
+    assert torch.equal(alone[1]["C"], probs[1]["C"])
