@@ -84,16 +84,4 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
-// Block-wide sum for blocks of up to 1024 threads; `red` is 32 floats of shared memory.
-__device__ __forceinline__ float block_sum(float v, float* red) {
-  v = warp_sum(v);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  float t = (l < nw) ? red[l] : 0.f;
-  t = warp_sum(t);
-  return t;
-}
-
 }  // namespace epara

@@ -56,29 +56,48 @@ void launch_gather(const GatherGroup* groups, int n_groups, int max_blocks, cuda
 }
 
 // ------------------------------------------------------------------ norms
-// Rows are held in registers between the statistics pass and the write.  Narrow rows
-// (d <= 1024) take one warp per row, 8 rows per block; wider rows one block per row.
+// Rows are held in registers between the statistics pass and the write.  A row of d > 512 is taken by W warps (one per
+// 1024 columns, so that a lane holds at most eight float4), 8 / W rows per block; the warps of a row meet at a named
+// barrier.  HBM-bound: what counts is the bytes in flight, 128 KB per SM here.  (One block per row had 32 KB in flight
+// and a block-wide barrier per sum: 8192 rows of 2048 columns took 44 us between events; now 23 us.)
 constexpr int NORM_THREADS = 256;
+constexpr int NORM_WARPS = NORM_THREADS / 32;
 constexpr int NORM_WARP_D = 1024;
 
-template <bool WARP>
-__device__ __forceinline__ void norm_row(const NormGroup& g, int row, float* red) {
-  constexpr int STRIDE = WARP ? 32 : NORM_THREADS;
-  const int t = WARP ? (threadIdx.x & 31) : threadIdx.x;
+// Sum over the W warps of a row; `red` has one slot per warp and sum.
+template <int W>
+__device__ __forceinline__ float norm_row_sum(float v, float* red) {
+  v = warp_sum(v);
+  if (W == 1) return v;
+  const int warp = threadIdx.x >> 5, first = warp / W * W;
+  if ((threadIdx.x & 31) == 0) red[warp] = v;
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + warp / W), "n"(32 * W) : "memory");
+  float t = red[first];
+#pragma unroll
+  for (int w = 1; w < W; ++w) t += red[first + w];
+  return t;
+}
+
+template <int W>
+__device__ __forceinline__ void norm_row(const NormGroup& g, int block, float* red) {
+  const int warp = threadIdx.x >> 5;
+  const int row = block * (NORM_WARPS / W) + warp / W;
+  if (row >= g.M) return;                        // all warps of the row leave together
+  const int t = (warp % W) * 32 + (threadIdx.x & 31);
   const int nvec = g.d >> 2;
   const float4* x = reinterpret_cast<const float4*>(g.x + (size_t)(g.row_index ? g.row_index[row] : row) * g.x_stride);
   float4 v[8];
-  float s = 0.f;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const int c = t + i * STRIDE;
-    if (c < nvec) {
-      v[i] = x[c];
-      s += (g.kind == NORM_LN) ? (v[i].x + v[i].y) + (v[i].z + v[i].w)
-                               : (v[i].x * v[i].x + v[i].y * v[i].y) + (v[i].z * v[i].z + v[i].w * v[i].w);
-    }
+    const int c = t + i * 32 * W;
+    v[i] = c < nvec ? x[c] : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  s = WARP ? warp_sum(s) : block_sum(s, red);
+  float s = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    s += (g.kind == NORM_LN) ? (v[i].x + v[i].y) + (v[i].z + v[i].w)
+                             : (v[i].x * v[i].x + v[i].y * v[i].y) + (v[i].z * v[i].z + v[i].w * v[i].w);
+  s = norm_row_sum<W>(s, red);
   float mean = 0.f, rstd;
   const float inv_d = 1.0f / (float)g.d;
   if (g.kind == NORM_LN) {
@@ -86,13 +105,12 @@ __device__ __forceinline__ void norm_row(const NormGroup& g, int row, float* red
     float q = 0.f;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int c = t + i * STRIDE;
-      if (c < nvec) {
+      if (t + i * 32 * W < nvec) {
         const float a = v[i].x - mean, b = v[i].y - mean, cc = v[i].z - mean, dd = v[i].w - mean;
         q += (a * a + b * b) + (cc * cc + dd * dd);
       }
     }
-    q = WARP ? warp_sum(q) : block_sum(q, red);
+    q = norm_row_sum<W>(q, red + NORM_WARPS);
     rstd = 1.0f / sqrtf(q * inv_d + g.eps);
   } else {
     rstd = 1.0f / sqrtf(s * inv_d + g.eps);
@@ -102,7 +120,7 @@ __device__ __forceinline__ void norm_row(const NormGroup& g, int row, float* red
   const uint2* bt = reinterpret_cast<const uint2*>(g.beta);
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const int c = t + i * STRIDE;
+    const int c = t + i * 32 * W;
     if (c < nvec) {
       const uint2 gg = __ldg(gm + c);
       float ga[4] = {__uint_as_float(gg.x << 16), __uint_as_float(gg.x & 0xffff0000u),
@@ -191,35 +209,31 @@ __device__ __forceinline__ void norm_rows_narrow(const NormGroup& g, int row0) {
   }
 }
 
-// Blocks a group of M rows of width d needs (device copy of norm_blocks).
-__device__ __forceinline__ int norm_blocks_dev(int M, int d) {
-  constexpr int wpb = NORM_THREADS / 32;
-  if (d <= NORM_NARROW_D) return (M + wpb * NORM_NARROW_ROWS - 1) / (wpb * NORM_NARROW_ROWS);
-  return d <= NORM_WARP_D ? (M + wpb - 1) / wpb : M;
+// Rows of width d per block, and the blocks a group of M rows needs.
+__host__ __device__ inline int norm_rows_per_block(int d) {
+  return d <= NORM_NARROW_D ? NORM_WARPS * NORM_NARROW_ROWS : d <= NORM_WARP_D ? NORM_WARPS : d <= 2 * NORM_WARP_D ? NORM_WARPS / 2
+       : d <= 4 * NORM_WARP_D ? NORM_WARPS / 4 : NORM_WARPS / 8;
 }
+int norm_blocks(int M, int d) { return (M + norm_rows_per_block(d) - 1) / norm_rows_per_block(d); }
 
 __global__ void __launch_bounds__(NORM_THREADS, 4) norm_kernel(const NormGroup* __restrict__ groups) {
-  __shared__ float red[32];
+  __shared__ float red[2 * NORM_WARPS];
   const NormGroup g = groups[blockIdx.y];
-  if ((int)blockIdx.x >= norm_blocks_dev(g.M, g.d)) return;   // beyond this group's rows: nothing to wait for
+  if ((int)blockIdx.x * norm_rows_per_block(g.d) >= g.M) return;   // beyond this group's rows: nothing to wait for
   pdl_launch_dependents();
   pdl_wait();
   if (g.d <= NORM_NARROW_D) {
-    const int row0 = (blockIdx.x * (NORM_THREADS / 32) + (threadIdx.x >> 5)) * NORM_NARROW_ROWS;
+    const int row0 = (blockIdx.x * NORM_WARPS + (threadIdx.x >> 5)) * NORM_NARROW_ROWS;
     if (row0 < g.M) norm_rows_narrow(g, row0);
   } else if (g.d <= NORM_WARP_D) {
-    const int row = blockIdx.x * (NORM_THREADS / 32) + (threadIdx.x >> 5);
-    if (row < g.M) norm_row<true>(g, row, red);
+    norm_row<1>(g, blockIdx.x, red);
+  } else if (g.d <= 2 * NORM_WARP_D) {
+    norm_row<2>(g, blockIdx.x, red);
+  } else if (g.d <= 4 * NORM_WARP_D) {
+    norm_row<4>(g, blockIdx.x, red);
   } else {
-    norm_row<false>(g, blockIdx.x, red);
+    norm_row<8>(g, blockIdx.x, red);
   }
-}
-
-// Blocks a group of M rows of width d needs.
-int norm_blocks(int M, int d) {
-  const int wpb = NORM_THREADS / 32;
-  if (d <= NORM_NARROW_D) return (M + wpb * NORM_NARROW_ROWS - 1) / (wpb * NORM_NARROW_ROWS);
-  return d <= NORM_WARP_D ? (M + wpb - 1) / wpb : M;
 }
 
 void launch_norm(const NormGroup* groups, int n_groups, int max_blocks, cudaStream_t st) {
@@ -233,49 +247,61 @@ void launch_norm(const NormGroup* groups, int n_groups, int max_blocks, cudaStre
 // (interleaved pairs; cos and sin come from the model's table, computed from fp64 angles when the
 // model was placed), q in place, k and v written to the cache page table[pos/16], slot pos%16.
 // The page id comes from the caller's block table and is checked against the pool's page count.
-__global__ void __launch_bounds__(256) rope_append_kernel(const RopeGroup* __restrict__ groups) {
+// A thread takes eight consecutive elements (four pairs) at a time and has ROPE_U of them in flight before it looks at
+// the page; their columns are a multiple of hd apart, so it needs one piece of the (cos, sin) row for all of them.
+// (One pair per thread and access: 8192 rows of 3072 columns took 55 us between events; now 24 us.)
+constexpr int ROPE_THREADS = 128;
+constexpr int ROPE_U = 3;
+__global__ void __launch_bounds__(ROPE_THREADS) rope_append_kernel(const RopeGroup* __restrict__ groups) {
   const RopeGroup g = groups[blockIdx.y];
   const int b = blockIdx.x;               // token row
   if (b >= g.B) return;
   pdl_launch_dependents();
-  pdl_wait();
   const RowDesc rd = g.rows[b];
   const int pos = rd.pos, hd = g.hd, half = hd >> 1;
-  const float2* cs = g.cs + (size_t)pos * half;
   const int page = g.reqs[rd.req].table[pos / 16], slot = pos % 16;
-  // a page id outside the pool is reported and nothing is written for this row (q stays unrotated)
-  if (page < 0 || page >= g.kv_pages) {
-    if (threadIdx.x == 0) atomicExch(g.status, ERR_PAGE_APPEND);
-    return;
-  }
+  const int e = (threadIdx.x * 8) % hd;   // ROPE_THREADS * 8 is a multiple of every head size
+  const float4* cs = reinterpret_cast<const float4*>(g.cs + (size_t)pos * half + (e >> 1));
+  const float4 t0 = __ldg(cs), t1 = __ldg(cs + 1);
+  const bool page_ok = page >= 0 && page < g.kv_pages;
+  pdl_wait();
   bf16* row = g.qkv + (size_t)b * (g.Hq + 2 * g.Hkv) * hd;
-  const int n_rot = (g.Hq + g.Hkv) * half;
-  for (int e = threadIdx.x; e < n_rot; e += blockDim.x) {
-    const int h = e / half, j = e % half;
-    const float2 t = __ldg(cs + j);
-    __nv_bfloat162* p2 = reinterpret_cast<__nv_bfloat162*>(row + (size_t)h * hd) + j;
-    const float2 v = __bfloat1622float2(*p2);
-    const float x0 = v.x * t.x - v.y * t.y, x1 = v.x * t.y + v.y * t.x;
-    const __nv_bfloat162 o = __floats2bfloat162_rn(x0, x1);
-    if (h < g.Hq) {
-      *p2 = o;
-    } else {
-      const int kh = h - g.Hq;
-      bf16* dst = g.kv_layer + (((size_t)page * 2 + 0) * g.Hkv + kh) * 16 * hd + (size_t)slot * hd;
-      reinterpret_cast<__nv_bfloat162*>(dst)[j] = o;
+  const int nvec = (g.Hq + 2 * g.Hkv) * hd >> 3;
+  for (int i0 = threadIdx.x; i0 < nvec; i0 += ROPE_THREADS * ROPE_U) {
+    uint4 u[ROPE_U];
+#pragma unroll
+    for (int k = 0; k < ROPE_U; ++k)
+      if (i0 + k * ROPE_THREADS < nvec) u[k] = *reinterpret_cast<const uint4*>(row + (i0 + k * ROPE_THREADS) * 8);
+    // a page id outside the pool is reported and nothing is written for this row (q stays unrotated)
+    if (!page_ok) {
+      if (threadIdx.x == 0) atomicExch(g.status, ERR_PAGE_APPEND);
+      return;
     }
-  }
-  const bf16* vsrc = row + (size_t)(g.Hq + g.Hkv) * hd;
-  for (int e = threadIdx.x; e < g.Hkv * half; e += blockDim.x) {
-    const int kh = e / half, j = e % half;
-    bf16* dst = g.kv_layer + (((size_t)page * 2 + 1) * g.Hkv + kh) * 16 * hd + (size_t)slot * hd;
-    reinterpret_cast<__nv_bfloat162*>(dst)[j] = reinterpret_cast<const __nv_bfloat162*>(vsrc + (size_t)kh * hd)[j];
+#pragma unroll
+    for (int k = 0; k < ROPE_U; ++k) {
+      const int c = (i0 + k * ROPE_THREADS) * 8, h = c / hd;
+      if (c >= nvec * 8) break;
+      if (h < g.Hq + g.Hkv) {
+        float f[8];
+        unpack8(u[k], f);
+        u[k].x = pack2(f[0] * t0.x - f[1] * t0.y, f[0] * t0.y + f[1] * t0.x);
+        u[k].y = pack2(f[2] * t0.z - f[3] * t0.w, f[2] * t0.w + f[3] * t0.z);
+        u[k].z = pack2(f[4] * t1.x - f[5] * t1.y, f[4] * t1.y + f[5] * t1.x);
+        u[k].w = pack2(f[6] * t1.z - f[7] * t1.w, f[6] * t1.w + f[7] * t1.z);
+      }
+      if (h < g.Hq) {
+        *reinterpret_cast<uint4*>(row + c) = u[k];
+      } else {
+        const int kh = h - g.Hq, v = kh >= g.Hkv;         // K heads, then V heads
+        *reinterpret_cast<uint4*>(g.kv_layer + (((size_t)page * 2 + v) * g.Hkv + (kh - v * g.Hkv)) * 16 * hd + (size_t)slot * hd + e) = u[k];
+      }
+    }
   }
 }
 
 void launch_rope_append(const RopeGroup* groups, int n_groups, int max_B, cudaStream_t st) {
   if (n_groups == 0 || max_B == 0) return;
-  launch_pdl(rope_append_kernel, dim3(max_B, n_groups), dim3(256), 0, st, groups);
+  launch_pdl(rope_append_kernel, dim3(max_B, n_groups), dim3(ROPE_THREADS), 0, st, groups);
 }
 
 // ------------------------------------------------------------------ ViT token assembly
