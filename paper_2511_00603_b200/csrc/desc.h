@@ -109,25 +109,26 @@ struct AttnReq {
   int row;               // activation row of the request's token (q is read and the output written there)
 };
 
-// Causal attention of prompt chunks (one layer): request i has n_tok query tokens in rows row_start ..,
-// token t at position kv_len + t attends to positions 0 .. kv_len + t of its paged cache (the chunk's own
-// k, v were appended by the kernel before).  One block per (request, query head, tile of 64 tokens).
-struct PrefillReq {
+// Causal attention of prompt chunks (one layer): a request has n_tok query tokens in consecutive rows, token t at position
+// kv_len + t attends to positions 0 .. kv_len + t of its paged cache (the chunk's own k, v were appended by the kernel
+// before).  A work item is 128 of its tokens and one or two query heads of one kv head; the list is sorted by the keys
+// an item walks, longest first.
+struct PrefillItem {
   const int32_t* table;
-  int row_start, n_tok, kv_len;
-  int blk_start;         // first block of this request within its group
+  int row, live;         // first activation row, tokens of the tile
+  int pos;               // position of the tile's first token
+  int head;              // first query head
+  int pad[2];
 };
-struct AttnPrefillGroup {
-  const bf16* qkv;       // [rows, q_stride], query head h at column h*hd
-  const bf16* kv_layer;
-  const PrefillReq* reqs;
+struct alignas(64) AttnPrefillGroup {
+  CUtensorMap tmQ;       // qkv [rows, (Hq+2Hkv)*hd] bf16, box 64 columns x 128 rows, 128-byte swizzle
+  CUtensorMap tmKV;      // one layer of the cache as [kv_pages * 2 * Hkv * 16, hd], box 64 columns x 16 rows
+  const PrefillItem* items;
   bf16* out;             // [rows, Hq*hd]
-  int* status;
   long long kv_pages;
-  int q_stride;
-  int n_reqs, Hq, Hkv, hd;
-  int blk_start;         // first block of this group in the launch
-  int n_blocks;
+  int n_items, Hq, Hkv, hd;
+  int item_start;        // first item of this group in the launch
+  int pad[5];
 };
 
 struct AttnDecGroup {
@@ -149,15 +150,14 @@ struct AttnDecGroup {
 
 struct alignas(64) AttnEncGroup {
   CUtensorMap tmQ;       // tensor-core kernel: qkv [rows, 3d] bf16, box 64 columns x 128 rows, 128-byte swizzle
-  CUtensorMap tmKV;      // same matrix, box 64 columns x KP rows
+  CUtensorMap tmKV;      // the same (K and V blocks are read with the box of Q)
   const bf16* qkv;       // [B*T, 3d]: q | k | v, head h at column h*hd within each
   bf16* out;             // [B*T, d]
   int B, T, H, hd;
   int blk_start;         // first block (item) of this group
-  int q_blocks;          // query blocks per (image, head); 1 for the tensor-core kernel
-  int tc;                // 1: runs in the tensor-core kernel (hd 64, T <= ENC_TC_MAX_T), fixed when the model is placed
-  int KP;                // T rounded up to a multiple of 16
-  int pad[8];
+  int q_blocks;          // query blocks per (image, head)
+  int tc;                // 1: runs in the tensor-core kernel, fixed when the model is placed
+  int pad[9];
 };
 
 // One transformer MLP block of an encoder as a single work unit of the fused kernel:
@@ -197,7 +197,7 @@ struct OutputGroup {     // copy logits rows to the requests' buffers and take t
 // Group arrays are packed back to back in the step blob: sizes must keep 8-byte alignment.
 namespace epara {
 static_assert(sizeof(GemmGroup) % 64 == 0, "GemmGroup holds 64-byte aligned TMA maps");
-static_assert(sizeof(AttnPrefillGroup) % 8 == 0 && sizeof(PrefillReq) % 8 == 0 && sizeof(RowDesc) == 16, "descriptor sizes");
+static_assert(sizeof(AttnPrefillGroup) % 64 == 0 && sizeof(PrefillItem) == 32 && sizeof(RowDesc) == 16, "descriptor sizes");
 static_assert(sizeof(NormGroup) % 8 == 0 && sizeof(GatherGroup) % 8 == 0 && sizeof(RopeGroup) % 8 == 0 &&
               sizeof(AttnDecGroup) % 8 == 0 && sizeof(AttnEncGroup) % 64 == 0 && sizeof(MlpGroup) % 64 == 0 && sizeof(AssembleGroup) % 8 == 0 &&
               sizeof(OutputGroup) % 8 == 0 && sizeof(ReqDesc) % 16 == 0 && sizeof(AttnReq) % 16 == 0,

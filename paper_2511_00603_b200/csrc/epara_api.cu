@@ -398,11 +398,10 @@ int build_model(Builder& bl, Model* m, const epara_config& cfg) {
       memset(&at, 0, sizeof(at));
       at.kind = EPARA_K_ATTN_ENC; at.rows_per_req = T;
       at.aenc.qkv = qkv; at.aenc.out = a; at.aenc.T = T; at.aenc.H = d.n_heads; at.aenc.hd = d.head_dim;
-      at.aenc.KP = round_up(T, 16);
-      at.aenc.tc = (d.head_dim == 64 && T <= ENC_TC_MAX_T && bl.gemm_impl != EPARA_GEMM_SIMT) ? 1 : 0;
+      at.aenc.tc = bl.gemm_impl != EPARA_GEMM_SIMT ? 1 : 0;
       if (at.aenc.tc && bl.c) {
-        if (!make_tmap(&at.aenc.tmQ, qkv, Mcap, 3 * dm, 3 * dm, 128)) return EPARA_E_CUDA;
-        if (!make_tmap(&at.aenc.tmKV, qkv, Mcap, 3 * dm, 3 * dm, at.aenc.KP)) return EPARA_E_CUDA;
+        if (!make_tmap(&at.aenc.tmQ, qkv, Mcap, 3 * dm, 3 * dm, FLASH_TILE)) return EPARA_E_CUDA;
+        at.aenc.tmKV = at.aenc.tmQ;
       }
       m->ops.push_back(at);
       if (!add_gemm(bl, m, a, dm, Mcap, w[4], dm, dm, z, dm, w[5], EPI_RESID_F32, T)) return EPARA_E_CUDA;
@@ -495,8 +494,11 @@ int build_model(Builder& bl, Model* m, const epara_config& cfg) {
     Op ap;                                   // causal attention of the step's prompt chunks (none in a pure decode step)
     memset(&ap, 0, sizeof(ap));
     ap.kind = EPARA_K_ATTN_PREFILL; ap.rows_per_req = 1;
-    ap.apre.qkv = qkv; ap.apre.q_stride = nq; ap.apre.kv_layer = kv_layer; ap.apre.out = a; ap.apre.kv_pages = d.kv_pages;
-    ap.apre.Hq = Hq; ap.apre.Hkv = Hkv; ap.apre.hd = hd;
+    ap.apre.out = a; ap.apre.kv_pages = d.kv_pages; ap.apre.Hq = Hq; ap.apre.Hkv = Hkv; ap.apre.hd = hd;
+    if (bl.c && hd >= 64) {
+      if (!make_tmap(&ap.apre.tmQ, qkv, Bcap, nq, nq, FLASH_TILE)) return EPARA_E_CUDA;
+      if (!make_tmap(&ap.apre.tmKV, kv_layer, d.kv_pages * 2 * Hkv * 16, hd, hd, 16)) return EPARA_E_CUDA;
+    }
     m->ops.push_back(ap);
     if (!add_gemm(bl, m, a, Hq * hd, Bcap, w[2], dm, Hq * hd, x, dm, nullptr, EPI_RESID_F32, 1)) return EPARA_E_CUDA;
     add_norm(m, x, dm, h, w[3], nullptr, dm, NORM_RMS, 1e-5f, 1);
@@ -793,17 +795,19 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
   // ---- admission (A0) ----
   // B requests; `rows` activation rows (one per token for a decoder, B otherwise); n_dec single-token and
   // n_pre prompt-chunk requests of a decoder, with their descriptor arrays in the blob
+  struct PrefillChunk { const int32_t* table; int row_start, n_tok, kv_len; };
   struct Active {
-    Model* m; int B; int rows; size_t req_off; size_t areq_off; size_t row_off; size_t preq_off; size_t last_off; size_t cursor;
-    int n_dec, n_pre, max_chunks_dec, pre_blocks;
+    Model* m; int B; int rows; size_t req_off; size_t areq_off; size_t row_off; size_t pitem_off; size_t last_off; size_t cursor;
+    int n_dec, n_pre, max_chunks_dec, pre_items;
+    std::vector<PrefillChunk> pre;
     std::vector<Request> reqs;
   };
   std::vector<Active> act;
   for (size_t mi = 0; mi < c->models.size(); ++mi) {
     Model* m = c->models[mi];
     Active a;
-    a.m = m; a.B = 0; a.rows = 0; a.cursor = 0; a.req_off = 0; a.areq_off = 0; a.row_off = 0; a.preq_off = 0; a.last_off = 0;
-    a.n_dec = a.n_pre = a.max_chunks_dec = a.pre_blocks = 0;
+    a.m = m; a.B = 0; a.rows = 0; a.cursor = 0; a.req_off = 0; a.areq_off = 0; a.row_off = 0; a.pitem_off = 0; a.last_off = 0;
+    a.n_dec = a.n_pre = a.max_chunks_dec = a.pre_items = 0;
     for (int cat = 0; cat < 2; ++cat) {
       std::deque<Request>& q = m->q[cat];
       if (q.empty()) continue;
@@ -874,7 +878,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
     const bool dec = a.m->d.kind == EPARA_MODEL_DECODER;
     std::vector<ReqDesc> rd(a.B);
     std::vector<AttnReq> ar;
-    std::vector<PrefillReq> pr;
+    std::vector<PrefillChunk>& pr = a.pre;
     std::vector<RowDesc> rows;
     std::vector<int> last(a.B);
     int row = 0;
@@ -898,10 +902,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
           ar.push_back(q1);
           a.max_chunks_dec = std::max(a.max_chunks_dec, (in.kv_len + 1 + ATTN_CHUNK - 1) / ATTN_CHUNK);
         } else {
-          PrefillReq p1;
-          p1.table = in.block_table; p1.row_start = row; p1.n_tok = nt; p1.kv_len = in.kv_len; p1.blk_start = a.pre_blocks;
-          a.pre_blocks += attn_prefill_blocks(nt, a.m->d.n_heads);
-          pr.push_back(p1);
+          pr.push_back({in.block_table, row, nt, in.kv_len});
           inf.prefill_tokens += nt;
         }
         // cached bytes the step must read at least once: the request's whole sequence, once per layer
@@ -917,11 +918,42 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       a.row_off = put(rows.data(), rows.size() * sizeof(RowDesc), 16);
       a.last_off = put(last.data(), last.size() * sizeof(int), 16);
       if (!ar.empty()) a.areq_off = put(ar.data(), ar.size() * sizeof(AttnReq), 16);
-      if (!pr.empty()) a.preq_off = put(pr.data(), pr.size() * sizeof(PrefillReq), 16);
     }
-    if (a.req_off == (size_t)-1 || a.areq_off == (size_t)-1 || a.row_off == (size_t)-1 || a.preq_off == (size_t)-1 ||
+    if (a.req_off == (size_t)-1 || a.areq_off == (size_t)-1 || a.row_off == (size_t)-1 ||
         a.last_off == (size_t)-1)
       overflow = true;
+  }
+
+  // ---- work items of the prompt chunks' attention: (request, 128-token tile, one or two heads), most keys first ----
+  int pre_mt[2] = {2, 2};                       // query tiles per item for head sizes 64 and 128
+  for (int hi = 0; hi < 2; ++hi) {
+    long long tiles = 0;
+    for (const Active& a : act)
+      if (a.n_pre > 0 && a.m->d.head_dim == (hi ? 128 : 64))
+        for (const PrefillChunk& p : a.pre) tiles += (long long)((p.n_tok + FLASH_TILE - 1) / FLASH_TILE) * a.m->d.n_heads;
+    pre_mt[hi] = attn_flash_tiles(tiles, c->sm_count);
+  }
+  for (Active& a : act) {
+    if (a.n_pre == 0 || overflow) continue;
+    const int G = a.m->d.n_heads / a.m->d.n_kv_heads, mt = pre_mt[a.m->d.head_dim == 128 ? 1 : 0];
+    struct Tile { int blocks, req, tile; };
+    std::vector<Tile> tiles;
+    for (int r = 0; r < a.n_pre; ++r)
+      for (int t = 0; t * FLASH_TILE < a.pre[r].n_tok; ++t)
+        tiles.push_back({(a.pre[r].kv_len + std::min(a.pre[r].n_tok, (t + 1) * FLASH_TILE) + FLASH_TILE - 1) / FLASH_TILE, r, t});
+    std::stable_sort(tiles.begin(), tiles.end(), [](const Tile& x, const Tile& y) { return x.blocks > y.blocks; });
+    std::vector<PrefillItem> items;
+    items.reserve(tiles.size() * a.m->d.n_heads);
+    for (const Tile& t : tiles)
+      for (int kvh = 0; kvh < a.m->d.n_kv_heads; ++kvh)
+        for (int h = 0; h < G; h += mt) {
+          const PrefillChunk& p = a.pre[t.req];
+          const int t0 = t.tile * FLASH_TILE;
+          items.push_back({p.table, p.row_start + t0, std::min(FLASH_TILE, p.n_tok - t0), p.kv_len + t0, kvh * G + h, {0, 0}});
+        }
+    a.pre_items = (int)items.size();
+    a.pitem_off = put(items.data(), items.size() * sizeof(PrefillItem), 16);
+    if (a.pitem_off == (size_t)-1) overflow = true;
   }
 
   // ---- plan (A1): sweep the kernel kinds until every model's op list is exhausted ----
@@ -1017,21 +1049,29 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
           LL.kind = kind;
           off = align_up(off, 64);
           LL.off = off;
-          int blocks = 0, n_put = 0;
+          int items = 0, n_put = 0;
           for (Active* a : who) {
+            if (a->m->ops[a->cursor].apre.hd != hd || a->n_pre == 0) continue;
             AttnPrefillGroup g = a->m->ops[a->cursor].apre;
-            if (g.hd != hd || a->n_pre == 0) continue;
-            g.reqs = (const PrefillReq*)(slot.dev + a->preq_off); g.n_reqs = a->n_pre; g.status = dev_status;
-            g.blk_start = blocks; g.n_blocks = a->pre_blocks;
-            blocks += a->pre_blocks;
+            g.items = (const PrefillItem*)(slot.dev + a->pitem_off);
+            g.item_start = items; g.n_items = a->pre_items;
+            items += a->pre_items;
             ++n_put;
-            if (put(&g, sizeof(g), 8) == (size_t)-1) overflow = true;
+            if (put(&g, sizeof(g), 64) == (size_t)-1) overflow = true;
           }
-          LL.n_groups = n_put; LL.p0 = blocks; LL.p1 = hd;
+          LL.n_groups = n_put; LL.p0 = items; LL.p1 = hd; LL.p2 = pre_mt[hd == 128 ? 1 : 0];
           if (n_put > 0) launches.push_back(LL);
         }
         for (Active* a : who) a->cursor++;
         continue;
+      }
+      if (kind == EPARA_K_ATTN_ENC) {
+        long long tiles = 0;                                   // query tiles of the tensor-core kernel's groups
+        for (Active* a : who) {
+          const AttnEncGroup& g = a->m->ops[a->cursor].aenc;
+          tiles += (long long)a->B * g.H * ((g.T + FLASH_TILE - 1) / FLASH_TILE);
+        }
+        L.p3 = attn_flash_tiles(tiles, c->sm_count);
       }
       int total = 0, mx = 0;
       for (Active* a : who) {
@@ -1122,7 +1162,8 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
           case EPARA_K_ATTN_ENC: {
             AttnEncGroup g = op.aenc;
             if ((g.tc != 0) != (pass == 0)) break;             // the other pass takes it
-            g.B = a->B; g.q_blocks = g.tc ? 1 : attn_encoder_q_blocks(g.T); g.blk_start = total;
+            g.B = a->B; g.blk_start = total;
+            g.q_blocks = g.tc ? (g.T + FLASH_TILE * L.p3 - 1) / (FLASH_TILE * L.p3) : attn_encoder_q_blocks(g.T);
             total += a->B * g.H * g.q_blocks;
             mx = std::max(mx, g.T);
             ++n_put;
@@ -1196,13 +1237,13 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
                                  L.p3 & 255, attn_decode_fused(L.p0, L.p1 & 0xffff, L.p2, c->sm_count) ? 1 : 0, st);
         break;
       case EPARA_K_ATTN_ENC:
-        if (L.p2 == 0) err = launch_attn_encoder_tc((const AttnEncGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st);
+        if (L.p2 == 0) err = launch_attn_encoder_tc((const AttnEncGroup*)gp, L.n_groups, L.p0, L.p3, dev_status, c->sm_count, st);
         else err = launch_attn_encoder((const AttnEncGroup*)gp, L.n_groups, L.p0, L.p1, st);
         break;
       case EPARA_K_OUTPUT: launch_output((const OutputGroup*)gp, L.n_groups, L.p1, st); break;
       case EPARA_K_TRACE: err = cudaMemcpyAsync(L.dst, L.src, L.bytes, cudaMemcpyDeviceToDevice, st); break;
       case EPARA_K_ATTN_PREFILL:
-        err = launch_attn_prefill((const AttnPrefillGroup*)gp, L.n_groups, L.p0, L.p1, st);
+        err = launch_attn_prefill((const AttnPrefillGroup*)gp, L.n_groups, L.p0, L.p2, L.p1, dev_status, c->sm_count, st);
         break;
     }
     if (prof) cudaEventRecord(slot.prof[2 * li + 1], st);

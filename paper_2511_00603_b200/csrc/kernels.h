@@ -62,15 +62,16 @@ void launch_attn_prepare(const AttnDecGroup& g, AttnDecGroup* dst, AttnReq* reqs
                          const int32_t* tables, int stride, int max_len, int n_counters, cudaStream_t st);
 constexpr int DEC_STATUS_OFFSET = 192;   // byte offset of the status word in a single-kernel call's scratch
 
-// Causal attention of prompt chunks (head size 64 or 128), one block per (request, query head, 64 query tokens).
-constexpr int PREFILL_TILE = 64;
-inline int attn_prefill_blocks(int n_tok, int Hq) { return (n_tok + PREFILL_TILE - 1) / PREFILL_TILE * Hq; }
-cudaError_t launch_attn_prefill(const AttnPrefillGroup* groups, int n_groups, int total_blocks, int hd, cudaStream_t st);
-
-// Encoder attention on tcgen05 for groups with AttnEncGroup::tc (hd 64, T <= ENC_TC_MAX_T): persistent,
-// one item per (image, head); total_items = sum of B * H.  `status` as for the GEMM.
-constexpr int ENC_TC_MAX_T = 224;
-cudaError_t launch_attn_encoder_tc(const AttnEncGroup* groups, int n_groups, int total_items, int* status, int sm_count,
+// Attention of many query rows on tcgen05, persistent over work items of `mt` (1 or 2) tiles of FLASH_TILE query rows;
+// `status` as for the GEMM.  Two tiles keep the tensor core and the softmax busy at once; attn_flash_tiles() picks one
+// when the launch's tiles do not outnumber the SMs.
+constexpr int FLASH_TILE = 128;
+inline int attn_flash_tiles(long long total_tiles, int sm_count) { return total_tiles <= sm_count ? 1 : 2; }
+// ... causal attention of prompt chunks (head size 64 or 128)
+cudaError_t launch_attn_prefill(const AttnPrefillGroup* groups, int n_groups, int total_items, int mt, int hd, int* status,
+                                int sm_count, cudaStream_t st);
+// ... encoder attention for groups with AttnEncGroup::tc (hd 64); total_items = sum of B * H * q_blocks.
+cudaError_t launch_attn_encoder_tc(const AttnEncGroup* groups, int n_groups, int total_items, int mt, int* status, int sm_count,
                                    cudaStream_t st);
 
 // Encoder (bidirectional) attention on mma.sync, one block per (image, head, query block).

@@ -108,6 +108,38 @@ def test_chunked_prefill_on_a_cached_prefix_and_head_size_128(mods):
     srv.close()
 
 
+@pytest.mark.parametrize("Hq,Hkv,hd,kv0,n,grow", [(32, 8, 128, 300, 650, 0.0), (24, 24, 64, 130, 900, 0.0), (8, 1, 64, 37, 200, 4.0),
+                                                 (16, 4, 64, 517, 131, 4.0), (4, 2, 128, 260, 129, 4.0), (2, 2, 64, 0, 385, 0.0)])
+def test_prompt_chunk_attention_items_and_running_maximum(mods, Hq, Hkv, hd, kv0, n, grow):
+    """Prompt chunks whose attention runs with two query tiles per work item (more tiles than SMs) and with one, heads
+    that pair up and heads that cannot (one query head per kv head), several key blocks with ragged ends, both head
+    sizes.  grow: the cached keys' magnitude rises along the sequence, so that a row's running maximum is raised, and its
+    output and sum rescaled, again and again.  (A score's standard deviation is 1.4 in log2 units at factor 1, so factor 5
+    takes the maximum from about 4 to about 20, past the 8 at which the kernel rescales.  It cannot be much larger: q and k
+    are rounded to bf16, which moves a score s by about 2^-9 s, and at factor 26 -- scores up to 120 -- that storage noise
+    alone, 2^-9 x 120 x ln 2 = 16 % of a probability, puts the oracle's two evaluations 2.4e-2 apart.)"""
+    E, server = mods
+    p = synth.make_decoder(d=256, n_layers=1, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=hd, ffn=256, vocab=300, seed=40, device=DEV,
+                           std=0.06)
+    rng = np.random.default_rng(Hq + n)
+    tokens = [int(t) for t in rng.integers(0, 300, n)]
+    table = _table(rng, kv0 + n, offset=1)
+    pool = synth.make_kv_pool(1, len(table) + 2, Hkv, hd, seed=41, device=DEV)
+    for i, pg in enumerate(table):
+        pool[0, int(pg), 0] *= 1.0 + grow * i / len(table)
+    pool0 = pool.clone()
+    srv = server.Server(workspace_bytes=256 << 20)
+    m = srv.add_model(p, kv_pool=pool, max_kv_len=kv0 + n, max_batch=n)
+    t = srv.submit(m, E.CAT_FS, tokens=tokens, kv_len=kv0, table=torch.as_tensor(table, device=DEV))
+    srv.step()
+    torch.cuda.synchronize()
+    s, logits, am = srv.collect(t)
+    assert s == E.OK
+    v = synth.bits_view({k: p[k] for k in p if k != "packed_layers"})
+    _check_prefill(v, pool, pool0, (logits, int(am.item())), tokens, kv0, table, f"chunk of {n} after {kv0} cached")
+    srv.close()
+
+
 def test_prompt_chunks_and_decode_requests_share_a_step(mods):
     """One decoder serving, in ONE step, two prompt chunks (37 tokens on an empty cache; 90 tokens after 21
     cached) and three decode requests, co-resident with a ViT.  Every request equals the oracle; and a
