@@ -78,15 +78,17 @@ __device__ __forceinline__ void finish_chunk(const AttnDecGroup& g, int b, int r
   if (n_chunks == 1 || !fused) return;
   __syncthreads();                      // all partials of the block are written ...
   if (threadIdx.x == 0) {
-    __threadfence();                    // ... and visible device-wide before the arrival is counted
+    // ... and, through the barrier and this release, visible device-wide before the arrival is counted; the block that
+    // finds itself last has acquired the others' partials the same way
     int* cnt = g.counters + (size_t)b * g.Hkv + kvh;
-    const int last = (atomicAdd(cnt, 1) == n_chunks - 1);
-    if (last) atomicExch(cnt, 0);
+    int old;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(cnt) : "memory");
+    const int last = old == n_chunks - 1;
+    if (last) *cnt = 0;
     s_last = last;
   }
   __syncthreads();
   if (!s_last) return;
-  __threadfence();
   for (int idx = threadIdx.x; idx < G * HD; idx += 128) {
     const int h = idx / HD, e = idx % HD;
     const float* p = g.partial + ((size_t)b * g.Hq + (kvh * G + h)) * g.max_chunks * (HD + 2);
@@ -249,11 +251,18 @@ __global__ void __launch_bounds__(128) attn_decode_kernel(const AttnDecGroup* __
 
 // Tensor-core variant for hd 64 / 128.  Same work split (chunk, kv head, request; 4 warps, warp w
 // takes pages w, w+4, w+8, w+12 of the chunk) and the same partial format, but the pages are
-// brought into shared memory with 16-byte cp.async copies -- all of a warp's pages are in flight
-// at once and no registers are tied up by loads -- and Q K^T and P V run on mma.sync m16n8k16
-// with the G query heads of the kv head as the first G rows of the 16-row A operand.  Rows of a
-// staged tile are 128-byte segments whose 16-byte pieces are XOR-swizzled by the token index, so
-// ldmatrix reads are free of bank conflicts.
+// brought into shared memory with 16-byte cp.async copies -- no registers are tied up by loads -- and
+// the products run on mma.sync m16n8k16 with the G query heads of the kv head as the 8 columns:
+// S^T = K Q^T (16 tokens x 8 heads), O^T += V^T P^T (16 dims x 8 heads).  (With the heads as rows half of
+// every accumulator was padding: 96 registers at hd 64, five blocks per SM, and HBM latency was not
+// covered; now 75 registers and six blocks: 113 -> 108 us per layer for the 1B decoder at 128 requests
+// with RoPE and append, which had 10 us of their own, included.)  The running maximum of a head is only raised, and O and the sum rescaled, when a
+// score passes it by more than 2^8.  Rows of a staged tile are 128-byte segments whose 16-byte pieces
+// are XOR-swizzled by the token index, so ldmatrix reads are free of bank conflicts.
+// With AttnDecGroup::cs the kernel also does RoPE and the append for its request: q is rotated as it is
+// read, the block that holds position len - 1 rotates k, writes k and v to the cache and into its
+// staged tile, and the cached pages, which no kernel of the step writes, are requested before the wait
+// on the QKV projection.  That takes a launch out of every layer.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
@@ -279,12 +288,24 @@ __device__ __forceinline__ void ldsm_x4_trans(uint32_t* r, uint32_t addr) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
 }
 
+__device__ __forceinline__ uint32_t transpose_8x8(uint32_t u) {
+  uint32_t r;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(u));
+  return r;
+}
+// RoPE of one interleaved pair of bf16
+__device__ __forceinline__ uint32_t rotate_pair(uint32_t u, float2 cs) {
+  const float a = __uint_as_float(u << 16), b = __uint_as_float(u & 0xffff0000u);
+  return pack2(a * cs.x - b * cs.y, a * cs.y + b * cs.x);
+}
+
 template <int HD, int G, int NSLOT>
 __global__ void __launch_bounds__(128) attn_decode_mma_kernel(const AttnDecGroup* __restrict__ groups, int n_groups, int fused) {
   constexpr int ROWB = HD * 2;              // bytes per token row
   constexpr int TILE = 16 * ROWB;           // bytes per (K or V) page tile
   constexpr int CPR = HD / 8;               // 16-byte pieces per row
-  constexpr int KS = HD / 16;               // k-steps of Q K^T
+  constexpr int KS = HD / 16;               // k-steps of K Q^T
+  constexpr float RAISE = 8.0f;             // log2 units a head's maximum may lag behind
   constexpr float LOG2E = 1.4426950408889634f;
   extern __shared__ __align__(128) unsigned char dsm[];
 
@@ -294,9 +315,10 @@ __global__ void __launch_bounds__(128) attn_decode_mma_kernel(const AttnDecGroup
   const int b = blockIdx.z - g.req_start;
   const int kvh = blockIdx.y;
   if (kvh >= g.Hkv) return;
+  const bool early = g.reqs_stable && g.cs != nullptr;
   if (g.reqs_stable && blockIdx.x * ATTN_CHUNK >= g.reqs[b].len) return;   // nothing to do and nothing to wait for
   pdl_launch_dependents();
-  pdl_wait();                 // q, the appended K/V row and (single-kernel entry) the request table come from earlier kernels
+  if (!early) pdl_wait();     // q, the appended K/V row and (single-kernel entry) the request table come from earlier kernels
   const AttnReq rq = g.reqs[b];
   const int chunk = blockIdx.x;
   const int t_begin = chunk * ATTN_CHUNK;
@@ -305,9 +327,12 @@ __global__ void __launch_bounds__(128) attn_decode_mma_kernel(const AttnDecGroup
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gq = lane >> 2, tq = lane & 3;
   const int Hkv = g.Hkv;
-  const bf16* kv_layer = g.kv_layer;
+  bf16* const kv_layer = g.kv_layer;
   const long long kv_pages = g.kv_pages;
+  const float2* const cs = g.cs;
+  const int pos = rq.len - 1;               // with cs: position of the token to rotate and append
   uint32_t bad_mask = 0;                    // pages of this warp whose id was outside the pool (warp-uniform)
+  int app_page = -1;                        // page of `pos` when this warp holds it
 
   // ---- issue all copies of this warp's pages (up to 4), one commit group per page
   unsigned char* wsm = dsm + warp * (NSLOT * 2 * TILE);
@@ -318,12 +343,14 @@ __global__ void __launch_bounds__(128) attn_decode_mma_kernel(const AttnDecGroup
     const int pg = page_begin + warp + 4 * i;
     if (i < 4 && pg < page_end) {
       const int page = rq.table[pg];
+      const bool app = cs != nullptr && pg == pos >> 4;
       if (page < 0 || page >= kv_pages) {            // outside the pool: reported, read as absent
-        if (lane == 0) atomicExch(g.status, ERR_PAGE_ATTEND);
+        if (lane == 0) atomicExch(g.status, app ? ERR_PAGE_APPEND : ERR_PAGE_ATTEND);
         bad_mask |= 1u << i;
         cp_async_commit();
         return;
       }
+      if (app) app_page = page;
       const unsigned char* kt = reinterpret_cast<const unsigned char*>(kv_layer + (((size_t)page * 2 + 0) * Hkv + kvh) * 16 * HD);
       const unsigned char* vt = reinterpret_cast<const unsigned char*>(kv_layer + (((size_t)page * 2 + 1) * Hkv + kvh) * 16 * HD);
       const uint32_t kd = wsm_u + (i % NSLOT) * 2 * TILE, vd = kd + TILE;
@@ -339,24 +366,31 @@ __global__ void __launch_bounds__(128) attn_decode_mma_kernel(const AttnDecGroup
   };
 #pragma unroll
   for (int i = 0; i < NSLOT; ++i) issue(i);
+  // (With cs the step's earlier kernels write nothing of the cache below `pos`: its pages are requested while the QKV
+  // projection may still be running.  The slot of `pos` holds something old and is overwritten in shared memory below.)
+  if (early) pdl_wait();
 
-  // ---- Q fragments: rows 0..G-1 of the A operand are the query heads of this kv head
-  uint32_t qa[KS][4];
+  // ---- Q fragments: the query heads of this kv head are the first G of the B operand's 8 columns
+  const bf16* const row0 = g.q + (size_t)rq.row * g.q_stride;
+  uint32_t qb[KS][2];
   {
-    const bf16* qrow = g.q + (size_t)rq.row * g.q_stride + (size_t)(kvh * G + gq) * HD;
+    const bf16* qrow = row0 + (size_t)(kvh * G + gq) * HD;
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) {
-      qa[ks][0] = (gq < G) ? *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 2 * tq) : 0u;
-      qa[ks][2] = (gq < G) ? *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 8 + 2 * tq) : 0u;
-      qa[ks][1] = 0u;
-      qa[ks][3] = 0u;
+      qb[ks][0] = (gq < G) ? *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 2 * tq) : 0u;
+      qb[ks][1] = (gq < G) ? *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 8 + 2 * tq) : 0u;
+      if (cs != nullptr) {                   // a lane's two elements are one rotation pair
+        const float2* c = cs + (size_t)pos * (HD / 2) + ks * 8 + tq;
+        qb[ks][0] = rotate_pair(qb[ks][0], __ldg(c));
+        qb[ks][1] = rotate_pair(qb[ks][1], __ldg(c + 4));
+      }
     }
   }
   const float scale = LOG2E * rsqrtf((float)HD);
-  float o[HD / 8][4];
+  float o[HD / 16][4];                       // O^T: dims np*16 + gq (+8), heads 2tq, 2tq+1
 #pragma unroll
-  for (int n = 0; n < HD / 8; ++n) { o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f; }
-  float m_run = -1e30f, l_run = 0.f;
+  for (int n = 0; n < HD / 16; ++n) { o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f; }
+  float m_run[2] = {-1e30f, -1e30f}, l_run[2] = {0.f, 0.f};     // heads 2tq, 2tq+1; the sums are this lane's tokens'
   const int lm_row = lane & 7, lm_mat = lane >> 3;
 
   auto process = [&](int i) {
@@ -364,6 +398,24 @@ __global__ void __launch_bounds__(128) attn_decode_mma_kernel(const AttnDecGroup
     if (pg >= page_end || (bad_mask & (1u << i))) return;
     const uint32_t kd = wsm_u + (i % NSLOT) * 2 * TILE, vd = kd + TILE;
     const int tok0 = pg * 16;
+    if (app_page >= 0 && pg == pos >> 4) {
+      // the new token: k (rotated) and v of this kv head to the cache and into the staged tile, a pair per lane and piece
+      const int r = pos & 15;
+      unsigned char* const kt = wsm + (i % NSLOT) * 2 * TILE + r * ROWB;
+      const uint32_t* const kr = reinterpret_cast<const uint32_t*>(row0 + (size_t)(g.Hq + kvh) * HD);
+      uint32_t* const dst = reinterpret_cast<uint32_t*>(kv_layer + (((size_t)app_page * 2) * Hkv + kvh) * 16 * HD + (size_t)r * HD);
+#pragma unroll
+      for (int p = 0; p < HD / 64; ++p) {
+        const int pair = p * 32 + lane, c = pair >> 2;
+        const uint32_t nk = rotate_pair(kr[pair], __ldg(cs + (size_t)pos * (HD / 2) + pair)), nv = kr[Hkv * (HD / 2) + pair];
+        dst[pair] = nk;
+        dst[Hkv * 8 * HD + pair] = nv;
+        const int off = (c & ~7) * 16 + (((c & 7) ^ (r & 7)) << 4) + (pair & 3) * 4;
+        *reinterpret_cast<uint32_t*>(kt + off) = nk;
+        *reinterpret_cast<uint32_t*>(kt + TILE + off) = nv;
+      }
+      __syncwarp();
+    }
     if (tok0 + 16 > t_end) {
       // slots past the length may hold anything (NaN included): zero those V rows
       const int valid = t_end - tok0;
@@ -375,52 +427,53 @@ __global__ void __launch_bounds__(128) attn_decode_mma_kernel(const AttnDecGroup
       }
       __syncwarp();
     }
-    // S = Q K^T for 16 tokens: two 8-token tiles
-    float sc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    // S^T = K Q^T for 16 tokens
+    float s[4] = {0.f, 0.f, 0.f, 0.f};       // (token gq, head 2tq), (gq, 2tq+1), (gq+8, 2tq), (gq+8, 2tq+1)
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) {
-      const int r = (lm_mat >> 1) * 8 + lm_row, c = ks * 2 + (lm_mat & 1);
+      const int r = (lm_mat & 1) * 8 + lm_row, c = ks * 2 + (lm_mat >> 1);
       uint32_t kr[4];
       ldsm_x4(kr, kd + r * ROWB + (c & ~7) * 16 + (((c & 7) ^ (r & 7)) << 4));
-      mma_bf16_m16n8k16(sc[0], qa[ks], kr[0], kr[1]);
-      mma_bf16_m16n8k16(sc[1], qa[ks], kr[2], kr[3]);
+      mma_bf16_m16n8k16(s, kr, qb[ks][0], qb[ks][1]);
     }
-    // row gq of the tile: tokens tok0 + j*8 + 2*tq (+1)
-    float s[4];
+    const bool lo_ok = tok0 + gq < t_end, hi_ok = tok0 + gq + 8 < t_end;
+    s[0] = lo_ok ? s[0] * scale : -INFINITY;
+    s[1] = lo_ok ? s[1] * scale : -INFINITY;
+    s[2] = hi_ok ? s[2] * scale : -INFINITY;
+    s[3] = hi_ok ? s[3] * scale : -INFINITY;
+    float mx0 = fmaxf(s[0], s[2]), mx1 = fmaxf(s[1], s[3]);
+    if (__any_sync(0xffffffffu, mx0 > m_run[0] + RAISE || mx1 > m_run[1] + RAISE)) {
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int t0 = tok0 + j * 8 + 2 * tq;
-      s[2 * j] = (t0 < t_end) ? sc[j][0] * scale : -INFINITY;
-      s[2 * j + 1] = (t0 + 1 < t_end) ? sc[j][1] * scale : -INFINITY;
+      for (int x = 4; x < 32; x <<= 1) {
+        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, x));
+        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, x));
+      }
+      mx0 = fmaxf(mx0, m_run[0]);
+      mx1 = fmaxf(mx1, m_run[1]);
+      const float f0 = exp2f(m_run[0] - mx0), f1 = exp2f(m_run[1] - mx1);
+      m_run[0] = mx0; m_run[1] = mx1;
+      l_run[0] *= f0; l_run[1] *= f1;
+#pragma unroll
+      for (int n = 0; n < HD / 16; ++n) { o[n][0] *= f0; o[n][1] *= f1; o[n][2] *= f0; o[n][3] *= f1; }
     }
-    float mx = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    const float mn = fmaxf(m_run, mx);
-    const float resc = exp2f(m_run - mn);
-    m_run = mn;
-    l_run *= resc;
-#pragma unroll
-    for (int n = 0; n < HD / 8; ++n) { o[n][0] *= resc; o[n][1] *= resc; }
-    const float p0 = exp2f(s[0] - mn), p1 = exp2f(s[1] - mn), p2 = exp2f(s[2] - mn), p3 = exp2f(s[3] - mn);
-    l_run += (p0 + p1) + (p2 + p3);
-    // P enters the tensor core as bf16; to keep fp32-level accuracy it is split into a bf16 head
-    // and a bf16 remainder (p = hi + lo up to 2^-17 relative), and P V is two MMAs per tile
-    uint32_t pa[4], pb[4];
-    pa[0] = pack2(p0, p1); pa[1] = 0u; pa[2] = pack2(p2, p3); pa[3] = 0u;
-    pb[0] = pack2(p0 - __uint_as_float(pa[0] << 16), p1 - __uint_as_float(pa[0] & 0xffff0000u));
-    pb[2] = pack2(p2 - __uint_as_float(pa[2] << 16), p3 - __uint_as_float(pa[2] & 0xffff0000u));
-    pb[1] = 0u; pb[3] = 0u;
-    // O += P V
+    const float p0 = exp2f(s[0] - m_run[0]), p1 = exp2f(s[1] - m_run[1]), p2 = exp2f(s[2] - m_run[0]), p3 = exp2f(s[3] - m_run[1]);
+    l_run[0] += p0 + p2;
+    l_run[1] += p1 + p3;
+    // P enters the tensor core as bf16; to keep fp32-level accuracy it is split into a bf16 head and a bf16 remainder
+    // (p = hi + lo up to 2^-17 relative), and O is two MMAs per tile.  A register holds (token, two heads); the
+    // transposed 8 x 8 block holds (two tokens, head): the B operand.
+    const uint32_t h0 = pack2(p0, p1), h1 = pack2(p2, p3);
+    const uint32_t pa0 = transpose_8x8(h0), pa1 = transpose_8x8(h1);
+    const uint32_t pb0 = transpose_8x8(pack2(p0 - __uint_as_float(h0 << 16), p1 - __uint_as_float(h0 & 0xffff0000u)));
+    const uint32_t pb1 = transpose_8x8(pack2(p2 - __uint_as_float(h1 << 16), p3 - __uint_as_float(h1 & 0xffff0000u)));
+    // O^T += V^T P^T
 #pragma unroll
     for (int np = 0; np < HD / 16; ++np) {
-      const int r = (lm_mat & 1) * 8 + lm_row, c = 2 * np + (lm_mat >> 1);
+      const int r = (lm_mat >> 1) * 8 + lm_row, c = 2 * np + (lm_mat & 1);
       uint32_t vr[4];
       ldsm_x4_trans(vr, vd + r * ROWB + (c & ~7) * 16 + (((c & 7) ^ (r & 7)) << 4));
-      mma_bf16_m16n8k16(o[2 * np], pa, vr[0], vr[1]);
-      mma_bf16_m16n8k16(o[2 * np + 1], pa, vr[2], vr[3]);
-      mma_bf16_m16n8k16(o[2 * np], pb, vr[0], vr[1]);
-      mma_bf16_m16n8k16(o[2 * np + 1], pb, vr[2], vr[3]);
+      mma_bf16_m16n8k16(o[np], vr, pa0, pa1);
+      mma_bf16_m16n8k16(o[np], vr, pb0, pb1);
     }
   };
 #pragma unroll
@@ -432,17 +485,24 @@ __global__ void __launch_bounds__(128) attn_decode_mma_kernel(const AttnDecGroup
     issue(i + NSLOT);
   }
 
-  l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
-  l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
+#pragma unroll
+  for (int x = 4; x < 32; x <<= 1) {
+    l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], x);
+    l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], x);
+  }
 
   // ---- merge the 4 warps through shared memory, in warp order (same layout as the SIMT kernel)
   __shared__ float sm_m[4][G], sm_l[4][G], sm_o[4][G][HD];
-  if (gq < G) {
-    if (tq == 0) { sm_m[warp][gq] = m_run; sm_l[warp][gq] = l_run; }
 #pragma unroll
-    for (int n = 0; n < HD / 8; ++n) {
-      sm_o[warp][gq][n * 8 + 2 * tq] = o[n][0];
-      sm_o[warp][gq][n * 8 + 2 * tq + 1] = o[n][1];
+  for (int e = 0; e < 2; ++e) {
+    const int h = 2 * tq + e;
+    if (h < G) {
+      if (gq == 0) { sm_m[warp][h] = m_run[e]; sm_l[warp][h] = l_run[e]; }
+#pragma unroll
+      for (int n = 0; n < HD / 16; ++n) {
+        sm_o[warp][h][n * 16 + gq] = o[n][e];
+        sm_o[warp][h][n * 16 + gq + 8] = o[n][2 + e];
+      }
     }
   }
   __syncthreads();
@@ -467,7 +527,8 @@ static cudaError_t launch_dec(const AttnDecGroup* groups, int n_groups, int tota
 
 // Few blocks (up to two waves): the last block of a (request, kv head) merges the chunks itself and the
 // step saves a launch.  Many blocks: the counter round trip at the end of every block costs more than
-// a second kernel, so the merge runs as attn_combine_kernel.
+// a second kernel, so the merge runs as attn_combine_kernel (1B decoder, 27 requests: 659 us of attention
+// per step merged in the kernel, 612 with the second one; 8B, 64 requests: 4252 and 3798).
 bool attn_decode_fused(int total_B, int max_Hkv, int max_chunks, int sm_count) {
   return (long long)total_B * max_Hkv * max_chunks <= 10ll * sm_count;
 }
@@ -767,7 +828,7 @@ extern "C" int epara_decode_attention_static(int device, void* cuda_stream, cons
   AttnDecGroup g;
   memset(&g, 0, sizeof(g));
   AttnReq* reqs = reinterpret_cast<AttnReq*>(s + 256);
-  g.q = (const bf16*)q; g.q_stride = q_stride; g.kv_layer = (const bf16*)kv_layer; g.reqs = reqs; g.out = (bf16*)out;
+  g.q = (const bf16*)q; g.q_stride = q_stride; g.kv_layer = (bf16*)const_cast<void*>(kv_layer); g.reqs = reqs; g.out = (bf16*)out;
   g.partial = reinterpret_cast<float*>(s + 256 + req_bytes);
   g.counters = reinterpret_cast<int*>(s + 256 + req_bytes + part_bytes);
   g.B = B; g.Hq = Hq; g.Hkv = Hkv; g.hd = hd; g.max_chunks = chunks; g.req_start = 0;

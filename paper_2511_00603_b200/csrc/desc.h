@@ -33,7 +33,8 @@ struct ReqDesc {
 // Decoder activations have one row per token.  Row r belongs to request `req`, sits at position `pos` of
 // its sequence and holds token id `token`.
 struct RowDesc {
-  int req, pos, token, pad;
+  int req, pos, token;
+  int single;            // 1: the only row of a decode request, 0: a prompt chunk's
 };
 
 // C = epi(A W^T + bias).  tmA/tmW are the TMA maps of A [rows, K] and W [N, K] (K innermost,
@@ -101,6 +102,8 @@ struct RopeGroup {
   int* status;           // device word: set to ERR_PAGE_APPEND when a block table names a page outside the pool
   long long kv_pages;    // pages of the pool; a page id outside [0, kv_pages) is reported, its write skipped
   int B, Hq, Hkv, hd;
+  int only_chunks;       // 1: decode rows are left alone (the attention kernel rotates and appends them itself)
+  int pad;
 };
 
 struct AttnReq {
@@ -133,8 +136,10 @@ struct alignas(64) AttnPrefillGroup {
 
 struct AttnDecGroup {
   const bf16* q;         // [B, q_stride], head h at column h*hd
-  const bf16* kv_layer;
+  bf16* kv_layer;
   const AttnReq* reqs;
+  const float2* cs;      // set: row b of q is followed by k and v (qkv), neither rotated nor appended yet; the kernel does
+                         // both for position len - 1 (RopeGroup::cs).  Null: q is rotated and the cache complete.
   bf16* out;             // [B, Hq*hd]
   float* partial;        // [B][Hq][max_chunks][hd + 2]  (m, l, o[hd]); requests of more than one chunk
   int* counters;         // [B][Hkv] chunks that have arrived; zero between launches

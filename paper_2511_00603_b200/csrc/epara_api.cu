@@ -482,6 +482,7 @@ int build_model(Builder& bl, Model* m, const epara_config& cfg) {
     r.kind = EPARA_K_ROPE; r.rows_per_req = 1;
     r.rope.qkv = qkv; r.rope.kv_layer = kv_layer; r.rope.cs = rope_cs;
     r.rope.Hq = Hq; r.rope.Hkv = Hkv; r.rope.hd = hd; r.rope.kv_pages = d.kv_pages;
+    r.rope.only_chunks = hd >= 64;           // (the tensor-core decode attention rotates and appends its rows itself)
     m->ops.push_back(r);
     Op at;
     memset(&at, 0, sizeof(at));
@@ -490,6 +491,7 @@ int build_model(Builder& bl, Model* m, const epara_config& cfg) {
     at.adec.counters = chunk_counters;
     at.adec.Hq = Hq; at.adec.Hkv = Hkv; at.adec.hd = hd; at.adec.max_chunks = m->max_chunks;
     at.adec.reqs_stable = 1; at.adec.kv_pages = d.kv_pages;
+    if (r.rope.only_chunks) at.adec.cs = rope_cs;
     m->ops.push_back(at);
     Op ap;                                   // causal attention of the step's prompt chunks (none in a pure decode step)
     memset(&ap, 0, sizeof(ap));
@@ -893,7 +895,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       if (dec) {
         for (int t = 0; t < nt; ++t) {
           RowDesc r;
-          r.req = b; r.pos = in.kv_len + t; r.token = nt > 1 ? rq.toks[t] : in.token; r.pad = 0;
+          r.req = b; r.pos = in.kv_len + t; r.token = nt > 1 ? rq.toks[t] : in.token; r.single = nt == 1;
           rows.push_back(r);
         }
         if (nt == 1) {
@@ -1151,11 +1153,13 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
             break;
           }
           case EPARA_K_ROPE: {
+            if (op.rope.only_chunks && a->n_pre == 0) break;   // nothing to rotate
             RopeGroup g = op.rope;
             g.reqs = (const ReqDesc*)(slot.dev + a->req_off); g.B = rows;
             g.rows = (const RowDesc*)(slot.dev + a->row_off);
             g.status = dev_status;
             mx = std::max(mx, rows);
+            ++n_put;
             if (put(&g, sizeof(g), 8) == (size_t)-1) overflow = true;
             break;
           }
@@ -1181,7 +1185,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
         if (pass == n_pass - 1) a->cursor++;
       }
       L.p0 = total; L.p1 = mx;
-      if (kind == EPARA_K_GEMM || kind == EPARA_K_ATTN_ENC) {
+      if (kind == EPARA_K_GEMM || kind == EPARA_K_ATTN_ENC || kind == EPARA_K_ROPE) {
         L.n_groups = n_put;
         if (n_put == 0) continue;
       }
@@ -1464,7 +1468,7 @@ int epara_decode_attention(int device, void* cuda_stream, const void* q, int q_s
   memset(&g, 0, sizeof(g));
   const int g_chunks = (max_len + ATTN_CHUNK - 1) / ATTN_CHUNK;
   AttnReq* reqs = (AttnReq*)(s + 256);
-  g.q = (const bf16*)q; g.q_stride = q_stride; g.kv_layer = (const bf16*)kv_layer; g.reqs = reqs; g.out = (bf16*)out;
+  g.q = (const bf16*)q; g.q_stride = q_stride; g.kv_layer = (bf16*)const_cast<void*>(kv_layer); g.reqs = reqs; g.out = (bf16*)out;
   g.partial = (float*)(s + 256 + align_up((size_t)B * sizeof(AttnReq), 256));
   g.counters = (int*)((unsigned char*)g.partial + align_up((size_t)B * Hq * g_chunks * (hd + 2) * 4, 256));
   g.B = B; g.Hq = Hq; g.Hkv = Hkv; g.hd = hd; g.max_chunks = g_chunks; g.req_start = 0;

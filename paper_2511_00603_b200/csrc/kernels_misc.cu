@@ -258,6 +258,7 @@ __global__ void __launch_bounds__(ROPE_THREADS) rope_append_kernel(const RopeGro
   if (b >= g.B) return;
   pdl_launch_dependents();
   const RowDesc rd = g.rows[b];
+  if (g.only_chunks && rd.single) return;
   const int pos = rd.pos, hd = g.hd, half = hd >> 1;
   const int page = g.reqs[rd.req].table[pos / 16], slot = pos % 16;
   const int e = (threadIdx.x * 8) % hd;   // ROPE_THREADS * 8 is a multiple of every head size
