@@ -99,7 +99,6 @@ __device__ __forceinline__ void finish_chunk(const AttnDecGroup& g, int b, int r
 // Separate merge for launches with many blocks: one block per (query head, request) of more than one chunk.
 template <int HD>
 __global__ void __launch_bounds__(HD) attn_combine_kernel(const AttnDecGroup* __restrict__ groups, int n_groups) {
-  pdl_launch_dependents();
   int gi = 0;
   for (int i = 1; i < n_groups; ++i) if ((int)blockIdx.y >= groups[i].req_start) gi = i;
   const AttnDecGroup& g = groups[gi];
@@ -128,7 +127,6 @@ __global__ void __launch_bounds__(128) attn_decode_kernel(const AttnDecGroup* __
   const int kvh = blockIdx.y;
   if (kvh >= g.Hkv) return;
   if (g.reqs_stable && blockIdx.x * ATTN_CHUNK >= g.reqs[b].len) return;   // nothing to do and nothing to wait for
-  pdl_launch_dependents();
   pdl_wait();                 // q, the appended K/V row and (single-kernel entry) the request table come from earlier kernels
   const AttnReq rq = g.reqs[b];
   const int chunk = blockIdx.x;
@@ -317,7 +315,6 @@ __global__ void __launch_bounds__(128) attn_decode_mma_kernel(const AttnDecGroup
   if (kvh >= g.Hkv) return;
   const bool early = g.reqs_stable && g.cs != nullptr;
   if (g.reqs_stable && blockIdx.x * ATTN_CHUNK >= g.reqs[b].len) return;   // nothing to do and nothing to wait for
-  pdl_launch_dependents();
   if (!early) pdl_wait();     // q, the appended K/V row and (single-kernel entry) the request table come from earlier kernels
   const AttnReq rq = g.reqs[b];
   const int chunk = blockIdx.x;
@@ -608,7 +605,6 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t* r, uint32_t addr) {
 __global__ void __launch_bounds__(ENC_ROWS * 2, 2) attn_encoder_kernel(const AttnEncGroup* __restrict__ groups, int n_groups) {
   constexpr int HD = 64;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pdl_launch_dependents();
   int gi = 0;
   for (int i = 1; i < n_groups; ++i) if ((int)blockIdx.x >= groups[i].blk_start) gi = i;
   const AttnEncGroup& g = groups[gi];

@@ -242,7 +242,6 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  pdl_launch_dependents();
   if (threadIdx.x == 0) {
     mbar_init(bar(FB_Q_FULL), 1); mbar_init(bar(FB_Q_EMPTY), 1);
     for (int i = 0; i < 4; ++i) { mbar_init(bar(FB_S_FULL + i), 1); mbar_init(bar(FB_P_READY + i), 4); mbar_init(bar(FB_PV_DONE + i), 1); }

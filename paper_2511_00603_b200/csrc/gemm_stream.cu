@@ -61,7 +61,6 @@ __global__ void __launch_bounds__(RS_WARPS * 32, NT == 1 ? 3 : 2)
 gemm_stream_kernel(const GemmGroup* __restrict__ groups, int n_groups) {
   __shared__ float red[RS_WARPS][NT][RS_ROWS][8];
   __shared__ float outv[NT][8][RS_ROWS + 1];
-  pdl_launch_dependents();
   const GemmGroup& g = groups[find_group_rs(groups, n_groups, blockIdx.x)];
   const int n0 = (blockIdx.x - g.tile_start) * RS_ROWS;
   const int M = g.M, N = g.N, K = g.K;

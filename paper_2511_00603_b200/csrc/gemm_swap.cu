@@ -83,7 +83,6 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
   bool acc_ok = true;
   const int rank = S == 1 ? 0 : (int)cluster_ctarank();
   const int item = blockIdx.x / S;
-  pdl_launch_dependents();
 
   const GemmGroup* g = groups + find_group_sw(groups, n_groups, item);
   const int nb = g->bn;                           // batch rows of a tile as the MMA's N: multiple of 16, at most 256

@@ -218,7 +218,6 @@ gemm_tc_pair_kernel(const GemmGroup* __restrict__ groups, int n_groups, int tota
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-  pdl_launch_dependents();
   if (threadIdx.x == 0) {
     for (int s = 0; s < PAIR_STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 2 * EPI_WARPS); }
@@ -466,7 +465,6 @@ gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int tota
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-  pdl_launch_dependents();
   if (threadIdx.x == 0) {
     for (int s = 0; s < MLP_SLOTS; ++s) { mbar_init(bar(MB_W_FULL + s), 1); mbar_init(bar(MB_W_EMPTY + s), 1); }
     mbar_init(bar(MB_X_FULL), 1); mbar_init(bar(MB_X_EMPTY), 1);

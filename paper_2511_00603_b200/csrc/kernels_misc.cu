@@ -13,7 +13,6 @@ namespace epara {
 __global__ void __launch_bounds__(128) gather_kernel(const GatherGroup* __restrict__ groups) {
   const GatherGroup g = groups[blockIdx.y];
   if ((int)blockIdx.x >= g.blocks) return;      // (descriptors are not written by kernels: no wait needed to leave)
-  pdl_launch_dependents();
   pdl_wait();
   if (g.kind == GATHER_ROWS) {
     const int b = blockIdx.x;
@@ -220,7 +219,6 @@ __global__ void __launch_bounds__(NORM_THREADS, 4) norm_kernel(const NormGroup* 
   __shared__ float red[2 * NORM_WARPS];
   const NormGroup g = groups[blockIdx.y];
   if ((int)blockIdx.x * norm_rows_per_block(g.d) >= g.M) return;   // beyond this group's rows: nothing to wait for
-  pdl_launch_dependents();
   pdl_wait();
   if (g.d <= NORM_NARROW_D) {
     const int row0 = (blockIdx.x * NORM_WARPS + (threadIdx.x >> 5)) * NORM_NARROW_ROWS;
@@ -256,7 +254,6 @@ __global__ void __launch_bounds__(ROPE_THREADS) rope_append_kernel(const RopeGro
   const RopeGroup g = groups[blockIdx.y];
   const int b = blockIdx.x;               // token row
   if (b >= g.B) return;
-  pdl_launch_dependents();
   const RowDesc rd = g.rows[b];
   if (g.only_chunks && rd.single) return;
   const int pos = rd.pos, hd = g.hd, half = hd >> 1;
@@ -311,7 +308,6 @@ __global__ void __launch_bounds__(256) assemble_kernel(const AssembleGroup* __re
   const AssembleGroup g = groups[blockIdx.y];
   const int row0 = blockIdx.x * ASSEMBLE_ROWS;
   if (row0 >= g.B * g.T) return;
-  pdl_launch_dependents();
   pdl_wait();
   const int nrows = min(ASSEMBLE_ROWS, g.B * g.T - row0), vecs = g.d / 8;
 #pragma unroll 2
@@ -343,7 +339,6 @@ __global__ void __launch_bounds__(OUT_THREADS) output_kernel(const OutputGroup* 
   const OutputGroup g = groups[blockIdx.y];
   const int b = blockIdx.x;
   if (b >= g.B) return;
-  pdl_launch_dependents();
   pdl_wait();
   const ReqDesc r = g.reqs[b];
   const bf16* src = g.logits + (size_t)b * g.ld;          // 16-byte aligned: ld is a multiple of 8
