@@ -20,10 +20,11 @@ namespace epara {
 // attention, small projections, all bound by latency -- waited for memory behind them.  One kernel ahead is enough to keep
 // HBM busy over a boundary (1B decoder: one request 972 -> 902 us a step, 27 requests 1385 -> 1331; one image through
 // ViT-B 671 -> 635; steps of large kernels unchanged).
-__device__ __forceinline__ void pdl_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // (one thread per block is enough; a block that exits counts)
-}
+// A kernel that streams weights to its end takes the two halves apart and triggers when its own requests are out.
+__device__ __forceinline__ void pdl_wait_only() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// (one thread per block is enough; a block that exits counts as having triggered)
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { pdl_wait_only(); pdl_trigger(); }
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {

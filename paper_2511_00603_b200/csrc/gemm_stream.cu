@@ -2,16 +2,23 @@
 // single decode request): C_g = epi(A_g W_g^T + bias_g) with M <= 16.
 //
 // With so few rows the work is reading W once; a 128-row tensor-core tile would leave most SMs idle
-// on the narrow matrices and spend its time on zero rows.  Here one block of 8 warps owns 16
+// on the narrow matrices and spend its time on zero rows.  Here one block of 16 warps owns 16
 // consecutive rows of W (16 output columns) over the whole K, so a GEMM gives N / 16 blocks and
 // every block has all of its loads in flight at once.  K is cut into 32-wide k-blocks dealt to the
-// warps round-robin (warp w takes k-blocks w, w + 8, ...): in one k-block lane (gq, tq) reads 16
+// warps round-robin (warp w takes k-blocks w, w + 16, ...): in one k-block lane (gq, tq) reads 16
 // contiguous bytes of W rows gq and gq + 8 and of activation row gq, which feed two
 // mma.sync.m16n8k16 (bf16 in, fp32 accumulate) with W as the 16-row operand and the batch as the
 // 8 columns.  The k order inside an MMA is a permutation of memory order, the same one for both
-// operands, which leaves every dot product unchanged.  The 8 warps' partial sums are added in warp
+// operands, which leaves every dot product unchanged.  The 16 warps' partial sums are added in warp
 // order in shared memory, then the epilogue (bias, GELU, SwiGLU, fp32 residual) writes the outputs.
 // An output row's value never depends on the other rows of the batch.
+//
+// HBM-bound: 513 MB of W (an LM head) take 79 us, 6.5 TB/s.  A short matrix is bound by how soon its blocks have all
+// their requests out: with 16 warps K = 2048 is requested at once (64 KB a block), K = 8192 in four rounds instead of
+// eight, and the next kernel, whose own first requests would queue in front of the rest of these, is let in only when
+// the last request of this one has been answered (one request through the 1B decoder: 8 warps 901 us a step, 16 warps
+// 883, with the late trigger 860; more in flight than that, in registers or through a bulk-copy ring of shared memory, reads
+// slower again, 5.2 TB/s).
 #include "common.cuh"
 #include "kernels.h"
 
@@ -20,7 +27,7 @@ namespace epara {
 namespace {
 
 constexpr int RS_ROWS = 16;       // W rows (output columns) per block
-constexpr int RS_WARPS = 8;
+constexpr int RS_WARPS = 16;
 constexpr int RS_U = 4;           // k-blocks in flight per warp
 
 __device__ __forceinline__ uint4 ldg_w(const bf16* p) {
@@ -57,7 +64,7 @@ __device__ __forceinline__ int find_group_rs(const GemmGroup* groups, int n, int
 
 // NT: batch tiles of 8 rows (1: M <= 8, 2: M <= 16).
 template <int NT>
-__global__ void __launch_bounds__(RS_WARPS * 32, NT == 1 ? 3 : 2)
+__global__ void __launch_bounds__(RS_WARPS * 32, NT == 1 ? 2 : 1)
 gemm_stream_kernel(const GemmGroup* __restrict__ groups, int n_groups) {
   __shared__ float red[RS_WARPS][NT][RS_ROWS][8];
   __shared__ float outv[NT][8][RS_ROWS + 1];
@@ -95,7 +102,7 @@ gemm_stream_kernel(const GemmGroup* __restrict__ groups, int n_groups) {
       wl[u] = (k_ok && w_lo_ok) ? ldg_w(w_lo + k) : zero4;
       wh[u] = (k_ok && w_hi_ok) ? ldg_w(w_hi + k) : zero4;
     }
-    if (first) { pdl_wait(); first = false; }
+    if (first) { pdl_wait_only(); first = false; }
 #pragma unroll
     for (int u = 0; u < RS_U; ++u) {
       const int k = (kb0 + u * RS_WARPS) * 32;
@@ -113,6 +120,7 @@ gemm_stream_kernel(const GemmGroup* __restrict__ groups, int n_groups) {
       }
     }
   }
+  pdl_trigger();
   // accumulator layout: acc[0], acc[1] = (W row gq, batch rows 2tq, 2tq+1); acc[2], acc[3] = (W row gq+8, same)
 #pragma unroll
   for (int t = 0; t < NT; ++t) {
