@@ -145,7 +145,7 @@ typedef struct {
   double gemm_flops;        /* 2 M N K over all GEMM groups */
   double weight_bytes;      /* bytes of weight matrices the step streams */
   double kv_bytes;          /* bytes of cached K/V the step reads */
-  double stream_gemm_flops;   /* the part of gemm_flops in weight-streaming launches (groups of at most 16 rows) */
+  double stream_gemm_flops;   /* the part of gemm_flops in weight-streaming launches (groups of few rows, small matrices) */
   double stream_weight_bytes; /* the part of weight_bytes in those launches */
   int prefill_tokens;         /* tokens of the step's prompt chunks */
 } epara_step_info;
@@ -166,7 +166,7 @@ typedef struct {
 enum {
   EPARA_K_GATHER = 0, EPARA_K_NORM = 1, EPARA_K_GEMM = 2, EPARA_K_ROPE = 3, EPARA_K_ATTN_DEC = 4,
   EPARA_K_ATTN_COMBINE = 5, EPARA_K_ATTN_ENC = 6, EPARA_K_ASSEMBLE = 7, EPARA_K_OUTPUT = 8,
-  EPARA_K_GEMM_STREAM = 9,  /* the weight-streaming GEMM launches (groups of at most 16 rows); EPARA_K_GEMM holds
+  EPARA_K_GEMM_STREAM = 9,  /* the weight-streaming GEMM launches (groups of few rows, small matrices); EPARA_K_GEMM holds
                                the tensor-core launches */
   EPARA_K_TRACE = 10,       /* copies into epara_model_desc.trace */
   EPARA_K_ATTN_PREFILL = 11, /* causal attention of prompt chunks */

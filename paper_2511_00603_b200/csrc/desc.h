@@ -56,8 +56,8 @@ struct alignas(64) GemmGroup {
   int tiles_m, tiles_n;
   int bn, ksplit;  // tile pairs: bn = tile width; swapped operands: bn = batch rows of a tile, ksplit = k ranges
   int c_rows;      // row extent of tmC (rows at and beyond it are never written)
-  int stream;      // 1: at most 16 rows ever, runs in the weight-streaming kernel (16 W rows per block,
-                   // tiles_n = ceil(N / 16), no TMA maps); 2: 256-row tiles on CTA pairs (tiles_m counts 256-row
+  int stream;      // 1: weight-streaming kernel (at most 16 rows ever, or a small matrix; 16 W rows per
+                   // block, tiles_n = ceil(N / 16), no TMA maps); 2: 256-row tiles on CTA pairs (tiles_m counts 256-row
                    // tiles and tmW's box holds bn / 2 rows); 3: swapped operands (tmA's box holds bn rows, tmW's
                    // 128); 0: plain CUDA-core comparator
   int pad1, pad2;

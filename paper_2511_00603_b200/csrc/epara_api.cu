@@ -236,7 +236,7 @@ bool add_gemm(Builder& bl, Model* m, const void* A, int lda, long long rows_cap,
   g.ksplit = 1;
   if (bl.gemm_impl == EPARA_GEMM_SIMT) {
     g.stream = 0;
-  } else if (max_rows <= GEMM_STREAM_MAX_ROWS) {
+  } else if (!one_sum && gemm_stream_eligible(max_rows, N, K)) {
     g.stream = 1; g.bn = 16;
   } else if (!one_sum && gemm_swap_eligible(max_rows, N, K, g.epi, sm_count)) {
     g.stream = 3;                              // W as the MMA's 128-row operand, the batch as its N
@@ -971,6 +971,12 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
         if (a.cursor < a.m->ops.size() && a.m->ops[a.cursor].kind == kind) who.push_back(&a);
       if (who.empty()) continue;
       more = true;
+      // the output is a model's last op: one launch serves every model once the last of them has got there
+      if (kind == EPARA_K_OUTPUT) {
+        bool all = true;
+        for (const Active& a : act) all = all && a.cursor + 1 >= a.m->ops.size();
+        if (!all) continue;
+      }
       if (kind == EPARA_K_TRACE) {               // debug copies of the residual stream: one plain copy per model
         for (Active* a : who) {
           const Op& op = a->m->ops[a->cursor];
@@ -984,7 +990,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
         continue;
       }
       // GEMM groups go out in one launch per kernel that has a group: CUDA cores (pass 0, comparator
-      // contexts only), the weight-streaming kernel for groups that never exceed 16 rows (pass 1) and
+      // contexts only), the weight-streaming kernel for groups of few rows or small matrices (pass 1) and
       // 256-row tiles on CTA pairs (pass 2); encoder attention in two: the tcgen05 kernel (pass 0) and the
       // mma.sync kernel for shapes it does not take (pass 1)
       // (passes 3 to 10: the swapped-operand kernel with 1 to 8 k ranges per tile)
@@ -1132,9 +1138,9 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
               g.tile_start = total;
               total += g.tiles_m * g.tiles_n;
             } else if (g.stream) {
-              g.tiles_m = 1; g.tiles_n = gemm_stream_tiles(g.N);
+              g.tiles_m = gemm_stream_tiles_m(rows); g.tiles_n = gemm_stream_tiles_n(g.N);
               g.tile_start = total;
-              total += g.tiles_n;
+              total += g.tiles_m * g.tiles_n;
               mx = std::max(mx, rows);
             } else {
               g.tiles_m = (rows + SIMT_TILE - 1) / SIMT_TILE; g.tiles_n = (g.N + SIMT_TILE - 1) / SIMT_TILE;
@@ -1366,11 +1372,11 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
     g.M = q.M; g.N = q.N; g.K = q.K; g.lda = q.lda; g.ldw = q.ldw; g.ldc = q.ldc; g.epi = q.epilogue;
     g.bn = 128; g.ksplit = 1;
     g.c_rows = q.M;
-    if (!simt && q.M <= GEMM_STREAM_MAX_ROWS && q.K % 8 == 0) {
+    if (!simt && gemm_stream_eligible(q.M, q.N, q.K)) {
       g.stream = 1; g.bn = 16;
-      g.tiles_m = 1; g.tiles_n = gemm_stream_tiles(q.N);
+      g.tiles_m = gemm_stream_tiles_m(q.M); g.tiles_n = gemm_stream_tiles_n(q.N);
       g.tile_start = total_stream;
-      if (q.M > 0) total_stream += g.tiles_n;
+      if (q.M > 0) total_stream += g.tiles_m * g.tiles_n;
       max_rows_stream = std::max(max_rows_stream, q.M);
       gs_stream.push_back(g);
       continue;

@@ -1,5 +1,5 @@
 // Weight-streaming grouped GEMM for groups of at most 16 rows (a latency-sensitive batch, a
-// single decode request): C_g = epi(A_g W_g^T + bias_g) with M <= 16.
+// single decode request): C_g = epi(A_g W_g^T + bias_g) with M <= 16, and for small matrices with up to 128 rows.
 //
 // With so few rows the work is reading W once; a 128-row tensor-core tile would leave most SMs idle
 // on the narrow matrices and spend its time on zero rows.  Here one block of 16 warps owns 16
@@ -62,15 +62,17 @@ __device__ __forceinline__ int find_group_rs(const GemmGroup* groups, int n, int
   return lo;
 }
 
-// NT: batch tiles of 8 rows (1: M <= 8, 2: M <= 16).
+// NT: batch tiles of 8 rows in a block's rows (1: M <= 8, 2: M <= 16, 4: any M, tiles_m tiles of 32 rows).
 template <int NT>
 __global__ void __launch_bounds__(RS_WARPS * 32, NT == 1 ? 2 : 1)
 gemm_stream_kernel(const GemmGroup* __restrict__ groups, int n_groups) {
   __shared__ float red[RS_WARPS][NT][RS_ROWS][8];
   __shared__ float outv[NT][8][RS_ROWS + 1];
   const GemmGroup& g = groups[find_group_rs(groups, n_groups, blockIdx.x)];
-  const int n0 = (blockIdx.x - g.tile_start) * RS_ROWS;
-  const int M = g.M, N = g.N, K = g.K;
+  const int local = blockIdx.x - g.tile_start;
+  const int n0 = (NT < 4 ? local : local / g.tiles_m) * RS_ROWS;
+  const int m0 = NT < 4 ? 0 : local % g.tiles_m * (8 * NT);
+  const int M = g.M - m0, N = g.N, K = g.K;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gq = lane >> 2, tq = lane & 3;
   const int nkb = (K + 31) >> 5;
@@ -83,7 +85,7 @@ gemm_stream_kernel(const GemmGroup* __restrict__ groups, int n_groups) {
 #pragma unroll
   for (int t = 0; t < NT; ++t) {
     x_ok[t] = t * 8 + gq < M;
-    x_row[t] = g.A + (size_t)(t * 8 + gq) * g.lda + tq * 8;
+    x_row[t] = g.A + (size_t)(m0 + t * 8 + gq) * g.lda + tq * 8;
   }
   float acc[NT][4];
 #pragma unroll
@@ -148,26 +150,37 @@ gemm_stream_kernel(const GemmGroup* __restrict__ groups, int n_groups) {
     if (m >= M || n >= N) continue;
     const float v = outv[t][bm][r];
     if (epi & EPI_RESID_F32) {
-      float* C = reinterpret_cast<float*>(g.C) + (size_t)m * g.ldc + n;
+      float* C = reinterpret_cast<float*>(g.C) + (size_t)(m0 + m) * g.ldc + n;
       *C += v;
     } else if (epi & EPI_SWIGLU) {
       if ((r & 1) == 0 && n + 1 < N)
-        reinterpret_cast<bf16*>(g.C)[(size_t)m * g.ldc + (n >> 1)] = f2bf(silu_f(v) * outv[t][bm][r + 1]);
+        reinterpret_cast<bf16*>(g.C)[(size_t)(m0 + m) * g.ldc + (n >> 1)] = f2bf(silu_f(v) * outv[t][bm][r + 1]);
     } else {
-      reinterpret_cast<bf16*>(g.C)[(size_t)m * g.ldc + n] = f2bf(v);
+      reinterpret_cast<bf16*>(g.C)[(size_t)(m0 + m) * g.ldc + n] = f2bf(v);
     }
   }
 }
 
 }  // namespace
 
-int gemm_stream_tiles(int N) { return (N + RS_ROWS - 1) / RS_ROWS; }
+// Up to 16 rows whatever the matrix.  A matrix of up to a million elements (the layers of an MLP classifier, a
+// classification head) is all latency: blocks of 16 columns and 32 rows that read it again from L2 need no cluster and no
+// tensor memory, and share a launch with the groups of few rows.  Two MLPs of 512- and 1024-wide layers, the second one
+// with 32 / 64 / 128 / 256 rows: 46 / 50 / 56 / 68 us a step with its layers in the swapped-operand kernel, 40 / 43 /
+// 47 / 68 here; one image through ViT-B, whose 197-row products of 768 x 768 would come here too: 627 against 650.
+bool gemm_stream_eligible(long long rows_cap, int N, int K) {
+  if (K % 8 != 0) return false;
+  return rows_cap <= GEMM_STREAM_MAX_ROWS || (rows_cap <= 128 && (long long)N * K <= 1 << 20);
+}
+int gemm_stream_tiles_n(int N) { return (N + RS_ROWS - 1) / RS_ROWS; }
+int gemm_stream_tiles_m(int M) { return M <= GEMM_STREAM_MAX_ROWS ? 1 : (M + 31) / 32; }
 
 cudaError_t launch_gemm_stream(const GemmGroup* groups, int n_groups, int total_items, int max_rows, cudaStream_t st) {
   if (n_groups == 0 || total_items == 0) return cudaSuccess;
-  if (max_rows > 16) return cudaErrorInvalidValue;
-  if (max_rows <= 8) return launch_pdl(gemm_stream_kernel<1>, dim3(total_items), dim3(RS_WARPS * 32), 0, st, groups, n_groups);
-  return launch_pdl(gemm_stream_kernel<2>, dim3(total_items), dim3(RS_WARPS * 32), 0, st, groups, n_groups);
+  const dim3 grid(total_items), block(RS_WARPS * 32);
+  if (max_rows <= 8) return launch_pdl(gemm_stream_kernel<1>, grid, block, 0, st, groups, n_groups);
+  if (max_rows <= 16) return launch_pdl(gemm_stream_kernel<2>, grid, block, 0, st, groups, n_groups);
+  return launch_pdl(gemm_stream_kernel<4>, grid, block, 0, st, groups, n_groups);
 }
 
 }  // namespace epara

@@ -42,10 +42,13 @@ int gemm_swap_tiles_n(int N);
 cudaError_t launch_gemm_swap(const GemmGroup* groups, int n_groups, int total_items, int ksplit, int max_nb, int* status,
                              int sm_count, cudaStream_t st);
 
-// Weight-streaming GEMM for groups that never exceed 16 rows (GemmGroup::stream): one block per 16
-// rows of W over the whole K, mma.sync, no tensor maps.  total_items = sum of gemm_stream_tiles(N).
+// Weight-streaming GEMM (GemmGroup::stream == 1) for groups that never exceed 16 rows, and for small matrices: one block
+// per 16 rows of W over the whole K and 32 batch rows, mma.sync, no tensor maps.  total_items = sum of
+// tiles_m * tiles_n; max_rows = the most rows of a group in the launch.
 constexpr int GEMM_STREAM_MAX_ROWS = 16;
-int gemm_stream_tiles(int N);
+bool gemm_stream_eligible(long long rows_cap, int N, int K);
+int gemm_stream_tiles_n(int N);
+int gemm_stream_tiles_m(int M);
 cudaError_t launch_gemm_stream(const GemmGroup* groups, int n_groups, int total_items, int max_rows, cudaStream_t st);
 
 // Decode attention, split-KV over 256-token chunks.  fused = 1: the block of a (request, kv head) that

@@ -109,6 +109,21 @@ def test_grouped_gemm_many_tiles_and_group_independence(E):
     assert torch.equal(alone[0]["C"], probs[0]["C"])
 
 
+@pytest.mark.parametrize("M", [17, 32, 33, 65, 127, 128])
+def test_grouped_gemm_small_matrices_in_tiles_of_32_rows(E, M):
+    """Matrices of up to a million elements with 17 to 128 rows run in the weight-streaming kernel in tiles of 32 rows:
+    row counts at the edges of a tile, N below one block and not a multiple of it, one 16-byte piece of K, K that is no
+    multiple of a k-block, every epilogue, the largest matrix; a group of few rows in the same launch and the problem
+    alone give the same bits."""
+    cases = [(M, 10, 512, ("bias",)), (M, 1000, 776, ("bias", "gelu")), (M, 24, 8, ()), (M, 512, 2048, ("resid",)),
+             (M, 512, 256, ("swiglu",)), (3, 520, 512, ("bias",))]
+    probs, refs = _run_gemm(E, E.GEMM_TCGEN05, cases, seed=M)
+    for p, ref, case in zip(probs, refs, cases):
+        assert_close(p["C"][:ref.shape[0], :ref.shape[1]], ref, what=f"small gemm {case}")
+    alone, _ = _run_gemm(E, E.GEMM_TCGEN05, cases[:1], seed=M)
+    assert torch.equal(alone[0]["C"][:, :10], probs[0]["C"][:, :10])     # (the columns that pad the rows stay NaN)
+
+
 def test_grouped_gemm_tile_pairs(E):
     """Dense bf16-output problems (more than 256 rows, 256-wide tiles) run as 256-row tiles on CTA pairs:
     ragged last pair (one CTA with no valid row), N tails inside the first and the second half of the W
