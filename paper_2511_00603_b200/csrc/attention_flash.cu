@@ -70,7 +70,7 @@ constexpr int FL_S_COL = 0, FL_O_COL = 256;
 // between two looks of its waiter.  K blocks sit in the even slots of the ring, V blocks in the odd ones, whose EMPTY
 // barriers count both P V warps (one that has no tile in the item arrives without an MMA).
 enum { FB_Q_FULL = 0, FB_Q_EMPTY, FB_S_FULL, FB_P_READY = FB_S_FULL + 4, FB_PV_DONE = FB_P_READY + 4, FB_KV_FULL = FB_PV_DONE + 4,
-       FB_KV_EMPTY = FB_KV_FULL + 8, FB_COUNT = FB_KV_EMPTY + 8 };
+       FB_KV_EMPTY = FB_KV_FULL + 8, FB_TURN = FB_KV_EMPTY + 8, FB_COUNT = FB_TURN + 8 };
 static_assert(8 * FB_COUNT + 16 <= FL_BAR_BYTES, "barrier area");
 
 __device__ __forceinline__ float fl_ex2(float x) {
@@ -245,6 +245,7 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
   if (threadIdx.x == 0) {
     mbar_init(bar(FB_Q_FULL), 1); mbar_init(bar(FB_Q_EMPTY), 1);
     for (int i = 0; i < 4; ++i) { mbar_init(bar(FB_S_FULL + i), 1); mbar_init(bar(FB_P_READY + i), 4); mbar_init(bar(FB_PV_DONE + i), 1); }
+    for (int i = 0; i < 8; ++i) mbar_init(bar(FB_TURN + i), 1);
     for (int s = 0; s < ST; ++s) { mbar_init(bar(FB_KV_FULL + s), 1); mbar_init(bar(FB_KV_EMPTY + s), 1 + (s & 1)); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -435,15 +436,27 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
     unsigned char* const stage = base_ptr + Geo::OFF_OUT + warp * 4096;
     bool ok = true;
     uint32_t cnt = 0;                            // steps of this tile done
+    uint32_t turns = 0;                          // turns waited for
     View view;
     view.g = nullptr;
-    for (int round = 0; ok; ++round) {
-      if (round * (int)gridDim.x >= total_items) break;
-      const int item = item_of_round(round);
-      if (item >= total_items) continue;
-      load_view(view, groups, n_groups, item, mt);
-      const Work w = get_work(view, item);
-      if (g >= w.n_mt) continue;
+    // this tile's next item; decoded while the last P V of the item before is under way
+    int round = 0;
+    Work next;
+    const Group* next_g = nullptr;
+    auto find_next = [&]() {
+      for (; round * (int)gridDim.x < total_items; ++round) {
+        const int item = item_of_round(round);
+        if (item >= total_items) continue;
+        load_view(view, groups, n_groups, item, mt);
+        next = get_work(view, item);
+        if (g < next.n_mt) { ++round; next_g = view.g; return true; }
+      }
+      return false;
+    };
+    bool more = find_next();
+    while (ok && more) {
+      const Work w = next;
+      const Group* const wg = next_g;
       const int steps = (w.n_keys + FL_STEP - 1) / FL_STEP;
       const int live = g ? w.live1 : w.live0;
       const bool warp_live = quarter * 32 < live;
@@ -451,40 +464,45 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
       const int lim = min(w.lim0 + min(row, live - 1), w.n_keys - 1);                        // last key of this row
       const int warp_first = min(w.lim0 + quarter * 32, w.n_keys - 1);                       // ... of the warp's first row
       const int warp_last = min(w.lim0 + min(quarter * 32 + 31, live - 1), w.n_keys - 1);    // ... and of its last
+      // the warp of the other tile on this scheduler has as many steps: the two take turns
+      const bool paired = w.n_mt == 2 && quarter * 32 < min(w.live0, w.live1);
       float m_ref = 0.f, l = 0.f;
       for (int j = 0; j < steps; ++j) {
         const uint32_t b = cnt & 1u, sb = s_addr + b * 64;
         if (!mbar_wait<false>(bar(FB_S_FULL + 2 * g + b), (cnt >> 1) & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 16); break; }
         tc_fence_after();
-        const int k0 = j * FL_STEP, n = min(FL_STEP, w.n_keys - k0);
-        if (warp_live) {
-          const int need = min(n, warp_last - k0 + 1);              // columns some row of the warp sees
-          const int nch = need <= 0 ? 0 : (need + 15) >> 4;         // ... in blocks of 16
+        const int k0 = j * FL_STEP;
+        // Columns that no row of the warp sees (the upper triangle of a prompt chunk): P is zero and nothing else changes.
+        const bool seen = warp_live && k0 <= warp_last;
+        if (warp_live && !seen) {
+          const uint32_t z[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+#pragma unroll
+          for (int c = 0; c < FL_STEP; c += 8) tmem_st8(sb + c, z);
+          tmem_st_wait();
+        }
+        // The two warps of a scheduler take turns at the exponentials, so that one's scores are read and reduced while the
+        // other keeps the special-function unit busy (in step they left it idle half of the time).
+        const bool take_turns = paired && (g == 1 || j > 0), give_turn = paired && (g == 0 || j + 1 < steps);
+        if (seen) {
           uint32_t v[FL_STEP];
-          if (nch > 0) tmem_ld32_nowait(sb, v);
-          if (nch > 2) tmem_ld32_nowait(sb + 32, v + 32);
+          tmem_ld32_nowait(sb, v);
+          tmem_ld32_nowait(sb + 32, v + 32);
           tmem_ld_wait();
 #pragma unroll
           for (int c = 0; c < 4; ++c) tmem_regs_ready16(v + 16 * c);
-          float mx = -INFINITY;
+          if (k0 + FL_STEP - 1 > warp_first) {                      // some row's limit lies in this step or before it
 #pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            if (2 * q >= nch) break;
-            uint32_t* const vq = v + 32 * q;
-            if (k0 + 32 * q + 31 > warp_first) {                    // some row's limit lies in this half or before it
-#pragma unroll
-              for (int i = 0; i < 32; ++i) if (k0 + 32 * q + i > lim) vq[i] = 0xff800000u;
-            }
-            float mx0 = mx, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
-#pragma unroll
-            for (int i = 0; i < 32; i += 8) {
-              mx0 = max3(mx0, __uint_as_float(vq[i]), __uint_as_float(vq[i + 1]));
-              mx1 = max3(mx1, __uint_as_float(vq[i + 2]), __uint_as_float(vq[i + 3]));
-              mx2 = max3(mx2, __uint_as_float(vq[i + 4]), __uint_as_float(vq[i + 5]));
-              mx3 = max3(mx3, __uint_as_float(vq[i + 6]), __uint_as_float(vq[i + 7]));
-            }
-            mx = fmaxf(max3(mx0, mx1, mx2), mx3);
+            for (int i = 0; i < FL_STEP; ++i) if (k0 + i > lim) v[i] = 0xff800000u;
           }
+          float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
+#pragma unroll
+          for (int i = 0; i < FL_STEP; i += 8) {
+            mx0 = max3(mx0, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
+            mx1 = max3(mx1, __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
+            mx2 = max3(mx2, __uint_as_float(v[i + 4]), __uint_as_float(v[i + 5]));
+            mx3 = max3(mx3, __uint_as_float(v[i + 6]), __uint_as_float(v[i + 7]));
+          }
+          const float mx = fmaxf(max3(mx0, mx1, mx2), mx3);
           if (j == 0) {
             m_ref = mx;                                             // (key 0 is in every row's reach)
           } else {
@@ -508,41 +526,47 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
           }
           const float nms = -m_ref * scale;
           const uint64_t nms2 = pack_f2(nms, nms), minus1 = pack_f2(-1.f, -1.f);
+          if (take_turns) {
+            if (!mbar_wait<false>(bar(FB_TURN + 4 * g + quarter), turns & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 19); break; }
+            ++turns;
+          }
           uint64_t l2a = 0, l2b = 0;
-          const int nall = (n + 15) >> 4;                           // 16-column blocks that P V reads
+          // p = 2^(s * scale - m * scale), its sum and its bf16 parts; one straight piece of code, so that the exponentials of
+          // a block of 16 columns run under the conversions of the block before
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            if (c >= nall) break;
             const uint32_t* const vc = v + 16 * c;
             uint32_t hi[8], lo[8];
-            if (c < nch) {
 #pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                float x, y;
-                unpack_f2(fma_f2(pack_f2(__uint_as_float(vc[2 * i]), __uint_as_float(vc[2 * i + 1])), scale2, nms2), x, y);
-                x = fl_ex2(x);
-                y = fl_ex2(y);
-                const uint64_t p2 = pack_f2(x, y);
-                if (i & 1) l2b = add_f2(l2b, p2); else l2a = add_f2(l2a, p2);
-                hi[i] = pack2(x, y);
-                if (SPLIT) {
-                  float rx, ry;
-                  unpack_f2(fma_f2(pack_f2(__uint_as_float(hi[i] << 16), __uint_as_float(hi[i] & 0xffff0000u)), minus1, p2), rx, ry);
-                  lo[i] = pack2(rx, ry);
-                }
+            for (int i = 0; i < 8; ++i) {
+              float x, y;
+              unpack_f2(fma_f2(pack_f2(__uint_as_float(vc[2 * i]), __uint_as_float(vc[2 * i + 1])), scale2, nms2), x, y);
+              x = fl_ex2(x);
+              y = fl_ex2(y);
+              const uint64_t p2 = pack_f2(x, y);
+              if (i & 1) l2b = add_f2(l2b, p2); else l2a = add_f2(l2a, p2);
+              hi[i] = pack2(x, y);
+              if (SPLIT) {
+                float rx, ry;
+                unpack_f2(fma_f2(pack_f2(__uint_as_float(hi[i] << 16), __uint_as_float(hi[i] & 0xffff0000u)), minus1, p2), rx, ry);
+                lo[i] = pack2(rx, ry);
               }
-            } else {
-#pragma unroll
-              for (int i = 0; i < 8; ++i) hi[i] = lo[i] = 0u;
             }
             tmem_st8(sb + 16 * c, hi);
             if (SPLIT) tmem_st8(sb + 16 * c + 8, lo);
           }
+          if (give_turn && lane == 0) mbar_arrive(bar(FB_TURN + 4 * (g ^ 1) + quarter));
           float a0, a1, a2, a3;
           unpack_f2(l2a, a0, a1);
           unpack_f2(l2b, a2, a3);
           l += (a0 + a1) + (a2 + a3);
           tmem_st_wait();
+        } else if (paired) {
+          if (take_turns) {
+            if (!mbar_wait<false>(bar(FB_TURN + 4 * g + quarter), turns & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 19); break; }
+            ++turns;
+          }
+          if (give_turn && lane == 0) mbar_arrive(bar(FB_TURN + 4 * (g ^ 1) + quarter));
         }
         tc_fence_before();
         __syncwarp();
@@ -551,13 +575,14 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
       }
       if (!ok) break;
       // ---- the tile's output: rows through this warp's staging area, then whole 128-byte lines
+      const float inv = 1.0f / l;
+      const int oy = w.qy + g * w.dy + quarter * 32, ox = w.qx + g * w.dx;
+      bf16* const out = wg->out;
+      const int ostride = out_stride(wg);
+      more = find_next();
       if (!warp_live) continue;
       if (!mbar_wait<false>(bar(FB_PV_DONE + 2 * g + ((cnt - 1u) & 1u)), ((cnt - 1u) >> 1) & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 18); break; }
       tc_fence_after();
-      const float inv = 1.0f / l;
-      const int oy = w.qy + g * w.dy + quarter * 32, ox = w.qx + g * w.dx;
-      bf16* const out = view.g->out;
-      const int ostride = out_stride(view.g);
 #pragma unroll 1
       for (int hh = 0; hh < Geo::NH; ++hh) {
         uint32_t o[64];
