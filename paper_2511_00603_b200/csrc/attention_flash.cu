@@ -13,7 +13,7 @@
 //   warps 10, 11  issue O_g += P_g V, g = 0 and 1, with P as the A operand from tensor memory and V consumed as the TMA
 //              wrote it (MN-major B operand).  (An MMA costs its issuer some 60 cycles here and a step as much again in
 //              waits and bookkeeping: one warp for all of them was the bound, 3350 cycles per step of two tiles.)
-//   warps 0-3  softmax of tile 0, warps 4-7 of tile 1: one thread per query row.  The thread reads its row of S once,
+//   warps 0-3  softmax of tile 0, warps 4-7 of tile 1: one thread per query row (but see `HALF` below).  The thread reads its row of S once,
 //              keeps it in registers for the maximum and the exponentials and writes P over S: 16 columns of S become 8
 //              of P as bf16 and, for prompt chunks, 8 of the bf16 remainder (p = hi + lo up to 2^-17 relative; O then
 //              takes two MMAs per step).  The running maximum is only raised, and O and the sum rescaled, when it has
@@ -24,11 +24,22 @@
 // V rows past the last key may hold anything; they meet P columns that are zero, but 0 x NaN is NaN: the P V warps zero
 // them before the P V of the last step.
 //
-// What bounds it: ex2.approx issues 16 per clock and SM, 1024 cycles for 128 x 128 scores; the MMAs of those take some 900
-// cycles at head size 64 (1100 with the remainder) and 1850 at 128.  With one S buffer of 128 columns per tile the two
-// tiles fell into step and waited for the tensor core together: 7000 cycles per 2 x 128 x 128 scores.
-// (Encoder, ViT-S, 203 images: 72 us per layer with one tile chain of S, P through shared memory and O; now 58.  Prompt
-// chunks, four of 2048 tokens, 1B decoder: 467 us per layer on mma.sync, 155 TFLOP/s; now 223.  Event-bracketed.)
+// What bounds it: ex2.approx issues 16 per clock and SM, 1024 cycles for a step of two tiles (2 x 128 x 64 scores); the MMAs
+// of those take some 450 cycles at head size 64 (550 with the remainder) and 930 at 128.  A softmax warp is one chain of
+// latencies around its 512 cycles of exponentials: 100 to see its scores, 140 to read them, 250 for the maximum, 150 to hand
+// P over and come around.  So a step is one straight piece of code (cut at every 16 columns it took 1250 cycles for the
+// exponentials alone, now 700), and the two warps of a scheduler take turns at them: in step both waited for the
+// special-function unit and then left it idle together (2450 cycles a step, now 1880; encoder 2000 and 1600).
+//
+// Launches with at most one query tile per SM (`HALF`): one tile per item, whose rows both groups of softmax warps share, 32
+// columns of a step each; the two tell each other the row's maximum.  A tile's chain of steps, which is all the time such a
+// launch takes, is that much shorter (512-token chunk after 1500 cached tokens, 1B decoder: 41 -> 34 us a layer; 509-token
+// prompt 21 -> 17).  Two sums per row, one of either half's columns, keep the order of the additions, so that a row has the
+// same bits in both forms.
+//
+// (Four prompts of 2048 tokens, 1B decoder: 467 us per layer on mma.sync, 223 with P in tensor memory, now 192.  Encoder,
+// ViT-S, 203 images: 72 us, 58, now 53.  Event-bracketed.  Splitting a tile's keys between the two groups, with a merge at the
+// end, shortened the small launches as much but doubled the copies of K and V, whose issue was then the bound: 240 us.)
 // Every mbarrier wait is bounded: when one runs out the kernel records a code in *status, all roles leave their loops,
 // tensor memory is freed and the kernel returns.
 #include <climits>
@@ -60,6 +71,7 @@ struct FlashGeo {
   static constexpr int OFF_KV = 2 * TILE_BYTES;
   static constexpr int OFF_OUT = OFF_KV + STAGES * TILE_BYTES;      // staging: 4 KB (32 rows of 128 bytes) per softmax warp
   static constexpr int OFF_BAR = OFF_OUT + FL_SOFT_WARPS * 4096;
+  // (HALF: the second Q tile's place holds what the two warps of a row tell each other: [3][2][128] floats)
   static constexpr size_t SMEM = 1024 + OFF_BAR + FL_BAR_BYTES;
   static_assert(SMEM <= 227 * 1024, "shared memory of one SM");
 };
@@ -70,7 +82,7 @@ constexpr int FL_S_COL = 0, FL_O_COL = 256;
 // between two looks of its waiter.  K blocks sit in the even slots of the ring, V blocks in the odd ones, whose EMPTY
 // barriers count both P V warps (one that has no tile in the item arrives without an MMA).
 enum { FB_Q_FULL = 0, FB_Q_EMPTY, FB_S_FULL, FB_P_READY = FB_S_FULL + 4, FB_PV_DONE = FB_P_READY + 4, FB_KV_FULL = FB_PV_DONE + 4,
-       FB_KV_EMPTY = FB_KV_FULL + 8, FB_TURN = FB_KV_EMPTY + 8, FB_COUNT = FB_TURN + 8 };
+       FB_KV_EMPTY = FB_KV_FULL + 8, FB_TURN = FB_KV_EMPTY + 8, FB_PAIR = FB_TURN + 8, FB_COUNT = FB_PAIR + 4 };
 static_assert(8 * FB_COUNT + 16 <= FL_BAR_BYTES, "barrier area");
 
 __device__ __forceinline__ float fl_ex2(float x) {
@@ -227,7 +239,7 @@ struct Cursor {
   __device__ __forceinline__ int keys() const { return min(FL_STEP, n_keys - step * FL_STEP); }
 };
 
-template <int HD, bool PAGED, class Group, class View>
+template <int HD, bool PAGED, bool HALF, class Group, class View>
 __global__ void __launch_bounds__(FL_THREADS, 1)
 attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_items, int mt, int* __restrict__ status) {
   using Geo = FlashGeo<HD>;
@@ -244,8 +256,9 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     mbar_init(bar(FB_Q_FULL), 1); mbar_init(bar(FB_Q_EMPTY), 1);
-    for (int i = 0; i < 4; ++i) { mbar_init(bar(FB_S_FULL + i), 1); mbar_init(bar(FB_P_READY + i), 4); mbar_init(bar(FB_PV_DONE + i), 1); }
+    for (int i = 0; i < 4; ++i) { mbar_init(bar(FB_S_FULL + i), 1); mbar_init(bar(FB_P_READY + i), HALF ? 8 : 4); mbar_init(bar(FB_PV_DONE + i), 1); }
     for (int i = 0; i < 8; ++i) mbar_init(bar(FB_TURN + i), 1);
+    for (int i = 0; i < 4; ++i) mbar_init(bar(FB_PAIR + i), 2);
     for (int s = 0; s < ST; ++s) { mbar_init(bar(FB_KV_FULL + s), 1); mbar_init(bar(FB_KV_EMPTY + s), 1 + (s & 1)); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -428,7 +441,10 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
   } else {
     // ------------------------------------------------------------------ softmax (warps 0 .. 7)
     pdl_wait();
-    const int g = warp >> 2, quarter = warp & 3, row = quarter * 32 + lane;
+    // (HALF: warps w and w + 4 share the rows of the one tile, 32 of a step's 64 columns each)
+    const int half = HALF ? warp >> 2 : 0, g = HALF ? 0 : warp >> 2, quarter = warp & 3, row = quarter * 32 + lane;
+    constexpr int NC = HALF ? FL_STEP / 2 : FL_STEP;                // columns of a step that this warp works on
+    float* const told = reinterpret_cast<float*>(base_ptr + Geo::TILE_BYTES) + row;   // [slot][half][128 rows]
     const float scale = 1.4426950408889634f * (HD == 64 ? 0.125f : 0.08838834764831845f);   // log2(e) / sqrt(HD)
     const uint64_t scale2 = pack_f2(scale, scale);
     const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
@@ -436,7 +452,7 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
     unsigned char* const stage = base_ptr + Geo::OFF_OUT + warp * 4096;
     bool ok = true;
     uint32_t cnt = 0;                            // steps of this tile done
-    uint32_t turns = 0;                          // turns waited for
+    uint32_t turns = 0, pairs = 0;               // turns and pair barriers waited for
     View view;
     view.g = nullptr;
     // this tile's next item; decoded while the last P V of the item before is under way
@@ -453,6 +469,16 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
       }
       return false;
     };
+    // What the other half's warp knows of the row: the larger maximum, or the sum of the halves in column order.
+    auto tell = [&](int slot, float mine, float& other) {
+      told[(slot * 2 + half) * FL_TILE] = mine;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(FB_PAIR + quarter));
+      if (!mbar_wait<false>(bar(FB_PAIR + quarter), pairs & 1u, abort_flag)) { if (lane == 0) atomicExch(status, 22); return false; }
+      ++pairs;
+      other = told[(slot * 2 + (half ^ 1)) * FL_TILE];
+      return true;
+    };
     bool more = find_next();
     while (ok && more) {
       const Work w = next;
@@ -465,8 +491,8 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
       const int warp_first = min(w.lim0 + quarter * 32, w.n_keys - 1);                       // ... of the warp's first row
       const int warp_last = min(w.lim0 + min(quarter * 32 + 31, live - 1), w.n_keys - 1);    // ... and of its last
       // the warp of the other tile on this scheduler has as many steps: the two take turns
-      const bool paired = w.n_mt == 2 && quarter * 32 < min(w.live0, w.live1);
-      float m_ref = 0.f, l = 0.f;
+      const bool paired = !HALF && w.n_mt == 2 && quarter * 32 < min(w.live0, w.live1);
+      float m_ref = 0.f, l[2] = {0.f, 0.f};      // sums of a step's first and second half of the columns
       for (int j = 0; j < steps; ++j) {
         const uint32_t b = cnt & 1u, sb = s_addr + b * 64;
         if (!mbar_wait<false>(bar(FB_S_FULL + 2 * g + b), (cnt >> 1) & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 16); break; }
@@ -477,32 +503,37 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
         if (warp_live && !seen) {
           const uint32_t z[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
 #pragma unroll
-          for (int c = 0; c < FL_STEP; c += 8) tmem_st8(sb + c, z);
+          for (int c = 0; c < NC; c += 8) tmem_st8(sb + half * NC + c, z);
           tmem_st_wait();
         }
         // The two warps of a scheduler take turns at the exponentials, so that one's scores are read and reduced while the
         // other keeps the special-function unit busy (in step they left it idle half of the time).
         const bool take_turns = paired && (g == 1 || j > 0), give_turn = paired && (g == 0 || j + 1 < steps);
         if (seen) {
-          uint32_t v[FL_STEP];
-          tmem_ld32_nowait(sb, v);
-          tmem_ld32_nowait(sb + 32, v + 32);
+          uint32_t v[NC];
+          tmem_ld32_nowait(sb + half * NC, v);
+          if (!HALF) tmem_ld32_nowait(sb + 32, v + NC - 32);
           tmem_ld_wait();
 #pragma unroll
-          for (int c = 0; c < 4; ++c) tmem_regs_ready16(v + 16 * c);
+          for (int c = 0; c < NC / 16; ++c) tmem_regs_ready16(v + 16 * c);
           if (k0 + FL_STEP - 1 > warp_first) {                      // some row's limit lies in this step or before it
 #pragma unroll
-            for (int i = 0; i < FL_STEP; ++i) if (k0 + i > lim) v[i] = 0xff800000u;
+            for (int i = 0; i < NC; ++i) if (k0 + half * NC + i > lim) v[i] = 0xff800000u;
           }
           float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
 #pragma unroll
-          for (int i = 0; i < FL_STEP; i += 8) {
+          for (int i = 0; i < NC; i += 8) {
             mx0 = max3(mx0, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
             mx1 = max3(mx1, __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
             mx2 = max3(mx2, __uint_as_float(v[i + 4]), __uint_as_float(v[i + 5]));
             mx3 = max3(mx3, __uint_as_float(v[i + 6]), __uint_as_float(v[i + 7]));
           }
-          const float mx = fmaxf(max3(mx0, mx1, mx2), mx3);
+          float mx = fmaxf(max3(mx0, mx1, mx2), mx3);
+          if (HALF) {
+            float other;
+            if (!tell(j & 1, mx, other)) { ok = false; break; }
+            mx = fmaxf(mx, other);
+          }
           if (j == 0) {
             m_ref = mx;                                             // (key 0 is in every row's reach)
           } else {
@@ -510,12 +541,13 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
             if (__any_sync(0xffffffffu, row_live && (m_new - m_ref) * scale > FL_RAISE)) {
               const float f = fl_ex2((m_ref - m_new) * scale);
               m_ref = m_new;
-              l *= f;
+              l[0] *= f;
+              l[1] *= f;
               // every P V up to the step before must be complete
               if (!mbar_wait<false>(bar(FB_PV_DONE + 2 * g + (b ^ 1u)), ((cnt - 1u) >> 1) & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 17); break; }
               tc_fence_after();
 #pragma unroll 1
-              for (int c = 0; c < HD; c += 16) {
+              for (int c = half * (HD / 2); c < (HALF ? (half + 1) * (HD / 2) : HD); c += 16) {
                 uint32_t o[16];
                 tmem_ld16(o_addr + c, o);
 #pragma unroll
@@ -530,36 +562,39 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
             if (!mbar_wait<false>(bar(FB_TURN + 4 * g + quarter), turns & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 19); break; }
             ++turns;
           }
-          uint64_t l2a = 0, l2b = 0;
           // p = 2^(s * scale - m * scale), its sum and its bf16 parts; one straight piece of code, so that the exponentials of
           // a block of 16 columns run under the conversions of the block before
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const uint32_t* const vc = v + 16 * c;
-            uint32_t hi[8], lo[8];
+          for (int h = 0; h < NC / 32; ++h) {
+            uint64_t l2a = 0, l2b = 0;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              float x, y;
-              unpack_f2(fma_f2(pack_f2(__uint_as_float(vc[2 * i]), __uint_as_float(vc[2 * i + 1])), scale2, nms2), x, y);
-              x = fl_ex2(x);
-              y = fl_ex2(y);
-              const uint64_t p2 = pack_f2(x, y);
-              if (i & 1) l2b = add_f2(l2b, p2); else l2a = add_f2(l2a, p2);
-              hi[i] = pack2(x, y);
-              if (SPLIT) {
-                float rx, ry;
-                unpack_f2(fma_f2(pack_f2(__uint_as_float(hi[i] << 16), __uint_as_float(hi[i] & 0xffff0000u)), minus1, p2), rx, ry);
-                lo[i] = pack2(rx, ry);
+            for (int c = 2 * h; c < 2 * h + 2; ++c) {
+              const uint32_t* const vc = v + 16 * c;
+              uint32_t hi[8], lo[8];
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                float x, y;
+                unpack_f2(fma_f2(pack_f2(__uint_as_float(vc[2 * i]), __uint_as_float(vc[2 * i + 1])), scale2, nms2), x, y);
+                x = fl_ex2(x);
+                y = fl_ex2(y);
+                const uint64_t p2 = pack_f2(x, y);
+                if (i & 1) l2b = add_f2(l2b, p2); else l2a = add_f2(l2a, p2);
+                hi[i] = pack2(x, y);
+                if (SPLIT) {
+                  float rx, ry;
+                  unpack_f2(fma_f2(pack_f2(__uint_as_float(hi[i] << 16), __uint_as_float(hi[i] & 0xffff0000u)), minus1, p2), rx, ry);
+                  lo[i] = pack2(rx, ry);
+                }
               }
+              tmem_st8(sb + half * NC + 16 * c, hi);
+              if (SPLIT) tmem_st8(sb + half * NC + 16 * c + 8, lo);
             }
-            tmem_st8(sb + 16 * c, hi);
-            if (SPLIT) tmem_st8(sb + 16 * c + 8, lo);
+            float a0, a1, a2, a3;
+            unpack_f2(l2a, a0, a1);
+            unpack_f2(l2b, a2, a3);
+            l[h] += (a0 + a1) + (a2 + a3);
           }
           if (give_turn && lane == 0) mbar_arrive(bar(FB_TURN + 4 * (g ^ 1) + quarter));
-          float a0, a1, a2, a3;
-          unpack_f2(l2a, a0, a1);
-          unpack_f2(l2b, a2, a3);
-          l += (a0 + a1) + (a2 + a3);
           tmem_st_wait();
         } else if (paired) {
           if (take_turns) {
@@ -575,39 +610,47 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
       }
       if (!ok) break;
       // ---- the tile's output: rows through this warp's staging area, then whole 128-byte lines
-      const float inv = 1.0f / l;
       const int oy = w.qy + g * w.dy + quarter * 32, ox = w.qx + g * w.dx;
       bf16* const out = wg->out;
       const int ostride = out_stride(wg);
       more = find_next();
       if (!warp_live) continue;
+      float sum = l[0] + l[1];
+      if (HALF) {
+        float other;
+        if (!tell(2, l[0], other)) { ok = false; break; }
+        sum = l[0] + other;
+      }
+      const float inv = 1.0f / sum;
       if (!mbar_wait<false>(bar(FB_PV_DONE + 2 * g + ((cnt - 1u) & 1u)), ((cnt - 1u) >> 1) & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 18); break; }
       tc_fence_after();
+      constexpr int EC = HALF && HD == 64 ? 32 : 64, PIECES = EC / 8;        // columns at a time, their 16-byte pieces
+      const int c_end = HALF ? (half + 1) * (HD / 2) : HD;
 #pragma unroll 1
-      for (int hh = 0; hh < Geo::NH; ++hh) {
-        uint32_t o[64];
-        tmem_ld32_nowait(o_addr + hh * 64, o);
-        tmem_ld32_nowait(o_addr + hh * 64 + 32, o + 32);
+      for (int c = half * (HD / 2); c < c_end; c += EC) {
+        uint32_t o[EC];
+        tmem_ld32_nowait(o_addr + c, o);
+        if (EC == 64) tmem_ld32_nowait(o_addr + c + 32, o + EC - 32);
         tmem_ld_wait();
 #pragma unroll
-        for (int c = 0; c < 4; ++c) tmem_regs_ready16(o + 16 * c);
+        for (int i = 0; i < EC / 16; ++i) tmem_regs_ready16(o + 16 * i);
+        auto place = [&](int r, int k) { return stage + r * (EC * 2) + ((k ^ (EC == 64 ? r & 7 : (r >> 1) & 3)) << 4); };
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
+        for (int k = 0; k < PIECES; ++k) {
           uint4 u;
           u.x = pack2(__uint_as_float(o[8 * k]) * inv, __uint_as_float(o[8 * k + 1]) * inv);
           u.y = pack2(__uint_as_float(o[8 * k + 2]) * inv, __uint_as_float(o[8 * k + 3]) * inv);
           u.z = pack2(__uint_as_float(o[8 * k + 4]) * inv, __uint_as_float(o[8 * k + 5]) * inv);
           u.w = pack2(__uint_as_float(o[8 * k + 6]) * inv, __uint_as_float(o[8 * k + 7]) * inv);
-          *reinterpret_cast<uint4*>(stage + lane * 128 + ((k ^ (lane & 7)) << 4)) = u;
+          *reinterpret_cast<uint4*>(place(lane, k)) = u;
         }
         __syncwarp();
-        const int piece = lane & 7;
+        const int piece = lane % PIECES;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int r = i * 4 + (lane >> 3);
+        for (int i = 0; i < PIECES; ++i) {
+          const int r = i * (32 / PIECES) + lane / PIECES;
           if (quarter * 32 + r < live)
-            *reinterpret_cast<uint4*>(out + (size_t)(oy + r) * ostride + ox + hh * 64 + piece * 8) =
-                *reinterpret_cast<const uint4*>(stage + r * 128 + ((piece ^ (r & 7)) << 4));
+            *reinterpret_cast<uint4*>(out + (size_t)(oy + r) * ostride + ox + c + piece * 8) = *reinterpret_cast<const uint4*>(place(r, piece));
         }
         __syncwarp();
       }
@@ -623,13 +666,20 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
   }
 }
 
+template <int HD, bool PAGED, bool HALF, class Group, class View>
+cudaError_t launch_flash_as(const Group* groups, int n_groups, int total_items, int mt, int* status, int sm_count, cudaStream_t st) {
+  const auto kernel = attn_flash_kernel<HD, PAGED, HALF, Group, View>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FlashGeo<HD>::SMEM);
+  if (e != cudaSuccess) return e;
+  const int grid = total_items < sm_count ? total_items : sm_count;
+  return launch_pdl(kernel, dim3(grid), dim3(FL_THREADS), FlashGeo<HD>::SMEM, st, groups, n_groups, total_items, mt, status);
+}
+
 template <int HD, bool PAGED, class Group, class View>
 cudaError_t launch_flash(const Group* groups, int n_groups, int total_items, int mt, int* status, int sm_count, cudaStream_t st) {
   if (n_groups == 0 || total_items == 0) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(attn_flash_kernel<HD, PAGED, Group, View>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FlashGeo<HD>::SMEM);
-  if (e != cudaSuccess) return e;
-  const int grid = total_items < sm_count ? total_items : sm_count;
-  return launch_pdl(attn_flash_kernel<HD, PAGED, Group, View>, dim3(grid), dim3(FL_THREADS), FlashGeo<HD>::SMEM, st, groups, n_groups, total_items, mt, status);
+  return mt == 1 ? launch_flash_as<HD, PAGED, true, Group, View>(groups, n_groups, total_items, mt, status, sm_count, st)
+                 : launch_flash_as<HD, PAGED, false, Group, View>(groups, n_groups, total_items, mt, status, sm_count, st);
 }
 
 }  // namespace

@@ -140,6 +140,39 @@ def test_prompt_chunk_attention_items_and_running_maximum(mods, Hq, Hkv, hd, kv0
     srv.close()
 
 
+@pytest.mark.parametrize("hd,Hq,Hkv,kv0,n", [(64, 24, 24, 33, 130), (64, 32, 8, 0, 64), (128, 16, 4, 70, 129)])
+def test_a_prompt_chunk_has_the_same_bits_alone_and_in_a_step_of_many_tiles(mods, hd, Hq, Hkv, kv0, n):
+    """Few query tiles (at most one per SM): two warps share a tile's rows and split every step's columns.  More tiles: a
+    warp has rows of its own and two tiles run side by side.  Maximum, exponentials and the order of the sums are the
+    same, hence so are the bits of a chunk alone and next to chunks that fill the chip; one step only, a ragged tile,
+    both head sizes."""
+    E, server = mods
+    p = synth.make_decoder(d=256, n_layers=1, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=hd, ffn=256, vocab=300, seed=50, device=DEV,
+                           std=0.06)
+    rng = np.random.default_rng(51)
+    fill = 1300                                                    # 11 tiles a head: 176 and more of them
+    chunks = [([int(t) for t in rng.integers(0, 300, n)], kv0), ([int(t) for t in rng.integers(0, 300, fill)], 0)]
+    tabs, off = [], 0
+    for tk, k in chunks:
+        tabs.append(torch.as_tensor(_table(rng, k + len(tk), offset=off), device=DEV))
+        off += len(tabs[-1])
+    pool0 = synth.make_kv_pool(1, off + 1, Hkv, hd, seed=52, device=DEV)
+    got = []
+    for together in (False, True):
+        pool = pool0.clone()
+        srv = server.Server(workspace_bytes=512 << 20)
+        m = srv.add_model(p, kv_pool=pool, max_kv_len=1400, max_batch=1500)
+        ts = [srv.submit(m, E.CAT_FS, tokens=tk, kv_len=k, table=tb)
+              for (tk, k), tb in list(zip(chunks, tabs))[:2 if together else 1]]
+        srv.step()
+        torch.cuda.synchronize()
+        s, logits, am = srv.collect(ts[0])
+        assert s == E.OK
+        got.append((logits.clone(), int(am.item())))
+        srv.close()
+    assert torch.equal(got[0][0], got[1][0]) and got[0][1] == got[1][1]
+
+
 def test_prompt_chunks_and_decode_requests_share_a_step(mods):
     """One decoder serving, in ONE step, two prompt chunks (37 tokens on an empty cache; 90 tokens after 21
     cached) and three decode requests, co-resident with a ViT.  Every request equals the oracle; and a
