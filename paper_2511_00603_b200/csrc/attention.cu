@@ -24,22 +24,42 @@ __device__ __forceinline__ uint4 ldg_stream(const uint4* p) {
   return v;
 }
 
-// Merge of the chunk partials of one (request, query head) element e, in chunk order.  Every load is
-// independent of the running sums: unrolled, they are all in flight together.
+// Merge of the chunk partials of one (request, query head), elements e and e + 1, in chunk order.  It is all latency: for
+// up to MERGE_CHUNKS chunks every load is requested before the first one is used.
+constexpr int MERGE_CHUNKS = 16;
 template <int HD>
-__device__ __forceinline__ float merge_chunks(const float* p, int n_chunks, int e) {
-  float mm = -1e30f;
+__device__ __forceinline__ float2 merge_chunks(const float* p, int n_chunks, int e) {
+  float mm = -1e30f, ll = 0.f;
+  float2 oo = make_float2(0.f, 0.f);
+  auto add = [&](float2 ml, float2 o) {
+    const float a = exp2f(ml.x - mm);
+    ll += ml.y * a;
+    oo.x += o.x * a;
+    oo.y += o.y * a;
+  };
+  auto load2 = [](const float* q) { return __ldcg(reinterpret_cast<const float2*>(q)); };
+  if (n_chunks <= MERGE_CHUNKS) {
+    float2 ml[MERGE_CHUNKS], o[MERGE_CHUNKS];
+#pragma unroll
+    for (int ch = 0; ch < MERGE_CHUNKS; ++ch) {
+      ml[ch] = o[ch] = make_float2(-1e30f, 0.f);
+      if (ch < n_chunks) {
+        ml[ch] = load2(p + (size_t)ch * (HD + 2));
+        o[ch] = load2(p + (size_t)ch * (HD + 2) + 2 + e);
+      }
+    }
+#pragma unroll
+    for (int ch = 0; ch < MERGE_CHUNKS; ++ch) mm = fmaxf(mm, ml[ch].x);
+#pragma unroll
+    for (int ch = 0; ch < MERGE_CHUNKS; ++ch)
+      if (ch < n_chunks) add(ml[ch], o[ch]);
+  } else {
 #pragma unroll 8
-  for (int ch = 0; ch < n_chunks; ++ch) mm = fmaxf(mm, __ldcg(p + (size_t)ch * (HD + 2)));
-  float ll = 0.f, oo = 0.f;
+    for (int ch = 0; ch < n_chunks; ++ch) mm = fmaxf(mm, __ldcg(p + (size_t)ch * (HD + 2)));
 #pragma unroll 8
-  for (int ch = 0; ch < n_chunks; ++ch) {
-    const float* pc = p + (size_t)ch * (HD + 2);
-    const float a = exp2f(__ldcg(pc) - mm);
-    ll += __ldcg(pc + 1) * a;
-    oo += __ldcg(pc + 2 + e) * a;
+    for (int ch = 0; ch < n_chunks; ++ch) add(load2(p + (size_t)ch * (HD + 2)), load2(p + (size_t)ch * (HD + 2) + 2 + e));
   }
-  return oo / ll;
+  return make_float2(oo.x / ll, oo.y / ll);
 }
 
 // Last step of a decode-attention block: the four warps' (m, l, o) of this chunk sit in shared
@@ -89,28 +109,35 @@ __device__ __forceinline__ void finish_chunk(const AttnDecGroup& g, int b, int r
   }
   __syncthreads();
   if (!s_last) return;
-  for (int idx = threadIdx.x; idx < G * HD; idx += 128) {
-    const int h = idx / HD, e = idx % HD;
+  for (int idx = threadIdx.x; idx < G * HD / 2; idx += 128) {
+    const int h = idx / (HD / 2), e = idx % (HD / 2) * 2;
     const float* p = g.partial + ((size_t)b * g.Hq + (kvh * G + h)) * g.max_chunks * (HD + 2);
-    g.out[((size_t)row * g.Hq + (kvh * G + h)) * HD + e] = f2bf(merge_chunks<HD>(p, n_chunks, e));
+    const float2 o = merge_chunks<HD>(p, n_chunks, e);
+    *reinterpret_cast<uint32_t*>(g.out + ((size_t)row * g.Hq + (kvh * G + h)) * HD + e) = pack2(o.x, o.y);
   }
 }
 
-// Separate merge for launches with many blocks: one block per (query head, request) of more than one chunk.
+// Separate merge for launches with many blocks: a block takes 256 / HD query heads of a request of more than one chunk.
+// (With a thread per element, the lengths read after the wait and two passes over the partials it took 9.5 us behind the
+// attention of 27 requests of the 1B decoder: 613 us of attention a step, now 522; one request, merged in the attention
+// kernel, 236 and 206.)
+constexpr int COMBINE_THREADS = 128;
 template <int HD>
-__global__ void __launch_bounds__(HD) attn_combine_kernel(const AttnDecGroup* __restrict__ groups, int n_groups) {
+__global__ void __launch_bounds__(COMBINE_THREADS) attn_combine_kernel(const AttnDecGroup* __restrict__ groups, int n_groups) {
   int gi = 0;
   for (int i = 1; i < n_groups; ++i) if ((int)blockIdx.y >= groups[i].req_start) gi = i;
   const AttnDecGroup& g = groups[gi];
-  const int b = blockIdx.y - g.req_start, hq = blockIdx.x;
-  pdl_wait();
-  if (hq >= g.Hq) return;
+  const int b = blockIdx.y - g.req_start, hq = blockIdx.x * (2 * COMBINE_THREADS / HD) + threadIdx.x / (HD / 2);
+  if (!g.reqs_stable) pdl_wait();
   const AttnReq rq = g.reqs[b];
   const int n_chunks = (rq.len + ATTN_CHUNK - 1) / ATTN_CHUNK;
-  if (n_chunks == 1) return;            // finished by the attention kernel itself
-  const float* p = g.partial + ((size_t)b * g.Hq + hq) * g.max_chunks * (HD + 2);
-  const int e = threadIdx.x;
-  g.out[((size_t)rq.row * g.Hq + hq) * HD + e] = f2bf(merge_chunks<HD>(p, n_chunks, e));
+  const float* const p = g.partial + ((size_t)b * g.Hq + hq) * g.max_chunks * (HD + 2);
+  bf16* const out = g.out + ((size_t)rq.row * g.Hq + hq) * HD;
+  if (g.reqs_stable) pdl_wait();
+  if (hq >= g.Hq || n_chunks <= 1) return;            // (one chunk: finished by the attention kernel itself)
+  const int e = threadIdx.x % (HD / 2) * 2;
+  const float2 o = merge_chunks<HD>(p, n_chunks, e);
+  *reinterpret_cast<uint32_t*>(out + e) = pack2(o.x, o.y);
 }
 
 template <int HD, int G>
@@ -524,8 +551,8 @@ static cudaError_t launch_dec(const AttnDecGroup* groups, int n_groups, int tota
 
 // Few blocks (up to two waves): the last block of a (request, kv head) merges the chunks itself and the
 // step saves a launch.  Many blocks: the counter round trip at the end of every block costs more than
-// a second kernel, so the merge runs as attn_combine_kernel (1B decoder, 27 requests: 659 us of attention
-// per step merged in the kernel, 612 with the second one; 8B, 64 requests: 4252 and 3798).
+// a second kernel, so the merge runs as attn_combine_kernel (with the merge as it was then, 1B decoder, 27
+// requests: 659 us of attention per step merged in the kernel, 612 with the second one; 8B, 64 requests: 4252 and 3798).
 bool attn_decode_fused(int total_B, int max_Hkv, int max_chunks, int sm_count) {
   return (long long)total_B * max_Hkv * max_chunks <= 10ll * sm_count;
 }
@@ -544,12 +571,13 @@ cudaError_t launch_attn_decode(const AttnDecGroup* groups, int n_groups, int tot
   EPARA_DEC(32, 1) EPARA_DEC(32, 2) EPARA_DEC(32, 4)
 #undef EPARA_DEC
   if (e != cudaSuccess || fused || max_chunks <= 1) return e;
-  const dim3 grid(max_Hq, total_B);
+  const int heads = 2 * COMBINE_THREADS / hd;
+  const dim3 grid((max_Hq + heads - 1) / heads, total_B), block(COMBINE_THREADS);
   switch (hd) {
-    case 16: return launch_pdl(attn_combine_kernel<16>, grid, dim3(16), 0, st, groups, n_groups);
-    case 32: return launch_pdl(attn_combine_kernel<32>, grid, dim3(32), 0, st, groups, n_groups);
-    case 64: return launch_pdl(attn_combine_kernel<64>, grid, dim3(64), 0, st, groups, n_groups);
-    case 128: return launch_pdl(attn_combine_kernel<128>, grid, dim3(128), 0, st, groups, n_groups);
+    case 16: return launch_pdl(attn_combine_kernel<16>, grid, block, 0, st, groups, n_groups);
+    case 32: return launch_pdl(attn_combine_kernel<32>, grid, block, 0, st, groups, n_groups);
+    case 64: return launch_pdl(attn_combine_kernel<64>, grid, block, 0, st, groups, n_groups);
+    case 128: return launch_pdl(attn_combine_kernel<128>, grid, block, 0, st, groups, n_groups);
   }
   return cudaErrorInvalidValue;
 }
