@@ -89,7 +89,8 @@ struct Op {
   int last_rows;      // norm: output row b reads the last token row of request b
   AttnPrefillGroup apre;
   GemmGroup gemm;
-  MlpGroup mlp;          // EPARA_K_GEMM with gemm.stream == 4: FC1, GELU, FC2 and the residual update in one kernel
+  MlpGroup mlp;          // EPARA_K_GEMM with gemm.stream == 4: FC1, GELU, FC2 and the residual update in one kernel ...
+  GemmGroup fc1, fc2;    // ... and the same as two GEMMs (same bits), for the tiles of a last round that few pairs would work
   NormGroup norm;
   GatherGroup gather;
   RopeGroup rope;
@@ -261,9 +262,15 @@ bool add_gemm(Builder& bl, Model* m, const void* A, int lda, long long rows_cap,
 // An encoder's MLP block as one fused op (see MlpGroup).  gemm.N / gemm.K carry the shapes for the step's
 // flop and byte accounting; gemm.stream == 4 routes the op to the fused kernel's launch.
 bool add_mlp(Builder& bl, Model* m, const void* X, long long rows_cap, const void* W1, const void* b1, const void* W2,
-             const void* b2, float* Z, int d, int F, int rows_per_req) {
+             const void* b2, float* Z, bf16* hidden, int d, int F, int rows_per_req) {
   Op op;
   memset(&op, 0, sizeof(op));
+  if (!add_gemm(bl, m, X, d, rows_cap, W1, F, d, hidden, F, b1, EPI_GELU, rows_per_req, true)) return false;
+  op.fc1 = m->ops.back().gemm;
+  m->ops.pop_back();
+  if (!add_gemm(bl, m, hidden, F, rows_cap, W2, d, F, Z, d, b2, EPI_RESID_F32, rows_per_req, true)) return false;
+  op.fc2 = m->ops.back().gemm;
+  m->ops.pop_back();
   op.kind = EPARA_K_GEMM;
   op.rows_per_req = rows_per_req;
   op.gemm.stream = 4; op.gemm.N = d; op.gemm.K = F; op.gemm.ksplit = 1; op.gemm.bn = d;
@@ -407,7 +414,7 @@ int build_model(Builder& bl, Model* m, const epara_config& cfg) {
       if (!add_gemm(bl, m, a, dm, Mcap, w[4], dm, dm, z, dm, w[5], EPI_RESID_F32, T)) return EPARA_E_CUDA;
       add_norm(m, z, dm, h, w[6], w[7], dm, NORM_LN, 1e-6f, T);
       if (bl.gemm_impl == EPARA_GEMM_TCGEN05 && gemm_mlp_eligible(Mcap, dm, d.ffn)) {
-        if (!add_mlp(bl, m, h, Mcap, w[8], w[9], w[10], w[11], z, dm, d.ffn, T)) return EPARA_E_CUDA;
+        if (!add_mlp(bl, m, h, Mcap, w[8], w[9], w[10], w[11], z, f, dm, d.ffn, T)) return EPARA_E_CUDA;
       } else {
         // (where the fused block exists, its two GEMMs on their own keep its order of summation)
         const bool one_sum = gemm_mlp_eligible(Mcap, dm, d.ffn);
@@ -1006,6 +1013,24 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       }
       for (int pass = 0; pass < n_pass; ++pass) {
       if (!((passes >> pass) & 1u)) continue;
+      // Tiles of the fused MLP kernel's last round, when they are few: the launch takes as long for one tile per pair as for
+      // a single one, so they go to the two GEMM kernels instead, which spread them over the chip (ViT-S, 12 blocks on 74 pairs: 2 tiles
+      // in the last round 2126 -> 1921 us a step, 9 3483 -> 3263, 26 3638 -> 3523, 37 3752 -> 3692, 49 3960 -> 4000).
+      Active* cut = nullptr;                                   // the model that gives them away
+      int cut_tiles = 0;
+      if (pass == PASS_MLP && kind == EPARA_K_GEMM) {
+        const int pairs = c->sm_count / 2;
+        int tiles = 0, most = 0;
+        for (Active* a : who) {
+          const Op& op = a->m->ops[a->cursor];
+          if (op.gemm.stream != 4) continue;
+          const int t = (a->B * op.rows_per_req + 2 * TC_BM - 1) / (2 * TC_BM);
+          tiles += t;
+          if (t > most) { most = t; cut = a; }
+        }
+        cut_tiles = tiles > pairs ? tiles % pairs : 0;
+        if (cut_tiles == 0 || cut_tiles > pairs / 2 || cut_tiles >= most) cut = nullptr;
+      }
       Launch L;
       memset(&L, 0, sizeof(L));
       L.kind = kind;
@@ -1117,6 +1142,10 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
               MlpGroup mg = op.mlp;
               mg.M = rows;
               mg.tiles_m = (rows + 2 * TC_BM - 1) / (2 * TC_BM);
+              if (a == cut) {
+                mg.tiles_m -= cut_tiles;
+                mg.M = mg.tiles_m * 2 * TC_BM;
+              }
               mg.tile_start = total;
               total += mg.tiles_m;
               ++n_put;
@@ -1196,6 +1225,22 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
         if (n_put == 0) continue;
       }
       launches.push_back(L);
+      if (cut) {
+        const Op& op = cut->m->ops[pass == n_pass - 1 ? cut->cursor - 1 : cut->cursor];
+        for (const GemmGroup* part : {&op.fc1, &op.fc2}) {
+          GemmGroup g = *part;
+          g.M = cut->B * op.rows_per_req;
+          g.tiles_m = (g.M + 2 * TC_BM - 1) / (2 * TC_BM); g.tiles_n = (g.N + g.bn - 1) / g.bn;
+          g.tile_start = -(g.tiles_m - cut_tiles) * g.tiles_n;           // items 0 .. are the last tiles
+          Launch R;
+          memset(&R, 0, sizeof(R));
+          R.kind = kind; R.n_groups = 1; R.p0 = cut_tiles * g.tiles_n; R.p2 = 2;
+          off = align_up(off, 64);
+          R.off = off;
+          if (put(&g, sizeof(g), 64) == (size_t)-1) overflow = true;
+          launches.push_back(R);
+        }
+      }
       }
     }
   }

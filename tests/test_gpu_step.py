@@ -454,3 +454,30 @@ def test_fused_encoder_mlp_block_equals_the_unfused_kernels_and_the_oracle(mods,
         ref, _, _ = O.vit_forward(synth.to_bits(imgs[i]), v)
         assert_close(fused[i][0], ref, what=f"fused MLP block, d={d}, image {i}")
         check_argmax(fused[i][1], fused[i][0], ref)
+
+
+@pytest.mark.parametrize("d,heads,mlp,B", [(128, 2, 256, 98), (384, 6, 1536, 99)])
+def test_last_round_of_fused_mlp_tiles_goes_to_the_gemm_kernels(mods, d, heads, mlp, B):
+    """More 256-row tiles than CTA pairs, by a few: the last ones (the very last ragged) run as two GEMMs next to the fused
+    kernel.  Every logit has the bits of the model whose GEMMs are all their own launches, and the last image, whose rows
+    are in those tiles, equals the oracle."""
+    E, server = mods
+    p = synth.make_vit(d=d, n_layers=1, n_heads=heads, mlp=mlp, n_cls=50, seed=7, device=DEV, std=0.05, perturb=0.2)
+    imgs = synth.make_images(B, seed=8, device=DEV)
+
+    def run(impl):
+        srv = server.Server(workspace_bytes=2 << 30, gemm_impl=impl)
+        m = srv.add_model(p, max_batch=B)
+        ts = [srv.submit(m, E.CAT_FS, x=imgs[i]) for i in range(B)]
+        info = srv.step()
+        res = _finish(srv, E, ts)
+        srv.close()
+        return info, res
+
+    fused_info, fused = run(E.GEMM_TCGEN05)
+    plain_info, plain = run(E.GEMM_TCGEN05_UNFUSED)
+    assert fused_info.launches == plain_info.launches + 1               # the fused launch and two for the last tiles
+    for i in range(B):
+        assert torch.equal(fused[i][0], plain[i][0]) and fused[i][1] == plain[i][1]
+    ref, _, _ = O.vit_forward(synth.to_bits(imgs[B - 1]), synth.bits_view(p))
+    assert_close(fused[B - 1][0], ref, what=f"last MLP tiles, d={d}")
