@@ -150,6 +150,9 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
   } else if (warp == SW_A_WARP) {
     // ------------------------------------------------------------ TMA producer of the activations (tmA: box of nb rows)
     tensormap_acquire(&g->tmA);
+    // the first copy after the wait finds its map (1B decoder, 27 requests: 1226 -> 1210 us a step; the larger tiles of the
+    // tile-pair kernel and attention gained nothing)
+    tensormap_prefetch_elect(&g->tmA);
     pdl_wait();
     int stage = 0;
     uint32_t phase = 0;

@@ -94,6 +94,11 @@ __device__ __forceinline__ void tensormap_acquire(const CUtensorMap* tm) {
   asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(tm) : "memory");
 }
 
+// One lane of a converged warp asks for the map ahead of its first copy.
+__device__ __forceinline__ void tensormap_prefetch_elect(const CUtensorMap* tm) {
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t@q prefetch.tensormap [%0];\n\t}" ::"l"(tm) : "memory");
+}
+
 // K-major operand tile in shared memory, rows of 128 bytes, 128-byte swizzle, 8-row groups 1024
 // bytes apart (what a TMA box of 64 bf16 x rows with SWIZZLE_128B produces).
 __device__ __forceinline__ uint64_t make_smem_desc(uint32_t addr) {
