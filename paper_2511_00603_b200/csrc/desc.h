@@ -60,8 +60,8 @@ struct alignas(64) GemmGroup {
                    // block, tiles_n = ceil(N / 16), no TMA maps); 2: 256-row tiles on CTA pairs (tiles_m counts 256-row
                    // tiles and tmW's box holds bn / 2 rows); 3: swapped operands (tmA's box holds bn rows, tmW's
                    // 128); 0: plain CUDA-core comparator
-  int pad1, pad2;
-  int pad3[4];
+  const ReqDesc* reqs;   // weight-streaming kernel: when set, row m of A is request m's input (an MLP's first layer)
+  int pad[4];
 };
 
 struct GemmLaunch {      // header followed by groups

@@ -87,6 +87,7 @@ struct Op {
   int rows_per_req;   // rows of this op = batch * rows_per_req ...
   int per_token;      // ... or, for a decoder's token-wise ops, the step's token rows (a prompt chunk has several)
   int last_rows;      // norm: output row b reads the last token row of request b
+  int from_requests;  // GEMM: the rows of A are the requests' inputs
   AttnPrefillGroup apre;
   GemmGroup gemm;
   MlpGroup mlp;          // EPARA_K_GEMM with gemm.stream == 4: FC1, GELU, FC2 and the residual update in one kernel ...
@@ -345,14 +346,16 @@ int build_model(Builder& bl, Model* m, const epara_config& cfg) {
     const int L = d.n_layers;
     int maxw = 0;
     for (int i = 1; i <= L; ++i) maxw = std::max(maxw, round_up(m->dims[i], 8));
-    bf16* x0 = (bf16*)bl.get((size_t)Bcap * m->dims[0] * 2);
+    // the weight-streaming kernel reads the requests' inputs where they are; the others want them in one matrix
+    const bool direct = bl.gemm_impl != EPARA_GEMM_SIMT && gemm_stream_eligible(m->max_batch, m->dims[1], m->dims[0]);
+    bf16* x0 = direct ? nullptr : (bf16*)bl.get((size_t)Bcap * m->dims[0] * 2);
     bf16* pp[2] = {(bf16*)bl.get((size_t)Bcap * maxw * 2), (bf16*)bl.get((size_t)Bcap * maxw * 2)};
     if (bl.fail) return EPARA_E_RESOURCE;
     Op g;
     memset(&g, 0, sizeof(g));
     g.kind = EPARA_K_GATHER; g.rows_per_req = 1;
     g.gather.kind = GATHER_ROWS; g.gather.out = x0; g.gather.width = m->dims[0]; g.gather.ld = m->dims[0];
-    m->ops.push_back(g);
+    if (!direct) m->ops.push_back(g);
     const bf16* in = x0;
     int ld_in = m->dims[0];
     for (int l = 0; l < L; ++l) {
@@ -360,6 +363,7 @@ int build_model(Builder& bl, Model* m, const epara_config& cfg) {
       bf16* out = pp[l & 1];
       if (!add_gemm(bl, m, in, ld_in, Bcap, t[2 * l], N, K, out, ldc, t[2 * l + 1], (l + 1 < L) ? EPI_GELU : 0, 1))
         return EPARA_E_CUDA;
+      if (l == 0 && direct) m->ops.back().from_requests = 1;
       in = out; ld_in = ldc;
     }
     Op o;
@@ -1171,6 +1175,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
               g.tile_start = total;
               total += g.tiles_m * g.tiles_n;
               mx = std::max(mx, rows);
+              if (op.from_requests) g.reqs = (const ReqDesc*)(slot.dev + a->req_off);
             } else {
               g.tiles_m = (rows + SIMT_TILE - 1) / SIMT_TILE; g.tiles_n = (g.N + SIMT_TILE - 1) / SIMT_TILE;
               g.tile_start = total;

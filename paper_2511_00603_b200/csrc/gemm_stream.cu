@@ -85,7 +85,8 @@ gemm_stream_kernel(const GemmGroup* __restrict__ groups, int n_groups) {
 #pragma unroll
   for (int t = 0; t < NT; ++t) {
     x_ok[t] = t * 8 + gq < M;
-    x_row[t] = g.A + (size_t)(m0 + t * 8 + gq) * g.lda + tq * 8;
+    const int m = m0 + t * 8 + gq;
+    x_row[t] = (g.reqs && x_ok[t] ? reinterpret_cast<const bf16*>(g.reqs[m].input) : g.A + (size_t)m * g.lda) + tq * 8;
   }
   float acc[NT][4];
 #pragma unroll

@@ -481,3 +481,25 @@ def test_last_round_of_fused_mlp_tiles_goes_to_the_gemm_kernels(mods, d, heads, 
         assert torch.equal(fused[i][0], plain[i][0]) and fused[i][1] == plain[i][1]
     ref, _, _ = O.vit_forward(synth.to_bits(imgs[B - 1]), synth.bits_view(p))
     assert_close(fused[B - 1][0], ref, what=f"last MLP tiles, d={d}")
+
+
+@pytest.mark.parametrize("cap,B", [(1, 1), (8, 8), (16, 11), (17, 17), (128, 100), (128, 128)])
+def test_first_mlp_layer_reads_the_requests_inputs_in_place(mods, cap, B):
+    """A model placed for up to 128 requests has no gather launch: its first layer reads every request's row where the
+    caller left it (rows of a larger array here, in another order than the requests), up to 16 rows and in tiles of
+    32; a launch less than the model's layers and the gather would take; every request equals the oracle."""
+    E, server = mods
+    p = synth.make_mlp([264, 136, 24], seed=9, device=DEV, perturb=0.3, std=0.1)
+    x = synth.make_mlp_inputs(2 * B, 264, seed=10, device=DEV)
+    order = np.random.default_rng(cap + B).permutation(2 * B)[:B]
+    srv = server.Server(workspace_bytes=64 << 20)
+    m = srv.add_model(p, max_batch=cap)
+    ts = [srv.submit(m, E.CAT_FS, x=x[int(i)]) for i in order]
+    info = srv.step()
+    assert info.launches == 3                                           # two layers and the output
+    v = synth.bits_view(p)
+    for i, (logits, am) in zip(order, _finish(srv, E, ts)):
+        ref, _ = O.mlp_forward(synth.to_bits(x[int(i)]), v["W"], v["b"])
+        assert_close(logits, ref, what=f"input {i} of {cap}")
+        check_argmax(am, logits, ref)
+    srv.close()
