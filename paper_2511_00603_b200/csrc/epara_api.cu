@@ -175,6 +175,7 @@ struct epara_ctx {
   std::unordered_map<uint64_t, Ticket> tickets;
   uint64_t next_ticket, next_step;
   Slot slots[N_SLOTS];
+  unsigned char* pinned;
   uint64_t last_step_slot;
   int max_profile_launches;
 };
@@ -675,6 +676,8 @@ int epara_init(const epara_config* cfg, epara_ctx** out) {
   int sm = 0;
   if (cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, cfg->device) != cudaSuccess) { delete c; return EPARA_E_CUDA; }
   c->sm_count = sm;
+  // one pinned block for every slot's blob and status word: pinning is most of what creating a context costs
+  if (cudaMallocHost((void**)&c->pinned, N_SLOTS * (BLOB_BYTES + 64)) != cudaSuccess) { delete c; return EPARA_E_CUDA; }
   for (int i = 0; i < N_SLOTS; ++i) {
     Slot& s = c->slots[i];
     s.dev = (unsigned char*)carve(c, BLOB_BYTES);
@@ -682,11 +685,9 @@ int epara_init(const epara_config* cfg, epara_ctx** out) {
     s.busy = false;
     s.profiled = false;
     s.launch_status = EPARA_OK;
-    if (cudaMallocHost((void**)&s.host, BLOB_BYTES) != cudaSuccess ||
-        cudaMallocHost((void**)&s.status_host, 64) != cudaSuccess ||
-        cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming) != cudaSuccess) {
-      return EPARA_E_CUDA;
-    }
+    s.host = c->pinned + i * (BLOB_BYTES + 64);
+    s.status_host = reinterpret_cast<int*>(s.host + BLOB_BYTES);
+    if (cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming) != cudaSuccess) return EPARA_E_CUDA;
     *s.status_host = 0;
   }
   *out = c;
@@ -701,9 +702,8 @@ int epara_destroy(epara_ctx* c) {
     if (s.busy) cudaEventSynchronize(s.done);
     for (cudaEvent_t e : s.prof) cudaEventDestroy(e);
     cudaEventDestroy(s.done);
-    cudaFreeHost(s.host);
-    cudaFreeHost(s.status_host);
   }
+  cudaFreeHost(c->pinned);
   for (Model* m : c->models) delete m;
   delete c;
   return EPARA_OK;
