@@ -23,12 +23,10 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
-# DRAM bytes (read + write) per tensor-core GEMM launch of the mixed step, from one ncu pass over the GEMM
-# launches of a step (65 tile-pair launches: 7.72 GB read + 3.69 GB written; 12 fused MLP-block launches:
-# 2.90 GB read + 1.18 GB written; the 65 weight-streaming launches moved 2.08 GB).  Not measured by this run:
-# the profile it comes from is named beside it in the JSON line.  Set to None when the GEMM kernels change.
-GEMM_TC_TRAFFIC_PER_LAUNCH_MIXED = 15488294144 / 77
-GEMM_TRAFFIC_SOURCE = "profiles/gemm_kernels_mixed_step_dram_traffic.md (one ncu pass, dram__bytes_read.sum + dram__bytes_write.sum)"
+# DRAM bytes (read + write) per tensor-core GEMM launch of the mixed step, from an ncu pass over the GEMM launches of
+# a step.  Not measured by this run.  None: no pass has been made since the GEMM kernels changed.
+GEMM_TC_TRAFFIC_PER_LAUNCH_MIXED = None
+GEMM_TRAFFIC_SOURCE = None
 
 E2E_BUFS = 4          # device input buffers per instance in the end-to-end loop
 PROFILE_EVERY = 5     # one step in five of the timed region carries per-launch events
@@ -555,8 +553,8 @@ def run_gpu(args):
         return 0
 
     # ---- roofline of the dominant kernel ----
-    # The GEMM launches of a step are two kinds of work: tensor-core launches (tile pairs and one-CTA tiles),
-    # judged against the tensor peak, and weight-streaming launches (groups of at most 16 rows), judged against
+    # The GEMM launches of a step are two kinds of work: tensor-core launches (tile pairs, swapped
+    # operands), judged against the tensor peak, and weight-streaming launches (few rows, small matrices), judged against
     # HBM.  The timed region is a fraction of a second; which bf16 peak applies depends on the clock it ran at,
     # so both fractions are given beside the sampled clock: the burst peak when the median SM clock stayed
     # within 10 % of the maximum, the sustained (power-capped) peak otherwise.
