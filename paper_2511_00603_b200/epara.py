@@ -282,7 +282,7 @@ class Context:
 
     def epara_collect(self, ticket: int):
         out = Output()
-        s = lib.epara_collect(self.h, ticket, C.byref(out))
+        s = lib.epara_collect(self.h, ticket, out)     # (ctypes takes the address; an explicit byref adds a quarter to the call)
         return s, out
 
     def epara_set_profile(self, on: bool):
