@@ -118,8 +118,10 @@ typedef struct {
 typedef struct {
   const void* input;        /* device: MLP bf16 [dims[0]]; VIT bf16 [3, img, img]; DECODER: NULL */
   int token;                /* decoder: id of the token being decoded */
-  int kv_len;               /* decoder: cached tokens L, written by earlier steps or by the caller before this one; the
-                               new token is written at slot L and attention runs over L + 1 tokens */
+  int kv_len;               /* decoder: cached tokens L; the new token is written at slot L and attention runs over
+                               L + 1 tokens.  They were written by earlier steps, by the caller before this one, or by
+                               other requests of this step: a step appends all its keys and values before any of its
+                               requests attends, so the tokens of one sequence may come as several requests of a step */
   const int32_t* block_table; /* device int32 [n_blocks], page ids; needs n_blocks >= (L + n - 1)/16 + 1 */
   int n_blocks;
   const int32_t* tokens;    /* decoder, HOST, read during epara_submit only: with n_tokens = n > 1 the request is a

@@ -10,6 +10,7 @@
 //
 // Encoder (ViT): full bidirectional attention of T tokens per (image, head).
 #include <cstring>
+#include <type_traits>
 
 #include "../../include/epara.h"
 #include "common.cuh"
@@ -286,8 +287,10 @@ __global__ void __launch_bounds__(128) attn_decode_kernel(const AttnDecGroup* __
 // are XOR-swizzled by the token index, so ldmatrix reads are free of bank conflicts.
 // With AttnDecGroup::cs the kernel also does RoPE and the append for its request: q is rotated as it is
 // read, the block that holds position len - 1 rotates k, writes k and v to the cache and into its
-// staged tile, and the cached pages, which no kernel of the step writes, are requested before the wait
-// on the QKV projection.  That takes a launch out of every layer.
+// staged tile, and the cached pages are requested before the wait on the QKV projection.  That takes a
+// launch out of every layer.  Requests of one sequence in one step (known tokens scored in one go, a token behind the
+// prompt chunk of the same step) attend to what the others append: the step's first kernel marks them (GATHER_LINK) and
+// they read those tokens out of qkv.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
@@ -318,10 +321,48 @@ __device__ __forceinline__ uint32_t transpose_8x8(uint32_t u) {
   asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(u));
   return r;
 }
-// RoPE of one interleaved pair of bf16
-__device__ __forceinline__ uint32_t rotate_pair(uint32_t u, float2 cs) {
-  const float a = __uint_as_float(u << 16), b = __uint_as_float(u & 0xffff0000u);
-  return pack2(a * cs.x - b * cs.y, a * cs.y + b * cs.x);
+
+// k (rotated to `cs_row`) and v of one kv head of an unrotated qkv row, to slot r of a staged tile (K, then V HD * 32 bytes
+// on) and, with dst, to the cache (V HD * 8 * Hkv words on): a pair per lane and piece.
+template <int HD>
+__device__ __forceinline__ void place_kv(unsigned char* tile, int r, const uint32_t* kr, int Hkv, const float2* cs_row, uint32_t* dst) {
+  const int lane = threadIdx.x & 31;
+  unsigned char* const kt = tile + r * (HD * 2);
+#pragma unroll
+  for (int p = 0; p < HD / 64; ++p) {
+    const int pair = p * 32 + lane, c = pair >> 2;
+    const uint32_t nk = rotate_pair(kr[pair], __ldg(cs_row + pair)), nv = kr[Hkv * (HD / 2) + pair];
+    if (dst != nullptr) {
+      dst[pair] = nk;
+      dst[Hkv * 8 * HD + pair] = nv;
+    }
+    const int off = (c & ~7) * 16 + (((c & 7) ^ (r & 7)) << 4) + (pair & 3) * 4;
+    *reinterpret_cast<uint32_t*>(kt + off) = nk;
+    *reinterpret_cast<uint32_t*>(kt + 16 * HD * 2 + off) = nv;
+  }
+}
+
+// Several requests of one sequence in one step: a staged tile's slots below n_slots that other rows of the step append to
+// this page are taken from those rows, since the append itself may stand before, beside or behind this block's read.
+template <int HD>
+__device__ __forceinline__ void place_step_rows(const AttnDecGroup& g, unsigned char* tile, int page, int kvh, int own_row, int n_slots) {
+  const int lane = threadIdx.x & 31;
+  for (int w0 = 0; w0 < g.n_rows; w0 += 32) {
+    const int w = w0 + lane;
+    int at = 0;
+    bool hit = false;
+    if (w < g.n_rows && w != own_row) {
+      const RowDesc rd = g.rows[w];
+      at = rd.pos;
+      hit = (at & 15) < n_slots && g.step_reqs[rd.req].table[at >> 4] == page;
+    }
+    for (unsigned m = __ballot_sync(0xffffffffu, hit); m != 0; m &= m - 1) {
+      const int l = __ffs(m) - 1, p = __shfl_sync(0xffffffffu, at, l);
+      const bf16* const row = g.q + (size_t)(w0 + l) * g.q_stride + (size_t)(g.Hq + kvh) * HD;
+      place_kv<HD>(tile, p & 15, reinterpret_cast<const uint32_t*>(row), g.Hkv, g.cs + (size_t)p * (HD / 2), nullptr);
+    }
+  }
+  __syncwarp();
 }
 
 template <int HD, int G, int NSLOT>
@@ -390,9 +431,11 @@ __global__ void __launch_bounds__(128) attn_decode_mma_kernel(const AttnDecGroup
   };
 #pragma unroll
   for (int i = 0; i < NSLOT; ++i) issue(i);
-  // (With cs the step's earlier kernels write nothing of the cache below `pos`: its pages are requested while the QKV
-  // projection may still be running.  The slot of `pos` holds something old and is overwritten in shared memory below.)
+  // (With cs the pages are requested while the QKV projection may still be running.  A slot that the step itself writes holds
+  // something old, or half of something: that of `pos`, and those of other requests of the same sequence (`linked`), which
+  // are replaced in shared memory below.  Everything else was written by earlier steps or by the caller.)
   if (early) pdl_wait();
+  const bool linked = g.linked != nullptr && __ldcg(g.linked + b) != 0;
 
   // ---- Q fragments: the query heads of this kv head are the first G of the B operand's 8 columns
   const bf16* const row0 = g.q + (size_t)rq.row * g.q_stride;
@@ -417,29 +460,20 @@ __global__ void __launch_bounds__(128) attn_decode_mma_kernel(const AttnDecGroup
   float m_run[2] = {-1e30f, -1e30f}, l_run[2] = {0.f, 0.f};     // heads 2tq, 2tq+1; the sums are this lane's tokens'
   const int lm_row = lane & 7, lm_mat = lane >> 3;
 
-  auto process = [&](int i) {
+  auto process = [&](int i, auto shared) {
     const int pg = page_begin + warp + 4 * i;
     if (pg >= page_end || (bad_mask & (1u << i))) return;
     const uint32_t kd = wsm_u + (i % NSLOT) * 2 * TILE, vd = kd + TILE;
     const int tok0 = pg * 16;
     if (app_page >= 0 && pg == pos >> 4) {
-      // the new token: k (rotated) and v of this kv head to the cache and into the staged tile, a pair per lane and piece
+      // the new token: k (rotated) and v of this kv head to the cache and into the staged tile
       const int r = pos & 15;
-      unsigned char* const kt = wsm + (i % NSLOT) * 2 * TILE + r * ROWB;
-      const uint32_t* const kr = reinterpret_cast<const uint32_t*>(row0 + (size_t)(g.Hq + kvh) * HD);
-      uint32_t* const dst = reinterpret_cast<uint32_t*>(kv_layer + (((size_t)app_page * 2) * Hkv + kvh) * 16 * HD + (size_t)r * HD);
-#pragma unroll
-      for (int p = 0; p < HD / 64; ++p) {
-        const int pair = p * 32 + lane, c = pair >> 2;
-        const uint32_t nk = rotate_pair(kr[pair], __ldg(cs + (size_t)pos * (HD / 2) + pair)), nv = kr[Hkv * (HD / 2) + pair];
-        dst[pair] = nk;
-        dst[Hkv * 8 * HD + pair] = nv;
-        const int off = (c & ~7) * 16 + (((c & 7) ^ (r & 7)) << 4) + (pair & 3) * 4;
-        *reinterpret_cast<uint32_t*>(kt + off) = nk;
-        *reinterpret_cast<uint32_t*>(kt + TILE + off) = nv;
-      }
+      place_kv<HD>(wsm + (i % NSLOT) * 2 * TILE, r, reinterpret_cast<const uint32_t*>(row0 + (size_t)(g.Hq + kvh) * HD), Hkv,
+                   cs + (size_t)pos * (HD / 2),
+                   reinterpret_cast<uint32_t*>(kv_layer + (((size_t)app_page * 2) * Hkv + kvh) * 16 * HD + (size_t)r * HD));
       __syncwarp();
     }
+    if constexpr (decltype(shared)::value) place_step_rows<HD>(g, wsm + (i % NSLOT) * 2 * TILE, rq.table[pg], kvh, rq.row, pos - tok0);
     if (tok0 + 16 > t_end) {
       // slots past the length may hold anything (NaN included): zero those V rows
       const int valid = t_end - tok0;
@@ -500,13 +534,19 @@ __global__ void __launch_bounds__(128) attn_decode_mma_kernel(const AttnDecGroup
       mma_bf16_m16n8k16(o[np], vr, pb0, pb1);
     }
   };
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  auto step = [&](int i, auto shared) {
     cp_async_wait<NSLOT - 1>();              // page i has landed (one group is committed per step)
     __syncwarp();
-    process(i);
+    process(i, shared);
     __syncwarp();                            // the slot is free again
     issue(i + NSLOT);
+  };
+  if (!linked) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) step(i, std::false_type());
+  } else {
+#pragma unroll 1
+    for (int i = 0; i < 4; ++i) step(i, std::true_type());
   }
 
 #pragma unroll

@@ -57,6 +57,13 @@ __device__ __forceinline__ unsigned pack2(float lo, float hi) {
   return *reinterpret_cast<unsigned*>(&v);
 }
 
+// RoPE of one interleaved pair of bf16.  The roundings are spelled out: a key has the same bits wherever it is rotated.
+__device__ __forceinline__ unsigned rotate_pair(unsigned u, float c, float s) {
+  const float a = __uint_as_float(u << 16), b = __uint_as_float(u & 0xffff0000u);
+  return pack2(__fmaf_rn(a, c, -__fmul_rn(b, s)), __fmaf_rn(a, s, __fmul_rn(b, c)));
+}
+__device__ __forceinline__ unsigned rotate_pair(unsigned u, float2 cs) { return rotate_pair(u, cs.x, cs.y); }
+
 // GELU in its erf form, 0.5 x (1 + erf(x / sqrt 2)), evaluated as 0.5 x (1 + tanh(x P(x^2))) with
 // P(t) = a + b t + c t^2 fitted (minimax over |x| <= 8) so that tanh(x P(x^2)) follows erf(x / sqrt 2):
 // the formula itself is within 2.6e-5 of the erf form everywhere.  t is clamped at 64, where the

@@ -81,16 +81,24 @@ struct NormGroup {
   float eps;
 };
 
-enum : int { GATHER_ROWS = 0, GATHER_EMB = 1, GATHER_PATCH = 2 };
+struct AttnReq {
+  const int32_t* table;
+  int len;               // tokens to attend (cached + appended)
+  int row;               // activation row of the request's token (q is read and the output written there)
+};
+
+// LINK: finds the decode requests that attend to tokens which other requests of the step append (see AttnDecGroup::linked).
+enum : int { GATHER_ROWS = 0, GATHER_EMB = 1, GATHER_PATCH = 2, GATHER_LINK = 3 };
 struct GatherGroup {
   const ReqDesc* reqs;
   const RowDesc* rows;   // EMB: one entry per output row
-  void* out;             // ROWS: bf16 [B, ld]; EMB: fp32 [rows, d]; PATCH: bf16 [B*np, 3*p*p]
+  const AttnReq* areqs;  // LINK: the decode requests, one block each; B counts all requests, n_pre of them prompt chunks
+  void* out;             // ROWS: bf16 [B, ld]; EMB: fp32 [rows, d]; PATCH: bf16 [B*np, 3*p*p]; LINK: int [decode requests]
   const bf16* emb;       // EMB
   int kind, B, width, ld;
   int img, patch;
   int blocks;            // blocks this group needs
-  int pad;
+  int n_pre;
 };
 
 struct RopeGroup {
@@ -104,12 +112,6 @@ struct RopeGroup {
   int B, Hq, Hkv, hd;
   int only_chunks;       // 1: decode rows are left alone (the attention kernel rotates and appends them itself)
   int pad;
-};
-
-struct AttnReq {
-  const int32_t* table;
-  int len;               // tokens to attend (cached + appended)
-  int row;               // activation row of the request's token (q is read and the output written there)
 };
 
 // Causal attention of prompt chunks (one layer): a request has n_tok query tokens in consecutive rows, token t at position
@@ -151,6 +153,13 @@ struct AttnDecGroup {
                          // length may leave without the dependency wait); 0: an earlier kernel writes it
   int* status;           // device word: set to ERR_PAGE_ATTEND when a block table names a page outside the pool
   long long kv_pages;    // pages of the pool; a page id outside [0, kv_pages) is reported and read as absent
+  // With cs, in a step of several requests: linked[b] != 0 when request b may attend to tokens that other rows of the
+  // step append (requests of one sequence in one step).  The block takes those from qkv then, wherever the append stands.
+  const int* linked;     // null: a single request
+  const RowDesc* rows;
+  const ReqDesc* step_reqs;
+  int n_rows;
+  int pad;
 };
 
 struct alignas(64) AttnEncGroup {

@@ -810,8 +810,9 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
   // n_pre prompt-chunk requests of a decoder, with their descriptor arrays in the blob
   struct PrefillChunk { const int32_t* table; int row_start, n_tok, kv_len; };
   struct Active {
-    Model* m; int B; int rows; size_t req_off; size_t areq_off; size_t row_off; size_t pitem_off; size_t last_off; size_t cursor;
+    Model* m; int B; int rows; size_t req_off; size_t areq_off; size_t row_off; size_t pitem_off; size_t last_off; size_t link_off; size_t cursor;
     int n_dec, n_pre, max_chunks_dec, pre_items;
+    bool append_first;   // decode rows are rotated and appended by a launch of their own, before any attention of the wave
     std::vector<PrefillChunk> pre;
     std::vector<Request> reqs;
   };
@@ -819,7 +820,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
   for (size_t mi = 0; mi < c->models.size(); ++mi) {
     Model* m = c->models[mi];
     Active a;
-    a.m = m; a.B = 0; a.rows = 0; a.cursor = 0; a.req_off = 0; a.areq_off = 0; a.row_off = 0; a.pitem_off = 0; a.last_off = 0;
+    a.m = m; a.B = 0; a.rows = 0; a.cursor = 0; a.req_off = 0; a.areq_off = 0; a.row_off = 0; a.pitem_off = 0; a.last_off = 0; a.link_off = 0; a.append_first = false;
     a.n_dec = a.n_pre = a.max_chunks_dec = a.pre_items = 0;
     for (int cat = 0; cat < 2; ++cat) {
       std::deque<Request>& q = m->q[cat];
@@ -931,11 +932,27 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       a.row_off = put(rows.data(), rows.size() * sizeof(RowDesc), 16);
       a.last_off = put(last.data(), last.size() * sizeof(int), 16);
       if (!ar.empty()) a.areq_off = put(ar.data(), ar.size() * sizeof(AttnReq), 16);
+      // several requests: each may attend to tokens that others append (AttnDecGroup::linked)
+      if (!ar.empty() && a.B > 1 && a.m->d.head_dim >= 64) {
+        const std::vector<int> none(ar.size(), 0);
+        a.link_off = put(none.data(), none.size() * sizeof(int), 16);
+      }
     }
     if (a.req_off == (size_t)-1 || a.areq_off == (size_t)-1 || a.row_off == (size_t)-1 ||
-        a.last_off == (size_t)-1)
+        a.last_off == (size_t)-1 || a.link_off == (size_t)-1)
       overflow = true;
   }
+  // Placements that share a cache (one service placed twice): a request of one may attend to what a request of the other
+  // appends in this step, and the rows of another model are not at hand in the attention kernel.
+  auto pool_end = [](const epara_model_desc& d) {
+    return (const char*)d.kv_pool + (size_t)d.kv_pages * 2 * d.n_kv_heads * EPARA_KV_PAGE * d.head_dim * d.n_layers * 2;
+  };
+  for (Active& a : act)
+    for (const Active& b : act) {
+      const epara_model_desc &x = a.m->d, &y = b.m->d;
+      if (&a == &b || x.kind != EPARA_MODEL_DECODER || y.kind != EPARA_MODEL_DECODER) continue;
+      a.append_first |= (const char*)x.kv_pool < pool_end(y) && (const char*)y.kv_pool < pool_end(x);
+    }
 
   // ---- work items of the prompt chunks' attention: (request, 128-token tile, one or two heads), most keys first ----
   int pre_mt[2] = {2, 2};                       // query tiles per item for head sizes 64 and 128
@@ -1065,6 +1082,13 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
             AttnDecGroup g = a->m->ops[a->cursor].adec;
             g.B = a->n_dec; g.reqs = (const AttnReq*)(slot.dev + a->areq_off); g.req_start = total_B;
             g.status = dev_status;
+            if (a->append_first) {
+              g.cs = nullptr;
+            } else if (a->link_off != 0) {
+              g.linked = (const int*)(slot.dev + a->link_off);
+              g.rows = (const RowDesc*)(slot.dev + a->row_off); g.step_reqs = (const ReqDesc*)(slot.dev + a->req_off);
+              g.n_rows = a->rows;
+            }
             total_B += a->n_dec;
             max_hkv = std::max(max_hkv, g.Hkv); max_hq = std::max(max_hq, g.Hq);
             max_chunks = std::max(max_chunks, a->max_chunks_dec);
@@ -1121,7 +1145,15 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
             g.rows = (const RowDesc*)(slot.dev + a->row_off);
             g.blocks = g.kind == GATHER_PATCH ? (rows + GATHER_PATCH_ROWS - 1) / GATHER_PATCH_ROWS : rows;
             mx = std::max(mx, g.blocks);
+            ++n_put;
             if (put(&g, sizeof(g), 8) == (size_t)-1) overflow = true;
+            if (a->link_off != 0 && !a->append_first) {
+              g.kind = GATHER_LINK; g.blocks = a->n_dec; g.n_pre = a->n_pre;
+              g.areqs = (const AttnReq*)(slot.dev + a->areq_off);
+              g.out = slot.dev + a->link_off;
+              ++n_put;
+              if (put(&g, sizeof(g), 8) == (size_t)-1) overflow = true;
+            }
             break;
           }
           case EPARA_K_ASSEMBLE: {
@@ -1193,8 +1225,9 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
             break;
           }
           case EPARA_K_ROPE: {
-            if (op.rope.only_chunks && a->n_pre == 0) break;   // nothing to rotate
+            if (op.rope.only_chunks && a->n_pre == 0 && !a->append_first) break;   // nothing to rotate
             RopeGroup g = op.rope;
+            if (a->append_first) g.only_chunks = 0;
             g.reqs = (const ReqDesc*)(slot.dev + a->req_off); g.B = rows;
             g.rows = (const RowDesc*)(slot.dev + a->row_off);
             g.status = dev_status;
@@ -1225,7 +1258,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
         if (pass == n_pass - 1) a->cursor++;
       }
       L.p0 = total; L.p1 = mx;
-      if (kind == EPARA_K_GEMM || kind == EPARA_K_ATTN_ENC || kind == EPARA_K_ROPE) {
+      if (kind == EPARA_K_GATHER || kind == EPARA_K_GEMM || kind == EPARA_K_ATTN_ENC || kind == EPARA_K_ROPE) {
         L.n_groups = n_put;
         if (n_put == 0) continue;
       }

@@ -10,6 +10,7 @@ namespace epara {
 // ------------------------------------------------------------------ gather
 // Row and embedding gathers take one block per row (a handful of rows per step); the patch gather takes
 // GATHER_PATCH_ROWS patch rows per block, so that a thread has several 16-byte loads in flight.
+constexpr int LINK_PAGES = 1024;
 __global__ void __launch_bounds__(128) gather_kernel(const GatherGroup* __restrict__ groups) {
   const GatherGroup g = groups[blockIdx.y];
   if ((int)blockIdx.x >= g.blocks) return;      // (descriptors are not written by kernels: no wait needed to leave)
@@ -30,6 +31,37 @@ __global__ void __launch_bounds__(128) gather_kernel(const GatherGroup* __restri
       dst[2 * i] = make_float4(f[0], f[1], f[2], f[3]);
       dst[2 * i + 1] = make_float4(f[4], f[5], f[6], f[7]);
     }
+  } else if (g.kind == GATHER_LINK) {
+    // Does the block table of decode request b, up to the request's own position, name a page that another request of the
+    // step appends to?  By whole pages: a request marked without need costs time only.
+    __shared__ int seen[LINK_PAGES];
+    const AttnReq rq = g.areqs[blockIdx.x];
+    const int n_pages = (rq.len - 1 + 15) >> 4;
+    bool hit = false;
+    for (int i0 = 0; i0 < n_pages; i0 += LINK_PAGES) {
+      const int n = min(LINK_PAGES, n_pages - i0);
+      __syncthreads();
+      for (int i = threadIdx.x; i < n; i += blockDim.x) seen[i] = rq.table[i0 + i];
+      __syncthreads();
+      for (int q = threadIdx.x; q < g.B; q += blockDim.x) {
+        const ReqDesc& r = g.reqs[q];
+        if (r.n_tok > 1 || r.row_start == rq.row) continue;
+        const int page = r.table[r.kv_len >> 4];
+#pragma unroll 8
+        for (int i = 0; i < n; ++i) hit |= seen[i] == page;
+      }
+      if (g.n_pre == 0) continue;
+      for (int q = 0; q < g.B; ++q) {                  // prompt chunks: a thread per page
+        const ReqDesc& r = g.reqs[q];
+        if (r.n_tok == 1) continue;
+        for (int pg = (r.kv_len >> 4) + threadIdx.x; pg <= (r.kv_len + r.n_tok - 1) >> 4; pg += blockDim.x) {
+          const int page = r.table[pg];
+#pragma unroll 8
+          for (int i = 0; i < n; ++i) hit |= seen[i] == page;
+        }
+      }
+    }
+    if (hit) reinterpret_cast<int*>(g.out)[blockIdx.x] = 1;      // (zero before the step)
   } else {  // GATHER_PATCH: row (b*np + i*gw + j), column c*p*p + u*p + v  <-  img[b][c][p*i+u][p*j+v]
     const int p = g.patch, gw = g.img / p, np = gw * gw;
     const int vec_per_row = p / 8, vecs = g.width / 8;
@@ -286,12 +318,10 @@ __global__ void __launch_bounds__(ROPE_THREADS) rope_append_kernel(const RopeGro
       const int c = (i0 + k * ROPE_THREADS) * 8, h = c / hd;
       if (c >= nvec * 8) break;
       if (h < g.Hq + g.Hkv) {
-        float f[8];
-        unpack8(u[k], f);
-        u[k].x = pack2(f[0] * t0.x - f[1] * t0.y, f[0] * t0.y + f[1] * t0.x);
-        u[k].y = pack2(f[2] * t0.z - f[3] * t0.w, f[2] * t0.w + f[3] * t0.z);
-        u[k].z = pack2(f[4] * t1.x - f[5] * t1.y, f[4] * t1.y + f[5] * t1.x);
-        u[k].w = pack2(f[6] * t1.z - f[7] * t1.w, f[6] * t1.w + f[7] * t1.z);
+        u[k].x = rotate_pair(u[k].x, t0.x, t0.y);
+        u[k].y = rotate_pair(u[k].y, t0.z, t0.w);
+        u[k].z = rotate_pair(u[k].z, t1.x, t1.y);
+        u[k].w = rotate_pair(u[k].w, t1.z, t1.w);
       }
       if (h < g.Hq) {
         *reinterpret_cast<uint4*>(row + c) = u[k];

@@ -322,3 +322,60 @@ def test_prefill_admission_by_token_rows_and_rejections(mods):
     m16 = srv.add_model(p16, kv_pool=pool16, max_kv_len=200, max_batch=64)
     assert status(tokens=[1, 2, 3], kv_len=0, table=big, model=m16) == E.E_UNSUPPORTED
     srv.close()
+
+
+@pytest.mark.parametrize("hd,Hq,Hkv,kv0,chunk,n_dec,placed_twice", [
+    (64, 8, 2, 37, 0, 2, False), (64, 8, 2, 254, 0, 5, False), (128, 4, 4, 511, 0, 3, False), (32, 4, 2, 30, 0, 4, False),
+    (64, 4, 1, 0, 40, 3, False), (128, 8, 2, 130, 130, 20, False), (64, 8, 2, 250, 0, 12, True), (64, 8, 2, 20, 33, 2, True)])
+def test_requests_of_one_sequence_in_one_step(mods, hd, Hq, Hkv, kv0, chunk, n_dec, placed_twice):
+    """A caller that scores known tokens: `n_dec` decode requests at successive positions of one sequence, alone or behind the
+    prompt chunk that fills the positions before them, all in ONE step, in an order that is not theirs, each with a block
+    table of its own, beside a request of another sequence.  Every request attends to what the requests before it append in
+    the same step, as if the step's keys and values were all appended before any attention reads them: logits and cache have
+    the bits of the same requests run one step after another.  (placed_twice: every other request goes to a second
+    placement of the same weights on the same cache.)  The slots they write hold NaN before the step."""
+    E, server = mods
+    p = synth.make_decoder(d=256, n_layers=2, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=hd, ffn=256, vocab=300, seed=60, device=DEV, std=0.06)
+    rng = np.random.default_rng(kv0 + n_dec)
+    total, other_len = kv0 + chunk + n_dec, 70
+    toks = [int(t) for t in rng.integers(0, 300, total)]
+    table = _table(rng, total)
+    other = torch.as_tensor(_table(rng, other_len + 1, offset=len(table)), device=DEV)
+    pool0 = synth.make_kv_pool(2, len(table) + len(other), Hkv, hd, seed=61, device=DEV)
+    for q in range(kv0, total):
+        pool0[:, int(table[q // 16]), :, :, q % 16, :] = float("nan")
+    got = []
+    for at_once in (True, False):
+        pool = pool0.clone()
+        srv = server.Server(workspace_bytes=512 << 20)
+        m = [srv.add_model(p, kv_pool=pool, max_kv_len=total + 64, max_batch=max(32, chunk + n_dec + 1)) for _ in range(1 + placed_twice)]
+        reqs = [dict(tokens=toks[kv0:kv0 + chunk], kv_len=kv0)] if chunk else []
+        reqs += [dict(token=toks[q], kv_len=q) for q in range(kv0 + chunk, total)]
+        order = rng.permutation(len(reqs)) if at_once else np.arange(len(reqs))
+        keep, ts = [], {}
+        for n, i in enumerate(order):
+            keep.append(torch.as_tensor(table, device=DEV))
+            ts[int(i)] = srv.submit(m[int(i) % len(m)], E.CAT_FS, table=keep[-1], **reqs[int(i)])
+            if n == 0:
+                ts["other"] = srv.submit(m[0], E.CAT_FS, token=7, kv_len=other_len, table=other)
+            if not at_once:
+                srv.step()
+        if at_once:
+            srv.step()
+        torch.cuda.synchronize()
+        res = {}
+        for i, t in ts.items():
+            s, logits, am = srv.collect(t)
+            assert s == E.OK
+            res[i] = (logits.clone(), int(am.item()))
+        got.append((res, pool))
+        srv.close()
+    for i in got[1][0]:
+        assert bool(torch.isfinite(got[1][0][i][0].float()).all())
+        assert torch.equal(got[0][0][i][0], got[1][0][i][0]) and got[0][0][i][1] == got[1][0][i][1], f"request {i}"
+    assert torch.equal(got[0][1].view(torch.int16), got[1][1].view(torch.int16))
+    v = synth.bits_view({k: p[k] for k in p if k != "packed_layers"})
+    fetch = lambda l, pg: synth.to_bits(pool0[l, pg])
+    ref = O.decoder_prefill(toks[kv0:], kv0, table, fetch, v, round_bf16=True)
+    last = max(i for i in got[0][0] if i != "other")
+    assert_close(got[0][0][last][0], ref["logits"], what="last token of the sequence")
