@@ -79,7 +79,7 @@ struct FlashGeo {
 constexpr int FL_S_COL = 0, FL_O_COL = 256;
 
 // S_FULL, P_READY, PV_DONE: one per tile and buffer (index 2 g + buffer), so that no barrier can complete two phases
-// between two looks of its waiter.  K blocks sit in the even slots of the ring, V blocks in the odd ones, whose EMPTY
+// between two looks of its waiter (TURN: see the softmax warps).  K blocks sit in the even slots of the ring, V blocks in the odd ones, whose EMPTY
 // barriers count both P V warps (one that has no tile in the item arrives without an MMA).
 enum { FB_Q_FULL = 0, FB_Q_EMPTY, FB_S_FULL, FB_P_READY = FB_S_FULL + 4, FB_PV_DONE = FB_P_READY + 4, FB_KV_FULL = FB_PV_DONE + 4,
        FB_KV_EMPTY = FB_KV_FULL + 8, FB_TURN = FB_KV_EMPTY + 8, FB_PAIR = FB_TURN + 8, FB_COUNT = FB_PAIR + 4 };
@@ -453,6 +453,7 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
     bool ok = true;
     uint32_t cnt = 0;                            // steps of this tile done
     uint32_t turns = 0, pairs = 0;               // turns and pair barriers waited for
+    bool turns_seen = false;                     // the first turn of this CTA's paired items is past
     View view;
     view.g = nullptr;
     // this tile's next item; decoded while the last P V of the item before is under way
@@ -508,7 +509,10 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
         }
         // The two warps of a scheduler take turns at the exponentials, so that one's scores are read and reduced while the
         // other keeps the special-function unit busy (in step they left it idle half of the time).
-        const bool take_turns = paired && (g == 1 || j > 0), give_turn = paired && (g == 0 || j + 1 < steps);
+        // (Strictly in turn, over the ends of items too: only the very first turn of tile 0 is not given to it.  Neither warp
+        // can be more than one turn ahead, so a TURN barrier never completes two phases between two looks of its waiter.)
+        const bool take_turns = paired && (g == 1 || turns_seen);
+        turns_seen |= paired;
         if (seen) {
           uint32_t v[NC];
           tmem_ld32_nowait(sb + half * NC, v);
@@ -594,14 +598,14 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
             unpack_f2(l2b, a2, a3);
             l[h] += (a0 + a1) + (a2 + a3);
           }
-          if (give_turn && lane == 0) mbar_arrive(bar(FB_TURN + 4 * (g ^ 1) + quarter));
+          if (paired && lane == 0) mbar_arrive(bar(FB_TURN + 4 * (g ^ 1) + quarter));
           tmem_st_wait();
         } else if (paired) {
           if (take_turns) {
             if (!mbar_wait<false>(bar(FB_TURN + 4 * g + quarter), turns & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 19); break; }
             ++turns;
           }
-          if (give_turn && lane == 0) mbar_arrive(bar(FB_TURN + 4 * (g ^ 1) + quarter));
+          if (lane == 0) mbar_arrive(bar(FB_TURN + 4 * (g ^ 1) + quarter));
         }
         tc_fence_before();
         __syncwarp();

@@ -379,3 +379,43 @@ def test_requests_of_one_sequence_in_one_step(mods, hd, Hq, Hkv, kv0, chunk, n_d
     ref = O.decoder_prefill(toks[kv0:], kv0, table, fetch, v, round_bf16=True)
     last = max(i for i in got[0][0] if i != "other")
     assert_close(got[0][0][last][0], ref["logits"], what="last token of the sequence")
+
+
+@pytest.mark.parametrize("hd,Hq,Hkv,chunks,kv0,n", [(64, 32, 8, 48, 0, 60), (128, 16, 4, 40, 0, 33), (64, 32, 4, 12, 200, 130),
+                                                    (128, 16, 8, 8, 330, 260), (64, 16, 8, 9, 517, 131)])
+def test_many_paired_items_in_a_row_with_raised_maxima(mods, hd, Hq, Hkv, chunks, kv0, n):
+    """Chunks that give every CTA several items of two query tiles (heads of one kv head) one after another, whose warps take
+    turns at the exponentials across the ends of items: items of a single step of keys, and items whose cached keys grow
+    along the sequence (factor 1 to 5), so that the running maximum is raised and output and sum are rescaled in the two-tile
+    form too; ragged tiles.  The first and the last chunk
+    have the bits they have alone (one tile per item) and equal the oracle."""
+    E, server = mods
+    p = synth.make_decoder(d=256, n_layers=1, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=hd, ffn=256, vocab=300, seed=70, device=DEV,
+                           std=0.06)
+    rng = np.random.default_rng(chunks + n)
+    per = (kv0 + n + 15) // 16
+    toks = [[int(t) for t in rng.integers(0, 300, n)] for _ in range(chunks)]
+    tabs = [_table(rng, kv0 + n, offset=per * i) for i in range(chunks)]
+    pool0 = synth.make_kv_pool(1, per * chunks, Hkv, hd, seed=71, device=DEV)
+    for tb in tabs:
+        for i, pg in enumerate(tb):
+            pool0[0, int(pg), 0] *= 1.0 + 4.0 * i / per
+    got, picked = [], [0, chunks - 1]
+    for which in (list(range(chunks)), picked[:1], picked[1:]):
+        pool = pool0.clone()
+        srv = server.Server(workspace_bytes=512 << 20, cap_fs=64)
+        m = srv.add_model(p, kv_pool=pool, max_kv_len=kv0 + n, max_batch=chunks * n)
+        dev_tabs = [torch.as_tensor(tabs[i], device=DEV) for i in which]
+        ts = {i: srv.submit(m, E.CAT_FS, tokens=toks[i], kv_len=kv0, table=tb) for i, tb in zip(which, dev_tabs)}
+        srv.step()
+        torch.cuda.synchronize()
+        res = {i: srv.collect(t) for i, t in ts.items()}
+        assert all(s == E.OK for s, _, _ in res.values())
+        got.append({i: (res[i][1].clone(), int(res[i][2].item())) for i in picked if i in res})
+        if len(which) == chunks:
+            pool_all = pool
+        srv.close()
+    v = synth.bits_view({k: p[k] for k in p if k != "packed_layers"})
+    for i, alone in zip(picked, got[1:]):
+        assert torch.equal(got[0][i][0], alone[i][0]) and got[0][i][1] == alone[i][1]
+        _check_prefill(v, pool_all, pool0, got[0][i], toks[i], kv0, tabs[i], f"chunk {i} of {chunks}")
