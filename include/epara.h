@@ -332,7 +332,7 @@ size_t epara_gemm_scratch_bytes_for(int device, const epara_gemm_problem* proble
 /* Split-KV paged decode attention with GQA (one layer).  q: bf16 [B, q_stride] (head h at
  * column h*hd); kv_layer: bf16 [kv_pages][2][Hkv][16][hd]; kv_lens int32 [B] = tokens to attend
  * (cached + appended; values outside [0, max_len] are clamped, a request of length 0 leaves its output
- * row unwritten); tables: int32 [B, table_stride]; out bf16 [B, Hq*hd];
+ * row unwritten); tables: int32 [B, table_stride]; out bf16 [B, Hq*hd], at any 2-byte boundary;
  * scratch: at least epara_decode_attention_scratch_bytes(B, Hq, hd, max_len) bytes (descriptor, request
  * table, fp32 chunk partials, chunk counters; the call clears what must start at zero itself).
  * A page id outside [0, kv_pages) is never dereferenced: the page is read as absent and the int32 at byte

@@ -63,6 +63,16 @@ __device__ __forceinline__ float2 merge_chunks(const float* p, int n_chunks, int
   return make_float2(oo.x / ll, oo.y / ll);
 }
 
+// Two neighbouring outputs.  The single-kernel entries take an `out` at any bf16 boundary; a step's is always aligned.
+__device__ __forceinline__ void store_pair(bf16* p, float2 o) {
+  if ((reinterpret_cast<uintptr_t>(p) & 3) == 0) {
+    *reinterpret_cast<uint32_t*>(p) = pack2(o.x, o.y);
+  } else {
+    p[0] = f2bf(o.x);
+    p[1] = f2bf(o.y);
+  }
+}
+
 // Last step of a decode-attention block: the four warps' (m, l, o) of this chunk sit in shared
 // memory.  They are merged in warp order.  A request of a single chunk is finished right here.
 // Otherwise the chunk's partial goes to scratch.  With `fused` a per-(request, kv head) counter is
@@ -114,7 +124,7 @@ __device__ __forceinline__ void finish_chunk(const AttnDecGroup& g, int b, int r
     const int h = idx / (HD / 2), e = idx % (HD / 2) * 2;
     const float* p = g.partial + ((size_t)b * g.Hq + (kvh * G + h)) * g.max_chunks * (HD + 2);
     const float2 o = merge_chunks<HD>(p, n_chunks, e);
-    *reinterpret_cast<uint32_t*>(g.out + ((size_t)row * g.Hq + (kvh * G + h)) * HD + e) = pack2(o.x, o.y);
+    store_pair(g.out + ((size_t)row * g.Hq + (kvh * G + h)) * HD + e, o);
   }
 }
 
@@ -137,8 +147,7 @@ __global__ void __launch_bounds__(COMBINE_THREADS) attn_combine_kernel(const Att
   if (g.reqs_stable) pdl_wait();
   if (hq >= g.Hq || n_chunks <= 1) return;            // (one chunk: finished by the attention kernel itself)
   const int e = threadIdx.x % (HD / 2) * 2;
-  const float2 o = merge_chunks<HD>(p, n_chunks, e);
-  *reinterpret_cast<uint32_t*>(out + e) = pack2(o.x, o.y);
+  store_pair(out + e, merge_chunks<HD>(p, n_chunks, e));
 }
 
 template <int HD, int G>
@@ -868,7 +877,8 @@ extern "C" int epara_decode_attention_static(int device, void* cuda_stream, cons
   if (!q || !kv_layer || !kv_lens || !tables || !out || B < 0 || Hkv <= 0 || Hq <= 0 || Hq % Hkv || max_len <= 0 || hd <= 0 ||
       kv_pages <= 0)
     return EPARA_E_INVALID;
-  if ((reinterpret_cast<uintptr_t>(q) & 15) || (reinterpret_cast<uintptr_t>(kv_layer) & 15) || (q_stride % 8))
+  if ((reinterpret_cast<uintptr_t>(q) & 15) || (reinterpret_cast<uintptr_t>(kv_layer) & 15) || (q_stride % 8) ||
+      (reinterpret_cast<uintptr_t>(out) & 1))
     return EPARA_E_INVALID;
   if (device < 0 || device >= MAX_DEVICES) return EPARA_E_INVALID;
   const int chunks = (max_len + ATTN_CHUNK - 1) / ATTN_CHUNK;

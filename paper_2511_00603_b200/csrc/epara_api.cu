@@ -1545,7 +1545,7 @@ int epara_decode_attention(int device, void* cuda_stream, const void* q, int q_s
       kv_pages <= 0)
     return EPARA_E_INVALID;
   if ((reinterpret_cast<uintptr_t>(q) & 15) || (reinterpret_cast<uintptr_t>(kv_layer) & 15) || (q_stride % 8) ||
-      (reinterpret_cast<uintptr_t>(scratch) & 255))
+      (reinterpret_cast<uintptr_t>(scratch) & 255) || (reinterpret_cast<uintptr_t>(out) & 1))
     return EPARA_E_INVALID;
   if (scratch_bytes < epara_decode_attention_scratch_bytes(B, Hq, hd, max_len)) return EPARA_E_RESOURCE;
   if (B == 0) return EPARA_OK;

@@ -262,3 +262,27 @@ def test_grouped_gemm_between_one_tile_and_a_full_chip(E, rows):
         assert_close(p["C"][:ref.shape[0], :ref.shape[1]], ref, what=f"gemm {case}")
     alone, _ = _run_gemm(E, E.GEMM_TCGEN05, cases[:2], seed=rows)
     assert torch.equal(alone[1]["C"], probs[1]["C"])
+
+
+@pytest.mark.parametrize("hd,Hq,Hkv", [(16, 4, 2), (64, 8, 2), (128, 4, 4)])
+@pytest.mark.parametrize("B", [5, 420])
+def test_decode_attention_writes_out_at_any_bf16_boundary(E, hd, Hq, Hkv, B):
+    """`out` one element past an aligned address: requests of one chunk and of several, merged by the last block to arrive
+    (5 requests) and by the second kernel (420).  The same bits as in an aligned tensor, and nothing beside it."""
+    dev = torch.device("cuda")
+    lens = np.resize(np.array([700, 1, 256, 257, 530], dtype=np.int32), B)
+    tables = torch.arange(44, dtype=torch.int32, device=dev).repeat(B, 1)
+    pool = synth.make_kv_pool(1, 44, Hkv, hd, seed=31, device=dev)[0]
+    q = torch.randn((B, Hq * hd), generator=torch.Generator(device=dev).manual_seed(32), device=dev).to(torch.bfloat16)
+    scratch = torch.empty(E.lib.epara_decode_attention_scratch_bytes(B, Hq, hd, 700), dtype=torch.uint8, device=dev)
+    buf = torch.full((B * Hq * hd + 2,), 9.0, device=dev, dtype=torch.bfloat16)
+    ref, odd = torch.empty_like(q), buf[1:-1].view(B, Hq * hd)
+    for out in (ref, odd):
+        E.epara_decode_attention(q, pool, torch.as_tensor(lens, device=dev), tables, out, Hq, Hkv, hd, 700, scratch, _stream())
+    torch.cuda.synchronize()
+    assert torch.equal(ref, odd) and float(buf[0]) == 9.0 and float(buf[-1]) == 9.0
+    if B == 5:
+        odd.zero_()
+        E.epara_decode_attention_static(q, pool, torch.as_tensor(lens, device=dev), tables, odd, Hq, Hkv, hd, 700, _stream())
+        torch.cuda.synchronize()
+        assert torch.equal(ref, odd) and float(buf[0]) == 9.0 and float(buf[-1]) == 9.0

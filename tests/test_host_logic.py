@@ -40,6 +40,14 @@ def test_strerror_and_null_arguments(E):
     assert E.lib.epara_destroy(None) == E.E_INVALID
 
 
+def test_decode_attention_refuses_an_output_between_two_bf16_elements(E):
+    """(nothing is launched, so any aligned number stands in for a device pointer)"""
+    for out, ok in ((4097, False), (4098, True)):
+        args = (4096, 512, 4096, 8, 4096, 4096, 4, out)
+        r = [E.lib.epara_decode_attention(0, None, *args, 0, 8, 2, 64, 64, 4096, 1 << 20), E.lib.epara_decode_attention_static(0, None, *args, 0, 8, 2, 64, 64)]
+        assert r == [E.OK if ok else E.E_INVALID] * 2
+
+
 def test_eq4_eq5_match_oracle(E):
     from oracle import epara_oracle as O
     for req, grp in [(97, 49), (98, 49), (99, 49), (60, 60), (1, 100), (120.5, 30)]:
