@@ -1432,14 +1432,8 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
   if (scratch_bytes < (impl == EPARA_GEMM_SIMT ? epara_gemm_scratch_bytes(n) : epara_gemm_scratch_bytes_for(device, p, n)))
     return EPARA_E_RESOURCE;
   if (n == 0) return EPARA_OK;
-  if (cudaSetDevice(device) != cudaSuccess) return EPARA_E_CUDA;
-  cudaStream_t st = (cudaStream_t)cuda_stream;
   const bool simt = impl == EPARA_GEMM_SIMT;
   const int sm_count = device_sm_count(device);
-  std::vector<GemmGroup> gs, gs_stream, gs_pair;   // CUDA-core groups; weight-streaming groups (M <= 16); CTA-pair groups
-  std::vector<GemmGroup> gs_swap[8];               // swapped-operand groups by k ranges per tile (1 to 8)
-  int total_swap[8] = {0}, nb_swap[8] = {0};
-  int total = 0, total_stream = 0, max_rows_stream = 0, total_pair = 0;
   for (int i = 0; i < n; ++i) {
     const epara_gemm_problem& q = p[i];
     if (!q.A || !q.W || !q.C || q.M < 0 || q.N <= 0 || q.K <= 0) return EPARA_E_INVALID;
@@ -1449,6 +1443,21 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
       return EPARA_E_INVALID;
     if ((q.epilogue & EPARA_EPI_SWIGLU) && (q.N % 2 || (q.epilogue & EPARA_EPI_RESID_F32))) return EPARA_E_INVALID;
     if ((q.epilogue & EPARA_EPI_BIAS) && !q.bias) return EPARA_E_INVALID;
+    // The CUDA-core and the weight-streaming kernel store single elements and take any ldc; the others store boxes whose
+    // rows start on 16 bytes or, up to 128 rows, vectors of four elements (SwiGLU: two).
+    if (simt || q.M == 0 || gemm_stream_eligible(q.M, q.N, q.K)) continue;
+    const bool f32 = (q.epilogue & EPARA_EPI_RESID_F32) != 0;
+    const int whole = q.M > TC_BM ? (f32 ? 4 : 8) : (q.epilogue & EPARA_EPI_SWIGLU) ? 2 : 4;
+    if (q.ldc % whole) return EPARA_E_INVALID;
+  }
+  if (cudaSetDevice(device) != cudaSuccess) return EPARA_E_CUDA;
+  cudaStream_t st = (cudaStream_t)cuda_stream;
+  std::vector<GemmGroup> gs, gs_stream, gs_pair;   // CUDA-core groups; weight-streaming groups (M <= 16); CTA-pair groups
+  std::vector<GemmGroup> gs_swap[8];               // swapped-operand groups by k ranges per tile (1 to 8)
+  int total_swap[8] = {0}, nb_swap[8] = {0};
+  int total = 0, total_stream = 0, max_rows_stream = 0, total_pair = 0;
+  for (int i = 0; i < n; ++i) {
+    const epara_gemm_problem& q = p[i];
     GemmGroup g;
     memset(&g, 0, sizeof(g));
     g.A = (const bf16*)q.A; g.W = (const bf16*)q.W; g.C = q.C; g.bias = (const bf16*)q.bias;

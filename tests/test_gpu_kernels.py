@@ -286,3 +286,29 @@ def test_decode_attention_writes_out_at_any_bf16_boundary(E, hd, Hq, Hkv, B):
         E.epara_decode_attention_static(q, pool, torch.as_tensor(lens, device=dev), tables, odd, Hq, Hkv, hd, 700, _stream())
         torch.cuda.synchronize()
         assert torch.equal(ref, odd) and float(buf[0]) == 9.0 and float(buf[-1]) == 9.0
+
+
+@pytest.mark.parametrize("M,N,K,fl,ldc", [(5, 100, 512, ("bias",), 101), (100, 250, 264, ("gelu", "bias"), 253), (64, 2048, 2048, ("resid",), 2052),
+                                          (100, 1030, 1544, (), 1036), (33, 4096, 512, ("swiglu",), 2050), (300, 264, 512, ("resid",), 268)])
+def test_grouped_gemm_takes_row_strides_of_c_that_its_kernels_can_store(E, M, N, K, fl, ldc):
+    """Strides of C that are no multiple of 8: any for the weight-streaming kernel, four (SwiGLU: two) elements for the
+    swapped operands up to 128 rows, 16 bytes above."""
+    dev = torch.device("cuda")
+    g = torch.Generator(device=dev).manual_seed(M)
+    A = torch.randn((M, K), generator=g, device=dev).to(torch.bfloat16)
+    W = (torch.randn((N, K), generator=g, device=dev) * 0.05).to(torch.bfloat16)
+    bias = torch.randn((N,), generator=g, device=dev).to(torch.bfloat16) if "bias" in fl else None
+    epi = sum({"bias": E.EPI_BIAS, "gelu": E.EPI_GELU, "swiglu": E.EPI_SWIGLU, "resid": E.EPI_RESID_F32}[f] for f in fl)
+    n_out = N // 2 if "swiglu" in fl else N
+    C0 = torch.randn((M, ldc), generator=g, device=dev) if "resid" in fl else torch.zeros((M, ldc), device=dev, dtype=torch.bfloat16)
+    wide = torch.zeros((M, (ldc + 7) // 8 * 8), device=dev, dtype=C0.dtype)
+    wide[:, :ldc] = C0
+    C = C0.clone()
+    for out in (C, wide):
+        prob = [{"A": A, "W": W, "C": out, "bias": bias, "M": M, "N": N, "K": K, "epilogue": epi}]
+        scratch = torch.empty(E.epara_gemm_scratch_bytes_for(prob), dtype=torch.uint8, device=dev)
+        E.epara_grouped_gemm(prob, _stream(), scratch)
+    torch.cuda.synchronize()
+    assert torch.equal(C[:, :n_out], wide[:, :n_out]) and bool((C[:, :n_out] != C0[:, :n_out]).any())
+    pad = n_out + (-n_out) % (4 if "resid" in fl else 8)              # columns up to there may be overwritten
+    assert torch.equal(C[:, pad:], C0[:, pad:])

@@ -48,6 +48,19 @@ def test_decode_attention_refuses_an_output_between_two_bf16_elements(E):
         assert r == [E.OK if ok else E.E_INVALID] * 2
 
 
+@pytest.mark.parametrize("M,N,K,epi,ldc", [(129, 768, 3072, "RESID", 770), (509, 2048, 8192, "RESID", 2050), (300, 1000, 768, "BIAS", 1004),
+                                           (512, 136, 4096, "BIAS", 140), (200, 4096, 1024, "SWIGLU", 2052), (64, 32000, 2048, "BIAS", 32002),
+                                           (17, 2048, 8192, "RESID", 2050), (100, 16384, 2048, "SWIGLU", 8193)])
+def test_grouped_gemm_refuses_an_ldc_its_vector_stores_cannot_take(E, M, N, K, epi, ldc):
+    """A bad row stride of C is refused before anything is built or launched (aligned numbers stand in for pointers), whichever
+    tensor-core kernel the sizes select, on its own and behind a good problem."""
+    flag = {"RESID": E.EPI_RESID_F32, "BIAS": E.EPI_BIAS, "SWIGLU": E.EPI_SWIGLU}[epi]
+    bad = E.GemmProblem(4096, 4096, 4096, 4096, M, N, K, K, K, ldc, flag)
+    good = E.GemmProblem(4096, 4096, 4096, 4096, 300, 512, 512, 512, 512, 512, E.EPI_BIAS)
+    for arr in ((E.GemmProblem * 1)(bad), (E.GemmProblem * 2)(good, bad)):
+        assert E.lib.epara_grouped_gemm(0, None, E.GEMM_TCGEN05, arr, len(arr), 4096, 1 << 20) == E.E_INVALID
+
+
 def test_eq4_eq5_match_oracle(E):
     from oracle import epara_oracle as O
     for req, grp in [(97, 49), (98, 49), (99, 49), (60, 60), (1, 100), (120.5, 30)]:
