@@ -363,7 +363,7 @@ __device__ __forceinline__ void place_step_rows(const AttnDecGroup& g, unsigned 
     if (w < g.n_rows && w != own_row) {
       const RowDesc rd = g.rows[w];
       at = rd.pos;
-      hit = (at & 15) < n_slots && g.step_reqs[rd.req].table[at >> 4] == page;
+      hit = (at & 15) < n_slots && g.step_reqs[rd.req()].table[at >> 4] == page;
     }
     for (unsigned m = __ballot_sync(0xffffffffu, hit); m != 0; m &= m - 1) {
       const int l = __ffs(m) - 1, p = __shfl_sync(0xffffffffu, at, l);

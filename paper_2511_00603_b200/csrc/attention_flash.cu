@@ -158,8 +158,9 @@ struct EncView {
 struct PreView {
   const AttnPrefillGroup* g;
   int start, end, G, hd;
-  int mt;
-  const PrefillItem* items;
+  int mt, head_shift, Hkv;
+  unsigned by_hkv;
+  const PrefillTile* tiles;
 };
 __device__ __forceinline__ void load_view(EncView& v, const AttnEncGroup* groups, int n_groups, int item, int mt) {
   if (v.g != nullptr && item >= v.start && item < v.end) return;
@@ -174,7 +175,8 @@ __device__ __forceinline__ void load_view(PreView& v, const AttnPrefillGroup* gr
   int gi = 0;
   for (int i = 1; i < n_groups; ++i) if (item >= groups[i].item_start) gi = i;
   const AttnPrefillGroup* g = groups + gi;
-  v.g = g; v.mt = mt; v.start = g->item_start; v.end = v.start + g->n_items; v.G = g->Hq / g->Hkv; v.hd = g->hd; v.items = g->items;
+  v.g = g; v.mt = mt; v.start = g->item_start; v.end = v.start + g->n_items; v.G = g->Hq / g->Hkv; v.hd = g->hd; v.tiles = g->tiles;
+  v.head_shift = g->head_shift; v.Hkv = g->Hkv; v.by_hkv = g->by_hkv;
 }
 __device__ __forceinline__ Work get_work(const EncView& v, int item) {
   const int local = item - v.start, bh = v.q_blocks == 1 ? local : local / v.q_blocks, qb = local - bh * v.q_blocks;
@@ -188,16 +190,24 @@ __device__ __forceinline__ Work get_work(const EncView& v, int item) {
   return w;
 }
 __device__ __forceinline__ Work get_work(const PreView& v, int item) {
-  const PrefillItem pi = v.items[item - v.start];
+  const int local = item - v.start, kv_item = local >> v.head_shift;
+  const int tile = v.by_hkv ? (int)__umulhi((unsigned)kv_item, v.by_hkv) : kv_item, kvh = kv_item - tile * v.Hkv;
+  const int h = (local - (kv_item << v.head_shift)) * v.mt;                         // the first of n_mt heads of kv head kvh
+  const PrefillTile pi = v.tiles[tile];
   Work w;
-  w.qx = pi.head * v.hd; w.qy = pi.row; w.dx = v.hd; w.dy = 0;
-  w.n_mt = min(v.mt, v.G - pi.head % v.G);
+  w.head = kvh * v.G + h;
+  w.qx = w.head * v.hd; w.qy = pi.row; w.dx = v.hd; w.dy = 0;
+  w.n_mt = min(v.mt, v.G - h);
   w.live0 = w.live1 = pi.live;
   w.n_keys = pi.pos + pi.live;
   w.lim0 = pi.pos;
-  w.head = pi.head; w.table = pi.table;
+  w.table = pi.table;
   return w;
 }
+__device__ __forceinline__ const CUtensorMap* map_q(const AttnEncGroup* g) { return &g->tmQ; }
+__device__ __forceinline__ const CUtensorMap* map_q(const AttnPrefillGroup* g) { return &g->maps->tmQ; }
+__device__ __forceinline__ const CUtensorMap* map_kv(const AttnEncGroup* g) { return &g->tmKV; }
+__device__ __forceinline__ const CUtensorMap* map_kv(const AttnPrefillGroup* g) { return &g->maps->tmKV; }
 __device__ __forceinline__ int out_stride(const AttnEncGroup* g) { return g->H * 64; }
 __device__ __forceinline__ int out_stride(const AttnPrefillGroup* g) { return g->Hq * g->hd; }
 
@@ -280,8 +290,9 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
     const Group* g_prev = nullptr;
     uint32_t kv = 0, it = 0;                     // ring tiles issued, items started
     bool waited = false;
-    int Hkv = 0;
+    int Hkv = 0, kv_row0 = 0, oob = 0;           // (oob: a row past the tensor: filled with zeros)
     long long kv_pages = 0;
+    const CUtensorMap *tmQ = nullptr, *tmKV = nullptr;
     for (int round = 0; ok; ++round) {
       const int item = item_of_round(round);
       if (round * (int)gridDim.x >= total_items) break;
@@ -289,12 +300,11 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
       load_view(view, groups, n_groups, item, mt);
       const Work w = get_work(view, item);
       const Group* g = view.g;
-      const CUtensorMap* const tmQ = &g->tmQ;
-      const CUtensorMap* const tmKV = &g->tmKV;
       if (g != g_prev) {
+        tmQ = map_q(g); tmKV = map_kv(g);
         tensormap_acquire(tmQ); tensormap_acquire(tmKV);
         g_prev = g;
-        if constexpr (PAGED) { Hkv = g->Hkv; kv_pages = g->kv_pages; }
+        if constexpr (PAGED) { Hkv = g->Hkv; kv_pages = g->kv_pages; kv_row0 = g->kv_row0; oob = g->kv_rows; }
       }
       const int nblk = (w.n_keys + FL_TILE - 1) / FL_TILE;
       int page = 0, kvh = 0, kx = 0, vx = 0, ky = 0;
@@ -308,11 +318,10 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
       if (!waited) { pdl_wait(); waited = true; }                 // q, k, v come from the kernels before this one
       for (int j = 0; j < nblk && ok; ++j) {
         const int n = min(FL_TILE, w.n_keys - j * FL_TILE), pages = (n + 15) >> 4;
-        const int oob = PAGED ? (int)(kv_pages * 2 * Hkv * 16) : 0;           // a row past the tensor: filled with zeros
         int yk = oob;
         if (PAGED) {
           if (lane < pages) {
-            if (page >= 0 && page < kv_pages) yk = (page * 2 * Hkv + kvh) * 16;
+            if (page >= 0 && page < kv_pages) yk = kv_row0 + (page * 2 * Hkv + kvh) * 16;
             else atomicExch(status, ERR_PAGE_ATTEND);
           }
           page = (lane < 8 && (j + 1) * FL_TILE + lane * 16 < w.n_keys) ? w.table[(j + 1) * 8 + lane] : 0;

@@ -33,8 +33,16 @@ struct ReqDesc {
 // Decoder activations have one row per token.  Row r belongs to request `req`, sits at position `pos` of
 // its sequence and holds token id `token`.
 struct RowDesc {
-  int req, pos, token;
-  int single;            // 1: the only row of a decode request, 0: a prompt chunk's
+  int req2;              // 2 * req, + 1 for the only row of a decode request (a prompt chunk's rows: + 0)
+  int pos, token;
+#ifdef __CUDACC__
+  __host__ __device__
+#endif
+  int req() const { return req2 >> 1; }
+#ifdef __CUDACC__
+  __host__ __device__
+#endif
+  bool single() const { return req2 & 1; }
 };
 
 // C = epi(A W^T + bias).  tmA/tmW are the TMA maps of A [rows, K] and W [N, K] (K innermost,
@@ -116,24 +124,32 @@ struct RopeGroup {
 
 // Causal attention of prompt chunks (one layer): a request has n_tok query tokens in consecutive rows, token t at position
 // kv_len + t attends to positions 0 .. kv_len + t of its paged cache (the chunk's own k, v were appended by the kernel
-// before).  A work item is 128 of its tokens and one or two query heads of one kv head; the list is sorted by the keys
-// an item walks, longest first.
-struct PrefillItem {
+// before).  A work item is 128 of its tokens (a tile) and one or two query heads of one kv head; the list holds one entry per
+// tile, sorted by the keys it walks, longest first, and a tile's heads are items one after another.  (With an entry per item
+// thousands of short chunks on a model of many heads, or a chunk of 180 thousand tokens, overflowed the step's blob.)
+struct PrefillTile {
   const int32_t* table;
   int row, live;         // first activation row, tokens of the tile
   int pos;               // position of the tile's first token
-  int head;              // first query head
-  int pad[2];
+  int pad;
 };
-struct alignas(64) AttnPrefillGroup {
+// One per model and step; the layers' groups point to it.
+struct alignas(64) PrefillMaps {
   CUtensorMap tmQ;       // qkv [rows, (Hq+2Hkv)*hd] bf16, box 64 columns x 128 rows, 128-byte swizzle
-  CUtensorMap tmKV;      // one layer of the cache as [kv_pages * 2 * Hkv * 16, hd], box 64 columns x 16 rows
-  const PrefillItem* items;
+  CUtensorMap tmKV;      // the cache as [n_layers * kv_pages * 2 * Hkv * 16, hd], box 64 columns x 16 rows
+};
+struct AttnPrefillGroup {
+  const PrefillMaps* maps;
+  const PrefillTile* tiles;
   bf16* out;             // [rows, Hq*hd]
   long long kv_pages;
+  int kv_row0, kv_rows;  // this layer's first row of tmKV, rows of tmKV (a box from there on arrives as zeros)
   int n_items, Hq, Hkv, hd;
   int item_start;        // first item of this group in the launch
-  int pad[5];
+  int head_shift;        // items of one kv head of a tile, as a power of two: its query heads by the query tiles of an item
+  unsigned by_hkv;       // 2^32 / Hkv rounded up (0 for Hkv = 1): items to tiles without a division, which every role of the
+                         // kernel would wait for at the start of an item (exact while items x Hkv < 2^32)
+  int pad;
 };
 
 struct AttnDecGroup {
@@ -211,7 +227,7 @@ struct OutputGroup {     // copy logits rows to the requests' buffers and take t
 // Group arrays are packed back to back in the step blob: sizes must keep 8-byte alignment.
 namespace epara {
 static_assert(sizeof(GemmGroup) % 64 == 0, "GemmGroup holds 64-byte aligned TMA maps");
-static_assert(sizeof(AttnPrefillGroup) % 64 == 0 && sizeof(PrefillItem) == 32 && sizeof(RowDesc) == 16, "descriptor sizes");
+static_assert(sizeof(AttnPrefillGroup) % 8 == 0 && sizeof(PrefillMaps) % 64 == 0 && sizeof(PrefillTile) == 24 && sizeof(RowDesc) == 12, "descriptor sizes");
 static_assert(sizeof(NormGroup) % 8 == 0 && sizeof(GatherGroup) % 8 == 0 && sizeof(RopeGroup) % 8 == 0 &&
               sizeof(AttnDecGroup) % 8 == 0 && sizeof(AttnEncGroup) % 64 == 0 && sizeof(MlpGroup) % 64 == 0 && sizeof(AssembleGroup) % 8 == 0 &&
               sizeof(OutputGroup) % 8 == 0 && sizeof(ReqDesc) % 16 == 0 && sizeof(AttnReq) % 16 == 0,

@@ -134,6 +134,7 @@ struct Model {
   std::vector<Op> ops;
   std::deque<Request> q[2];
   int max_chunks;       // decoder
+  PrefillMaps pre_maps; // decoder, head sizes 64 and 128
   double kv_bytes_per_token;
 };
 
@@ -484,6 +485,12 @@ int build_model(Builder& bl, Model* m, const epara_config& cfg) {
   };
   add_trace(0);
   const size_t layer_elems = (size_t)d.kv_pages * 2 * Hkv * 16 * hd;
+  const long long layer_rows = d.kv_pages * 2 * Hkv * 16;    // (all layers' rows fit an int: a cache of 2^31 of them is 275 GB)
+  if (bl.c && hd >= 64) {
+    if (layer_rows * d.n_layers > 0x7fffffffll) return EPARA_E_RESOURCE;
+    if (!make_tmap(&m->pre_maps.tmQ, qkv, Bcap, nq, nq, FLASH_TILE)) return EPARA_E_CUDA;
+    if (!make_tmap(&m->pre_maps.tmKV, d.kv_pool, layer_rows * d.n_layers, hd, hd, 16)) return EPARA_E_CUDA;
+  }
   for (int l = 0; l < d.n_layers; ++l) {
     const void* const* w = t + 1 + 6 * l;
     bf16* kv_layer = (bf16*)d.kv_pool + layer_elems * l;
@@ -509,10 +516,7 @@ int build_model(Builder& bl, Model* m, const epara_config& cfg) {
     memset(&ap, 0, sizeof(ap));
     ap.kind = EPARA_K_ATTN_PREFILL; ap.rows_per_req = 1;
     ap.apre.out = a; ap.apre.kv_pages = d.kv_pages; ap.apre.Hq = Hq; ap.apre.Hkv = Hkv; ap.apre.hd = hd;
-    if (bl.c && hd >= 64) {
-      if (!make_tmap(&ap.apre.tmQ, qkv, Bcap, nq, nq, FLASH_TILE)) return EPARA_E_CUDA;
-      if (!make_tmap(&ap.apre.tmKV, kv_layer, d.kv_pages * 2 * Hkv * 16, hd, hd, 16)) return EPARA_E_CUDA;
-    }
+    ap.apre.kv_row0 = (int)(layer_rows * l); ap.apre.kv_rows = (int)(layer_rows * d.n_layers);
     m->ops.push_back(ap);
     if (!add_gemm(bl, m, a, Hq * hd, Bcap, w[2], dm, Hq * hd, x, dm, nullptr, EPI_RESID_F32, 1)) return EPARA_E_CUDA;
     add_norm(m, x, dm, h, w[3], nullptr, dm, NORM_RMS, 1e-5f, 1);
@@ -810,7 +814,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
   // n_pre prompt-chunk requests of a decoder, with their descriptor arrays in the blob
   struct PrefillChunk { const int32_t* table; int row_start, n_tok, kv_len; };
   struct Active {
-    Model* m; int B; int rows; size_t req_off; size_t areq_off; size_t row_off; size_t pitem_off; size_t last_off; size_t link_off; size_t cursor;
+    Model* m; int B; int rows; size_t req_off; size_t areq_off; size_t row_off; size_t ptile_off; size_t pmaps_off; size_t last_off; size_t link_off; size_t cursor;
     int n_dec, n_pre, max_chunks_dec, pre_items;
     bool append_first;   // decode rows are rotated and appended by a launch of their own, before any attention of the wave
     std::vector<PrefillChunk> pre;
@@ -820,7 +824,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
   for (size_t mi = 0; mi < c->models.size(); ++mi) {
     Model* m = c->models[mi];
     Active a;
-    a.m = m; a.B = 0; a.rows = 0; a.cursor = 0; a.req_off = 0; a.areq_off = 0; a.row_off = 0; a.pitem_off = 0; a.last_off = 0; a.link_off = 0; a.append_first = false;
+    a.m = m; a.B = 0; a.rows = 0; a.cursor = 0; a.req_off = 0; a.areq_off = 0; a.row_off = 0; a.ptile_off = 0; a.pmaps_off = 0; a.last_off = 0; a.link_off = 0; a.append_first = false;
     a.n_dec = a.n_pre = a.max_chunks_dec = a.pre_items = 0;
     for (int cat = 0; cat < 2; ++cat) {
       std::deque<Request>& q = m->q[cat];
@@ -907,7 +911,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       if (dec) {
         for (int t = 0; t < nt; ++t) {
           RowDesc r;
-          r.req = b; r.pos = in.kv_len + t; r.token = nt > 1 ? rq.toks[t] : in.token; r.single = nt == 1;
+          r.req2 = 2 * b + (nt == 1); r.pos = in.kv_len + t; r.token = nt > 1 ? rq.toks[t] : in.token;
           rows.push_back(r);
         }
         if (nt == 1) {
@@ -954,7 +958,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       a.append_first |= (const char*)x.kv_pool < pool_end(y) && (const char*)y.kv_pool < pool_end(x);
     }
 
-  // ---- work items of the prompt chunks' attention: (request, 128-token tile, one or two heads), most keys first ----
+  // ---- tiles of the prompt chunks' attention, most keys first; an item is a tile and one or two of its heads ----
   int pre_mt[2] = {2, 2};                       // query tiles per item for head sizes 64 and 128
   for (int hi = 0; hi < 2; ++hi) {
     long long tiles = 0;
@@ -972,18 +976,17 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       for (int t = 0; t * FLASH_TILE < a.pre[r].n_tok; ++t)
         tiles.push_back({(a.pre[r].kv_len + std::min(a.pre[r].n_tok, (t + 1) * FLASH_TILE) + FLASH_TILE - 1) / FLASH_TILE, r, t});
     std::stable_sort(tiles.begin(), tiles.end(), [](const Tile& x, const Tile& y) { return x.blocks > y.blocks; });
-    std::vector<PrefillItem> items;
-    items.reserve(tiles.size() * a.m->d.n_heads);
-    for (const Tile& t : tiles)
-      for (int kvh = 0; kvh < a.m->d.n_kv_heads; ++kvh)
-        for (int h = 0; h < G; h += mt) {
-          const PrefillChunk& p = a.pre[t.req];
-          const int t0 = t.tile * FLASH_TILE;
-          items.push_back({p.table, p.row_start + t0, std::min(FLASH_TILE, p.n_tok - t0), p.kv_len + t0, kvh * G + h, {0, 0}});
-        }
-    a.pre_items = (int)items.size();
-    a.pitem_off = put(items.data(), items.size() * sizeof(PrefillItem), 16);
-    if (a.pitem_off == (size_t)-1) overflow = true;
+    std::vector<PrefillTile> list;
+    list.reserve(tiles.size());
+    for (const Tile& t : tiles) {
+      const PrefillChunk& p = a.pre[t.req];
+      const int t0 = t.tile * FLASH_TILE;
+      list.push_back({p.table, p.row_start + t0, std::min(FLASH_TILE, p.n_tok - t0), p.kv_len + t0, 0});
+    }
+    a.pre_items = (int)list.size() * a.m->d.n_kv_heads * ((G + mt - 1) / mt);
+    a.ptile_off = put(list.data(), list.size() * sizeof(PrefillTile), 16);
+    a.pmaps_off = put(&a.m->pre_maps, sizeof(PrefillMaps), 64);
+    if (a.ptile_off == (size_t)-1 || a.pmaps_off == (size_t)-1) overflow = true;
   }
 
   // ---- plan (A1): sweep the kernel kinds until every model's op list is exhausted ----
@@ -1114,11 +1117,14 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
           for (Active* a : who) {
             if (a->m->ops[a->cursor].apre.hd != hd || a->n_pre == 0) continue;
             AttnPrefillGroup g = a->m->ops[a->cursor].apre;
-            g.items = (const PrefillItem*)(slot.dev + a->pitem_off);
+            g.tiles = (const PrefillTile*)(slot.dev + a->ptile_off); g.maps = (const PrefillMaps*)(slot.dev + a->pmaps_off);
+            const int head_items = (g.Hq / g.Hkv + pre_mt[hd == 128 ? 1 : 0] - 1) / pre_mt[hd == 128 ? 1 : 0];   // (Hq / Hkv is 1, 2, 4 or 8)
+            for (g.head_shift = 0; 1 << g.head_shift < head_items;) ++g.head_shift;
+            g.by_hkv = g.Hkv == 1 ? 0u : (unsigned)(((1ull << 32) + g.Hkv - 1) / g.Hkv);
             g.item_start = items; g.n_items = a->pre_items;
             items += a->pre_items;
             ++n_put;
-            if (put(&g, sizeof(g), 64) == (size_t)-1) overflow = true;
+            if (put(&g, sizeof(g), 8) == (size_t)-1) overflow = true;
           }
           LL.n_groups = n_put; LL.p0 = items; LL.p1 = hd; LL.p2 = pre_mt[hd == 128 ? 1 : 0];
           if (n_put > 0) launches.push_back(LL);

@@ -293,9 +293,9 @@ __global__ void __launch_bounds__(ROPE_THREADS) rope_append_kernel(const RopeGro
   const int b = blockIdx.x;               // token row
   if (b >= g.B) return;
   const RowDesc rd = g.rows[b];
-  if (g.only_chunks && rd.single) return;
+  if (g.only_chunks && rd.single()) return;
   const int pos = rd.pos, hd = g.hd, half = hd >> 1;
-  const int page = g.reqs[rd.req].table[pos / 16], slot = pos % 16;
+  const int page = g.reqs[rd.req()].table[pos / 16], slot = pos % 16;
   const int e = (threadIdx.x * 8) % hd;   // ROPE_THREADS * 8 is a multiple of every head size
   const float4* cs = reinterpret_cast<const float4*>(g.cs + (size_t)pos * half + (e >> 1));
   const float4 t0 = __ldg(cs), t1 = __ldg(cs + 1);

@@ -419,3 +419,29 @@ def test_many_paired_items_in_a_row_with_raised_maxima(mods, hd, Hq, Hkv, chunks
     for i, alone in zip(picked, got[1:]):
         assert torch.equal(got[0][i][0], alone[i][0]) and got[0][i][1] == alone[i][1]
         _check_prefill(v, pool_all, pool0, got[0][i], toks[i], kv0, tabs[i], f"chunk {i} of {chunks}")
+
+
+def test_thousands_of_short_chunks_fit_one_step(mods):
+    """3900 prompt chunks of two tokens on a model of 32 heads: their descriptors (request, rows, one tile each) take a tenth
+    of the step's blob.  Sampled answers equal the oracle."""
+    E, server = mods
+    n_req, n = 3900, 2
+    p = synth.make_decoder(d=64, n_layers=2, n_q_heads=32, n_kv_heads=32, head_dim=64, ffn=64, vocab=50, seed=80, device=DEV, std=0.1)
+    rng = np.random.default_rng(81)
+    toks = rng.integers(0, 50, (n_req, n))
+    order = rng.permutation(n_req).astype(np.int32)
+    tables = torch.as_tensor(order, device=DEV)
+    pool = torch.zeros((2, n_req, 2, 32, 16, 64), dtype=torch.bfloat16, device=DEV)
+    pool0 = pool[:, :1].clone()                                          # (every page is empty)
+    srv = server.Server(workspace_bytes=2 << 30, cap_fs=4096)
+    m = srv.add_model(p, kv_pool=pool, max_kv_len=16, max_batch=n_req * n)
+    ts = [srv.submit(m, E.CAT_FS, tokens=toks[i], kv_len=0, table=tables[i:i + 1]) for i in range(n_req)]
+    assert srv.step().prefill_tokens == n_req * n
+    torch.cuda.synchronize()
+    res = [srv.collect(t) for t in ts]
+    assert all(s == E.OK for s, _, _ in res)
+    v = synth.bits_view({k: p[k] for k in p if k != "packed_layers"})
+    for i in (0, 1, 1777, n_req - 1):
+        ref = O.decoder_prefill([int(t) for t in toks[i]], 0, order[i:i + 1], lambda l, pg: synth.to_bits(pool0[l, 0]), v, round_bf16=True)
+        assert_close(res[i][1], ref["logits"], what=f"chunk {i}")
+    srv.close()
