@@ -378,9 +378,10 @@ int epara_decode_attention_static_status(int device, int* code);
 size_t epara_static_scratch_bytes(void);
 
 /* Self-test of the bounded waits (the paper has no counterpart; it exists so that the give-up path of the
- * kernels' waits can be run without making a real kernel misbehave).  Launches one thread that waits, for
- * at most limit_ns (<= 1 s), on a barrier nothing ever arrives at, then synchronises the stream.  Expected
- * answer: EPARA_E_DEVICE with *code = 90 (the wait ran out and the kernel returned by itself).
+ * kernels' waits can be run without making a real kernel misbehave).  Launches one warp that waits, for
+ * at most limit_ns (<= 1 s), half of its lanes on a barrier nothing ever arrives at, then synchronises the
+ * stream.  Expected answer: EPARA_E_DEVICE with *code = 90 (the wait ran out for every lane and the kernel
+ * returned by itself; 91: only some lanes gave up).
  * status_dev: device int32 used as the status word; code: host. */
 int epara_selftest_bounded_wait(int device, void* cuda_stream, unsigned long long limit_ns, int* status_dev, int* code);
 

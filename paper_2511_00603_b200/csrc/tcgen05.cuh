@@ -25,7 +25,9 @@ __device__ __forceinline__ unsigned long long globaltimer() {
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
   return t;
 }
-// Bounded wait for the phase with the given parity.  Returns false when it gave up.
+// Bounded wait of a whole converged warp for the phase with the given parity.  Returns false when it gave up, to all lanes
+// alike: a lane that gave up beside one that saw the phase complete would leave that one at the next `elect.sync` or vote,
+// which have no limit.
 // SLEEP: back off with nanosleep after a few polls (for waits that are long while other warps of the
 // CTA need the issue slots); without it the wait is the hardware's own suspending try_wait in a loop.
 // limit_ns: how long the wait may last (measured from its first check of the clock, about a thousand polls in).
@@ -40,18 +42,19 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    if (done) return true;
+    if (__all_sync(0xffffffffu, done)) return true;
     if (SLEEP && it >= 8) __nanosleep(32);    // a long wait: stop competing with the epilogue warps for issue slots
     if ((it & 1023u) == 1023u) {
-      if (*abort_flag) return false;
+      bool give_up = *abort_flag != 0;
       const unsigned long long now = globaltimer();
       if (t0 == 0) t0 = now;
-      else if (now - t0 > limit_ns) return false;
+      else give_up |= now - t0 > limit_ns;
+      if (__any_sync(0xffffffffu, give_up)) return false;
     }
   }
 }
 
-// Non-blocking look at a barrier's phase.
+// Non-blocking look of a converged warp at a barrier's phase; one answer for all lanes.
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   uint32_t done;
   asm volatile(
@@ -59,7 +62,7 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
       "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-  return done != 0;
+  return __all_sync(0xffffffffu, done);
 }
 
 // Used on the give-up path only: lets TMA copies that are still in flight towards this CTA's shared memory
