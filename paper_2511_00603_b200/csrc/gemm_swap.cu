@@ -171,8 +171,12 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
     uint32_t wphase = 0, aphase = 0;
     bool ok = true;
     for (int kb = kb0; kb < kb1; ++kb) {
-      if (!mbar_wait<false>(afull_bar(as), aphase, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 45); break; }
-      if (!mbar_wait<false>(wfull_bar(ws), wphase, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 42); break; }
+      if (!mbar_wait_both(afull_bar(as), aphase, wfull_bar(ws), wphase, abort_flag)) {
+        ok = false;
+        const int code = mbar_test(afull_bar(as), aphase) ? 42 : 45;
+        if (lane == 0) atomicExch(status, code);
+        break;
+      }
       const uint64_t dw = make_smem_desc(w_base + ws * SW_W_BYTES), da = make_smem_desc(base + as * a_bytes);
 #pragma unroll
       for (int k = 0; k < TC_BK / 16; ++k)

@@ -54,6 +54,30 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// The same for two barriers at once (one vote when both phases are complete).
+__device__ __forceinline__ bool mbar_wait_both(uint32_t bar_a, uint32_t parity_a, uint32_t bar_b, uint32_t parity_b, volatile int* abort_flag,
+                                               unsigned long long limit_ns = WAIT_LIMIT_NS) {
+  unsigned long long t0 = 0;
+  for (unsigned it = 0;; ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 q, [%3], %4;\n\t"
+        "and.pred p, p, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done) : "r"(bar_a), "r"(parity_a), "r"(bar_b), "r"(parity_b) : "memory");
+    if (__all_sync(0xffffffffu, done)) return true;
+    if ((it & 1023u) == 1023u) {
+      bool give_up = *abort_flag != 0;
+      const unsigned long long now = globaltimer();
+      if (t0 == 0) t0 = now;
+      else give_up |= now - t0 > limit_ns;
+      if (__any_sync(0xffffffffu, give_up)) return false;
+    }
+  }
+}
+
 // Non-blocking look of a converged warp at a barrier's phase; one answer for all lanes.
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   uint32_t done;
