@@ -312,3 +312,34 @@ def test_grouped_gemm_takes_row_strides_of_c_that_its_kernels_can_store(E, M, N,
     assert torch.equal(C[:, :n_out], wide[:, :n_out]) and bool((C[:, :n_out] != C0[:, :n_out]).any())
     pad = n_out + (-n_out) % (4 if "resid" in fl else 8)              # columns up to there may be overwritten
     assert torch.equal(C[:, pad:], C0[:, pad:])
+
+
+@pytest.mark.parametrize("hd,Hq,Hkv", [(64, 8, 2), (128, 4, 4), (32, 4, 1)])
+def test_decode_attention_merges_any_number_of_chunks(E, hd, Hq, Hkv):
+    """16, 17, 32, 33 and 41 chunks of 256 tokens, whose partials are merged 16 at a time, and few: against the oracle, merged
+    by the last block to arrive, and with the same bits by the second kernel (more requests in the call).  The keys of the
+    later chunks are larger, so that the maximum of a later group of chunks is the larger one."""
+    dev = torch.device("cuda")
+    lens = np.array([4096, 4097, 8192, 8193, 10300, 700, 30], dtype=np.int32)
+    B, n_pages = len(lens), (10300 + 15) // 16
+    table = np.random.default_rng(41).permutation(n_pages).astype(np.int32)
+    pool = synth.make_kv_pool(1, n_pages, Hkv, hd, seed=42, device=dev)[0]
+    for i, pg in enumerate(table):
+        pool[int(pg), 0] *= 0.5 + 2.0 * i / n_pages
+    outs = []
+    for times in (1, 40):
+        n = B * times
+        q = torch.randn((B, Hq * hd), generator=torch.Generator(device=dev).manual_seed(43), device=dev).to(torch.bfloat16).repeat(times, 1)
+        out = torch.empty_like(q)
+        scratch = torch.empty(E.lib.epara_decode_attention_scratch_bytes(n, Hq, hd, 10300), dtype=torch.uint8, device=dev)
+        E.epara_decode_attention(q, pool, torch.as_tensor(np.tile(lens, times), device=dev), torch.as_tensor(table, device=dev).repeat(n, 1), out,
+                                 Hq, Hkv, hd, 10300, scratch, _stream())
+        torch.cuda.synchronize()
+        outs.append((q, out))
+    q, out = outs[0]
+    assert torch.equal(outs[1][1], out.repeat(40, 1))
+    pool_bits, qf = synth.to_bits(pool), O.bf16_to_f64(synth.to_bits(q)).reshape(B, Hq, hd)
+    for b, L in enumerate(lens):
+        K, V = O.gather_kv(lambda l, pg: pool_bits[pg], 0, table, int(L))
+        ref = np.stack([O.attention(qf[b, h], K[h // (Hq // Hkv)], V[h // (Hq // Hkv)]) for h in range(Hq)])
+        assert_close(out[b].reshape(Hq, hd), ref, what=f"decode attention of {L} tokens")
