@@ -691,7 +691,12 @@ int epara_init(const epara_config* cfg, epara_ctx** out) {
     s.launch_status = EPARA_OK;
     s.host = c->pinned + i * (BLOB_BYTES + 64);
     s.status_host = reinterpret_cast<int*>(s.host + BLOB_BYTES);
-    if (cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming) != cudaSuccess) return EPARA_E_CUDA;
+    if (cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming) != cudaSuccess) {
+      while (i > 0) cudaEventDestroy(c->slots[--i].done);
+      cudaFreeHost(c->pinned);
+      delete c;
+      return EPARA_E_CUDA;
+    }
     *s.status_host = 0;
   }
   *out = c;
