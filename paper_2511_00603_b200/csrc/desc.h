@@ -72,11 +72,6 @@ struct alignas(64) GemmGroup {
   int pad[4];
 };
 
-struct GemmLaunch {      // header followed by groups
-  int n_groups;
-  int total_tiles;
-};
-
 enum : int { NORM_LN = 0, NORM_RMS = 1 };
 struct NormGroup {
   const float* x;        // fp32 [M rows, row stride x_stride]

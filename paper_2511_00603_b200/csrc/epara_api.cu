@@ -30,7 +30,10 @@ namespace {
 constexpr int N_SLOTS = 4;
 constexpr size_t BLOB_BYTES = 4u << 20;
 constexpr int MAX_PROFILE_LAUNCHES = 4096;
-constexpr int PASS_MLP = 11;   // last of a GEMM wave's launches (see epara_step)
+constexpr int PASS_SWAP = 3, PASS_MLP = 7;   // launches of a GEMM wave (see epara_step); PASS_MLP is the last
+constexpr int N_SWAP = PASS_MLP - PASS_SWAP;  // swapped-operand launches: 1, 2, 4 or 8 k ranges per tile
+
+inline int swap_index(int ksplit) { return ksplit >= 8 ? 3 : ksplit >= 4 ? 2 : ksplit >= 2 ? 1 : 0; }
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 inline int round_up(int v, int a) { return (v + a - 1) / a * a; }
@@ -1029,15 +1032,15 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       // contexts only), the weight-streaming kernel for groups of few rows or small matrices (pass 1) and
       // 256-row tiles on CTA pairs (pass 2); encoder attention in two: the tcgen05 kernel (pass 0) and the
       // mma.sync kernel for shapes it does not take (pass 1)
-      // (passes 3 to 10: the swapped-operand kernel with 1 to 8 k ranges per tile)
-      // (pass 11: encoder MLP blocks in the fused kernel)
+      // (passes 3 to 6: the swapped-operand kernel with 1, 2, 4 and 8 k ranges per tile)
+      // (pass 7: encoder MLP blocks in the fused kernel)
       const int n_pass = kind == EPARA_K_GEMM ? PASS_MLP + 1 : (kind == EPARA_K_ATTN_ENC ? 2 : 1);
       unsigned passes = ~0u;                                   // GEMM passes that some model needs
       if (kind == EPARA_K_GEMM) {
         passes = 1u << (n_pass - 1);                           // (the last pass also moves the cursors on)
         for (Active* a : who) {
           const GemmGroup& g = a->m->ops[a->cursor].gemm;
-          passes |= 1u << (g.stream == 3 ? 2 + g.ksplit : g.stream == 4 ? PASS_MLP : g.stream);
+          passes |= 1u << (g.stream == 3 ? PASS_SWAP + swap_index(g.ksplit) : g.stream == 4 ? PASS_MLP : g.stream);
         }
       }
       for (int pass = 0; pass < n_pass; ++pass) {
@@ -1183,7 +1186,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
             break;
           }
           case EPARA_K_GEMM: {
-            const int gpass = op.gemm.stream == 3 ? 2 + op.gemm.ksplit : op.gemm.stream == 4 ? PASS_MLP : op.gemm.stream;
+            const int gpass = op.gemm.stream == 3 ? PASS_SWAP + swap_index(op.gemm.ksplit) : op.gemm.stream == 4 ? PASS_MLP : op.gemm.stream;
             if (gpass != pass) break;                          // another pass takes it
             if (op.gemm.stream == 4) {
               MlpGroup mg = op.mlp;
@@ -1330,7 +1333,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       case EPARA_K_NORM: launch_norm((const NormGroup*)gp, L.n_groups, L.p1, st); break;
       case EPARA_K_GEMM:
         if (L.p2 == PASS_MLP) err = launch_gemm_mlp_pair((const MlpGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st);
-        else if (L.p2 >= 3) err = launch_gemm_swap((const GemmGroup*)gp, L.n_groups, L.p0, L.p2 - 2, L.p3, dev_status, c->sm_count, st);
+        else if (L.p2 >= PASS_SWAP) err = launch_gemm_swap((const GemmGroup*)gp, L.n_groups, L.p0, 1 << (L.p2 - PASS_SWAP), L.p3, dev_status, c->sm_count, st);
         else if (L.p2 == 1) err = launch_gemm_stream((const GemmGroup*)gp, L.n_groups, L.p0, L.p1, st);
         else if (L.p2 == 2) err = launch_gemm_tc_pair((const GemmGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st);
         else launch_gemm_simt((const GemmGroup*)gp, L.n_groups, L.p0, st);
@@ -1464,8 +1467,8 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
   if (cudaSetDevice(device) != cudaSuccess) return EPARA_E_CUDA;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   std::vector<GemmGroup> gs, gs_stream, gs_pair;   // CUDA-core groups; weight-streaming groups (M <= 16); CTA-pair groups
-  std::vector<GemmGroup> gs_swap[8];               // swapped-operand groups by k ranges per tile (1 to 8)
-  int total_swap[8] = {0}, nb_swap[8] = {0};
+  std::vector<GemmGroup> gs_swap[N_SWAP];          // swapped-operand groups by k ranges per tile
+  int total_swap[N_SWAP] = {0}, nb_swap[N_SWAP] = {0};
   int total = 0, total_stream = 0, max_rows_stream = 0, total_pair = 0;
   for (int i = 0; i < n; ++i) {
     const epara_gemm_problem& q = p[i];
@@ -1488,7 +1491,7 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
     if (!simt && gemm_swap_eligible(q.M, q.N, q.K, q.epilogue, sm_count)) {
       g.stream = 3;
       gemm_swap_config(q.M, q.N, q.K, sm_count, &g.bn, &g.ksplit);
-      const int si = g.ksplit - 1;
+      const int si = swap_index(g.ksplit);
       g.tiles_m = (q.M + g.bn - 1) / g.bn; g.tiles_n = gemm_swap_tiles_n(q.N);
       g.tile_start = total_swap[si];
       total_swap[si] += g.tiles_m * g.tiles_n;
@@ -1519,10 +1522,10 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
   GemmGroup* dev_groups = (GemmGroup*)((unsigned char*)scratch + 256);
   GemmGroup* dev_stream = dev_groups + gs.size();
   GemmGroup* dev_pair = dev_stream + gs_stream.size();
-  GemmGroup* dev_swap[8];
+  GemmGroup* dev_swap[N_SWAP];
   dev_swap[0] = dev_pair + gs_pair.size();
-  for (int i = 1; i < 8; ++i) dev_swap[i] = dev_swap[i - 1] + gs_swap[i - 1].size();
-  for (int i = 0; i < 8; ++i)
+  for (int i = 1; i < N_SWAP; ++i) dev_swap[i] = dev_swap[i - 1] + gs_swap[i - 1].size();
+  for (int i = 0; i < N_SWAP; ++i)
     if (!gs_swap[i].empty() &&
         cudaMemcpyAsync(dev_swap[i], gs_swap[i].data(), gs_swap[i].size() * sizeof(GemmGroup), cudaMemcpyHostToDevice, st) != cudaSuccess)
       return EPARA_E_CUDA;
@@ -1546,8 +1549,8 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
     err = launch_gemm_stream(dev_stream, (int)gs_stream.size(), total_stream, max_rows_stream, st);
     if (err == cudaSuccess)
       err = launch_gemm_tc_pair(dev_pair, (int)gs_pair.size(), total_pair, status, sm, st);
-    for (int i = 0; i < 8 && err == cudaSuccess; ++i)
-      err = launch_gemm_swap(dev_swap[i], (int)gs_swap[i].size(), total_swap[i], i + 1, nb_swap[i], status, sm, st);
+    for (int i = 0; i < N_SWAP && err == cudaSuccess; ++i)
+      err = launch_gemm_swap(dev_swap[i], (int)gs_swap[i].size(), total_swap[i], 1 << i, nb_swap[i], status, sm, st);
   }
   return err == cudaSuccess ? EPARA_OK : EPARA_E_CUDA;
 }

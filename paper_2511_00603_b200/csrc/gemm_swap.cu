@@ -356,7 +356,7 @@ cudaError_t launch_swap(const GemmGroup* groups, int n_groups, int total_items, 
 // Above, one CTA takes an SM and the clusters have to be resident together: 74 of two CTAs, 33 of four and 15 of eight
 // fit on 148 SMs (sizes between them fit no more CTAs; one cluster too many costs a second wave: 2048 x 2048 at 256
 // rows 27 us with 16 clusters of eight, 15 on tile pairs).  A k-block costs 0.23 us + 1.1 ns per row, the exchange of
-// the partial sums runs at 22 bytes a cycle per SM.
+// the partial sums runs at 41.8 KB a microsecond per SM.
 double gemm_swap_config(long long rows_cap, int N, int K, int sm_count, int* nb, int* ksplit) {
   const int tiles_n = (N + SW_BM - 1) / SW_BM, kblocks = (K + TC_BK - 1) / TC_BK;
   const int tiles_m = (int)((rows_cap + GEMM_SWAP_TILE_ROWS - 1) / GEMM_SWAP_TILE_ROWS);
@@ -374,7 +374,7 @@ double gemm_swap_config(long long rows_cap, int N, int K, int sm_count, int* nb,
     if (tiles <= fit[i] && kblocks >= 3 << i) s = 1 << i;
   *ksplit = s;
   const double rounds = (double)((tiles + fit[0] - 1) / fit[0]);
-  return 10.0 + rounds * ((kblocks + s - 1) / s) * (0.23 + 0.0011 * *nb) + (s > 1 ? *nb * 512.0 * (s - 1) / s / 22.0 / 1900.0 : 0.0);
+  return 10.0 + rounds * ((kblocks + s - 1) / s) * (0.23 + 0.0011 * *nb) + (s > 1 ? *nb * 512.0 * (s - 1) / s / 41800.0 : 0.0);
 }
 
 // Up to 128 rows a tile of A would be mostly padding for the tile-pair kernel.  Above, the estimates decide: the split
@@ -394,11 +394,7 @@ cudaError_t launch_gemm_swap(const GemmGroup* groups, int n_groups, int total_it
   switch (ksplit) {
     case 1: return launch_swap<1>(groups, n_groups, total_items, max_nb, status, sm_count, st);
     case 2: return launch_swap<2>(groups, n_groups, total_items, max_nb, status, sm_count, st);
-    case 3: return launch_swap<3>(groups, n_groups, total_items, max_nb, status, sm_count, st);
     case 4: return launch_swap<4>(groups, n_groups, total_items, max_nb, status, sm_count, st);
-    case 5: return launch_swap<5>(groups, n_groups, total_items, max_nb, status, sm_count, st);
-    case 6: return launch_swap<6>(groups, n_groups, total_items, max_nb, status, sm_count, st);
-    case 7: return launch_swap<7>(groups, n_groups, total_items, max_nb, status, sm_count, st);
     case 8: return launch_swap<8>(groups, n_groups, total_items, max_nb, status, sm_count, st);
   }
   return cudaErrorInvalidValue;
