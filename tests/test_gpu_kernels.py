@@ -34,12 +34,12 @@ GEMM_CASES = [
     (77, 768, 3072, ("bias", "resid")),
     (0, 64, 64, ()),                    # empty group
     (257, 136, 64, ("gelu", "bias")),   # single k-block, N tail of 8
-    (40, 1024, 1024, ("swiglu",)),      # split along K with a SwiGLU epilogue
-    (256, 2048, 4096, ("resid",)),      # two row tiles, long K
-    (64, 512, 8192, ("bias", "resid")), # few tiles, very long K: split along K with the last-arriver reduction
+    (40, 1024, 1024, ("swiglu",)),      # the largest matrix of the weight-streaming kernel at more than 16 rows
+    (256, 2048, 4096, ("resid",)),      # long K, split over a cluster of four
+    (64, 512, 8192, ("bias", "resid")), # few tiles, very long K: split over a cluster of eight
     (20, 768, 4096, ("gelu", "bias")),  # split along K, bf16 output
-    (9, 256, 5120, ("swiglu",)),        # split along K, SwiGLU, uneven ranges
-    # at most 16 rows: the weight-streaming kernel (16 W rows per block, k-blocks of 32 dealt to 8 warps)
+    # at most 16 rows: the weight-streaming kernel (16 W rows per block, k-blocks of 32 dealt to 16 warps)
+    (9, 256, 5120, ("swiglu",)),        # long K, SwiGLU
     (16, 1000, 776, ("bias",)),         # ragged N, K not a multiple of 32
     (3, 10, 512, ("bias",)),            # N below one block
     (5, 64, 8, ()),                     # a single 16-byte piece of K
@@ -125,10 +125,10 @@ def test_grouped_gemm_small_matrices_in_tiles_of_32_rows(E, M):
 
 
 def test_grouped_gemm_tile_pairs(E):
-    """Dense bf16-output problems (more than 256 rows, 256-wide tiles) run as 256-row tiles on CTA pairs:
-    ragged last pair (one CTA with no valid row), N tails inside the first and the second half of the W
-    rows, SwiGLU, one k-block, a long K beyond the six-stage ring, more pairs than SM pairs, fp32-residual
-    outputs with 192- and 256-wide tiles, 128-wide tiles of problems with 129 to 256 rows, N below one tile."""
+    """Problems of more than 128 rows run as 256-row tiles on CTA pairs, these in tiles of 128 columns (wider ones:
+    test_grouped_gemm_wide_tile_pairs): ragged last pair (one CTA with no valid row), N tails inside the first and the
+    second half of the W rows, SwiGLU, one k-block, a K beyond the six-stage ring, more pairs than SM pairs, fp32-residual
+    outputs, 129 to 256 rows, N below one tile; and one long K with few tiles, which the swapped operands take."""
     cases = [(1000, 1152, 384, ("bias",)), (513, 2048, 256, ("swiglu",)), (700, 264, 1536, ("bias", "gelu")),
              (257, 392, 64, ()), (20000, 512, 128, ("bias",)), (384, 256, 4096, ("gelu", "bias")),
              (900, 384, 384, ("bias", "resid")), (515, 768, 1536, ("resid",)), (1300, 576, 192, ("bias", "resid")),
@@ -141,11 +141,11 @@ def test_grouped_gemm_tile_pairs(E):
 
 
 def test_grouped_gemm_swapped_operands_17_to_128_rows(E):
-    """Problems of 17 to 128 rows run with W as the tensor core's 128-row operand and the batch as its N, a cluster
-    of 1, 2, 4 or 8 CTAs per tile of 128 output columns splitting K (reduced through distributed shared memory in
-    rank order): every epilogue, N below and not a multiple of a tile, K not a multiple of a k-block, batch sizes
-    on both sides of the multiples of 16, one k-block, and the decode shapes of the 1B decoder.  The same problem
-    alone and among others gives the same bits."""
+    """Problems of 17 to 128 rows with matrices of more than a million elements run with W as the tensor core's 128-row
+    operand and the batch as its N, a cluster of 1, 2, 4 or 8 CTAs per tile of 128 output columns splitting K (reduced
+    through distributed shared memory in rank order): the decode shapes of the 1B decoder, batch sizes on both sides of
+    the multiples of 16, beside smaller matrices, which go to the weight-streaming kernel in the same call (tails of N and K:
+    test_grouped_gemm_swapped_operands_tails).  The same problem alone and among others gives the same bits."""
     cases = [(17, 10, 512, ("bias",)), (128, 3072, 2048, ()), (100, 1000, 776, ("bias",)), (48, 2048, 8192, ("resid",)),
              (33, 512, 256, ("swiglu",)), (64, 2048, 2048, ("resid", "bias")), (127, 16384, 2048, ("swiglu",)),
              (32, 1024, 256, ("bias", "gelu")), (96, 136, 64, ("gelu", "bias")), (20, 768, 4096, ("gelu", "bias")),
@@ -169,6 +169,45 @@ def test_grouped_gemm_swapped_operands_17_to_128_rows(E):
     torch.cuda.synchronize()
     assert bool((part[40:] == 7.0).all())
     assert_close(part[:40], to_f64(full[:40]), what="first 40 rows", tol=1e-6)
+
+
+def test_grouped_gemm_swapped_operands_tails(E):
+    """17 to 128 rows and matrices of more than a million elements (smaller ones go to the weight-streaming kernel): N no
+    multiple of a tile, of a vector store or of two, K no multiple of a k-block, clusters of 1, 2, 4 and 8, every epilogue,
+    row counts on both sides of the multiples of 16.  Alone and among others: the same bits.  Rows past the live ones, in
+    a matrix that has more, keep what they hold."""
+    cases = [(17, 1000, 1544, ("bias",)), (33, 4100, 264, ("gelu", "bias")), (64, 4102, 520, ("swiglu",)), (100, 8200, 2056, ()),
+             (128, 1030, 4104, ("resid",)), (96, 264, 8200, ("bias", "resid")), (50, 32001, 72, ("bias",)), (40, 1034, 1160, ("swiglu",))]
+    probs, refs = _run_gemm(E, E.GEMM_TCGEN05, cases, seed=21)
+    for p, ref, case in zip(probs, refs, cases):
+        assert_close(p["C"][:ref.shape[0], :ref.shape[1]], ref, what=f"swapped gemm {case}")
+    alone, _ = _run_gemm(E, E.GEMM_TCGEN05, cases[:2], seed=21)
+    assert torch.equal(alone[1]["C"][:, :4100], probs[1]["C"][:, :4100])
+    M, N, K = 128, 1032, 4104
+    g = torch.Generator(device="cuda").manual_seed(22)
+    A = torch.randn((M, K), generator=g, device="cuda").to(torch.bfloat16)
+    W = (torch.randn((N, K), generator=g, device="cuda") * 0.05).to(torch.bfloat16)
+    for rows in (40, 17, 113):
+        full = torch.full((M, N), 7.0, device="cuda", dtype=torch.bfloat16)
+        part = full.clone()
+        for C_, n in ((full, M), (part, rows)):
+            pr = [{"A": A, "W": W, "C": C_, "bias": None, "M": n, "N": N, "K": K, "epilogue": 0}]
+            sc = torch.empty(E.epara_gemm_scratch_bytes_for(pr), dtype=torch.uint8, device="cuda")
+            E.epara_grouped_gemm(pr, _stream(), sc)
+        torch.cuda.synchronize()
+        assert bool((part[rows:] == 7.0).all()) and torch.equal(part[:rows], full[:rows])
+
+
+def test_grouped_gemm_wide_tile_pairs(E):
+    """Tile pairs 256 and 192 columns wide: N tails in either half of the W rows, ragged last rows, more tiles than pairs (a
+    pair's second tile uses the other accumulator), K no multiple of a k-block, every epilogue."""
+    cases = [(900, 8200, 520, ("bias", "gelu")), (1537, 4200, 1096, ("swiglu",)), (1025, 6000, 1160, ("bias", "resid")),
+             (1500, 3264, 1160, ("resid",)), (900, 5184, 712, ("bias", "resid"))]
+    probs, refs = _run_gemm(E, E.GEMM_TCGEN05, cases, seed=23)
+    for p, ref, case in zip(probs, refs, cases):
+        assert_close(p["C"][:ref.shape[0], :ref.shape[1]], ref, what=f"wide pair gemm {case}")
+    alone, _ = _run_gemm(E, E.GEMM_TCGEN05, cases[:1], seed=23)
+    assert torch.equal(alone[0]["C"], probs[0]["C"])
 
 
 def test_grouped_gemm_rejects_bad_arguments(E):
@@ -229,7 +268,7 @@ def test_gelu_epilogue_sweep_through_identity_gemm(E, rows):
     GEMM with the identity as weights, so the accumulator holds x exactly and the epilogue alone decides the
     output.  Bound: the fitted form's 2.6e-5, the hardware tanh's relative error 2^-11 scaled by 0.5 |x|
     (2.5e-4 |x|), and the rounding of the bf16 store (half an ulp: at most 2^-8 of the result).  The row counts select the
-    weight-streaming kernel, the swapped-operand kernel, the one-CTA tile kernel and the tile-pair kernel."""
+    weight-streaming kernel (16 rows and 100) and the tile-pair kernel; the swapped operands have a sweep of their own."""
     dev = torch.device("cuda")
     K = N = 256
     x = torch.linspace(-8.0, 8.0, rows * K, device=dev).reshape(rows, K)
@@ -248,6 +287,23 @@ def test_gelu_epilogue_sweep_through_identity_gemm(E, rows):
     bad = np.abs(got - ref) > bound
     assert not bad.any(), f"{int(bad.sum())} of {bad.size} outside the bound; worst excess " \
                           f"{float(np.max(np.abs(got - ref) - bound)):.3e} at x = {float(xs[np.unravel_index(np.argmax(np.abs(got - ref) - bound), xs.shape)])}"
+
+
+def test_gelu_epilogue_sweep_through_the_swapped_operands(E):
+    """The sweep of the test above through the swapped-operand kernel, which takes identities of more than a million elements at
+    100 rows."""
+    dev = torch.device("cuda")
+    rows, K = 100, 1032
+    x = torch.linspace(-8.0, 8.0, rows * K, device=dev).reshape(rows, K)
+    x = x[:, torch.randperm(K, generator=torch.Generator(device=dev).manual_seed(rows), device=dev)].to(torch.bfloat16)
+    C = torch.full((rows, K), float("nan"), device=dev, dtype=torch.bfloat16)
+    prob = [{"A": x, "W": torch.eye(K, device=dev).to(torch.bfloat16), "C": C, "bias": None, "M": rows, "N": K, "K": K, "epilogue": E.EPI_GELU}]
+    scratch = torch.empty(E.epara_gemm_scratch_bytes_for(prob), dtype=torch.uint8, device=dev)
+    E.epara_grouped_gemm(prob, _stream(), scratch)
+    torch.cuda.synchronize()
+    xs = O.bf16_to_f64(synth.to_bits(x))
+    ref = O.gelu(xs)
+    assert not (np.abs(to_f64(C) - ref) > 2.6e-5 + 2.5e-4 * np.abs(xs) + 2.0 ** -8 * np.abs(ref) + 1e-7).any()
 
 
 @pytest.mark.parametrize("rows", [129, 197, 256, 257, 509, 1024])
