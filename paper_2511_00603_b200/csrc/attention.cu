@@ -5,8 +5,8 @@
 // all G query heads that share the kv head, so every K/V byte is read once.  The chunk size is
 // a constant, hence a request's reduction order never depends on what else is in the step.
 // A page's (K or V, head) tile is 16 x hd contiguous bf16; a warp reads it with 128-bit loads,
-// lanes covering consecutive 16-byte pieces.  Partials (m, l, o) go to scratch; the block of a
-// (request, kv head) that finishes last merges the chunks in chunk order (finish_chunk).
+// lanes covering consecutive 16-byte pieces.  Partials (m, l, o) go to scratch and are merged in chunk order by a second
+// kernel (attn_combine_kernel), for few and short requests by the block of a (request, kv head) that finishes last.
 //
 // Encoder (ViT): full bidirectional attention of T tokens per (image, head).
 #include <cstring>
@@ -137,10 +137,9 @@ __device__ __forceinline__ void finish_chunk(const AttnDecGroup& g, int b, int r
   }
 }
 
-// Separate merge for launches with many blocks: a block takes 256 / HD query heads of a request of more than one chunk.
+// Separate merge: a block takes 256 / HD query heads of a request of more than one chunk.
 // (With a thread per element, the lengths read after the wait and two passes over the partials it took 9.5 us behind the
-// attention of 27 requests of the 1B decoder: 613 us of attention a step, now 522; one request, merged in the attention
-// kernel, 236 and 206.)
+// attention of 27 requests of the 1B decoder: 613 us of attention a step, then 522.)
 constexpr int COMBINE_THREADS = 128;
 template <int HD>
 __global__ void __launch_bounds__(COMBINE_THREADS, 6) attn_combine_kernel(const AttnDecGroup* __restrict__ groups, int n_groups) {
@@ -607,12 +606,16 @@ static cudaError_t launch_dec(const AttnDecGroup* groups, int n_groups, int tota
   return launch_pdl(attn_decode_kernel<HD, G>, dim3(max_chunks, max_Hkv, total_B), dim3(128), 0, st, groups, n_groups, fused);
 }
 
-// Few blocks (up to two waves): the last block of a (request, kv head) merges the chunks itself and the
-// step saves a launch.  Many blocks: the counter round trip at the end of every block costs more than
-// a second kernel, so the merge runs as attn_combine_kernel (with the merge as it was then, 1B decoder, 27
-// requests: 659 us of attention per step merged in the kernel, 612 with the second one; 8B, 64 requests: 4252 and 3798).
-bool attn_decode_fused(int total_B, int max_Hkv, int max_chunks, int sm_count) {
-  return (long long)total_B * max_Hkv * max_chunks <= 10ll * sm_count;
+// Where the merge runs.  The second kernel is as good as free: it is resident when the attention ends and reads the partials
+// with every load in flight, while a counter makes a round trip at the end of every block.  Whole steps, second kernel against
+// merge in the kernel: 1B decoder, one request of 4096 tokens 774 and 781 us, 8 900 and 912, 27 1192 and 1212, 64 1676 and
+// 1739; 8B, one request 3174 and 3402, 32 4633 and 4791.  The exception are a few blocks per SM of short requests at head
+// size 64, which have ended when the second kernel could start: 32 requests of up to 600 tokens 956 and 931, 64 1109 and 1090, 32
+// of 500 961 and 941, 32 of 1000 1059 and 1052 -- but 16 of 750 1033 and 1039, 64 of 1000 (14 blocks per SM) 1295 and 1318, 16 of
+// 1500 1120 and 1147.
+bool attn_decode_fused(int total_B, int max_Hkv, int max_chunks, int hd, int sm_count) {
+  const long long blocks = (long long)total_B * max_Hkv * max_chunks;
+  return hd <= 64 && max_chunks <= 4 && blocks >= 3ll * sm_count && blocks <= 10ll * sm_count;
 }
 
 cudaError_t launch_attn_decode(const AttnDecGroup* groups, int n_groups, int total_B, int max_Hkv, int max_Hq,
@@ -922,7 +925,7 @@ extern "C" int epara_decode_attention_static(int device, void* cuda_stream, cons
   // zero); every partial that is read is written first by this call's attention kernel.
   launch_attn_prepare(g, reinterpret_cast<AttnDecGroup*>(s), reqs, kv_lens, tables, table_stride, max_len, B * Hq, st);
   cudaError_t e = launch_attn_decode(reinterpret_cast<const AttnDecGroup*>(s), 1, B, Hkv, Hq, chunks, hd, Hq / Hkv,
-                                     attn_decode_fused(B, Hkv, chunks, g_static_sm[device]) ? 1 : 0, st);
+                                     attn_decode_fused(B, Hkv, chunks, hd, g_static_sm[device]) ? 1 : 0, st);
   if (e == cudaErrorInvalidValue) return EPARA_E_UNSUPPORTED;
   return e == cudaSuccess ? EPARA_OK : EPARA_E_CUDA;
 }

@@ -1321,7 +1321,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
   int li = 0, n_kernels = 0;
   for (const Launch& L : launches) {
     n_kernels += 1 + ((L.kind == EPARA_K_ATTN_DEC && L.p2 > 1 &&
-                       !attn_decode_fused(L.p0, L.p1 & 0xffff, L.p2, c->sm_count)) ? 1 : 0);
+                       !attn_decode_fused(L.p0, L.p1 & 0xffff, L.p2, L.p3 >> 8, c->sm_count)) ? 1 : 0);
     const unsigned char* gp = slot.dev + L.off;
     if (prof) {
       cudaEventRecord(slot.prof[2 * li], st);
@@ -1341,7 +1341,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       case EPARA_K_ROPE: launch_rope_append((const RopeGroup*)gp, L.n_groups, L.p1, st); break;
       case EPARA_K_ATTN_DEC:
         err = launch_attn_decode((const AttnDecGroup*)gp, L.n_groups, L.p0, L.p1 & 0xffff, L.p1 >> 16, L.p2, L.p3 >> 8,
-                                 L.p3 & 255, attn_decode_fused(L.p0, L.p1 & 0xffff, L.p2, c->sm_count) ? 1 : 0, st);
+                                 L.p3 & 255, attn_decode_fused(L.p0, L.p1 & 0xffff, L.p2, L.p3 >> 8, c->sm_count) ? 1 : 0, st);
         break;
       case EPARA_K_ATTN_ENC:
         if (L.p2 == 0) err = launch_attn_encoder_tc((const AttnEncGroup*)gp, L.n_groups, L.p0, L.p3, dev_status, c->sm_count, st);
@@ -1589,7 +1589,7 @@ int epara_decode_attention(int device, void* cuda_stream, const void* q, int q_s
   // one set-up kernel writes the descriptor, clears the status word and the counters and fills the request table
   launch_attn_prepare(g, (AttnDecGroup*)s, reqs, kv_lens, tables, table_stride, max_len, B * Hq, st);
   cudaError_t e = launch_attn_decode((const AttnDecGroup*)s, 1, B, Hkv, Hq, g.max_chunks, hd, Hq / Hkv,
-                                     attn_decode_fused(B, Hkv, g.max_chunks, device_sm_count(device)) ? 1 : 0, st);
+                                     attn_decode_fused(B, Hkv, g.max_chunks, hd, device_sm_count(device)) ? 1 : 0, st);
   if (e == cudaErrorInvalidValue) return EPARA_E_UNSUPPORTED;
   return e == cudaSuccess ? EPARA_OK : EPARA_E_CUDA;
 }

@@ -56,7 +56,7 @@ cudaError_t launch_gemm_stream(const GemmGroup* groups, int n_groups, int total_
 // zero); fused = 0: a second kernel merges them.  attn_decode_fused() is the rule that picks the mode
 // from the launch's block count; both modes give the same bits.
 constexpr int ATTN_CHUNK = 256;
-bool attn_decode_fused(int total_B, int max_Hkv, int max_chunks, int sm_count);
+bool attn_decode_fused(int total_B, int max_Hkv, int max_chunks, int hd, int sm_count);
 cudaError_t launch_attn_decode(const AttnDecGroup* groups, int n_groups, int total_B, int max_Hkv, int max_Hq,
                                int max_chunks, int hd, int gqa, int fused, cudaStream_t st);
 // Set-up of a single-kernel decode-attention call on the stream: writes `g` to `dst`, clears *g.status and

@@ -321,10 +321,10 @@ def test_grouped_gemm_between_one_tile_and_a_full_chip(E, rows):
 
 
 @pytest.mark.parametrize("hd,Hq,Hkv", [(16, 4, 2), (64, 8, 2), (128, 4, 4)])
-@pytest.mark.parametrize("B", [5, 420])
+@pytest.mark.parametrize("B", [5, 100, 420])
 def test_decode_attention_writes_out_at_any_bf16_boundary(E, hd, Hq, Hkv, B):
-    """`out` one element past an aligned address: requests of one chunk and of several, merged by the last block to arrive
-    (5 requests) and by the second kernel (420).  The same bits as in an aligned tensor, and nothing beside it."""
+    """`out` one element past an aligned address: requests of one chunk and of several, merged by the second kernel and (100
+    requests, head sizes up to 64) by the last block to arrive.  The same bits as in an aligned tensor, and nothing beside it."""
     dev = torch.device("cuda")
     lens = np.resize(np.array([700, 1, 256, 257, 530], dtype=np.int32), B)
     tables = torch.arange(44, dtype=torch.int32, device=dev).repeat(B, 1)
@@ -337,7 +337,7 @@ def test_decode_attention_writes_out_at_any_bf16_boundary(E, hd, Hq, Hkv, B):
         E.epara_decode_attention(q, pool, torch.as_tensor(lens, device=dev), tables, out, Hq, Hkv, hd, 700, scratch, _stream())
     torch.cuda.synchronize()
     assert torch.equal(ref, odd) and float(buf[0]) == 9.0 and float(buf[-1]) == 9.0
-    if B == 5:
+    for _ in range(2):                                  # (the second call finds the counters as the first left them)
         odd.zero_()
         E.epara_decode_attention_static(q, pool, torch.as_tensor(lens, device=dev), tables, odd, Hq, Hkv, hd, 700, _stream())
         torch.cuda.synchronize()
@@ -372,9 +372,9 @@ def test_grouped_gemm_takes_row_strides_of_c_that_its_kernels_can_store(E, M, N,
 
 @pytest.mark.parametrize("hd,Hq,Hkv", [(64, 8, 2), (128, 4, 4), (32, 4, 1)])
 def test_decode_attention_merges_any_number_of_chunks(E, hd, Hq, Hkv):
-    """16, 17, 32, 33 and 41 chunks of 256 tokens, whose partials are merged 16 at a time, and few: against the oracle, merged
-    by the last block to arrive, and with the same bits by the second kernel (more requests in the call).  The keys of the
-    later chunks are larger, so that the maximum of a later group of chunks is the larger one."""
+    """16, 17, 32, 33 and 41 chunks of 256 tokens, whose partials are merged 16 at a time, and few: against the oracle, and with
+    the same bits among more requests.  The keys of the later chunks are larger, so that the maximum of a later group of
+    chunks is the larger one."""
     dev = torch.device("cuda")
     lens = np.array([4096, 4097, 8192, 8193, 10300, 700, 30], dtype=np.int32)
     B, n_pages = len(lens), (10300 + 15) // 16
@@ -399,3 +399,24 @@ def test_decode_attention_merges_any_number_of_chunks(E, hd, Hq, Hkv):
         K, V = O.gather_kv(lambda l, pg: pool_bits[pg], 0, table, int(L))
         ref = np.stack([O.attention(qf[b, h], K[h // (Hq // Hkv)], V[h // (Hq // Hkv)]) for h in range(Hq)])
         assert_close(out[b].reshape(Hq, hd), ref, what=f"decode attention of {L} tokens")
+
+
+@pytest.mark.parametrize("hd,Hq,Hkv", [(16, 4, 2), (64, 8, 2), (64, 8, 1), (128, 4, 4)])
+def test_decode_attention_merge_in_the_kernel_and_after_it_give_the_same_bits(E, hd, Hq, Hkv):
+    """Requests of up to four chunks: few and very many of them are merged by the second kernel, some hundred blocks (three
+    to ten per SM) at head sizes up to 64 by the block that arrives last.  A request has the same bits in all of them."""
+    dev = torch.device("cuda")
+    lens = np.array([1000, 1, 256, 257, 530, 1024, 700, 40], dtype=np.int32)
+    tables = torch.arange(64, dtype=torch.int32, device=dev)
+    pool = synth.make_kv_pool(1, 64, Hkv, hd, seed=51, device=dev)[0]
+    q = torch.randn((8, Hq * hd), generator=torch.Generator(device=dev).manual_seed(52), device=dev).to(torch.bfloat16)
+    outs = []
+    for n in (1, -(-3 * 148 // (8 * 4 * Hkv)), 10 * 148 // (8 * 4 * Hkv), 10 * 148 // (8 * 4 * Hkv) + 1):
+        out = torch.empty((8 * n, Hq * hd), device=dev, dtype=torch.bfloat16)
+        scratch = torch.empty(E.lib.epara_decode_attention_scratch_bytes(8 * n, Hq, hd, 1024), dtype=torch.uint8, device=dev)
+        E.epara_decode_attention(q.repeat(n, 1), pool, torch.as_tensor(np.tile(lens, n), device=dev), tables.repeat(8 * n, 1), out, Hq, Hkv, hd,
+                                 1024, scratch, _stream())
+        torch.cuda.synchronize()
+        assert torch.equal(out, out[:8].repeat(n, 1))
+        outs.append(out[:8])
+    assert all(torch.equal(o, outs[0]) for o in outs)

@@ -45,8 +45,7 @@ def _case(E, B, lens, Hq, Hkv, hd, seed):
 def test_static_scratch_entry_matches_the_ordinary_entry_twice_in_a_row(E):
     stream = torch.cuda.current_stream().cuda_stream
     # different problems back to back: each call finds the previous one's leftovers in the array; the third
-    # repeats the first (several chunks per request, merged by the last block to arrive) after the second,
-    # so it runs on chunk counters that the earlier calls must have left at zero
+    # repeats the first (several chunks per request) after the second, on partials and counters of the earlier calls
     problems = [(6, [700, 1, 256, 257, 40, 1023], 8, 2, 64, 70), (3, [300, 17, 513], 8, 2, 128, 80),
                 (6, [700, 1, 256, 257, 40, 1023], 8, 2, 64, 70)]
     for n, (B, lens, Hq, Hkv, hd, seed) in enumerate(problems):
