@@ -159,7 +159,7 @@ typedef struct {
   int n_out;
   int32_t* argmax;
   int device_error;         /* with EPARA_E_DEVICE: the code a kernel of the step left in the step's status word.
-                               1..49: a bounded wait ran out (which role gave up); 101: a block table named a page
+                               1..59: a bounded wait ran out (which role gave up); 101: a block table named a page
                                outside the model's kv_pages at the append; 102: the same at an attention read.
                                The accesses behind 101 / 102 are skipped, never performed. */
 } epara_output;

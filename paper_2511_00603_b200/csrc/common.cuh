@@ -20,7 +20,8 @@ namespace epara {
 // attention, small projections, all bound by latency -- waited for memory behind them.  One kernel ahead is enough to keep
 // HBM busy over a boundary (1B decoder: one request 972 -> 902 us a step, 27 requests 1385 -> 1331; one image through
 // ViT-B 671 -> 635; steps of large kernels unchanged).
-// A kernel that streams weights to its end takes the two halves apart and triggers when its own requests are out.
+// A kernel that streams weights to its end takes the two halves apart: a block of it triggers when the first of its warps
+// has nothing left to request.
 __device__ __forceinline__ void pdl_wait_only() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // (one thread per block is enough; a block that exits counts as having triggered)
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

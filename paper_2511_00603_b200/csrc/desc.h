@@ -12,7 +12,7 @@ typedef __nv_bfloat16 bf16;
 
 enum : int { EPI_BIAS = 1, EPI_GELU = 2, EPI_SWIGLU = 4, EPI_RESID_F32 = 8 };
 
-// Codes a kernel leaves in the step's device status word (0 = none).  1..49 are bounded waits that ran
+// Codes a kernel leaves in the step's device status word (0 = none).  1..59 are bounded waits that ran
 // out (the role that gave up); the others are indices found out of range, whose access was skipped.
 enum : int { ERR_PAGE_APPEND = 101, ERR_PAGE_ATTEND = 102, ERR_SELFTEST_WAIT = 90, ERR_SELFTEST_SPLIT = 91 };
 

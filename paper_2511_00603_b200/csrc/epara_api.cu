@@ -1466,7 +1466,7 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
   }
   if (cudaSetDevice(device) != cudaSuccess) return EPARA_E_CUDA;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  std::vector<GemmGroup> gs, gs_stream, gs_pair;   // CUDA-core groups; weight-streaming groups (M <= 16); CTA-pair groups
+  std::vector<GemmGroup> gs, gs_stream, gs_pair;   // CUDA-core groups; weight-streaming groups; CTA-pair groups
   std::vector<GemmGroup> gs_swap[N_SWAP];          // swapped-operand groups by k ranges per tile
   int total_swap[N_SWAP] = {0}, nb_swap[N_SWAP] = {0};
   int total = 0, total_stream = 0, max_rows_stream = 0, total_pair = 0;

@@ -1,5 +1,5 @@
-// Weight-streaming grouped GEMM for groups of at most 16 rows (a latency-sensitive batch, a
-// single decode request): C_g = epi(A_g W_g^T + bias_g) with M <= 16, and for small matrices with up to 128 rows.
+// Weight-streaming grouped GEMM, C_g = epi(A_g W_g^T + bias_g), for groups of at most 16 rows (a latency-sensitive batch,
+// a single decode request) and for matrices of up to a million elements with at most 128 rows.
 //
 // With so few rows the work is reading W once; a 128-row tensor-core tile would leave most SMs idle
 // on the narrow matrices and spend its time on zero rows.  Here one block of 16 warps owns 16
@@ -15,9 +15,9 @@
 //
 // HBM-bound: 513 MB of W (an LM head) take 79 us, 6.5 TB/s.  A short matrix is bound by how soon its blocks have all
 // their requests out: with 16 warps K = 2048 is requested at once (64 KB a block), K = 8192 in four rounds instead of
-// eight, and the next kernel, whose own first requests would queue in front of the rest of these, is let in only when
-// the last request of this one has been answered (one request through the 1B decoder: 8 warps 901 us a step, 16 warps
-// 883, with the late trigger 860; more in flight than that, in registers or through a bulk-copy ring of shared memory, reads
+// eight, and the next kernel, whose own first requests would queue in front of the rest of these, is let in late: a block
+// triggers when the first of its warps is through its k-blocks (one request through the 1B decoder: 8 warps 901 us a step,
+// 16 warps 883, with the late trigger 860; more in flight than that, in registers or through a bulk-copy ring of shared memory, reads
 // slower again, 5.2 TB/s).
 #include "common.cuh"
 #include "kernels.h"

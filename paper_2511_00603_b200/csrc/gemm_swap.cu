@@ -9,8 +9,8 @@
 // At small batches what bounds these kernels is how many bytes of W a CTA has in flight: at full rate HBM answers a
 // request after about 5 us, so the whole device needs some 30 MB outstanding, about 200 KB per SM (measured: a CTA's
 // ingest is its ring size divided by that latency, whatever the tile shape).  Activation tiles come from L2, a
-// fraction of that latency away, and must not take ring space from W: the two operands have rings of their own, ten
-// stages of 16 KB for W and two to four short-lived stages for the activations (tiles of more than 128 rows: four
+// fraction of that latency away, and must not take ring space from W: the two operands have rings of their own, up to ten
+// stages of 16 KB for W and two to eight short-lived stages for the activations (tiles of more than 128 rows: four
 // stages of activations, the rest for W, since there the MMA time of a k-block is what has to be covered).
 //
 // A matrix has only N / 128 such tiles (16 to 24 for the projections of a 1B-scale decoder), too few CTAs to pull
@@ -23,9 +23,9 @@
 // columns contiguous.  No partial ever travels through global memory and the reduction order is fixed, so a
 // request's bits do not depend on timing or on what else is in the launch.
 //
-// Roles per CTA: warp 0 (one lane) TMA producer of W -- it does not wait for the earlier kernels of the stream,
-// weights being static, so its ring is full when they finish; the last warp (one lane) TMA producer of the
-// activations; warp 1 (one lane) tcgen05.mma issuer; warps 2..9 read the accumulator (two warps per TMEM lane
+// Roles per CTA (converged warps, an elected lane issues): warp 0 TMA producer of W -- it does not wait for the earlier
+// kernels of the stream, weights being static, so its ring is full when they finish; the last warp TMA producer of the
+// activations; warp 1 tcgen05.mma issuer; warps 2..9 read the accumulator (two warps per TMEM lane
 // quarter) and run the epilogue.  Every mbarrier wait is bounded; a CTA that gives up records a code in *status and
 // still meets its cluster at the barriers.
 #include "common.cuh"

@@ -406,8 +406,12 @@ gemm_tc_pair_kernel(const GemmGroup* __restrict__ groups, int n_groups, int tota
 // the k order of both contractions is ascending), so a request's bits do not change with the kernel.
 // The two contractions have an issuing thread each (warp 1 for S, the last warp for O): the chains only meet
 // through the epilogue warps (S -> P), so the tensor core works on the next chunk's S while this chunk's GELU is
-// computed and on this chunk's O while the next S is read out, and neither thread's issue time (some 80 cycles
-// per tcgen05.mma) delays the other chain.  Weights stream through two rings of two 24 KB slots (W1: three k-blocks
+// computed and on this chunk's O while the next S is read out, and neither thread's issue time delays the other chain.
+// What bounds it: S and P have one buffer each, so that O of a chunk, the writing of the next P and that P's O are one
+// chain.  Cycles per chunk and role at d 384 (5.9 thousand in all, a twelfth of the tile's 11.5 thousand for its output
+// included; 3.07 thousand of tensor work): S issuer 1.9 issuing, 2.8 waiting for the read-out; O issuer 2.4 issuing, 2.5
+// waiting for P; an epilogue warp 0.6 waiting for S, 0.1 reading, 1.6 of bias and GELU, 1.8 waiting for P's buffer.
+// Weights stream through two rings of two 24 KB slots (W1: three k-blocks
 // of a chunk half per slot; W2: one k-block of a chunk half per slot), each with its own producer thread.
 // P's 32 KB double as the staging area of the final epilogue (P is idle by then).
 constexpr int MLP_SLOT_BYTES = 24 * 1024;

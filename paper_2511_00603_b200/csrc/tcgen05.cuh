@@ -164,7 +164,8 @@ __device__ __forceinline__ uint32_t make_idesc_pair(int bn) {
 // that tcgen05.commit covers the MMAs before it).  Measured per k-block of four MMAs with its barrier wait and commit
 // (M 128, N 32 / 128 / 256, operands resident): 484 / 484 / 516 cycles with the loop inside `if (lane == 0)`, 288 /
 // 310 / 511 like this: a wait on a barrier that is ready already takes 200 cycles in the divergent branch and each
-// MMA 58 instead of 40, so that no tile narrower than 256 columns could keep the tensor pipe busy.
+// MMA 58 instead of 40, so that no tile narrower than 256 columns could keep the tensor pipe busy.  (Measured with every
+// lane leaving a wait on its own; the vote costs a k-block with one wait nothing that a launch shows.)
 __device__ __forceinline__ void mbar_expect_tx_elect(uint32_t bar, uint32_t bytes) {
   asm volatile(
       "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
