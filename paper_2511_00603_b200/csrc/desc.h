@@ -121,7 +121,7 @@ struct RopeGroup {
 // kv_len + t attends to positions 0 .. kv_len + t of its paged cache (the chunk's own k, v were appended by the kernel
 // before).  A work item is 128 of its tokens (a tile) and one or two query heads of one kv head; the list holds one entry per
 // tile, sorted by the keys it walks, longest first, and a tile's heads are items one after another.  (With an entry per item
-// thousands of short chunks on a model of many heads, or a chunk of 180 thousand tokens, overflowed the step's blob.)
+// 3900 chunks of two tokens on a model of 32 heads overflowed the step's blob.)
 struct PrefillTile {
   const int32_t* table;
   int row, live;         // first activation row, tokens of the tile
