@@ -363,19 +363,19 @@ __device__ __forceinline__ void place_kv(unsigned char* tile, int r, const uint3
 template <int HD>
 __device__ __forceinline__ void place_step_rows(const AttnDecGroup& g, unsigned char* tile, int page, int kvh, int own_row, int n_slots) {
   const int lane = threadIdx.x & 31;
-  for (int w0 = 0; w0 < g.n_rows; w0 += 32) {
-    const int w = w0 + lane;
-    int at = 0;
-    bool hit = false;
-    if (w < g.n_rows && w != own_row) {
-      const RowDesc rd = g.rows[w];
-      at = rd.pos;
-      hit = (at & 15) < n_slots && g.step_reqs[rd.req()].table[at >> 4] == page;
-    }
+#pragma unroll 1
+  for (int w0 = 0; w0 < g.n_written; w0 += 32) {
+    WrittenPage wp = {nullptr, 0, 0};
+    if (w0 + lane < g.n_written) wp = g.written[w0 + lane];
+    const bool hit = wp.id != nullptr && wp.row() != own_row && (wp.pos & 15) < n_slots && *wp.id == page;
     for (unsigned m = __ballot_sync(0xffffffffu, hit); m != 0; m &= m - 1) {
-      const int l = __ffs(m) - 1, p = __shfl_sync(0xffffffffu, at, l);
-      const bf16* const row = g.q + (size_t)(w0 + l) * g.q_stride + (size_t)(g.Hq + kvh) * HD;
-      place_kv<HD>(tile, p & 15, reinterpret_cast<const uint32_t*>(row), g.Hkv, g.cs + (size_t)p * (HD / 2), nullptr);
+      const int l = __ffs(m) - 1, pos = __shfl_sync(0xffffffffu, wp.pos, l), row_n = __shfl_sync(0xffffffffu, wp.row_n, l);
+      const int n = min(row_n & 31, n_slots - (pos & 15));
+#pragma unroll 1
+      for (int r = 0; r < n; ++r) {
+        const bf16* const row = g.q + (size_t)((row_n >> 5) + r) * g.q_stride + (size_t)(g.Hq + kvh) * HD;
+        place_kv<HD>(tile, (pos + r) & 15, reinterpret_cast<const uint32_t*>(row), g.Hkv, g.cs + (size_t)(pos + r) * (HD / 2), nullptr);
+      }
     }
   }
   __syncwarp();

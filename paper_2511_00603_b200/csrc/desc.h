@@ -90,18 +90,34 @@ struct AttnReq {
   int row;               // activation row of the request's token (q is read and the output written there)
 };
 
+// A cache page that the step appends to: `n` token rows from `row` on, at positions from `pos` on.
+struct WrittenPage {
+  const int32_t* id;     // where the caller's block table holds the page's id
+  int pos;
+  int row_n;             // 32 * row + n
+#ifdef __CUDACC__
+  __host__ __device__
+#endif
+  int row() const { return row_n >> 5; }
+#ifdef __CUDACC__
+  __host__ __device__
+#endif
+  int n() const { return row_n & 31; }
+};
+
 // LINK: finds the decode requests that attend to tokens which other requests of the step append (see AttnDecGroup::linked).
 enum : int { GATHER_ROWS = 0, GATHER_EMB = 1, GATHER_PATCH = 2, GATHER_LINK = 3 };
 struct GatherGroup {
   const ReqDesc* reqs;
   const RowDesc* rows;   // EMB: one entry per output row
-  const AttnReq* areqs;  // LINK: the decode requests, one block each; B counts all requests, n_pre of them prompt chunks
+  const AttnReq* areqs;  // LINK: the decode requests, one block each
+  const WrittenPage* written;   // LINK: the decode requests' pages, in their order, then those of the prompt chunks; B counts them
   void* out;             // ROWS: bf16 [B, ld]; EMB: fp32 [rows, d]; PATCH: bf16 [B*np, 3*p*p]; LINK: int [decode requests]
   const bf16* emb;       // EMB
   int kind, B, width, ld;
   int img, patch;
   int blocks;            // blocks this group needs
-  int n_pre;
+  int pad;
 };
 
 struct RopeGroup {
@@ -167,9 +183,8 @@ struct AttnDecGroup {
   // With cs, in a step of several requests: linked[b] != 0 when request b may attend to tokens that other rows of the
   // step append (requests of one sequence in one step).  The block takes those from qkv then, wherever the append stands.
   const int* linked;     // null: a single request
-  const RowDesc* rows;
-  const ReqDesc* step_reqs;
-  int n_rows;
+  const WrittenPage* written;
+  int n_written;
   int pad;
 };
 
@@ -222,7 +237,7 @@ struct OutputGroup {     // copy logits rows to the requests' buffers and take t
 // Group arrays are packed back to back in the step blob: sizes must keep 8-byte alignment.
 namespace epara {
 static_assert(sizeof(GemmGroup) % 64 == 0, "GemmGroup holds 64-byte aligned TMA maps");
-static_assert(sizeof(AttnPrefillGroup) % 8 == 0 && sizeof(PrefillMaps) % 64 == 0 && sizeof(PrefillTile) == 24 && sizeof(RowDesc) == 12, "descriptor sizes");
+static_assert(sizeof(AttnPrefillGroup) % 8 == 0 && sizeof(PrefillMaps) % 64 == 0 && sizeof(PrefillTile) == 24 && sizeof(RowDesc) == 12 && sizeof(WrittenPage) == 16, "descriptor sizes");
 static_assert(sizeof(NormGroup) % 8 == 0 && sizeof(GatherGroup) % 8 == 0 && sizeof(RopeGroup) % 8 == 0 &&
               sizeof(AttnDecGroup) % 8 == 0 && sizeof(AttnEncGroup) % 64 == 0 && sizeof(MlpGroup) % 64 == 0 && sizeof(AssembleGroup) % 8 == 0 &&
               sizeof(OutputGroup) % 8 == 0 && sizeof(ReqDesc) % 16 == 0 && sizeof(AttnReq) % 16 == 0,

@@ -822,8 +822,8 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
   // n_pre prompt-chunk requests of a decoder, with their descriptor arrays in the blob
   struct PrefillChunk { const int32_t* table; int row_start, n_tok, kv_len; };
   struct Active {
-    Model* m; int B; int rows; size_t req_off; size_t areq_off; size_t row_off; size_t ptile_off; size_t pmaps_off; size_t last_off; size_t link_off; size_t cursor;
-    int n_dec, n_pre, max_chunks_dec, pre_items;
+    Model* m; int B; int rows; size_t req_off; size_t areq_off; size_t row_off; size_t ptile_off; size_t pmaps_off; size_t last_off; size_t link_off; size_t written_off; size_t cursor;
+    int n_dec, n_pre, max_chunks_dec, pre_items, n_written;
     bool append_first;   // decode rows are rotated and appended by a launch of their own, before any attention of the wave
     std::vector<PrefillChunk> pre;
     std::vector<Request> reqs;
@@ -832,7 +832,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
   for (size_t mi = 0; mi < c->models.size(); ++mi) {
     Model* m = c->models[mi];
     Active a;
-    a.m = m; a.B = 0; a.rows = 0; a.cursor = 0; a.req_off = 0; a.areq_off = 0; a.row_off = 0; a.ptile_off = 0; a.pmaps_off = 0; a.last_off = 0; a.link_off = 0; a.append_first = false;
+    a.m = m; a.B = 0; a.rows = 0; a.cursor = 0; a.req_off = 0; a.areq_off = 0; a.row_off = 0; a.ptile_off = 0; a.pmaps_off = 0; a.last_off = 0; a.link_off = 0; a.written_off = 0; a.n_written = 0; a.append_first = false;
     a.n_dec = a.n_pre = a.max_chunks_dec = a.pre_items = 0;
     for (int cat = 0; cat < 2; ++cat) {
       std::deque<Request>& q = m->q[cat];
@@ -948,10 +948,20 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       if (!ar.empty() && a.B > 1 && a.m->d.head_dim >= 64) {
         const std::vector<int> none(ar.size(), 0);
         a.link_off = put(none.data(), none.size() * sizeof(int), 16);
+        std::vector<WrittenPage> written;
+        for (const AttnReq& q : ar) written.push_back({q.table + (q.len - 1) / EPARA_KV_PAGE, q.len - 1, 32 * q.row + 1});
+        for (const PrefillChunk& p : pr)
+          for (int t = 0, n; t < p.n_tok; t += n) {
+            const int pos = p.kv_len + t;
+            n = std::min(p.n_tok - t, EPARA_KV_PAGE - pos % EPARA_KV_PAGE);
+            written.push_back({p.table + pos / EPARA_KV_PAGE, pos, 32 * (p.row_start + t) + n});
+          }
+        a.n_written = (int)written.size();
+        a.written_off = put(written.data(), written.size() * sizeof(written[0]), 16);
       }
     }
     if (a.req_off == (size_t)-1 || a.areq_off == (size_t)-1 || a.row_off == (size_t)-1 ||
-        a.last_off == (size_t)-1 || a.link_off == (size_t)-1)
+        a.last_off == (size_t)-1 || a.link_off == (size_t)-1 || a.written_off == (size_t)-1)
       overflow = true;
   }
   // Placements that share a cache (one service placed twice): a request of one may attend to what a request of the other
@@ -1097,8 +1107,8 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
               g.cs = nullptr;
             } else if (a->link_off != 0) {
               g.linked = (const int*)(slot.dev + a->link_off);
-              g.rows = (const RowDesc*)(slot.dev + a->row_off); g.step_reqs = (const ReqDesc*)(slot.dev + a->req_off);
-              g.n_rows = a->rows;
+              g.written = (const WrittenPage*)(slot.dev + a->written_off);
+              g.n_written = a->n_written;
             }
             total_B += a->n_dec;
             max_hkv = std::max(max_hkv, g.Hkv); max_hq = std::max(max_hq, g.Hq);
@@ -1162,7 +1172,8 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
             ++n_put;
             if (put(&g, sizeof(g), 8) == (size_t)-1) overflow = true;
             if (a->link_off != 0 && !a->append_first) {
-              g.kind = GATHER_LINK; g.blocks = a->n_dec; g.n_pre = a->n_pre;
+              g.kind = GATHER_LINK; g.blocks = a->n_dec; g.B = a->n_written;
+              g.written = (const WrittenPage*)(slot.dev + a->written_off);
               g.areqs = (const AttnReq*)(slot.dev + a->areq_off);
               g.out = slot.dev + a->link_off;
               ++n_put;

@@ -2,6 +2,8 @@
 // RMSNorm, RoPE + KV append, ViT token assembly, logits scatter + argmax.
 // Every launch is grouped: blockIdx.y selects the group (one model), blockIdx.x a unit of work
 // inside it; blocks beyond a group's extent return at once.
+#include <climits>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -10,7 +12,7 @@ namespace epara {
 // ------------------------------------------------------------------ gather
 // Row and embedding gathers take one block per row (a handful of rows per step); the patch gather takes
 // GATHER_PATCH_ROWS patch rows per block, so that a thread has several 16-byte loads in flight.
-constexpr int LINK_PAGES = 1024;
+constexpr int LINK_PAGES = 1024, LINK_ROWS = 4;
 __global__ void __launch_bounds__(128) gather_kernel(const GatherGroup* __restrict__ groups) {
   const GatherGroup g = groups[blockIdx.y];
   if ((int)blockIdx.x >= g.blocks) return;      // (descriptors are not written by kernels: no wait needed to leave)
@@ -34,30 +36,28 @@ __global__ void __launch_bounds__(128) gather_kernel(const GatherGroup* __restri
   } else if (g.kind == GATHER_LINK) {
     // Does the block table of decode request b, up to the request's own position, name a page that another request of the
     // step appends to?  By whole pages: a request marked without need costs time only.
-    __shared__ int seen[LINK_PAGES];
+    __shared__ __align__(16) int seen[LINK_PAGES];
     const AttnReq rq = g.areqs[blockIdx.x];
     const int n_pages = (rq.len - 1 + 15) >> 4;
     bool hit = false;
     for (int i0 = 0; i0 < n_pages; i0 += LINK_PAGES) {
       const int n = min(LINK_PAGES, n_pages - i0);
       __syncthreads();
-      for (int i = threadIdx.x; i < n; i += blockDim.x) seen[i] = rq.table[i0 + i];
+      for (int i = threadIdx.x; i < (n + 3 & ~3); i += blockDim.x) seen[i] = i < n ? rq.table[i0 + i] : INT_MAX;
       __syncthreads();
-      for (int q = threadIdx.x; q < g.B; q += blockDim.x) {
-        const ReqDesc& r = g.reqs[q];
-        if (r.n_tok > 1 || r.row_start == rq.row) continue;
-        const int page = r.table[r.kv_len >> 4];
-#pragma unroll 8
-        for (int i = 0; i < n; ++i) hit |= seen[i] == page;
-      }
-      if (g.n_pre == 0) continue;
-      for (int q = 0; q < g.B; ++q) {                  // prompt chunks: a thread per page
-        const ReqDesc& r = g.reqs[q];
-        if (r.n_tok == 1) continue;
-        for (int pg = (r.kv_len >> 4) + threadIdx.x; pg <= (r.kv_len + r.n_tok - 1) >> 4; pg += blockDim.x) {
-          const int page = r.table[pg];
-#pragma unroll 8
-          for (int i = 0; i < n; ++i) hit |= seen[i] == page;
+      // a thread takes LINK_ROWS page ids at a time
+      for (int w0 = threadIdx.x; w0 < g.B; w0 += blockDim.x * LINK_ROWS) {
+        int page[LINK_ROWS];
+#pragma unroll
+        for (int k = 0; k < LINK_ROWS; ++k) {
+          const int w = w0 + k * blockDim.x;
+          page[k] = w < g.B && w != (int)blockIdx.x ? *g.written[w].id : INT_MIN;
+        }
+#pragma unroll 2
+        for (int i = 0; i < n; i += 4) {
+          const int4 s = *reinterpret_cast<const int4*>(seen + i);
+#pragma unroll
+          for (int k = 0; k < LINK_ROWS; ++k) hit |= s.x == page[k] | s.y == page[k] | s.z == page[k] | s.w == page[k];
         }
       }
     }

@@ -326,7 +326,7 @@ def test_prefill_admission_by_token_rows_and_rejections(mods):
 
 @pytest.mark.parametrize("hd,Hq,Hkv,kv0,chunk,n_dec,placed_twice", [
     (64, 8, 2, 37, 0, 2, False), (64, 8, 2, 254, 0, 5, False), (128, 4, 4, 511, 0, 3, False), (32, 4, 2, 30, 0, 4, False),
-    (64, 4, 1, 0, 40, 3, False), (128, 8, 2, 130, 130, 20, False), (64, 8, 2, 250, 0, 12, True), (64, 8, 2, 20, 33, 2, True)])
+    (64, 4, 1, 0, 40, 3, False), (128, 8, 2, 130, 130, 20, False), (64, 8, 2, 77, 600, 40, False), (64, 8, 2, 250, 0, 12, True), (64, 8, 2, 20, 33, 2, True)])
 def test_requests_of_one_sequence_in_one_step(mods, hd, Hq, Hkv, kv0, chunk, n_dec, placed_twice):
     """A caller that scores known tokens: `n_dec` decode requests at successive positions of one sequence, alone or behind the
     prompt chunk that fills the positions before them, all in ONE step, in an order that is not theirs, each with a block
