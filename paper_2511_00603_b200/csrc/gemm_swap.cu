@@ -140,7 +140,8 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
     uint32_t phase = 0;
     bool ok = true;
     for (int kb = kb0; kb < kb1; ++kb) {
-      if (!mbar_wait(wempty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 41); break; }
+      // (a stage's first use has nothing to wait for)
+      if (kb - kb0 >= w_stages && !mbar_wait(wempty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 41); break; }
       mbar_expect_tx_elect(wfull_bar(stage), (uint32_t)SW_W_BYTES);
       tma_load_2d_elect(w_base + stage * SW_W_BYTES, &g->tmW, kb * TC_BK, n0, wfull_bar(stage));
       if (++stage == w_stages) { stage = 0; phase ^= 1u; }
@@ -158,7 +159,7 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
     uint32_t phase = 0;
     bool ok = true;
     for (int kb = kb0; kb < kb1; ++kb) {
-      if (!mbar_wait(aempty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 44); break; }
+      if (kb - kb0 >= a_stages && !mbar_wait(aempty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 44); break; }
       mbar_expect_tx_elect(afull_bar(stage), (uint32_t)a_bytes);
       tma_load_2d_elect(base + stage * a_bytes, &g->tmA, kb * TC_BK, m0, afull_bar(stage));
       if (++stage == a_stages) { stage = 0; phase ^= 1u; }

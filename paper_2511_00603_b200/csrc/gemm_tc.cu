@@ -238,7 +238,7 @@ gemm_tc_pair_kernel(const GemmGroup* __restrict__ groups, int n_groups, int tota
     // ------------------------------------------------------------ TMA producer of A (one per CTA)
     // (A and W have a warp each: a k-block costs its issuer a wait and a TMA issue, and with both operands on one
     // warp that is more than the MMAs of a k-block take once tiles are short.)
-    int stage = 0;
+    int stage = 0, used = 0;                   // (a stage's first use has nothing to wait for)
     uint32_t phase = 0;
     bool ok = true;
     const GemmGroup* g_prev = nullptr;
@@ -257,7 +257,7 @@ gemm_tc_pair_kernel(const GemmGroup* __restrict__ groups, int n_groups, int tota
       if (g != g_prev) { tensormap_acquire(&g->tmA); g_prev = g; }
       const uint32_t bytes = 2u * (A_BYTES + (uint32_t)(gc.bn >> 1) * TC_BK * 2);   // both CTAs' boxes of a k-block
       for (int kb = 0; kb < gc.kblocks; ++kb) {
-        if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 31); break; }
+        if (++used > PAIR_STAGES && !mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 31); break; }
         if (rank == 0) mbar_expect_tx_elect(full_bar(stage), bytes);
         tma_load_2d_pair_elect(base + stage * PAIR_STAGE_BYTES, &g->tmA, kb * TC_BK, it.m0, mapa_shared(full_bar(stage), 0));
         if (++stage == PAIR_STAGES) { stage = 0; phase ^= 1u; }
@@ -270,7 +270,7 @@ gemm_tc_pair_kernel(const GemmGroup* __restrict__ groups, int n_groups, int tota
     // stream: the first stages' W boxes are on their way while those still run.  (Bytes that land before
     // rank 0 has announced them leave the barrier's count negative for a while, which is allowed; the
     // phase cannot complete before that thread's own arrival.)
-    int stage = 0;
+    int stage = 0, used = 0;                   // (a stage's first use has nothing to wait for)
     uint32_t phase = 0;
     bool ok = true;
     const GemmGroup* g_prev = nullptr;
@@ -283,7 +283,7 @@ gemm_tc_pair_kernel(const GemmGroup* __restrict__ groups, int n_groups, int tota
       if (g != g_prev) { tensormap_acquire(&g->tmW); g_prev = g; }
       const int n_half = it.n0 + rank * (gc.bn >> 1);
       for (int kb = 0; kb < gc.kblocks; ++kb) {
-        if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 35); break; }
+        if (++used > PAIR_STAGES && !mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 35); break; }
         tma_load_2d_pair_elect(base + stage * PAIR_STAGE_BYTES + A_BYTES, &g->tmW, kb * TC_BK, n_half, mapa_shared(full_bar(stage), 0));
         if (++stage == PAIR_STAGES) { stage = 0; phase ^= 1u; }
       }
