@@ -206,7 +206,7 @@ __device__ __forceinline__ Work get_work(const PreView& v, int item) {
 }
 __device__ __forceinline__ const CUtensorMap* map_q(const AttnEncGroup* g) { return &g->tmQ; }
 __device__ __forceinline__ const CUtensorMap* map_q(const AttnPrefillGroup* g) { return &g->maps->tmQ; }
-__device__ __forceinline__ const CUtensorMap* map_kv(const AttnEncGroup* g) { return &g->tmKV; }
+__device__ __forceinline__ const CUtensorMap* map_kv(const AttnEncGroup* g) { return &g->tmQ; }
 __device__ __forceinline__ const CUtensorMap* map_kv(const AttnPrefillGroup* g) { return &g->maps->tmKV; }
 __device__ __forceinline__ int out_stride(const AttnEncGroup* g) { return g->H * 64; }
 __device__ __forceinline__ int out_stride(const AttnPrefillGroup* g) { return g->Hq * g->hd; }

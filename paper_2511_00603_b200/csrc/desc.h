@@ -45,9 +45,14 @@ struct RowDesc {
   bool single() const { return req2 & 1; }
 };
 
+// Descriptors that hold TMA maps start on 128 bytes, a map's size.  (64 is all a map needs, but one that lies across two lines is
+// slower to fetch: the 65 GEMM launches of a step of 128 requests through the 1B decoder 1310 us between events, 1306 like
+// this.)
+constexpr int TMAP_ALIGN = 128;
+
 // C = epi(A W^T + bias).  tmA/tmW are the TMA maps of A [rows, K] and W [N, K] (K innermost,
 // 128-byte swizzle, 64 columns x the rows a CTA loads of each).
-struct alignas(64) GemmGroup {
+struct alignas(TMAP_ALIGN) GemmGroup {
   CUtensorMap tmA;
   CUtensorMap tmW;
   CUtensorMap tmC;   // output, written by TMA from the epilogue's staging rows: bf16 [rows, N] with a
@@ -145,7 +150,7 @@ struct PrefillTile {
   int pad;
 };
 // One per model and step; the layers' groups point to it.
-struct alignas(64) PrefillMaps {
+struct alignas(TMAP_ALIGN) PrefillMaps {
   CUtensorMap tmQ;       // qkv [rows, (Hq+2Hkv)*hd] bf16, box 64 columns x 128 rows, 128-byte swizzle
   CUtensorMap tmKV;      // the cache as [n_layers * kv_pages * 2 * Hkv * 16, hd], box 64 columns x 16 rows
 };
@@ -188,23 +193,21 @@ struct AttnDecGroup {
   int pad;
 };
 
-struct alignas(64) AttnEncGroup {
-  CUtensorMap tmQ;       // tensor-core kernel: qkv [rows, 3d] bf16, box 64 columns x 128 rows, 128-byte swizzle
-  CUtensorMap tmKV;      // the same (K and V blocks are read with the box of Q)
+struct alignas(TMAP_ALIGN) AttnEncGroup {
+  CUtensorMap tmQ;       // tensor-core kernel: qkv [rows, 3d] bf16, box 64 columns x 128 rows, 128-byte swizzle (K and V blocks too)
   const bf16* qkv;       // [B*T, 3d]: q | k | v, head h at column h*hd within each
   bf16* out;             // [B*T, d]
   int B, T, H, hd;
   int blk_start;         // first block (item) of this group
   int q_blocks;          // query blocks per (image, head)
   int tc;                // 1: runs in the tensor-core kernel, fixed when the model is placed
-  int pad[9];
 };
 
 // One transformer MLP block of an encoder as a single work unit of the fused kernel:
 // z += GELU(h W1^T + b1) W2^T + b2 with h bf16 [rows, d], W1 [F, d], W2 [d, F], z fp32 [rows, d].
 // d is a multiple of 64 and at most 384 (the output accumulator of a 128-row tile must fit the tensor memory
 // beside one 128-column chunk of the hidden layer), F a multiple of 128.
-struct alignas(64) MlpGroup {
+struct alignas(TMAP_ALIGN) MlpGroup {
   CUtensorMap tmX;       // h [rows, d] bf16, box 64 columns x 128 rows, 128-byte swizzle
   CUtensorMap tmW1;      // W1 [F, d] bf16, box 64 x 64 rows (one CTA of a pair loads half of a chunk's 128 rows)
   CUtensorMap tmW2;      // W2 [d, F] bf16, box 64 x n2/2 rows (n2 = d, or d / 2 when d > 256: two MMAs per k step)
@@ -236,10 +239,11 @@ struct OutputGroup {     // copy logits rows to the requests' buffers and take t
 
 // Group arrays are packed back to back in the step blob: sizes must keep 8-byte alignment.
 namespace epara {
-static_assert(sizeof(GemmGroup) % 64 == 0, "GemmGroup holds 64-byte aligned TMA maps");
-static_assert(sizeof(AttnPrefillGroup) % 8 == 0 && sizeof(PrefillMaps) % 64 == 0 && sizeof(PrefillTile) == 24 && sizeof(RowDesc) == 12 && sizeof(WrittenPage) == 16, "descriptor sizes");
+static_assert(sizeof(GemmGroup) % TMAP_ALIGN == 0 && sizeof(PrefillMaps) % TMAP_ALIGN == 0 && sizeof(AttnEncGroup) % TMAP_ALIGN == 0 &&
+              sizeof(MlpGroup) % TMAP_ALIGN == 0, "TMA maps on lines of their own");
+static_assert(sizeof(AttnPrefillGroup) % 8 == 0 && sizeof(PrefillTile) == 24 && sizeof(RowDesc) == 12 && sizeof(WrittenPage) == 16, "descriptor sizes");
 static_assert(sizeof(NormGroup) % 8 == 0 && sizeof(GatherGroup) % 8 == 0 && sizeof(RopeGroup) % 8 == 0 &&
-              sizeof(AttnDecGroup) % 8 == 0 && sizeof(AttnEncGroup) % 64 == 0 && sizeof(MlpGroup) % 64 == 0 && sizeof(AssembleGroup) % 8 == 0 &&
+              sizeof(AttnDecGroup) % 8 == 0 && sizeof(AssembleGroup) % 8 == 0 &&
               sizeof(OutputGroup) % 8 == 0 && sizeof(ReqDesc) % 16 == 0 && sizeof(AttnReq) % 16 == 0,
               "descriptor sizes");
 }  // namespace epara

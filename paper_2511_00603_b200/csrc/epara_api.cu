@@ -417,7 +417,6 @@ int build_model(Builder& bl, Model* m, const epara_config& cfg) {
       at.aenc.tc = bl.gemm_impl != EPARA_GEMM_SIMT ? 1 : 0;
       if (at.aenc.tc && bl.c) {
         if (!make_tmap(&at.aenc.tmQ, qkv, Mcap, 3 * dm, 3 * dm, FLASH_TILE)) return EPARA_E_CUDA;
-        at.aenc.tmKV = at.aenc.tmQ;
       }
       m->ops.push_back(at);
       if (!add_gemm(bl, m, a, dm, Mcap, w[4], dm, dm, z, dm, w[5], EPI_RESID_F32, T)) return EPARA_E_CUDA;
@@ -1003,7 +1002,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
     }
     a.pre_items = (int)list.size() * a.m->d.n_kv_heads * ((G + mt - 1) / mt);
     a.ptile_off = put(list.data(), list.size() * sizeof(PrefillTile), 16);
-    a.pmaps_off = put(&a.m->pre_maps, sizeof(PrefillMaps), 64);
+    a.pmaps_off = put(&a.m->pre_maps, sizeof(PrefillMaps), TMAP_ALIGN);
     if (a.ptile_off == (size_t)-1 || a.pmaps_off == (size_t)-1) overflow = true;
   }
 
@@ -1079,7 +1078,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       L.n_groups = (int)who.size();
       L.p2 = pass;
       int n_put = 0;
-      off = align_up(off, 64);
+      off = align_up(off, TMAP_ALIGN);
       L.off = off;
       if (kind == EPARA_K_ATTN_DEC) {
         // decode attention is templated on (hd, G): one launch per distinct pair
@@ -1095,7 +1094,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
           Launch LL;
           memset(&LL, 0, sizeof(LL));
           LL.kind = kind; LL.n_groups = (int)same.size();
-          off = align_up(off, 64);
+          off = align_up(off, TMAP_ALIGN);
           LL.off = off;
           int total_B = 0, max_hkv = 0, max_hq = 0, max_chunks = 0, n_put = 0;
           for (Active* a : same) {
@@ -1129,7 +1128,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
           Launch LL;
           memset(&LL, 0, sizeof(LL));
           LL.kind = kind;
-          off = align_up(off, 64);
+          off = align_up(off, TMAP_ALIGN);
           LL.off = off;
           int items = 0, n_put = 0;
           for (Active* a : who) {
@@ -1213,7 +1212,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
               inf.gemm_groups++;
               inf.gemm_flops += 2.0 * 2.0 * rows * mg.d * mg.F;
               inf.weight_bytes += op.weight_bytes;
-              if (put(&mg, sizeof(mg), 64) == (size_t)-1) overflow = true;
+              if (put(&mg, sizeof(mg), TMAP_ALIGN) == (size_t)-1) overflow = true;
               break;
             }
             GemmGroup g = op.gemm;
@@ -1246,7 +1245,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
               inf.stream_gemm_flops += 2.0 * rows * g.N * g.K;
               inf.stream_weight_bytes += op.weight_bytes;
             }
-            if (put(&g, sizeof(g), 64) == (size_t)-1) overflow = true;
+            if (put(&g, sizeof(g), TMAP_ALIGN) == (size_t)-1) overflow = true;
             break;
           }
           case EPARA_K_ROPE: {
@@ -1269,7 +1268,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
             total += a->B * g.H * g.q_blocks;
             mx = std::max(mx, g.T);
             ++n_put;
-            if (put(&g, sizeof(g), 64) == (size_t)-1) overflow = true;
+            if (put(&g, sizeof(g), TMAP_ALIGN) == (size_t)-1) overflow = true;
             break;
           }
           case EPARA_K_OUTPUT: {
@@ -1298,9 +1297,9 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
           Launch R;
           memset(&R, 0, sizeof(R));
           R.kind = kind; R.n_groups = 1; R.p0 = cut_tiles * g.tiles_n; R.p2 = 2;
-          off = align_up(off, 64);
+          off = align_up(off, TMAP_ALIGN);
           R.off = off;
-          if (put(&g, sizeof(g), 64) == (size_t)-1) overflow = true;
+          if (put(&g, sizeof(g), TMAP_ALIGN) == (size_t)-1) overflow = true;
           launches.push_back(R);
         }
       }
