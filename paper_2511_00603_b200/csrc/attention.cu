@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(128) attn_decode_kernel(const AttnDecGroup* __
 // the products run on mma.sync m16n8k16 with the G query heads of the kv head as the 8 columns:
 // S^T = K Q^T (16 tokens x 8 heads), O^T += V^T P^T (16 dims x 8 heads).  (With the heads as rows half of
 // every accumulator was padding: 113 us per layer for the 1B decoder at 128 requests, 108 without it with RoPE and
-// append, which had 10 us of their own, included; 99 and 4 of the merge now, at 96 registers and five blocks per SM.)  The running maximum of a head is only raised, and O and the sum rescaled, when a
+// append, which had 10 us of their own, included; 99 and 8 of the merge now, at 96 registers and five blocks per SM.)  The running maximum of a head is only raised, and O and the sum rescaled, when a
 // score passes it by more than 2^8.  Rows of a staged tile are 128-byte segments whose 16-byte pieces
 // are XOR-swizzled by the token index, so ldmatrix reads are free of bank conflicts.
 // With AttnDecGroup::cs the kernel also does RoPE and the append for its request: q is rotated as it is

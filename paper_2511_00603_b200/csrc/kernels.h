@@ -54,7 +54,7 @@ cudaError_t launch_gemm_stream(const GemmGroup* groups, int n_groups, int total_
 // Decode attention, split-KV over 256-token chunks.  fused = 1: the block of a (request, kv head) that
 // finishes last merges the chunk partials (AttnDecGroup::counters must be zero at launch and is left
 // zero); fused = 0: a second kernel merges them.  attn_decode_fused() is the rule that picks the mode
-// from the launch's block count; both modes give the same bits.
+// from the launch's block count, the chunks of a request and the head size; both modes give the same bits.
 constexpr int ATTN_CHUNK = 256;
 bool attn_decode_fused(int total_B, int max_Hkv, int max_chunks, int hd, int sm_count);
 cudaError_t launch_attn_decode(const AttnDecGroup* groups, int n_groups, int total_B, int max_Hkv, int max_Hq,
