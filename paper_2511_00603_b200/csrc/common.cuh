@@ -65,6 +65,11 @@ __device__ __forceinline__ unsigned rotate_pair(unsigned u, float c, float s) {
 }
 __device__ __forceinline__ unsigned rotate_pair(unsigned u, float2 cs) { return rotate_pair(u, cs.x, cs.y); }
 
+__device__ __forceinline__ unsigned long long pair_of(float v) {
+  const unsigned long long u = __float_as_uint(v);
+  return u << 32 | u;
+}
+
 // GELU in its erf form, 0.5 x (1 + erf(x / sqrt 2)), evaluated as 0.5 x (1 + tanh(x P(x^2))) with
 // P(t) = a + b t + c t^2 fitted (minimax over |x| <= 8) so that tanh(x P(x^2)) follows erf(x / sqrt 2):
 // the formula itself is within 2.6e-5 of the erf form everywhere.  t is clamped at 64, where the
@@ -81,6 +86,28 @@ __device__ __forceinline__ float gelu_erf(float x) {
   asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(x * p));
   const float hx = 0.5f * x;
   return fmaf(hx, th, hx);
+}
+// The same for two values, two fp32 operations per instruction (the same roundings): the loops of an epilogue are bound by
+// issue slots, 13 an element with a scalar form and 9 like this.
+__device__ __forceinline__ void gelu_erf2(float& a, float& b) {
+  asm("{\n\t.reg .b64 x, t, p, h;\n\t.reg .f32 t0, t1;\n\t"
+      "mov.b64 x, {%0, %1};\n\t"
+      "mul.rn.f32x2 t, x, x;\n\t"
+      "mov.b64 {t0, t1}, t;\n\tmin.f32 t0, t0, 0f42800000;\n\tmin.f32 t1, t1, 0f42800000;\n\tmov.b64 t, {t0, t1};\n\t"
+      "fma.rn.f32x2 p, t, %2, %3;\n\t"
+      "fma.rn.f32x2 p, t, p, %4;\n\t"
+      "mul.rn.f32x2 p, x, p;\n\t"
+      "mov.b64 {t0, t1}, p;\n\ttanh.approx.f32 t0, t0;\n\ttanh.approx.f32 t1, t1;\n\tmov.b64 p, {t0, t1};\n\t"
+      "mul.rn.f32x2 h, x, %5;\n\t"
+      "fma.rn.f32x2 x, h, p, h;\n\t"
+      "mov.b64 {%0, %1}, x;\n\t}"
+      : "+f"(a), "+f"(b)
+      : "l"(pair_of(-3.51516781e-4f)), "l"(pair_of(3.70056460e-2f)), "l"(pair_of(7.97507884e-1f)), "l"(pair_of(0.5f)));
+}
+// a, b plus the two bf16 in w
+__device__ __forceinline__ void add_bias2(float& a, float& b, unsigned w) {
+  asm("{\n\t.reg .b64 x, y;\n\t.reg .b32 lo, hi;\n\tshl.b32 lo, %2, 16;\n\tand.b32 hi, %2, 0xffff0000;\n\t"
+      "mov.b64 x, {%0, %1};\n\tmov.b64 y, {lo, hi};\n\tadd.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}" : "+f"(a), "+f"(b) : "r"(w));
 }
 // x / (1 + e^-x) with the fast division (2 ulp; the denominator is at least 1, and an overflowed e^-x gives 0,
 // the limit).  The IEEE division's special-case path, which a zero numerator takes, measured 3x slower in

@@ -211,7 +211,7 @@ struct alignas(TMAP_ALIGN) MlpGroup {
   CUtensorMap tmX;       // h [rows, d] bf16, box 64 columns x 128 rows, 128-byte swizzle
   CUtensorMap tmW1;      // W1 [F, d] bf16, box 64 x 64 rows (one CTA of a pair loads half of a chunk's 128 rows)
   CUtensorMap tmW2;      // W2 [d, F] bf16, box 64 x n2/2 rows (n2 = d, or d / 2 when d > 256: two MMAs per k step)
-  CUtensorMap tmC;       // z [rows, d] fp32, box 16 columns x 32 rows (TMA reduce-add of the epilogue)
+  CUtensorMap tmC;       // z [rows, d] fp32, box 32 columns x 16 rows, 128-byte swizzle (TMA reduce-add of the epilogue)
   const bf16* b1;        // [F] or null
   const bf16* b2;        // [d] or null
   int M, d, F;

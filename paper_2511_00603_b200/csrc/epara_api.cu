@@ -85,6 +85,18 @@ bool make_tmap_c(CUtensorMap* tm, void* C, long long rows, int N, int ldc, int e
             CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Output map of the fused MLP block: fp32 boxes of 32 columns x 16 rows.
+bool make_tmap_z(CUtensorMap* tm, void* Z, long long rows, int d) {
+  EncodeTiledFn fn = get_encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)d * 4};
+  cuuint32_t box[2] = {32, 16};
+  cuuint32_t estr[2] = {1, 1};
+  return fn(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, Z, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 struct Op {
   int kind;           // EPARA_K_*
   int rows_per_req;   // rows of this op = batch * rows_per_req ...
@@ -288,7 +300,7 @@ bool add_mlp(Builder& bl, Model* m, const void* X, long long rows_cap, const voi
     if (!make_tmap(&g.tmX, X, rows_cap, d, d, TC_BM)) return false;
     if (!make_tmap(&g.tmW1, W1, F, d, d, 64)) return false;
     if (!make_tmap(&g.tmW2, W2, d, F, F, n2 / 2)) return false;
-    if (!make_tmap_c(&g.tmC, Z, rows_cap, d, d, EPI_RESID_F32)) return false;
+    if (!make_tmap_z(&g.tmC, Z, rows_cap, d)) return false;
   }
   m->ops.push_back(op);
   return true;

@@ -141,7 +141,7 @@ __device__ __forceinline__ void epi_direct(const GView& g, const Item& it, uint3
     }
     if (g.epi & EPI_GELU) {
 #pragma unroll
-      for (int j = 0; j < CW; ++j) v[j] = gelu_erf(v[j]);
+      for (int j = 0; j < CW; j += 2) gelu_erf2(v[j], v[j + 1]);
     }
     // the previous box of this warp must have been read out of the staging area
     if (lane == 0) bulk_wait_read0();
@@ -399,37 +399,41 @@ gemm_tc_pair_kernel(const GemmGroup* __restrict__ groups, int n_groups, int tota
 // of 128 columns:
 //   S = h W1_c^T         (M 256, N 128, K d)  into tensor-memory columns 384..511,
 //   P = bf16(GELU(S + b1_c)) by the 16 epilogue warps, written to shared memory in the K-major 128-byte-swizzled
-//                        layout an A operand has (two blocks of 128 rows x 64 columns),
+//                        layout an A operand has (two units of 128 rows x 64 columns),
 //   O += P W2_c^T        (M 256, N d, K 128)  into columns 0..d-1 (two MMAs of N = d / 2 per k step when d > 256),
-// and after the last chunk O + b2 is added to z through the same TMA reduce-add epilogue as any fp32-residual
-// GEMM.  The rounding points are those of the unfused pair of GEMMs (the hidden tensor is rounded to bf16 once,
+// and after the last chunk O + b2 is added to z by TMA reduce-adds, as in any fp32-residual GEMM.  The rounding points are those of the unfused pair of GEMMs (the hidden tensor is rounded to bf16 once,
 // the k order of both contractions is ascending), so a request's bits do not change with the kernel.
 // The two contractions have an issuing thread each (warp 1 for S, the last warp for O): the chains only meet
 // through the epilogue warps (S -> P), so the tensor core works on the next chunk's S while this chunk's GELU is
 // computed and on this chunk's O while the next S is read out, and neither thread's issue time delays the other chain.
-// What bounds it: S and P have one buffer each, so that O of a chunk, the writing of the next P and that P's O are one
-// chain.  Cycles per chunk and role at d 384 (5.9 thousand in all, a twelfth of the tile's 11.5 thousand for its output
-// included; 3.07 thousand of tensor work): S issuer 1.9 issuing, 2.8 waiting for the read-out; O issuer 2.4 issuing, 2.5
-// waiting for P; an epilogue warp 0.6 waiting for S, 0.1 reading, 1.6 of bias and GELU, 1.8 waiting for P's buffer.
-// Weights stream through two rings of two 24 KB slots (W1: three k-blocks
-// of a chunk half per slot; W2: one k-block of a chunk half per slot), each with its own producer thread.
-// P's 32 KB double as the staging area of the final epilogue (P is idle by then).
-constexpr int MLP_SLOT_BYTES = 24 * 1024;
-constexpr int MLP_SLOTS = 4;                                   // two for W1 (0, 1), two for W2 (2, 3)
+// P is a ring of three units of 64 hidden columns, so that a chunk's P is written while the O of the chunk before still runs
+// (with one buffer of a whole chunk that was one chain: 5.5 thousand cycles a chunk, 2.8 of them an epilogue warp's wait for the
+// buffer; with the ring 4.3, with GELU two values an instruction and biases by load instead of shuffle 3.5).
+// What bounds it: per chunk 3.07 thousand cycles of tensor work and about as many of shared memory (h is read again for every
+// S, P for every O: 290 KB of operands, 100 KB of arriving weights, 32 KB of P at 128 bytes a cycle); an epilogue warp spends 1.0
+// thousand waiting for S, 0.2 reading it, 1.5 on bias and GELU, 0.6 on P.  A tile's output takes 11 thousand, 2 to 3 of them until O is
+// complete: 196 KB a CTA at the rate of the reductions at L2, all CTAs at once (boxes of 16-column rows: 15 thousand).
+// 203 images of ViT-S: 94 us a launch before, 80 now, at 1.69 GHz under the power cap (1.77 before).
+// Weights stream through two rings (W1: four slots of one k-block of a chunk half, 8 KB; W2: two of 24 KB), each with its own
+// producer thread.  P's ring doubles as the staging area of the final epilogue (P is idle by then).
+constexpr int MLP_W1_BYTES = 64 * 128, MLP_W2_BYTES = 24 * 1024;   // a k-block of a chunk half
+constexpr int MLP_W1_SLOTS = 4, MLP_W2_SLOTS = 2, MLP_SLOTS = MLP_W1_SLOTS + MLP_W2_SLOTS;
 constexpr int MLP_O_WARP = PAIR_W_WARP + 1;                    // issues the second contraction
 constexpr int MLP_THREADS = PAIR_THREADS + 32;
 constexpr int MLP_X_BYTES = 6 * A_BYTES;                       // d <= 384: at most six k-blocks of 128 x 64
-constexpr int MLP_P_BYTES = 2 * A_BYTES;                       // 128 rows x 128 hidden columns, bf16
+constexpr int MLP_P_UNITS = 3;                                 // 128 rows x 64 hidden columns each, bf16
+constexpr int MLP_P_BYTES = MLP_P_UNITS * A_BYTES;
 constexpr int MLP_OFF_P = MLP_X_BYTES;
 constexpr int MLP_OFF_RING = MLP_OFF_P + MLP_P_BYTES;
-constexpr int MLP_OFF_BAR = MLP_OFF_RING + MLP_SLOTS * MLP_SLOT_BYTES;
+constexpr int MLP_OFF_W2 = MLP_OFF_RING + MLP_W1_SLOTS * MLP_W1_BYTES;
+constexpr int MLP_OFF_BAR = MLP_OFF_W2 + MLP_W2_SLOTS * MLP_W2_BYTES;
 constexpr size_t MLP_SMEM_BYTES = 1024 + (size_t)MLP_OFF_BAR + 256;
 static_assert(MLP_SMEM_BYTES <= 227 * 1024, "shared memory of one SM");
-static_assert(STAGE_OUT_BYTES <= MLP_P_BYTES, "the final epilogue stages its boxes in P");
+static_assert(EPI_WARPS * 2048 <= MLP_P_BYTES, "the final epilogue stages its boxes in P");
 constexpr int MLP_S_COL = 384;                                 // S behind the output accumulator
 constexpr int MLP_CHUNK = 128;
-enum { MB_W_FULL = 0, MB_W_EMPTY = MLP_SLOTS, MB_X_FULL = 2 * MLP_SLOTS, MB_X_EMPTY, MB_S_FULL, MB_S_EMPTY, MB_P_FULL,
-       MB_P_EMPTY, MB_O_FULL, MB_O_EMPTY, MB_STAGE_FREE, MB_COUNT };
+enum { MB_W_FULL = 0, MB_W_EMPTY = MLP_SLOTS, MB_X_FULL = 2 * MLP_SLOTS, MB_X_EMPTY, MB_S_FULL, MB_S_EMPTY, MB_O_FULL, MB_O_EMPTY,
+       MB_STAGE_FREE, MB_P_FULL, MB_P_EMPTY = MB_P_FULL + MLP_P_UNITS, MB_COUNT = MB_P_EMPTY + MLP_P_UNITS };
 static_assert(8 * MB_COUNT + 16 <= 256, "barrier area");
 
 __device__ __forceinline__ int find_group_mlp(const MlpGroup* groups, int n, int item) {
@@ -440,7 +444,7 @@ __device__ __forceinline__ int find_group_mlp(const MlpGroup* groups, int n, int
 // Geometry of a group in registers (the single-thread roles cannot hide descriptor loads).
 struct MlpGeo {
   const MlpGroup* g;
-  int start, end, kb1, nc, n2, n2i, slots1;
+  int start, end, kb1, nc, n2, n2i;
 };
 __device__ __forceinline__ void mlp_geo(MlpGeo& c, const MlpGroup* groups, int n_groups, int item) {
   if (c.g != nullptr && item >= c.start && item < c.end) return;
@@ -453,7 +457,6 @@ __device__ __forceinline__ void mlp_geo(MlpGeo& c, const MlpGroup* groups, int n
   c.nc = g->F / MLP_CHUNK;              // chunks of the hidden layer
   c.n2i = d > 256 ? 2 : 1;              // MMAs per k step of the second contraction
   c.n2 = d / c.n2i;                     // and their N
-  c.slots1 = (c.kb1 + 2) / 3;           // ring slots of one W1 chunk (three k-blocks of 64 rows each per slot)
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MLP_THREADS, 1)
@@ -473,7 +476,7 @@ gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int tota
     for (int s = 0; s < MLP_SLOTS; ++s) { mbar_init(bar(MB_W_FULL + s), 1); mbar_init(bar(MB_W_EMPTY + s), 1); }
     mbar_init(bar(MB_X_FULL), 1); mbar_init(bar(MB_X_EMPTY), 1);
     mbar_init(bar(MB_S_FULL), 1); mbar_init(bar(MB_S_EMPTY), 2 * EPI_WARPS);
-    mbar_init(bar(MB_P_FULL), 2 * EPI_WARPS); mbar_init(bar(MB_P_EMPTY), 1);
+    for (int u = 0; u < MLP_P_UNITS; ++u) { mbar_init(bar(MB_P_FULL + u), EPI_WARPS); mbar_init(bar(MB_P_EMPTY + u), 1); }
     mbar_init(bar(MB_O_FULL), 1); mbar_init(bar(MB_O_EMPTY), 2 * EPI_WARPS);
     mbar_init(bar(MB_STAGE_FREE), EPI_WARPS);
     *abort_flag = 0;
@@ -510,14 +513,11 @@ gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int tota
       for (int kb = 0; kb < gc.kb1; ++kb)
         tma_load_2d_pair_elect(base + kb * A_BYTES, &g->tmX, kb * TC_BK, m0, mapa_shared(bar(MB_X_FULL), 0));
       for (int c = 0; c < gc.nc && ok; ++c) {
-        for (int s1 = 0; s1 < gc.slots1; ++s1) {
+        for (int kb = 0; kb < gc.kb1; ++kb) {
           if (!mbar_wait(bar(MB_W_EMPTY + slot), phase ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 42); break; }
-          const int kb_lo = s1 * 3, kb_hi = min(gc.kb1, kb_lo + 3);
-          if (rank == 0) mbar_expect_tx_elect(bar(MB_W_FULL + slot), 2u * (uint32_t)(kb_hi - kb_lo) * (64 * 128));
-          for (int kb = kb_lo; kb < kb_hi; ++kb)
-            tma_load_2d_pair_elect(base + MLP_OFF_RING + slot * MLP_SLOT_BYTES + (kb - kb_lo) * (64 * 128), &g->tmW1, kb * TC_BK,
-                                   c * MLP_CHUNK + rank * 64, mapa_shared(bar(MB_W_FULL + slot), 0));
-          if (++slot == 2) { slot = 0; phase ^= 1u; }
+          if (rank == 0) mbar_expect_tx_elect(bar(MB_W_FULL + slot), 2u * MLP_W1_BYTES);
+          tma_load_2d_pair_elect(base + MLP_OFF_RING + slot * MLP_W1_BYTES, &g->tmW1, kb * TC_BK, c * MLP_CHUNK + rank * 64, mapa_shared(bar(MB_W_FULL + slot), 0));
+          if (++slot == MLP_W1_SLOTS) { slot = 0; phase ^= 1u; }
         }
       }
     }
@@ -538,12 +538,12 @@ gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int tota
       const int half = gc.n2 >> 1;                         // rows of one MMA's B operand held by this CTA
       for (int c = 0; c < gc.nc && ok; ++c) {
         for (int j = 0; j < 2; ++j) {                      // the chunk's two k-blocks
-          if (!mbar_wait(bar(MB_W_EMPTY + 2 + slot), phase ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 43); break; }
-          if (rank == 0) mbar_expect_tx_elect(bar(MB_W_FULL + 2 + slot), 2u * (uint32_t)gc.n2i * (uint32_t)half * 128u);
+          if (!mbar_wait(bar(MB_W_EMPTY + MLP_W1_SLOTS + slot), phase ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 43); break; }
+          if (rank == 0) mbar_expect_tx_elect(bar(MB_W_FULL + MLP_W1_SLOTS + slot), 2u * (uint32_t)gc.n2i * (uint32_t)half * 128u);
           for (int i = 0; i < gc.n2i; ++i)
-            tma_load_2d_pair_elect(base + MLP_OFF_RING + (2 + slot) * MLP_SLOT_BYTES + i * half * 128, &g->tmW2, (2 * c + j) * TC_BK,
-                                   i * gc.n2 + rank * half, mapa_shared(bar(MB_W_FULL + 2 + slot), 0));
-          if (++slot == 2) { slot = 0; phase ^= 1u; }
+            tma_load_2d_pair_elect(base + MLP_OFF_W2 + slot * MLP_W2_BYTES + i * half * 128, &g->tmW2, (2 * c + j) * TC_BK,
+                                   i * gc.n2 + rank * half, mapa_shared(bar(MB_W_FULL + MLP_W1_SLOTS + slot), 0));
+          if (++slot == MLP_W2_SLOTS) { slot = 0; phase ^= 1u; }
         }
       }
     }
@@ -565,18 +565,14 @@ gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int tota
           // S is free once the epilogue warps have read the chunk before out of it
           if (n_s > 0 && !mbar_wait<false>(bar(MB_S_EMPTY), (n_s - 1) & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 44); break; }
           tc_fence_after();
-          for (int s1 = 0; s1 < gc.slots1; ++s1) {
+          for (int kb = 0; kb < gc.kb1; ++kb) {
             if (!mbar_wait<false>(bar(MB_W_FULL + slot), phase, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 45); break; }
-            const int kb_lo = s1 * 3, kb_hi = min(gc.kb1, kb_lo + 3);
-            for (int kb = kb_lo; kb < kb_hi; ++kb) {
-              const uint64_t da = make_smem_desc(base + kb * A_BYTES);
-              const uint64_t db = make_smem_desc(base + MLP_OFF_RING + slot * MLP_SLOT_BYTES + (kb - kb_lo) * (64 * 128));
+            const uint64_t da = make_smem_desc(base + kb * A_BYTES), db = make_smem_desc(base + MLP_OFF_RING + slot * MLP_W1_BYTES);
 #pragma unroll
-              for (int k = 0; k < TC_BK / 16; ++k)
-                mma_f16_pair_elect(tmem_base + MLP_S_COL, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc_s, (kb > 0 || k > 0) ? 1u : 0u);
-            }
+            for (int k = 0; k < TC_BK / 16; ++k)
+              mma_f16_pair_elect(tmem_base + MLP_S_COL, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc_s, (kb > 0 || k > 0) ? 1u : 0u);
             mma_commit_pair_elect(bar(MB_W_EMPTY + slot));
-            if (++slot == 2) { slot = 0; phase ^= 1u; }
+            if (++slot == MLP_W1_SLOTS) { slot = 0; phase ^= 1u; }
           }
           if (!ok) break;
           mma_commit_pair_elect(bar(MB_S_FULL));
@@ -590,7 +586,7 @@ gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int tota
     if (rank == 0) {
       int slot = 0;
       uint32_t phase = 0;
-      uint32_t n_o = 0, t = 0;
+      uint32_t unit = 0, unit_phase = 0, t = 0;
       bool ok = true;
       MlpGeo gc;
       gc.g = nullptr;
@@ -598,26 +594,27 @@ gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int tota
         mlp_geo(gc, groups, n_groups, item);
         const uint32_t idesc_o = make_idesc_pair(gc.n2);
         const int half = gc.n2 >> 1;
-        for (int c = 0; c < gc.nc && ok; ++c, ++n_o) {
-          if (!mbar_wait<false>(bar(MB_P_FULL), n_o & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 46); break; }
+        for (int c = 0; c < gc.nc && ok; ++c) {
           // the first chunk overwrites O: the tile before must have been read out of it
           if (c == 0 && t > 0 && !mbar_wait<false>(bar(MB_O_EMPTY), (t - 1) & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 47); break; }
-          tc_fence_after();
           for (int j = 0; j < 2; ++j) {
-            if (!mbar_wait<false>(bar(MB_W_FULL + 2 + slot), phase, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 48); break; }
-            const uint64_t da = make_smem_desc(base + MLP_OFF_P + j * A_BYTES);
+            if (!mbar_wait<false>(bar(MB_P_FULL + unit), unit_phase, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 46); break; }
+            tc_fence_after();
+            if (!mbar_wait<false>(bar(MB_W_FULL + MLP_W1_SLOTS + slot), phase, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 48); break; }
+            const uint64_t da = make_smem_desc(base + MLP_OFF_P + unit * A_BYTES);
 #pragma unroll
             for (int k = 0; k < TC_BK / 16; ++k)
               for (int i = 0; i < gc.n2i; ++i) {
-                const uint64_t db = make_smem_desc(base + MLP_OFF_RING + (2 + slot) * MLP_SLOT_BYTES + i * half * 128);
+                const uint64_t db = make_smem_desc(base + MLP_OFF_W2 + slot * MLP_W2_BYTES + i * half * 128);
                 mma_f16_pair_elect(tmem_base + (uint32_t)(i * gc.n2), da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc_o,
                                    (c > 0 || j > 0 || k > 0) ? 1u : 0u);
               }
-            mma_commit_pair_elect(bar(MB_W_EMPTY + 2 + slot));
-            if (++slot == 2) { slot = 0; phase ^= 1u; }
+            mma_commit_pair_elect(bar(MB_W_EMPTY + MLP_W1_SLOTS + slot));
+            mma_commit_pair_elect(bar(MB_P_EMPTY + unit));
+            if (++slot == MLP_W2_SLOTS) { slot = 0; phase ^= 1u; }
+            if (++unit == MLP_P_UNITS) { unit = 0; unit_phase ^= 1u; }
           }
           if (!ok) break;
-          mma_commit_pair_elect(bar(MB_P_EMPTY));
           if (c == gc.nc - 1) mma_commit_pair_elect(bar(MB_O_FULL));
         }
       }
@@ -636,9 +633,10 @@ gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int tota
     int g_start = 0, g_end = -1, nc = 0, d = 0, c_rows = 0;
     const bf16 *b1 = nullptr, *b2 = nullptr;
     const uint32_t s_taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(MLP_S_COL + part * 32);
-    unsigned char* prow = base_ptr + MLP_OFF_P + (part >> 1) * A_BYTES + row * 128;
+    unsigned char* const prow0 = base_ptr + MLP_OFF_P + row * 128;
+    uint32_t unit = part >> 1, unit_phase = 1;                // this warp's next unit of P: every other one, from its half of the chunk on
     const int piece0 = (part & 1) * 4, sw = row & 7;
-    const uint32_t s_empty_r = mapa_shared(bar(MB_S_EMPTY), 0), p_full_r = mapa_shared(bar(MB_P_FULL), 0);
+    const uint32_t s_empty_r = mapa_shared(bar(MB_S_EMPTY), 0), p_full_r = mapa_shared(bar(MB_P_FULL), 0);   // (of unit 0)
     const uint32_t o_empty_r = mapa_shared(bar(MB_O_EMPTY), 0);
     for (int item = pair; item < total_items && ok; item += n_pairs, ++t) {
       if (item >= g_end || item < g_start) {
@@ -648,9 +646,11 @@ gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int tota
         if (lane == 0) tensormap_acquire(&g->tmC);
       }
       for (int c = 0; c < nc && ok; ++c, ++n_c) {
-        // this warp's 32 hidden columns of the chunk: bias values four per lane in lanes 0..7
-        uint2 bias_reg = make_uint2(0u, 0u);
-        if (b1 != nullptr && lane < 8) bias_reg = __ldg(reinterpret_cast<const uint2*>(b1 + c * MLP_CHUNK + part * 32 + lane * 4));
+        // this warp's 32 hidden columns of the chunk: every lane has all their bias values (requested before the wait; handed
+        // around with shuffles they took a quarter of the loop's issue slots)
+        uint4 bias[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) bias[j] = b1 != nullptr ? __ldg(reinterpret_cast<const uint4*>(b1 + c * MLP_CHUNK + part * 32) + j) : make_uint4(0u, 0u, 0u, 0u);
         if (!mbar_wait(bar(MB_S_FULL), n_c & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 50); break; }
         tc_fence_after();
         float v[32];
@@ -663,20 +663,20 @@ gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int tota
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(s_empty_r);       // the next chunk's S may be issued
-        if (b1 != nullptr) {
 #pragma unroll
-          for (int jj = 0; jj < 16; ++jj) {
-            const uint32_t w = __shfl_sync(0xffffffffu, (jj & 1) ? bias_reg.y : bias_reg.x, jj >> 1);
-            v[2 * jj] += __uint_as_float(w << 16);
-            v[2 * jj + 1] += __uint_as_float(w & 0xffff0000u);
-          }
+        for (int j = 0; j < 4; ++j) {
+          add_bias2(v[8 * j], v[8 * j + 1], bias[j].x);
+          add_bias2(v[8 * j + 2], v[8 * j + 3], bias[j].y);
+          add_bias2(v[8 * j + 4], v[8 * j + 5], bias[j].z);
+          add_bias2(v[8 * j + 6], v[8 * j + 7], bias[j].w);
         }
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = gelu_erf(v[j]);
-        // P still feeds the second contraction of the chunk before; at a tile's first chunk it also was the
+        for (int j = 0; j < 32; j += 2) gelu_erf2(v[j], v[j + 1]);
+        // the unit may still feed the second contraction of an earlier chunk; at a tile's first chunk P also was the
         // staging area of the final epilogue of the tile before, which every warp of this CTA must have left
-        if (n_c > 0 && !mbar_wait(bar(MB_P_EMPTY), (n_c - 1) & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 51); break; }
+        if (!mbar_wait(bar(MB_P_EMPTY + unit), unit_phase, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 51); break; }
         if (c == 0 && t > 0 && !mbar_wait(bar(MB_STAGE_FREE), (t - 1) & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 52); break; }
+        unsigned char* const prow = prow0 + unit * A_BYTES;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           uint4 o;
@@ -686,24 +686,61 @@ gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int tota
         }
         fence_async_smem();                     // P must be visible to the tensor core's reads
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(p_full_r);
+        if (lane == 0) mbar_arrive_cluster(p_full_r + 8u * unit);
+        unit += 2;
+        if (unit >= MLP_P_UNITS) { unit -= MLP_P_UNITS; unit_phase ^= 1u; }
       }
       if (!ok) break;
-      // ---- the tile's output: O + b2 added to z (TMA reduce-add), staged in P
-      GView gv;
-      gv.bias = b2; gv.tmC = &g->tmC; gv.N = d; gv.epi = EPI_RESID_F32 | (b2 != nullptr ? EPI_BIAS : 0);
-      gv.tile_start = g_start; gv.tiles_m = g_end - g_start; gv.tiles_n = 1; gv.bn = d; gv.c_rows = c_rows;
-      Item it;
-      it.m0 = (item - g_start) * (2 * TC_BM) + rank * TC_BM; it.n0 = 0;
+      // ---- the tile's output: O + b2 added to z, in boxes of 16 rows x 32 columns staged in P: the rows of a box are whole
+      // 128-byte lines, which is what the reduction at L2 is fast with
       uint2 bias_reg = make_uint2(0u, 0u);
-      if (b2 != nullptr) {
-        const int nb = part * (d >> 2) + lane * 4;
-        if (lane * 4 < (d >> 2)) bias_reg = __ldg(reinterpret_cast<const uint2*>(b2 + nb));
-      }
+      const int n_out = (d >> 5) - part;                       // this warp's blocks of 32 columns: part, part + 4, ...
+      if (b2 != nullptr && (lane >> 3) * 4 < n_out) bias_reg = __ldg(reinterpret_cast<const uint2*>(b2 + part * 32 + (lane >> 3) * 128 + (lane & 7) * 4));
       if (!mbar_wait(bar(MB_O_FULL), t & 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 53); break; }
       tc_fence_after();
-      const uint32_t o_taddr = tmem_base + ((uint32_t)(quarter * 32) << 16);
-      epi_direct<2>(gv, it, o_taddr, base_ptr + MLP_OFF_P + ew * 2048, quarter, part, lane, bias_reg, o_empty_r);
+      const uint32_t o_taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(part * 32);
+      unsigned char* const wst = base_ptr + MLP_OFF_P + ew * 2048;
+      const int y0 = (item - g_start) * (2 * TC_BM) + rank * TC_BM + quarter * 32;
+#pragma unroll 1
+      for (int i = 0; i * 4 < n_out; ++i) {
+        float v[32];
+        {
+          uint32_t r[32];
+          tmem_ld32(o_taddr + (uint32_t)(i * 128), r);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+        }
+        if ((i + 1) * 4 >= n_out) {                            // that was this warp's last read of O
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(o_empty_r);
+        }
+        if (b2 != nullptr) {
+#pragma unroll
+          for (int jj = 0; jj < 16; ++jj) {
+            const uint32_t w = __shfl_sync(0xffffffffu, (jj & 1) ? bias_reg.y : bias_reg.x, i * 8 + (jj >> 1));
+            v[2 * jj] += __uint_as_float(w << 16);
+            v[2 * jj + 1] += __uint_as_float(w & 0xffff0000u);
+          }
+        }
+#pragma unroll
+        for (int hr = 0; hr < 2; ++hr) {                       // rows 0 .. 15, then 16 .. 31
+          if (lane == 0) bulk_wait_read0();                    // the box before has left the staging area
+          __syncwarp();
+          if (lane >> 4 == hr) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+              *reinterpret_cast<float4*>(wst + (lane & 15) * 128 + ((k ^ (lane & 7)) << 4)) = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+          }
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0 && y0 + hr * 16 < c_rows) {
+            tma_reduce_add_2d(&g->tmC, smem_u32(wst), part * 32 + i * 128, y0 + hr * 16);
+            bulk_commit();
+          }
+        }
+      }
+      if (n_out <= 0) { if (lane == 0) mbar_arrive_cluster(o_empty_r); }
       if (lane == 0) { bulk_wait_read0(); mbar_arrive(bar(MB_STAGE_FREE)); }   // this warp's boxes have left P
     }
     if (lane == 0) bulk_wait_done0();
