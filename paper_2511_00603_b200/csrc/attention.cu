@@ -338,16 +338,20 @@ __device__ __forceinline__ uint32_t transpose_8x8(uint32_t u) {
   return r;
 }
 
+// What the kernels before this one wrote: past L1 where no dependency wait has emptied it.
+template <bool BESIDE>
+__device__ __forceinline__ uint32_t ld_step(const uint32_t* p) { return BESIDE ? __ldcg(p) : *p; }
+
 // k (rotated to `cs_row`) and v of one kv head of an unrotated qkv row, to slot r of a staged tile (K, then V HD * 32 bytes
 // on) and, with dst, to the cache (V HD * 8 * Hkv words on): a pair per lane and piece.
-template <int HD>
+template <int HD, bool BESIDE>
 __device__ __forceinline__ void place_kv(unsigned char* tile, int r, const uint32_t* kr, int Hkv, const float2* cs_row, uint32_t* dst) {
   const int lane = threadIdx.x & 31;
   unsigned char* const kt = tile + r * (HD * 2);
 #pragma unroll
   for (int p = 0; p < HD / 64; ++p) {
     const int pair = p * 32 + lane, c = pair >> 2;
-    const uint32_t nk = rotate_pair(kr[pair], __ldg(cs_row + pair)), nv = kr[Hkv * (HD / 2) + pair];
+    const uint32_t nk = rotate_pair(ld_step<BESIDE>(kr + pair), __ldg(cs_row + pair)), nv = ld_step<BESIDE>(kr + Hkv * (HD / 2) + pair);
     if (dst != nullptr) {
       dst[pair] = nk;
       dst[Hkv * 8 * HD + pair] = nv;
@@ -360,28 +364,29 @@ __device__ __forceinline__ void place_kv(unsigned char* tile, int r, const uint3
 
 // Several requests of one sequence in one step: a staged tile's slots below n_slots that other rows of the step append to
 // this page are taken from those rows, since the append itself may stand before, beside or behind this block's read.
-template <int HD>
+template <int HD, bool BESIDE>
 __device__ __forceinline__ void place_step_rows(const AttnDecGroup& g, unsigned char* tile, int page, int kvh, int own_row, int n_slots) {
   const int lane = threadIdx.x & 31;
 #pragma unroll 1
   for (int w0 = 0; w0 < g.n_written; w0 += 32) {
     WrittenPage wp = {nullptr, 0, 0};
     if (w0 + lane < g.n_written) wp = g.written[w0 + lane];
-    const bool hit = wp.id != nullptr && wp.row() != own_row && (wp.pos & 15) < n_slots && *wp.id == page;
+    const bool hit = wp.id != nullptr && wp.row != own_row && (wp.pos & 15) < n_slots && *wp.id == page;
     for (unsigned m = __ballot_sync(0xffffffffu, hit); m != 0; m &= m - 1) {
-      const int l = __ffs(m) - 1, pos = __shfl_sync(0xffffffffu, wp.pos, l), row_n = __shfl_sync(0xffffffffu, wp.row_n, l);
-      const int n = min(row_n & 31, n_slots - (pos & 15));
+      const int l = __ffs(m) - 1, pos = __shfl_sync(0xffffffffu, wp.pos, l), row = __shfl_sync(0xffffffffu, wp.row, l);
+      const int n = min(1, n_slots - (pos & 15));               // one token: a rolled loop all the same, straight code here costs the caller spills
 #pragma unroll 1
       for (int r = 0; r < n; ++r) {
-        const bf16* const row = g.q + (size_t)((row_n >> 5) + r) * g.q_stride + (size_t)(g.Hq + kvh) * HD;
-        place_kv<HD>(tile, (pos + r) & 15, reinterpret_cast<const uint32_t*>(row), g.Hkv, g.cs + (size_t)(pos + r) * (HD / 2), nullptr);
+        const bf16* const kv = g.q + (size_t)(row + r) * g.q_stride + (size_t)(g.Hq + kvh) * HD;
+        place_kv<HD, BESIDE>(tile, (pos + r) & 15, reinterpret_cast<const uint32_t*>(kv), g.Hkv, g.cs + (size_t)(pos + r) * (HD / 2), nullptr);
       }
     }
   }
   __syncwarp();
 }
 
-template <int HD, int G, int NSLOT>
+// BESIDE: runs beside the launch before it (see pdl_begin(); q, k and v then come past L1).
+template <int HD, int G, int NSLOT, bool BESIDE>
 __global__ void __launch_bounds__(128, HD == 64 && G <= 4 ? 5 : 4) attn_decode_mma_kernel(const AttnDecGroup* __restrict__ groups, int n_groups, int fused) {
   constexpr int ROWB = HD * 2;              // bytes per token row
   constexpr int TILE = 16 * ROWB;           // bytes per (K or V) page tile
@@ -399,7 +404,7 @@ __global__ void __launch_bounds__(128, HD == 64 && G <= 4 ? 5 : 4) attn_decode_m
   if (kvh >= g.Hkv) return;
   const bool early = g.reqs_stable && g.cs != nullptr;
   if (g.reqs_stable && blockIdx.x * ATTN_CHUNK >= g.reqs[b].len) return;   // nothing to do and nothing to wait for
-  if (!early) pdl_wait();     // q, the appended K/V row and (single-kernel entry) the request table come from earlier kernels
+  if (!early) pdl_begin(BESIDE);     // q, the appended K/V row and (single-kernel entry) the request table come from earlier kernels
   const AttnReq rq = g.reqs[b];
   const int chunk = blockIdx.x;
   const int t_begin = chunk * ATTN_CHUNK;
@@ -450,7 +455,7 @@ __global__ void __launch_bounds__(128, HD == 64 && G <= 4 ? 5 : 4) attn_decode_m
   // (With cs the pages are requested while the QKV projection may still be running.  A slot that the step itself writes holds
   // something old, or half of something: that of `pos`, and those of other requests of the same sequence (`linked`), which
   // are replaced in shared memory below.  Everything else was written by earlier steps or by the caller.)
-  if (early) pdl_wait();
+  if (early) pdl_begin(BESIDE);
   const bool linked = g.linked != nullptr && __ldcg(g.linked + b) != 0;
 
   // ---- Q fragments: the query heads of this kv head are the first G of the B operand's 8 columns
@@ -460,8 +465,8 @@ __global__ void __launch_bounds__(128, HD == 64 && G <= 4 ? 5 : 4) attn_decode_m
     const bf16* qrow = row0 + (size_t)(kvh * G + gq) * HD;
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) {
-      qb[ks][0] = (gq < G) ? *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 2 * tq) : 0u;
-      qb[ks][1] = (gq < G) ? *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 8 + 2 * tq) : 0u;
+      qb[ks][0] = (gq < G) ? ld_step<BESIDE>(reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 2 * tq)) : 0u;
+      qb[ks][1] = (gq < G) ? ld_step<BESIDE>(reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 8 + 2 * tq)) : 0u;
       if (cs != nullptr) {                   // a lane's two elements are one rotation pair
         const float2* c = cs + (size_t)pos * (HD / 2) + ks * 8 + tq;
         qb[ks][0] = rotate_pair(qb[ks][0], __ldg(c));
@@ -484,12 +489,12 @@ __global__ void __launch_bounds__(128, HD == 64 && G <= 4 ? 5 : 4) attn_decode_m
     if (app_page >= 0 && pg == pos >> 4) {
       // the new token: k (rotated) and v of this kv head to the cache and into the staged tile
       const int r = pos & 15;
-      place_kv<HD>(wsm + (i % NSLOT) * 2 * TILE, r, reinterpret_cast<const uint32_t*>(row0 + (size_t)(g.Hq + kvh) * HD), Hkv,
+      place_kv<HD, BESIDE>(wsm + (i % NSLOT) * 2 * TILE, r, reinterpret_cast<const uint32_t*>(row0 + (size_t)(g.Hq + kvh) * HD), Hkv,
                    cs + (size_t)pos * (HD / 2),
                    reinterpret_cast<uint32_t*>(kv_layer + (((size_t)app_page * 2) * Hkv + kvh) * 16 * HD + (size_t)r * HD));
       __syncwarp();
     }
-    if constexpr (decltype(shared)::value) place_step_rows<HD>(g, wsm + (i % NSLOT) * 2 * TILE, rq.table[pg], kvh, rq.row, pos - tok0);
+    if constexpr (decltype(shared)::value) place_step_rows<HD, BESIDE>(g, wsm + (i % NSLOT) * 2 * TILE, rq.table[pg], kvh, rq.row, pos - tok0);
     if (tok0 + 16 > t_end) {
       // slots past the length may hold anything (NaN included): zero those V rows
       const int valid = t_end - tok0;
@@ -587,16 +592,18 @@ __global__ void __launch_bounds__(128, HD == 64 && G <= 4 ? 5 : 4) attn_decode_m
   }
   __syncthreads();
   finish_chunk<HD, G>(g, b, rq.row, kvh, chunk, rq.len, fused, sm_m, sm_l, sm_o);
+  pdl_end(BESIDE);
 }
 
 template <int HD, int G>
 static cudaError_t launch_dec_mma(const AttnDecGroup* groups, int n_groups, int total_B, int max_Hkv, int max_chunks,
-                                  int fused, cudaStream_t st) {
+                                  int fused, cudaStream_t st, int beside) {
   constexpr int NSLOT = 2;                           // pages in flight per warp
   constexpr int SMEM = 4 * NSLOT * 2 * 16 * HD * 2;  // 4 warps x NSLOT pages x (K + V) tiles
-  cudaError_t e = cudaFuncSetAttribute(attn_decode_mma_kernel<HD, G, NSLOT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+  const auto kernel = beside ? attn_decode_mma_kernel<HD, G, NSLOT, true> : attn_decode_mma_kernel<HD, G, NSLOT, false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
   if (e != cudaSuccess) return e;
-  return launch_pdl(attn_decode_mma_kernel<HD, G, NSLOT>, dim3(max_chunks, max_Hkv, total_B), dim3(128), SMEM, st, groups, n_groups, fused);
+  return launch_pdl(kernel, dim3(max_chunks, max_Hkv, total_B), dim3(128), SMEM, st, groups, n_groups, fused);
 }
 
 template <int HD, int G>
@@ -618,12 +625,12 @@ bool attn_decode_fused(int total_B, int max_Hkv, int max_chunks, int hd, int sm_
 }
 
 cudaError_t launch_attn_decode(const AttnDecGroup* groups, int n_groups, int total_B, int max_Hkv, int max_Hq,
-                               int max_chunks, int hd, int gqa, int fused, cudaStream_t st) {
+                               int max_chunks, int hd, int gqa, int fused, cudaStream_t st, int beside) {
   if (n_groups == 0 || total_B == 0) return cudaSuccess;
   if (total_B > 65535 || max_Hkv > 65535) return cudaErrorInvalidValue;
   cudaError_t e = cudaErrorInvalidValue;
 #define EPARA_DEC(HD_, G_) if (hd == HD_ && gqa == G_) e = launch_dec<HD_, G_>(groups, n_groups, total_B, max_Hkv, max_chunks, fused, st);
-#define EPARA_DEC_MMA(HD_, G_) if (hd == HD_ && gqa == G_) e = launch_dec_mma<HD_, G_>(groups, n_groups, total_B, max_Hkv, max_chunks, fused, st);
+#define EPARA_DEC_MMA(HD_, G_) if (hd == HD_ && gqa == G_) e = launch_dec_mma<HD_, G_>(groups, n_groups, total_B, max_Hkv, max_chunks, fused, st, beside);
   EPARA_DEC_MMA(64, 1) EPARA_DEC_MMA(64, 2) EPARA_DEC_MMA(64, 4) EPARA_DEC_MMA(64, 8)
   EPARA_DEC_MMA(128, 1) EPARA_DEC_MMA(128, 2) EPARA_DEC_MMA(128, 4) EPARA_DEC_MMA(128, 8)
 #undef EPARA_DEC_MMA

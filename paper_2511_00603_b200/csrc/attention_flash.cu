@@ -251,7 +251,7 @@ struct Cursor {
 
 template <int HD, bool PAGED, bool HALF, class Group, class View>
 __global__ void __launch_bounds__(FL_THREADS, 1)
-attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_items, int mt, int* __restrict__ status) {
+attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_items, int mt, int* __restrict__ status, int beside) {
   using Geo = FlashGeo<HD>;
   constexpr int ST = Geo::STAGES;
   constexpr bool SPLIT = PAGED;                  // P as head + remainder
@@ -315,7 +315,7 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
         kx = (view.H + w.head) * 64; vx = kx + view.H * 64;
         ky = (w.qy / view.T) * view.T;
       }
-      if (!waited) { pdl_wait(); waited = true; }                 // q, k, v come from the kernels before this one
+      if (!waited) { pdl_begin(beside); waited = true; }                 // q, k, v come from the kernels before this one
       for (int j = 0; j < nblk && ok; ++j) {
         const int n = min(FL_TILE, w.n_keys - j * FL_TILE), pages = (n + 15) >> 4;
         int yk = oob;
@@ -358,7 +358,7 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
       }
       ++it;
     }
-    if (!waited) pdl_wait();
+    if (!waited) pdl_begin(beside);
     if (!ok) { *abort_flag = 1; drain_sleep(200000ull); }
   } else if (warp == FL_S_WARP) {
     // ------------------------------------------------------------------ issuer of S
@@ -400,7 +400,7 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
       if (last) mma_commit_elect(bar(FB_Q_EMPTY));                              // ... Q at the item's
     }
     if (!ok) *abort_flag = 1;
-    pdl_wait();
+    pdl_begin(beside);
   } else if (warp >= FL_PV_WARP) {
     // ------------------------------------------------------------------ issuers of O_g += P_g V
     const int g = warp - FL_PV_WARP;
@@ -446,10 +446,10 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
       if (done) mma_commit_elect(bar(FB_KV_EMPTY + slot));
     }
     if (!ok) *abort_flag = 1;
-    pdl_wait();
+    pdl_begin(beside);
   } else {
     // ------------------------------------------------------------------ softmax (warps 0 .. 7)
-    pdl_wait();
+    pdl_begin(beside);
     // (HALF: warps w and w + 4 share the rows of the one tile, 32 of a step's 64 columns each)
     const int half = HALF ? warp >> 2 : 0, g = HALF ? 0 : warp >> 2, quarter = warp & 3, row = quarter * 32 + lane;
     constexpr int NC = HALF ? FL_STEP / 2 : FL_STEP;                // columns of a step that this warp works on
@@ -673,6 +673,7 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
   }
   tc_fence_before();
   __syncthreads();
+  pdl_end(beside);
   if (warp == FL_S_WARP) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
@@ -680,32 +681,32 @@ attn_flash_kernel(const Group* __restrict__ groups, int n_groups, int total_item
 }
 
 template <int HD, bool PAGED, bool HALF, class Group, class View>
-cudaError_t launch_flash_as(const Group* groups, int n_groups, int total_items, int mt, int* status, int sm_count, cudaStream_t st) {
+cudaError_t launch_flash_as(const Group* groups, int n_groups, int total_items, int mt, int* status, int sm_count, cudaStream_t st, int beside) {
   const auto kernel = attn_flash_kernel<HD, PAGED, HALF, Group, View>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FlashGeo<HD>::SMEM);
   if (e != cudaSuccess) return e;
   const int grid = total_items < sm_count ? total_items : sm_count;
-  return launch_pdl(kernel, dim3(grid), dim3(FL_THREADS), FlashGeo<HD>::SMEM, st, groups, n_groups, total_items, mt, status);
+  return launch_pdl(kernel, dim3(grid), dim3(FL_THREADS), FlashGeo<HD>::SMEM, st, groups, n_groups, total_items, mt, status, beside);
 }
 
 template <int HD, bool PAGED, class Group, class View>
-cudaError_t launch_flash(const Group* groups, int n_groups, int total_items, int mt, int* status, int sm_count, cudaStream_t st) {
+cudaError_t launch_flash(const Group* groups, int n_groups, int total_items, int mt, int* status, int sm_count, cudaStream_t st, int beside) {
   if (n_groups == 0 || total_items == 0) return cudaSuccess;
-  return mt == 1 ? launch_flash_as<HD, PAGED, true, Group, View>(groups, n_groups, total_items, mt, status, sm_count, st)
-                 : launch_flash_as<HD, PAGED, false, Group, View>(groups, n_groups, total_items, mt, status, sm_count, st);
+  return mt == 1 ? launch_flash_as<HD, PAGED, true, Group, View>(groups, n_groups, total_items, mt, status, sm_count, st, beside)
+                 : launch_flash_as<HD, PAGED, false, Group, View>(groups, n_groups, total_items, mt, status, sm_count, st, beside);
 }
 
 }  // namespace
 
 cudaError_t launch_attn_encoder_tc(const AttnEncGroup* groups, int n_groups, int total_items, int mt, int* status, int sm_count,
-                                   cudaStream_t st) {
-  return launch_flash<64, false, AttnEncGroup, EncView>(groups, n_groups, total_items, mt, status, sm_count, st);
+                                   cudaStream_t st, int beside) {
+  return launch_flash<64, false, AttnEncGroup, EncView>(groups, n_groups, total_items, mt, status, sm_count, st, beside);
 }
 
 cudaError_t launch_attn_prefill(const AttnPrefillGroup* groups, int n_groups, int total_items, int mt, int hd, int* status,
-                                int sm_count, cudaStream_t st) {
-  if (hd == 64) return launch_flash<64, true, AttnPrefillGroup, PreView>(groups, n_groups, total_items, mt, status, sm_count, st);
-  if (hd == 128) return launch_flash<128, true, AttnPrefillGroup, PreView>(groups, n_groups, total_items, mt, status, sm_count, st);
+                                int sm_count, cudaStream_t st, int beside) {
+  if (hd == 64) return launch_flash<64, true, AttnPrefillGroup, PreView>(groups, n_groups, total_items, mt, status, sm_count, st, beside);
+  if (hd == 128) return launch_flash<128, true, AttnPrefillGroup, PreView>(groups, n_groups, total_items, mt, status, sm_count, st, beside);
   return cudaErrorInvalidValue;
 }
 

@@ -95,19 +95,10 @@ struct AttnReq {
   int row;               // activation row of the request's token (q is read and the output written there)
 };
 
-// A cache page that the step appends to: `n` token rows from `row` on, at positions from `pos` on.
+// A cache page that a decode request of the step appends to, at position `pos`, from token row `row`.
 struct WrittenPage {
   const int32_t* id;     // where the caller's block table holds the page's id
-  int pos;
-  int row_n;             // 32 * row + n
-#ifdef __CUDACC__
-  __host__ __device__
-#endif
-  int row() const { return row_n >> 5; }
-#ifdef __CUDACC__
-  __host__ __device__
-#endif
-  int n() const { return row_n & 31; }
+  int pos, row;
 };
 
 // LINK: finds the decode requests that attend to tokens which other requests of the step append (see AttnDecGroup::linked).
@@ -116,7 +107,7 @@ struct GatherGroup {
   const ReqDesc* reqs;
   const RowDesc* rows;   // EMB: one entry per output row
   const AttnReq* areqs;  // LINK: the decode requests, one block each
-  const WrittenPage* written;   // LINK: the decode requests' pages, in their order, then those of the prompt chunks; B counts them
+  const WrittenPage* written;   // LINK: the decode requests' pages, in their order; B counts them
   void* out;             // ROWS: bf16 [B, ld]; EMB: fp32 [rows, d]; PATCH: bf16 [B*np, 3*p*p]; LINK: int [decode requests]
   const bf16* emb;       // EMB
   int kind, B, width, ld;

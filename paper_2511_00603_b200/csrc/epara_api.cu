@@ -175,6 +175,7 @@ struct Launch {
   size_t off;
   int n_groups;
   int p0, p1, p2, p3;
+  int beside;        // runs beside the launch before it (see pdl_begin())
   const void* src;   // EPARA_K_TRACE
   void* dst;
   size_t bytes;
@@ -517,6 +518,12 @@ int build_model(Builder& bl, Model* m, const epara_config& cfg) {
     r.rope.Hq = Hq; r.rope.Hkv = Hkv; r.rope.hd = hd; r.rope.kv_pages = d.kv_pages;
     r.rope.only_chunks = hd >= 64;           // (the tensor-core decode attention rotates and appends its rows itself)
     m->ops.push_back(r);
+    Op ap;                                   // causal attention of the step's prompt chunks (none in a pure decode step)
+    memset(&ap, 0, sizeof(ap));
+    ap.kind = EPARA_K_ATTN_PREFILL; ap.rows_per_req = 1;
+    ap.apre.out = a; ap.apre.kv_pages = d.kv_pages; ap.apre.Hq = Hq; ap.apre.Hkv = Hkv; ap.apre.hd = hd;
+    ap.apre.kv_row0 = (int)(layer_rows * l); ap.apre.kv_rows = (int)(layer_rows * d.n_layers);
+    m->ops.push_back(ap);
     Op at;
     memset(&at, 0, sizeof(at));
     at.kind = EPARA_K_ATTN_DEC; at.rows_per_req = 1;
@@ -526,12 +533,6 @@ int build_model(Builder& bl, Model* m, const epara_config& cfg) {
     at.adec.reqs_stable = 1; at.adec.kv_pages = d.kv_pages;
     if (r.rope.only_chunks) at.adec.cs = rope_cs;
     m->ops.push_back(at);
-    Op ap;                                   // causal attention of the step's prompt chunks (none in a pure decode step)
-    memset(&ap, 0, sizeof(ap));
-    ap.kind = EPARA_K_ATTN_PREFILL; ap.rows_per_req = 1;
-    ap.apre.out = a; ap.apre.kv_pages = d.kv_pages; ap.apre.Hq = Hq; ap.apre.Hkv = Hkv; ap.apre.hd = hd;
-    ap.apre.kv_row0 = (int)(layer_rows * l); ap.apre.kv_rows = (int)(layer_rows * d.n_layers);
-    m->ops.push_back(ap);
     if (!add_gemm(bl, m, a, Hq * hd, Bcap, w[2], dm, Hq * hd, x, dm, nullptr, EPI_RESID_F32, 1)) return EPARA_E_CUDA;
     add_norm(m, x, dm, h, w[3], nullptr, dm, NORM_RMS, 1e-5f, 1);
     if (!add_gemm(bl, m, h, dm, Bcap, w[4], 2 * F, dm, f, F, nullptr, EPI_SWIGLU, 1)) return EPARA_E_CUDA;
@@ -911,6 +912,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
     return at;
   };
   bool overflow = false;
+  long long dec_blocks = 0;                    // blocks of the step's decode attention (a layer)
   for (Active& a : act) {
     const bool dec = a.m->d.kind == EPARA_MODEL_DECODER;
     std::vector<ReqDesc> rd(a.B);
@@ -937,7 +939,9 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
           AttnReq q1;
           q1.table = in.block_table; q1.len = in.kv_len + 1; q1.row = row;
           ar.push_back(q1);
-          a.max_chunks_dec = std::max(a.max_chunks_dec, (in.kv_len + 1 + ATTN_CHUNK - 1) / ATTN_CHUNK);
+          const int chunks = (in.kv_len + 1 + ATTN_CHUNK - 1) / ATTN_CHUNK;
+          a.max_chunks_dec = std::max(a.max_chunks_dec, chunks);
+          dec_blocks += (long long)chunks * a.m->d.n_kv_heads;
         } else {
           pr.push_back({in.block_table, row, nt, in.kv_len});
           inf.prefill_tokens += nt;
@@ -955,18 +959,15 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       a.row_off = put(rows.data(), rows.size() * sizeof(RowDesc), 16);
       a.last_off = put(last.data(), last.size() * sizeof(int), 16);
       if (!ar.empty()) a.areq_off = put(ar.data(), ar.size() * sizeof(AttnReq), 16);
-      // several requests: each may attend to tokens that others append (AttnDecGroup::linked)
-      if (!ar.empty() && a.B > 1 && a.m->d.head_dim >= 64) {
+      // Prompt chunks beside decode requests: the RoPE launch, which the chunks need, appends the decode rows too, so that both
+      // attentions find the cache complete and can run side by side.
+      a.append_first = !ar.empty() && !pr.empty();
+      // several decode requests: each may attend to tokens that others append (AttnDecGroup::linked)
+      if (ar.size() > 1 && pr.empty() && a.m->d.head_dim >= 64) {
         const std::vector<int> none(ar.size(), 0);
         a.link_off = put(none.data(), none.size() * sizeof(int), 16);
         std::vector<WrittenPage> written;
-        for (const AttnReq& q : ar) written.push_back({q.table + (q.len - 1) / EPARA_KV_PAGE, q.len - 1, 32 * q.row + 1});
-        for (const PrefillChunk& p : pr)
-          for (int t = 0, n; t < p.n_tok; t += n) {
-            const int pos = p.kv_len + t;
-            n = std::min(p.n_tok - t, EPARA_KV_PAGE - pos % EPARA_KV_PAGE);
-            written.push_back({p.table + pos / EPARA_KV_PAGE, pos, 32 * (p.row_start + t) + n});
-          }
+        for (const AttnReq& q : ar) written.push_back({q.table + (q.len - 1) / EPARA_KV_PAGE, q.len - 1, q.row});
         a.n_written = (int)written.size();
         a.written_off = put(written.data(), written.size() * sizeof(written[0]), 16);
       }
@@ -994,7 +995,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
     for (const Active& a : act)
       if (a.n_pre > 0 && a.m->d.head_dim == (hi ? 128 : 64))
         for (const PrefillChunk& p : a.pre) tiles += (long long)((p.n_tok + FLASH_TILE - 1) / FLASH_TILE) * a.m->d.n_heads;
-    pre_mt[hi] = attn_flash_tiles(tiles, c->sm_count);
+    pre_mt[hi] = attn_flash_tiles(tiles, c->sm_count, dec_blocks);
   }
   for (Active& a : act) {
     if (a.n_pre == 0 || overflow) continue;
@@ -1020,11 +1021,15 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
 
   // ---- plan (A1): sweep the kernel kinds until every model's op list is exhausted ----
   static const int sweep[] = {EPARA_K_GATHER, EPARA_K_TRACE, EPARA_K_ASSEMBLE, EPARA_K_NORM, EPARA_K_GEMM, EPARA_K_ROPE,
-                              EPARA_K_ATTN_DEC, EPARA_K_ATTN_PREFILL, EPARA_K_ATTN_ENC, EPARA_K_OUTPUT};
+                              EPARA_K_ATTN_PREFILL, EPARA_K_ATTN_ENC, EPARA_K_ATTN_DEC, EPARA_K_OUTPUT};
   std::vector<Launch> launches;
   bool more = true;
   while (more && !overflow) {
     more = false;
+    // A sweep's attention launches do not depend on one another (a step's keys and values that another of its launches reads are
+    // appended before), nor do its GEMM launches: all but the first of either run beside the one before.  Order: what holds
+    // whole SMs first, the decode attention's small blocks fill the SMs that it leaves.
+    int attn_launches = 0, gemm_launches = 0;
     for (int kind : sweep) {
       std::vector<Active*> who;
       for (Active& a : act)
@@ -1129,7 +1134,8 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
           }
           LL.n_groups = n_put;
           LL.p0 = total_B; LL.p1 = max_hkv | (max_hq << 16); LL.p2 = max_chunks; LL.p3 = (hd << 8) | G;
-          if (n_put > 0) launches.push_back(LL);
+          LL.beside = attn_launches > 0;
+          if (n_put > 0) { launches.push_back(LL); ++attn_launches; }
           rest.swap(other);
         }
         for (Active* a : who) a->cursor++;
@@ -1156,7 +1162,8 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
             if (put(&g, sizeof(g), 8) == (size_t)-1) overflow = true;
           }
           LL.n_groups = n_put; LL.p0 = items; LL.p1 = hd; LL.p2 = pre_mt[hd == 128 ? 1 : 0];
-          if (n_put > 0) launches.push_back(LL);
+          LL.beside = attn_launches > 0;
+          if (n_put > 0) { launches.push_back(LL); ++attn_launches; }
         }
         for (Active* a : who) a->cursor++;
         continue;
@@ -1298,6 +1305,8 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
         L.n_groups = n_put;
         if (n_put == 0) continue;
       }
+      if (kind == EPARA_K_ATTN_ENC) L.beside = attn_launches++ > 0;
+      if (kind == EPARA_K_GEMM) L.beside = gemm_launches++ > 0;
       launches.push_back(L);
       if (cut) {
         const Op& op = cut->m->ops[pass == n_pass - 1 ? cut->cursor - 1 : cut->cursor];
@@ -1309,6 +1318,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
           Launch R;
           memset(&R, 0, sizeof(R));
           R.kind = kind; R.n_groups = 1; R.p0 = cut_tiles * g.tiles_n; R.p2 = 2;
+          R.beside = part == &op.fc1;              // (other rows than the fused launch; the second GEMM needs the first)
           off = align_up(off, TMAP_ALIGN);
           R.off = off;
           if (put(&g, sizeof(g), TMAP_ALIGN) == (size_t)-1) overflow = true;
@@ -1354,25 +1364,25 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       case EPARA_K_ASSEMBLE: launch_assemble((const AssembleGroup*)gp, L.n_groups, L.p1, st); break;
       case EPARA_K_NORM: launch_norm((const NormGroup*)gp, L.n_groups, L.p1, st); break;
       case EPARA_K_GEMM:
-        if (L.p2 == PASS_MLP) err = launch_gemm_mlp_pair((const MlpGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st);
-        else if (L.p2 >= PASS_SWAP) err = launch_gemm_swap((const GemmGroup*)gp, L.n_groups, L.p0, 1 << (L.p2 - PASS_SWAP), L.p3, dev_status, c->sm_count, st);
+        if (L.p2 == PASS_MLP) err = launch_gemm_mlp_pair((const MlpGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st, L.beside);
+        else if (L.p2 >= PASS_SWAP) err = launch_gemm_swap((const GemmGroup*)gp, L.n_groups, L.p0, 1 << (L.p2 - PASS_SWAP), L.p3, dev_status, c->sm_count, st, L.beside);
         else if (L.p2 == 1) err = launch_gemm_stream((const GemmGroup*)gp, L.n_groups, L.p0, L.p1, st);
-        else if (L.p2 == 2) err = launch_gemm_tc_pair((const GemmGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st);
+        else if (L.p2 == 2) err = launch_gemm_tc_pair((const GemmGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st, L.beside);
         else launch_gemm_simt((const GemmGroup*)gp, L.n_groups, L.p0, st);
         break;
       case EPARA_K_ROPE: launch_rope_append((const RopeGroup*)gp, L.n_groups, L.p1, st); break;
       case EPARA_K_ATTN_DEC:
         err = launch_attn_decode((const AttnDecGroup*)gp, L.n_groups, L.p0, L.p1 & 0xffff, L.p1 >> 16, L.p2, L.p3 >> 8,
-                                 L.p3 & 255, attn_decode_fused(L.p0, L.p1 & 0xffff, L.p2, L.p3 >> 8, c->sm_count) ? 1 : 0, st);
+                                 L.p3 & 255, attn_decode_fused(L.p0, L.p1 & 0xffff, L.p2, L.p3 >> 8, c->sm_count) ? 1 : 0, st, L.beside);
         break;
       case EPARA_K_ATTN_ENC:
-        if (L.p2 == 0) err = launch_attn_encoder_tc((const AttnEncGroup*)gp, L.n_groups, L.p0, L.p3, dev_status, c->sm_count, st);
+        if (L.p2 == 0) err = launch_attn_encoder_tc((const AttnEncGroup*)gp, L.n_groups, L.p0, L.p3, dev_status, c->sm_count, st, L.beside);
         else err = launch_attn_encoder((const AttnEncGroup*)gp, L.n_groups, L.p0, L.p1, st);
         break;
       case EPARA_K_OUTPUT: launch_output((const OutputGroup*)gp, L.n_groups, L.p1, st); break;
       case EPARA_K_TRACE: err = cudaMemcpyAsync(L.dst, L.src, L.bytes, cudaMemcpyDeviceToDevice, st); break;
       case EPARA_K_ATTN_PREFILL:
-        err = launch_attn_prefill((const AttnPrefillGroup*)gp, L.n_groups, L.p0, L.p2, L.p1, dev_status, c->sm_count, st);
+        err = launch_attn_prefill((const AttnPrefillGroup*)gp, L.n_groups, L.p0, L.p2, L.p1, dev_status, c->sm_count, st, L.beside);
         break;
     }
     if (prof) cudaEventRecord(slot.prof[2 * li + 1], st);

@@ -63,7 +63,9 @@ __device__ __forceinline__ int find_group_sw(const GemmGroup* groups, int n, int
 }
 
 // S: CTAs per cluster = k ranges per tile.  One cluster per (group, tile of 128 output columns, tile of nb rows).
-template <int S>
+// BESIDE: runs beside the launch before it (see pdl_begin(); the residual then comes past L1.  A run-time switch cost 6 us of 1195 in
+// a step of 27 requests through the 1B decoder).
+template <int S, bool BESIDE>
 __global__ void __launch_bounds__(SW_THREADS, 2)
 gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __restrict__ status, int ring_bytes) {
   extern __shared__ unsigned char smem_dyn[];
@@ -146,7 +148,7 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
       tma_load_2d_elect(w_base + stage * SW_W_BYTES, &g->tmW, kb * TC_BK, n0, wfull_bar(stage));
       if (++stage == w_stages) { stage = 0; phase ^= 1u; }
     }
-    pdl_wait();                                    // (every thread of the kernel waits once, see common.cuh)
+    pdl_begin(BESIDE);                                    // (every thread of the kernel waits once, see common.cuh)
     if (!ok) { *abort_flag = 1; drain_sleep(200000ull); }
   } else if (warp == SW_A_WARP) {
     // ------------------------------------------------------------ TMA producer of the activations (tmA: box of nb rows)
@@ -154,7 +156,7 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
     // the first copy after the wait finds its map (1B decoder, 27 requests: 1226 -> 1210 us a step; the larger tiles of the
     // tile-pair kernel and attention gained nothing)
     tensormap_prefetch_elect(&g->tmA);
-    pdl_wait();
+    pdl_begin(BESIDE);
     int stage = 0;
     uint32_t phase = 0;
     bool ok = true;
@@ -191,7 +193,7 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
     else if (!empty) mma_commit_elect(tfull_bar);
   } else {
     // ------------------------------------------------------------ wait for this CTA's accumulator (warps 2..9)
-    pdl_wait();
+    pdl_begin(BESIDE);
     acc_ok = empty || mbar_wait(tfull_bar, 0u, abort_flag);
     if (!acc_ok) {
       if (lane == 0) atomicExch(status, 43);
@@ -260,8 +262,8 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
         old[u] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (resid && l < nrows && some) {
           const float* cf = reinterpret_cast<const float*>(Cptr) + (size_t)(m0 + r0 + l) * ldc + n;
-          if (full) old[u] = *reinterpret_cast<const float4*>(cf);
-          else { old[u].x = cf[0]; if (n + 1 < N) old[u].y = cf[1]; if (n + 2 < N) old[u].z = cf[2]; }
+          if (full) old[u] = BESIDE ? __ldcg(reinterpret_cast<const float4*>(cf)) : *reinterpret_cast<const float4*>(cf);
+          else { old[u].x = BESIDE ? __ldcg(cf) : cf[0]; if (n + 1 < N) old[u].y = BESIDE ? __ldcg(cf + 1) : cf[1]; if (n + 2 < N) old[u].z = BESIDE ? __ldcg(cf + 2) : cf[2]; }
         }
       }
       // (rows past the live ones read stale shared memory and are not stored: the U rows stay one straight piece of code)
@@ -316,6 +318,7 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
     }
   }
   // (after the barrier above nobody touches another CTA's shared memory, so the CTAs may leave one by one)
+  pdl_end(BESIDE);
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -325,8 +328,9 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
 }
 
 template <int S>
-cudaError_t launch_swap(const GemmGroup* groups, int n_groups, int total_items, int max_nb, int* status, int sm_count, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(gemm_swap_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw_smem(SW_RING_BYTES_1));
+cudaError_t launch_swap(const GemmGroup* groups, int n_groups, int total_items, int max_nb, int* status, int sm_count, cudaStream_t st, int beside) {
+  const auto kernel = beside ? gemm_swap_kernel<S, true> : gemm_swap_kernel<S, false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw_smem(SW_RING_BYTES_1));
   if (e != cudaSuccess) return e;
   // Tiles of more than 128 rows need the large ring (the reduction lands nb x 512 bytes in it).
   // (clusters of eight one-SM CTAs were slow to place: 25.8 us against 15.4 with two CTAs per SM, 2048 x 8192 at 128 rows)
@@ -345,7 +349,7 @@ cudaError_t launch_swap(const GemmGroup* groups, int n_groups, int total_items, 
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, gemm_swap_kernel<S>, groups, n_groups, status, ring_bytes);
+  return cudaLaunchKernelEx(&cfg, kernel, groups, n_groups, status, ring_bytes);
 }
 
 }  // namespace
@@ -390,13 +394,13 @@ bool gemm_swap_eligible(long long rows_cap, int N, int K, int epi, int sm_count)
 int gemm_swap_tiles_n(int N) { return (N + SW_BM - 1) / SW_BM; }
 
 cudaError_t launch_gemm_swap(const GemmGroup* groups, int n_groups, int total_items, int ksplit, int max_nb, int* status,
-                             int sm_count, cudaStream_t st) {
+                             int sm_count, cudaStream_t st, int beside) {
   if (n_groups == 0 || total_items == 0) return cudaSuccess;
   switch (ksplit) {
-    case 1: return launch_swap<1>(groups, n_groups, total_items, max_nb, status, sm_count, st);
-    case 2: return launch_swap<2>(groups, n_groups, total_items, max_nb, status, sm_count, st);
-    case 4: return launch_swap<4>(groups, n_groups, total_items, max_nb, status, sm_count, st);
-    case 8: return launch_swap<8>(groups, n_groups, total_items, max_nb, status, sm_count, st);
+    case 1: return launch_swap<1>(groups, n_groups, total_items, max_nb, status, sm_count, st, beside);
+    case 2: return launch_swap<2>(groups, n_groups, total_items, max_nb, status, sm_count, st, beside);
+    case 4: return launch_swap<4>(groups, n_groups, total_items, max_nb, status, sm_count, st, beside);
+    case 8: return launch_swap<8>(groups, n_groups, total_items, max_nb, status, sm_count, st, beside);
   }
   return cudaErrorInvalidValue;
 }

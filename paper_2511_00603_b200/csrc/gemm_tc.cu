@@ -202,7 +202,7 @@ constexpr int PAIR_W_WARP = 2 + EPI_WARPS;                     // the warp after
 constexpr int PAIR_THREADS = N_THREADS + 32;
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PAIR_THREADS, 1)
-gemm_tc_pair_kernel(const GemmGroup* __restrict__ groups, int n_groups, int total_items, int* __restrict__ status) {
+gemm_tc_pair_kernel(const GemmGroup* __restrict__ groups, int n_groups, int total_items, int* __restrict__ status, int beside) {
   extern __shared__ unsigned char smem_dyn[];
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   unsigned char* base_ptr = smem_dyn + (base - smem_u32(smem_dyn));
@@ -249,7 +249,7 @@ gemm_tc_pair_kernel(const GemmGroup* __restrict__ groups, int n_groups, int tota
       tensormap_acquire(&gc.g->tmA);
       g_prev = gc.g;
     }
-    pdl_wait();
+    pdl_begin(beside);
     for (int item = pair; item < total_items && ok; item += n_pairs) {
       group_cache(gc, groups, n_groups, item);
       const GemmGroup* g = gc.g;
@@ -324,7 +324,7 @@ gemm_tc_pair_kernel(const GemmGroup* __restrict__ groups, int n_groups, int tota
       // ---------------------------------------------------------- L2 prefetch of residual tiles
       // The fp32 residual of both CTAs' rows is added to at L2 by the epilogue's reduce stores: this otherwise idle
       // warp asks for those lines ahead of time so that the additions do not wait on HBM.
-      pdl_wait();
+      pdl_begin(beside);
       for (int item = pair; item < total_items; item += n_pairs) {
         const GemmGroup& g = groups[find_group_tc(groups, n_groups, item)];
         if (!(g.epi & EPI_RESID_F32)) continue;
@@ -339,7 +339,7 @@ gemm_tc_pair_kernel(const GemmGroup* __restrict__ groups, int n_groups, int tota
     }
   } else {
     // ------------------------------------------------------------ epilogue (warps 2..17 of both CTAs)
-    pdl_wait();
+    pdl_begin(beside);
     const int ew = warp - 2;
     const int quarter = warp & 3;
     const int part = ew >> 2;
@@ -386,6 +386,7 @@ gemm_tc_pair_kernel(const GemmGroup* __restrict__ groups, int n_groups, int tota
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();                        // neither CTA leaves while the other may still read its operands or signal it
+  pdl_end(beside);
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)TMEM_COLS) : "memory");
@@ -460,7 +461,7 @@ __device__ __forceinline__ void mlp_geo(MlpGeo& c, const MlpGroup* groups, int n
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MLP_THREADS, 1)
-gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int total_items, int* __restrict__ status) {
+gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int total_items, int* __restrict__ status, int beside) {
   extern __shared__ unsigned char smem_dyn[];
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   unsigned char* base_ptr = smem_dyn + (base - smem_u32(smem_dyn));
@@ -508,7 +509,7 @@ gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int tota
       if (g != g_prev) { tensormap_acquire(&g->tmX); tensormap_acquire(&g->tmW1); g_prev = g; }
       const int m0 = (item - gc.start) * (2 * TC_BM) + rank * TC_BM;
       if (!mbar_wait(bar(MB_X_EMPTY), (t & 1u) ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 41); break; }
-      if (!waited) { pdl_wait(); waited = true; }   // h is written by the kernel before this one
+      if (!waited) { pdl_begin(beside); waited = true; }   // h is written by the kernel before this one
       if (rank == 0) mbar_expect_tx_elect(bar(MB_X_FULL), 2u * (uint32_t)gc.kb1 * A_BYTES);
       for (int kb = 0; kb < gc.kb1; ++kb)
         tma_load_2d_pair_elect(base + kb * A_BYTES, &g->tmX, kb * TC_BK, m0, mapa_shared(bar(MB_X_FULL), 0));
@@ -622,7 +623,7 @@ gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int tota
     }
   } else {
     // ------------------------------------------------------------ epilogue warps (2..17 of both CTAs)
-    pdl_wait();
+    pdl_begin(beside);
     const int ew = warp - 2;
     const int quarter = warp & 3;
     const int part = ew >> 2;
@@ -749,6 +750,7 @@ gemm_mlp_pair_kernel(const MlpGroup* __restrict__ groups, int n_groups, int tota
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();                        // neither CTA leaves while the other may still read its operands or signal it
+  pdl_end(beside);
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)TMEM_COLS) : "memory");
@@ -781,12 +783,12 @@ double gemm_pair_config(long long rows_cap, int N, int K, int epi, int sm_count,
 }
 
 cudaError_t launch_gemm_tc_pair(const GemmGroup* groups, int n_groups, int total_items, int* status, int sm_count,
-                                cudaStream_t st) {
+                                cudaStream_t st, int beside) {
   if (n_groups == 0 || total_items == 0) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(gemm_tc_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
   if (e != cudaSuccess) return e;
   const int pairs = total_items < sm_count / 2 ? total_items : sm_count / 2;
-  return launch_pdl(gemm_tc_pair_kernel, dim3(2 * pairs), dim3(PAIR_THREADS), SMEM_BYTES, st, groups, n_groups, total_items, status);
+  return launch_pdl(gemm_tc_pair_kernel, dim3(2 * pairs), dim3(PAIR_THREADS), SMEM_BYTES, st, groups, n_groups, total_items, status, beside);
 }
 
 // The fused MLP kernel takes an encoder block when its accumulators fit the tensor memory (d <= 384 beside one
@@ -796,12 +798,12 @@ bool gemm_mlp_eligible(long long rows_cap, int d, int F) {
 }
 
 cudaError_t launch_gemm_mlp_pair(const MlpGroup* groups, int n_groups, int total_items, int* status, int sm_count,
-                                 cudaStream_t st) {
+                                 cudaStream_t st, int beside) {
   if (n_groups == 0 || total_items == 0) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(gemm_mlp_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MLP_SMEM_BYTES);
   if (e != cudaSuccess) return e;
   const int pairs = total_items < sm_count / 2 ? total_items : sm_count / 2;
-  return launch_pdl(gemm_mlp_pair_kernel, dim3(2 * pairs), dim3(MLP_THREADS), MLP_SMEM_BYTES, st, groups, n_groups, total_items, status);
+  return launch_pdl(gemm_mlp_pair_kernel, dim3(2 * pairs), dim3(MLP_THREADS), MLP_SMEM_BYTES, st, groups, n_groups, total_items, status, beside);
 }
 
 }  // namespace epara

@@ -5,6 +5,8 @@
 
 namespace epara {
 
+// (beside: see pdl_begin() in common.cuh)
+
 constexpr int GATHER_PATCH_ROWS = 8;   // patch rows per block of the patch gather
 void launch_gather(const GatherGroup* groups, int n_groups, int max_blocks, cudaStream_t st);
 int norm_blocks(int M, int d);
@@ -25,10 +27,10 @@ constexpr int TC_BN_MAX = 256;
 constexpr int TC_BK = 64;
 double gemm_pair_config(long long rows_cap, int N, int K, int epi, int sm_count, int* bn);
 cudaError_t launch_gemm_tc_pair(const GemmGroup* groups, int n_groups, int total_items, int* status, int sm_count,
-                                cudaStream_t st);
+                                cudaStream_t st, int beside = 0);
 bool gemm_mlp_eligible(long long rows_cap, int d, int F);
 cudaError_t launch_gemm_mlp_pair(const MlpGroup* groups, int n_groups, int total_items, int* status, int sm_count,
-                                 cudaStream_t st);
+                                 cudaStream_t st, int beside = 0);
 
 // Swapped-operand tensor-core GEMM (GemmGroup::stream == 3): a cluster of `ksplit` CTAs per tile of 128 output
 // columns and bn batch rows; all groups of a launch share ksplit.  gemm_swap_config() picks bn (a multiple of 16, at
@@ -40,7 +42,7 @@ double gemm_swap_config(long long rows_cap, int N, int K, int sm_count, int* nb,
 bool gemm_swap_eligible(long long rows_cap, int N, int K, int epi, int sm_count);
 int gemm_swap_tiles_n(int N);
 cudaError_t launch_gemm_swap(const GemmGroup* groups, int n_groups, int total_items, int ksplit, int max_nb, int* status,
-                             int sm_count, cudaStream_t st);
+                             int sm_count, cudaStream_t st, int beside = 0);
 
 // Weight-streaming GEMM (GemmGroup::stream == 1) for groups that never exceed 16 rows, and for small matrices: one block
 // per 16 rows of W over the whole K and 32 batch rows, mma.sync, no tensor maps.  total_items = sum of
@@ -58,7 +60,7 @@ cudaError_t launch_gemm_stream(const GemmGroup* groups, int n_groups, int total_
 constexpr int ATTN_CHUNK = 256;
 bool attn_decode_fused(int total_B, int max_Hkv, int max_chunks, int hd, int sm_count);
 cudaError_t launch_attn_decode(const AttnDecGroup* groups, int n_groups, int total_B, int max_Hkv, int max_Hq,
-                               int max_chunks, int hd, int gqa, int fused, cudaStream_t st);
+                               int max_chunks, int hd, int gqa, int fused, cudaStream_t st, int beside = 0);
 // Set-up of a single-kernel decode-attention call on the stream: writes `g` to `dst`, clears *g.status and
 // g.counters[0 .. n_counters), fills reqs[b] = {tables + b*stride, kv_lens[b] clamped to [0, max_len]}.
 void launch_attn_prepare(const AttnDecGroup& g, AttnDecGroup* dst, AttnReq* reqs, const int32_t* kv_lens,
@@ -69,13 +71,20 @@ constexpr int DEC_STATUS_OFFSET = 192;   // byte offset of the status word in a 
 // `status` as for the GEMM.  Two tiles keep the tensor core and the softmax busy at once; attn_flash_tiles() picks one
 // when the launch's tiles do not outnumber the SMs.
 constexpr int FLASH_TILE = 128;
-inline int attn_flash_tiles(long long total_tiles, int sm_count) { return total_tiles <= sm_count ? 1 : 2; }
+// With decode attention beside it the launch also leaves SMs to that one's blocks: one tile keeps the launch short while they
+// are few, two tiles leave more SMs (1B decoder, a 512-token chunk, 128 tiles: with 4 / 12 / 24 / 60 decode requests, 14 / 42 /
+// 84 / 210 blocks per SM left over, 2306 / 2409 / 2560 / 2818 us a step with one tile and 2467 / 2485 / 2525 / 2779 with two; a
+// 256-token chunk with 24 / 60 requests, 20 / 50 blocks: 1822 / 2271 and 1955 / 2236).
+constexpr int FLASH_DEC_BLOCKS = 48;
+inline int attn_flash_tiles(long long total_tiles, int sm_count, long long dec_blocks = 0) {
+  return total_tiles <= sm_count && dec_blocks <= FLASH_DEC_BLOCKS * (sm_count - total_tiles) ? 1 : 2;
+}
 // ... causal attention of prompt chunks (head size 64 or 128)
 cudaError_t launch_attn_prefill(const AttnPrefillGroup* groups, int n_groups, int total_items, int mt, int hd, int* status,
-                                int sm_count, cudaStream_t st);
+                                int sm_count, cudaStream_t st, int beside = 0);
 // ... encoder attention for groups with AttnEncGroup::tc (hd 64); total_items = sum of B * H * q_blocks.
 cudaError_t launch_attn_encoder_tc(const AttnEncGroup* groups, int n_groups, int total_items, int mt, int* status, int sm_count,
-                                   cudaStream_t st);
+                                   cudaStream_t st, int beside = 0);
 
 // Encoder (bidirectional) attention on mma.sync, one block per (image, head, query block).
 cudaError_t launch_attn_encoder(const AttnEncGroup* groups, int n_groups, int total_blocks, int max_T,
