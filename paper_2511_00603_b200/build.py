@@ -7,6 +7,7 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -15,6 +16,7 @@ OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libepara.so")
 SOURCES = ["epara_api.cu", "kernels_misc.cu", "gemm_simt.cu", "gemm_tc.cu", "gemm_stream.cu", "gemm_swap.cu", "attention.cu", "attention_flash.cu", "policy.cu",
            "selftest.cu"]
+FAST_SRC, FAST_LIB = os.path.join(CSRC, "fastcall.cpp"), os.path.join(HERE, "_fastcall.so")   # Python side of epara_collect
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC"]
 
 
@@ -35,7 +37,19 @@ def _stale() -> bool:
     return _newer(LIB, [os.path.join(CSRC, s) for s in SOURCES] + _headers())
 
 
+def build_fastcall(force: bool = False) -> None:
+    """The binding works without it (through ctypes), so a machine without Python's headers goes without."""
+    include = sysconfig.get_paths()["include"]
+    if not os.path.exists(os.path.join(include, "Python.h")) or not (force or _newer(FAST_LIB, [FAST_SRC])):
+        return
+    r = subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-I", include, FAST_SRC, "-o", FAST_LIB],
+                       capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("fastcall.cpp:\n" + r.stdout + r.stderr)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_fastcall(force)
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

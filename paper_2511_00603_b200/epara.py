@@ -250,6 +250,7 @@ class Context:
         self._keep = [workspace]
         self.h = C.c_void_p()
         _check(lib.epara_init(C.byref(self.cfg), C.byref(self.h)), "epara_init")
+        self._handle = self.h.value
 
     def model_workspace_bytes(self, desc: ModelDesc) -> int:
         return lib.epara_model_workspace_bytes(C.byref(self.cfg), C.byref(desc))
@@ -298,12 +299,21 @@ class Context:
         if self.h:
             lib.epara_destroy(self.h)
             self.h = C.c_void_p()
+            self._handle = 0
 
     def __del__(self):
         try:
             self.close()
         except Exception:
             pass
+
+
+# The same method without a foreign-function call per answer (csrc/fastcall.cpp).
+try:
+    from . import _fastcall
+    Context.epara_collect = _fastcall.collect_method(C.cast(lib.epara_collect, C.c_void_p).value, Output, Context.epara_collect, "_handle")
+except ImportError:
+    pass
 
 
 # ----------------------------------------------------------------------------- single kernels

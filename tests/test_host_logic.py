@@ -111,3 +111,19 @@ def test_product_path_does_not_import_the_oracle():
                 assert not re.search(r"^\s*(from|import)\s+oracle|epara_oracle|oracle[/.]", txt, flags=re.M), f
     otxt = open(os.path.join(ROOT, "oracle", "epara_oracle.py")).read()
     assert "paper_2511_00603_b200" not in otxt and "ctypes" not in otxt
+
+
+def test_collect_method_without_ctypes_takes_what_the_general_one_takes(E):
+    """The binding's compiled epara_collect: positional, by keyword, ticket as a ctypes integer, wrong types; on a context without a
+    handle every form answers INVALID."""
+    class NoContext(E.Context):
+        def __init__(self):
+            self.h, self._handle = E.C.c_void_p(), 0
+    c = NoContext()
+    for s, out in (c.epara_collect(7), c.epara_collect(ticket=7), c.epara_collect(E.C.c_uint64(7)), c.epara_collect(2**64 - 1), c.epara_collect(-1),
+                   E.Context.epara_collect(c, 7)):
+        assert s == E.E_INVALID and isinstance(out, E.Output)
+    with pytest.raises(Exception):
+        c.epara_collect("7")
+    with pytest.raises(TypeError):
+        c.epara_collect()
