@@ -304,9 +304,9 @@ __global__ void __launch_bounds__(128) attn_decode_kernel(const AttnDecGroup* __
 // With AttnDecGroup::cs the kernel also does RoPE and the append for its request: q is rotated as it is
 // read, the block that holds position len - 1 rotates k, writes k and v to the cache and into its
 // staged tile, and the cached pages are requested before the wait on the QKV projection.  That takes a
-// launch out of every layer.  Requests of one sequence in one step (known tokens scored in one go, a token behind the
-// prompt chunk of the same step) attend to what the others append: the step's first kernel marks them (GATHER_LINK) and
-// they read those tokens out of qkv.
+// launch out of every layer.  Decode requests of one sequence in one step (known tokens scored in one go) attend
+// to what the others append: the step's first kernel marks them (GATHER_LINK) and they read those tokens out of qkv.  (In a step
+// that has prompt chunks too the RoPE launch appends everything and cs is null.)
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }

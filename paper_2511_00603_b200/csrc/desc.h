@@ -55,7 +55,7 @@ constexpr int TMAP_ALIGN = 128;
 struct alignas(TMAP_ALIGN) GemmGroup {
   CUtensorMap tmA;
   CUtensorMap tmW;
-  CUtensorMap tmC;   // output, written by TMA from the epilogue's staging rows: bf16 [rows, N] with a
+  CUtensorMap tmC;   // (swapped operands on pairs: the activations for a tile's second MMA)  output, written by TMA from the epilogue's staging rows: bf16 [rows, N] with a
                      // 32 x 32 box (SwiGLU: [rows, N/2], 16 x 32), or fp32 [rows, N] with a 16 x 32 box
                      // for the residual update (TMA reduce-add)
   const bf16* A;
@@ -72,7 +72,7 @@ struct alignas(TMAP_ALIGN) GemmGroup {
   int stream;      // 1: weight-streaming kernel (at most 16 rows ever, or a small matrix; 16 W rows per
                    // block, tiles_n = ceil(N / 16), no TMA maps); 2: 256-row tiles on CTA pairs (tiles_m counts 256-row
                    // tiles and tmW's box holds bn / 2 rows); 3: swapped operands (tmA's box holds bn rows, tmW's
-                   // 128); 0: plain CUDA-core comparator
+                   // 128); 5: swapped operands on CTA pairs (see kernels.h); 0: plain CUDA-core comparator
   const ReqDesc* reqs;   // weight-streaming kernel: when set, row m of A is request m's input (an MLP's first layer)
   int pad[4];
 };

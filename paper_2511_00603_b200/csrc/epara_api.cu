@@ -30,10 +30,14 @@ namespace {
 constexpr int N_SLOTS = 4;
 constexpr size_t BLOB_BYTES = 4u << 20;
 constexpr int MAX_PROFILE_LAUNCHES = 4096;
-constexpr int PASS_SWAP = 3, PASS_MLP = 7;   // launches of a GEMM wave (see epara_step); PASS_MLP is the last
-constexpr int N_SWAP = PASS_MLP - PASS_SWAP;  // swapped-operand launches: 1, 2, 4 or 8 k ranges per tile
+constexpr int PASS_SWAP = 3, PASS_SWAP2 = 7, PASS_MLP = 9;   // launches of a GEMM wave (see epara_step); PASS_MLP is the last
+constexpr int N_SWAP = PASS_SWAP2 - PASS_SWAP, N_SWAP2 = PASS_MLP - PASS_SWAP2;  // swapped-operand launches: 1, 2, 4 or 8 k ranges per tile
 
 inline int swap_index(int ksplit) { return ksplit >= 8 ? 3 : ksplit >= 4 ? 2 : ksplit >= 2 ? 1 : 0; }
+// The launch of a GEMM wave that takes a group.
+inline int gemm_pass(const GemmGroup& g) {
+  return g.stream == GEMM_SWAP ? PASS_SWAP + swap_index(g.ksplit) : g.stream == GEMM_SWAP2 ? PASS_SWAP2 + swap_index(g.ksplit) : g.stream == 4 ? PASS_MLP : g.stream;
+}
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 inline int round_up(int v, int a) { return (v + a - 1) / a * a; }
@@ -95,6 +99,21 @@ bool make_tmap_z(CUtensorMap* tm, void* Z, long long rows, int d) {
   cuuint32_t estr[2] = {1, 1};
   return fn(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, Z, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The TMA maps that a group's kernel wants; rows: of A and C.
+bool make_gemm_maps(GemmGroup& g, long long rows) {
+  if (g.stream == GEMM_SWAP)                    // W as the MMA's 128-row operand, the batch as its N
+    return make_tmap(&g.tmA, g.A, rows, g.K, g.lda, g.bn) && make_tmap(&g.tmW, g.W, g.N, g.K, g.ldw, TC_BM);
+  if (g.stream == GEMM_SWAP2) {                 // ... on pairs of CTAs: each loads half of an MMA's batch rows
+    const int nb1 = gemm_swap2_first(g.bn);
+    return make_tmap(&g.tmA, g.A, rows, g.K, g.lda, nb1 / 2) && make_tmap(&g.tmW, g.W, g.N, g.K, g.ldw, TC_BM) &&
+           (nb1 == g.bn || make_tmap(&g.tmC, g.A, rows, g.K, g.lda, (g.bn - nb1) / 2));
+  }
+  if (g.stream == GEMM_PAIR)                    // 256-row tiles on CTA pairs: a pair's CTA loads half of the W rows
+    return make_tmap(&g.tmA, g.A, rows, g.K, g.lda, TC_BM) && make_tmap(&g.tmW, g.W, g.N, g.K, g.ldw, g.bn / 2) &&
+           make_tmap_c(&g.tmC, g.C, rows, g.N, g.ldc, g.epi);
+  return true;
 }
 
 struct Op {
@@ -258,21 +277,13 @@ bool add_gemm(Builder& bl, Model* m, const void* A, int lda, long long rows_cap,
     g.stream = 0;
   } else if (!one_sum && gemm_stream_eligible(max_rows, N, K)) {
     g.stream = 1; g.bn = 16;
-  } else if (!one_sum && gemm_swap_eligible(max_rows, N, K, g.epi, sm_count)) {
-    g.stream = 3;                              // W as the MMA's 128-row operand, the batch as its N
-    gemm_swap_config(max_rows, N, K, sm_count, &g.bn, &g.ksplit);
-  } else {
-    g.stream = 2;                              // 256-row tiles on CTA pairs
+  } else if (one_sum) {
+    g.stream = GEMM_PAIR;
     gemm_pair_config(max_rows, N, K, g.epi, sm_count, &g.bn);
+  } else {
+    g.stream = gemm_tc_choice(max_rows, N, K, g.epi, sm_count, &g.bn, &g.ksplit);
   }
-  if (bl.c && g.stream == 3) {
-    if (!make_tmap(&g.tmA, A, rows_cap, K, lda, g.bn)) return false;
-    if (!make_tmap(&g.tmW, W, N, K, K, TC_BM)) return false;
-  } else if (bl.c && g.stream == 2) {
-    if (!make_tmap(&g.tmA, A, rows_cap, K, lda, TC_BM)) return false;
-    if (!make_tmap(&g.tmW, W, N, K, K, g.bn / 2)) return false;   // a pair's CTA loads half of the W rows
-    if (!make_tmap_c(&g.tmC, C, rows_cap, N, ldc, g.epi)) return false;
-  }
+  if (bl.c && !make_gemm_maps(g, rows_cap)) return false;
   g.c_rows = (int)rows_cap;
   m->ops.push_back(op);
   return true;
@@ -1058,15 +1069,14 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       // contexts only), the weight-streaming kernel for groups of few rows or small matrices (pass 1) and
       // 256-row tiles on CTA pairs (pass 2); encoder attention in two: the tcgen05 kernel (pass 0) and the
       // mma.sync kernel for shapes it does not take (pass 1)
-      // (passes 3 to 6: the swapped-operand kernel with 1, 2, 4 and 8 k ranges per tile)
-      // (pass 7: encoder MLP blocks in the fused kernel)
+      // (passes 3 to 6: the swapped-operand kernel with 1, 2, 4 and 8 k ranges per tile; 7 and 8: on pairs of CTAs, with 1 and 2)
+      // (pass 9: encoder MLP blocks in the fused kernel)
       const int n_pass = kind == EPARA_K_GEMM ? PASS_MLP + 1 : (kind == EPARA_K_ATTN_ENC ? 2 : 1);
       unsigned passes = ~0u;                                   // GEMM passes that some model needs
       if (kind == EPARA_K_GEMM) {
         passes = 1u << (n_pass - 1);                           // (the last pass also moves the cursors on)
         for (Active* a : who) {
-          const GemmGroup& g = a->m->ops[a->cursor].gemm;
-          passes |= 1u << (g.stream == 3 ? PASS_SWAP + swap_index(g.ksplit) : g.stream == 4 ? PASS_MLP : g.stream);
+          passes |= 1u << gemm_pass(a->m->ops[a->cursor].gemm);
         }
       }
       for (int pass = 0; pass < n_pass; ++pass) {
@@ -1215,8 +1225,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
             break;
           }
           case EPARA_K_GEMM: {
-            const int gpass = op.gemm.stream == 3 ? PASS_SWAP + swap_index(op.gemm.ksplit) : op.gemm.stream == 4 ? PASS_MLP : op.gemm.stream;
-            if (gpass != pass) break;                          // another pass takes it
+            if (gemm_pass(op.gemm) != pass) break;             // another pass takes it
             if (op.gemm.stream == 4) {
               MlpGroup mg = op.mlp;
               mg.M = rows;
@@ -1241,6 +1250,10 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
               g.tile_start = total;
               total += g.tiles_m * g.tiles_n;
               L.p3 = std::max(L.p3, g.bn);
+            } else if (g.stream == GEMM_SWAP2) {
+              g.tiles_m = (rows + g.bn - 1) / g.bn; g.tiles_n = gemm_swap2_tiles_n(g.N);
+              g.tile_start = total;
+              total += g.tiles_m * g.tiles_n;
             } else if (g.stream == 2) {
               g.tiles_m = (rows + 2 * TC_BM - 1) / (2 * TC_BM); g.tiles_n = (g.N + g.bn - 1) / g.bn;
               g.tile_start = total;
@@ -1365,6 +1378,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
       case EPARA_K_NORM: launch_norm((const NormGroup*)gp, L.n_groups, L.p1, st); break;
       case EPARA_K_GEMM:
         if (L.p2 == PASS_MLP) err = launch_gemm_mlp_pair((const MlpGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st, L.beside);
+        else if (L.p2 >= PASS_SWAP2) err = launch_gemm_swap2((const GemmGroup*)gp, L.n_groups, L.p0, 1 << (L.p2 - PASS_SWAP2), dev_status, c->sm_count, st, L.beside);
         else if (L.p2 >= PASS_SWAP) err = launch_gemm_swap((const GemmGroup*)gp, L.n_groups, L.p0, 1 << (L.p2 - PASS_SWAP), L.p3, dev_status, c->sm_count, st, L.beside);
         else if (L.p2 == 1) err = launch_gemm_stream((const GemmGroup*)gp, L.n_groups, L.p0, L.p1, st);
         else if (L.p2 == 2) err = launch_gemm_tc_pair((const GemmGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st, L.beside);
@@ -1499,8 +1513,9 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
   if (cudaSetDevice(device) != cudaSuccess) return EPARA_E_CUDA;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   std::vector<GemmGroup> gs, gs_stream, gs_pair;   // CUDA-core groups; weight-streaming groups; CTA-pair groups
-  std::vector<GemmGroup> gs_swap[N_SWAP];          // swapped-operand groups by k ranges per tile
-  int total_swap[N_SWAP] = {0}, nb_swap[N_SWAP] = {0};
+  constexpr int KINDS = N_SWAP + N_SWAP2;
+  std::vector<GemmGroup> gs_swap[KINDS];           // swapped-operand groups by k ranges per tile, then those on pairs of CTAs
+  int total_swap[KINDS] = {0}, nb_swap[KINDS] = {0};
   int total = 0, total_stream = 0, max_rows_stream = 0, total_pair = 0;
   for (int i = 0; i < n; ++i) {
     const epara_gemm_problem& q = p[i];
@@ -1520,29 +1535,23 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
       continue;
     }
     if (!simt && q.M == 0) continue;
-    if (!simt && gemm_swap_eligible(q.M, q.N, q.K, q.epilogue, sm_count)) {
-      g.stream = 3;
-      gemm_swap_config(q.M, q.N, q.K, sm_count, &g.bn, &g.ksplit);
-      const int si = swap_index(g.ksplit);
-      g.tiles_m = (q.M + g.bn - 1) / g.bn; g.tiles_n = gemm_swap_tiles_n(q.N);
+    if (!simt) {
+      g.stream = gemm_tc_choice(q.M, q.N, q.K, q.epilogue, sm_count, &g.bn, &g.ksplit);
+      if (!make_gemm_maps(g, q.M)) return EPARA_E_CUDA;
+      if (g.stream == GEMM_PAIR) {
+        g.tiles_m = (q.M + 2 * TC_BM - 1) / (2 * TC_BM); g.tiles_n = (q.N + g.bn - 1) / g.bn;
+        g.tile_start = total_pair;
+        total_pair += g.tiles_m * g.tiles_n;
+        gs_pair.push_back(g);
+        continue;
+      }
+      const bool two = g.stream == GEMM_SWAP2;
+      const int si = swap_index(g.ksplit) + (two ? N_SWAP : 0);
+      g.tiles_m = (q.M + g.bn - 1) / g.bn; g.tiles_n = two ? gemm_swap2_tiles_n(q.N) : gemm_swap_tiles_n(q.N);
       g.tile_start = total_swap[si];
       total_swap[si] += g.tiles_m * g.tiles_n;
       nb_swap[si] = std::max(nb_swap[si], g.bn);
-      if (!make_tmap(&g.tmA, q.A, q.M, q.K, q.lda, g.bn)) return EPARA_E_CUDA;
-      if (!make_tmap(&g.tmW, q.W, q.N, q.K, q.ldw, TC_BM)) return EPARA_E_CUDA;
       gs_swap[si].push_back(g);
-      continue;
-    }
-    if (!simt) {
-      g.stream = 2;
-      gemm_pair_config(q.M, q.N, q.K, q.epilogue, sm_count, &g.bn);
-      g.tiles_m = (q.M + 2 * TC_BM - 1) / (2 * TC_BM); g.tiles_n = (q.N + g.bn - 1) / g.bn;
-      g.tile_start = total_pair;
-      total_pair += g.tiles_m * g.tiles_n;
-      if (!make_tmap(&g.tmA, q.A, q.M, q.K, q.lda, TC_BM)) return EPARA_E_CUDA;
-      if (!make_tmap(&g.tmW, q.W, q.N, q.K, q.ldw, g.bn / 2)) return EPARA_E_CUDA;
-      if (!make_tmap_c(&g.tmC, q.C, q.M, q.N, q.ldc, q.epilogue)) return EPARA_E_CUDA;
-      gs_pair.push_back(g);
       continue;
     }
     g.tiles_m = (q.M + SIMT_TILE - 1) / SIMT_TILE; g.tiles_n = (q.N + SIMT_TILE - 1) / SIMT_TILE;
@@ -1554,10 +1563,10 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
   GemmGroup* dev_groups = (GemmGroup*)((unsigned char*)scratch + 256);
   GemmGroup* dev_stream = dev_groups + gs.size();
   GemmGroup* dev_pair = dev_stream + gs_stream.size();
-  GemmGroup* dev_swap[N_SWAP];
+  GemmGroup* dev_swap[KINDS];
   dev_swap[0] = dev_pair + gs_pair.size();
-  for (int i = 1; i < N_SWAP; ++i) dev_swap[i] = dev_swap[i - 1] + gs_swap[i - 1].size();
-  for (int i = 0; i < N_SWAP; ++i)
+  for (int i = 1; i < KINDS; ++i) dev_swap[i] = dev_swap[i - 1] + gs_swap[i - 1].size();
+  for (int i = 0; i < KINDS; ++i)
     if (!gs_swap[i].empty() &&
         cudaMemcpyAsync(dev_swap[i], gs_swap[i].data(), gs_swap[i].size() * sizeof(GemmGroup), cudaMemcpyHostToDevice, st) != cudaSuccess)
       return EPARA_E_CUDA;
@@ -1583,6 +1592,8 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
       err = launch_gemm_tc_pair(dev_pair, (int)gs_pair.size(), total_pair, status, sm, st);
     for (int i = 0; i < N_SWAP && err == cudaSuccess; ++i)
       err = launch_gemm_swap(dev_swap[i], (int)gs_swap[i].size(), total_swap[i], 1 << i, nb_swap[i], status, sm, st);
+    for (int i = N_SWAP; i < KINDS && err == cudaSuccess; ++i)
+      err = launch_gemm_swap2(dev_swap[i], (int)gs_swap[i].size(), total_swap[i], 1 << (i - N_SWAP), status, sm, st);
   }
   return err == cudaSuccess ? EPARA_OK : EPARA_E_CUDA;
 }

@@ -1,5 +1,5 @@
 // Grouped bf16 GEMM for groups of 17 to about a thousand rows (decode batches, classification heads, single images,
-// short prompts): C = epi(A W^T + bias) with the operands swapped on the tensor core.
+// prompts of some hundred tokens): C = epi(A W^T + bias) with the operands swapped on the tensor core.
 //
 // With so few rows the work is streaming W once, or too few output tiles to fill the chip.  The MMA's 128-row
 // operand is a tile of W (128 output columns) and the batch is the MMA's N: one tile of up to 256 rows, several of
@@ -23,11 +23,24 @@
 // columns contiguous.  No partial ever travels through global memory and the reduction order is fixed, so a
 // request's bits do not depend on timing or on what else is in the launch.
 //
+// Pairs (PAIR; some 150 to a thousand rows).  With hundreds of rows what counts is what a CTA takes in: a tile of 128 columns and 256
+// rows asks for 48 KB a k-block, as much as the MMAs of one SM can use in 512 cycles, and L2 delivers 61 bytes a cycle to an SM.
+// Here a tile has 256 columns and two CTAs (cta_group::2): each loads its own 128 rows of W and half of the batch rows, the first
+// one issues M = 256 MMAs for both (two per step when the tile has more than 256 rows), and each accumulates, exchanges and writes
+// out its own 128 columns as above, with the CTAs of the same half in the other k ranges.  Against tiles of 256 batch rows on
+// CTA pairs (the tile-pair kernel) the row tile is free: 536 rows are four of 160 and not two of 256 and a third that is nearly
+// empty, and K can be split where the tiles are few.  (One barrier a stage for both operands: with one each, as in the form on one
+// CTA, a k-block cost the issuer 650 cycles, now 360; 16 epilogue warps instead of eight gained nothing.)  512-token chunk beside
+// 24 decode requests, 1B decoder: 2498 -> 2367 us a step; a prompt of 509 tokens 1648 -> 1560, of 250 1419 -> 1271; two of 300, 8B,
+// 11310 -> 10600; one image through ViT-B 602 -> 548.
+//
 // Roles per CTA (converged warps, an elected lane issues): warp 0 TMA producer of W -- it does not wait for the earlier
 // kernels of the stream, weights being static, so its ring is full when they finish; the last warp TMA producer of the
 // activations; warp 1 tcgen05.mma issuer; warps 2..9 read the accumulator (two warps per TMEM lane
 // quarter) and run the epilogue.  Every mbarrier wait is bounded; a CTA that gives up records a code in *status and
 // still meets its cluster at the barriers.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 #include "tcgen05.cuh"
@@ -62,11 +75,15 @@ __device__ __forceinline__ int find_group_sw(const GemmGroup* groups, int n, int
   return lo;
 }
 
+// Rows of the first MMA of a PAIR tile: all of up to 256, the larger half of more.
+__host__ __device__ inline int swap2_first(int nb) { return nb <= 256 ? nb : (nb + 63) / 64 * 32; }
+
 // S: CTAs per cluster = k ranges per tile.  One cluster per (group, tile of 128 output columns, tile of nb rows).
 // BESIDE: runs beside the launch before it (see pdl_begin(); the residual then comes past L1.  A run-time switch cost 6 us of 1195 in
 // a step of 27 requests through the 1B decoder).
-template <int S, bool BESIDE>
-__global__ void __launch_bounds__(SW_THREADS, 2)
+// PAIR: a tile has 256 output columns and up to 384 batch rows and each of its k ranges two CTAs (see above).
+template <int S, bool BESIDE, bool PAIR>
+__global__ void __launch_bounds__(SW_THREADS, PAIR ? 1 : 2)
 gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __restrict__ status, int ring_bytes) {
   extern __shared__ unsigned char smem_dyn[];
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
@@ -83,14 +100,17 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   bool acc_ok = true;
-  const int rank = S == 1 ? 0 : (int)cluster_ctarank();
-  const int item = blockIdx.x / S;
+  constexpr int CTAS = PAIR ? 2 * S : S;          // of a cluster
+  const int crank = CTAS == 1 ? 0 : (int)cluster_ctarank();
+  const int rank = PAIR ? crank >> 1 : crank;     // k range
+  const int half = PAIR ? crank & 1 : 0;          // which 128 of the tile's 256 output columns, and which half of its batch rows to load
+  const int item = blockIdx.x / CTAS;
 
   const GemmGroup* g = groups + find_group_sw(groups, n_groups, item);
-  const int nb = g->bn;                           // batch rows of a tile as the MMA's N: multiple of 16, at most 256
+  const int nb = g->bn;                           // batch rows of a tile as the MMA's N: multiple of 16, at most 256 (PAIR: of 32, 384)
   const int tiles_m = g->tiles_m;
   const int local = item - g->tile_start;
-  const int n0 = (local / tiles_m) * SW_BM;       // first output column (W row) of the tile; the row tiles of one
+  const int n0 = (local / tiles_m) * (PAIR ? 2 * SW_BM : SW_BM) + half * SW_BM;   // first output column (W row); the row tiles of one
   const int m0 = (local % tiles_m) * nb;          // W tile are neighbours in the launch and share it through L2
   const int rows = min(nb, g->M - m0);            // live rows of this tile (at least one)
   const int kblocks = (g->K + TC_BK - 1) / TC_BK;
@@ -98,15 +118,16 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
   const int kb0 = rank * per, kb1 = min(kblocks, kb0 + per);
   const bool empty = kb0 >= kb1;                  // K too short for this rank: its partial is zero
   // activation ring first (a_stages tiles of nb x 64), then the W ring (w_stages tiles of 128 x 64)
-  const int a_bytes = nb * TC_BK * 2;
+  const int nb1 = PAIR ? swap2_first(nb) : nb, nb2 = nb - nb1;        // PAIR: the tile's rows in one MMA or two
+  const int a_bytes = PAIR ? nb * TC_BK : nb * TC_BK * 2;
   // (a load from L2 takes some 1100 cycles to land and its stage another 300 to come back, a k-block's MMAs a tenth of
   // that: with few rows the whole k range of a split tile fits the ring, so nothing waits for a stage)
   // (two CTAs per SM: the smaller ring stays with W)
-  const int a_stages = ring_bytes < SW_RING_BYTES_1 ? (nb > 64 ? 2 : 4) : nb > 128 ? 4 : nb > 64 ? 3 : nb > 32 ? 6 : SW_A_STAGES_MAX;
-  const int w_stages = min(SW_W_STAGES_MAX, (ring_bytes - a_stages * a_bytes) / SW_W_BYTES);
+  const int a_stages = PAIR ? min(SW_A_STAGES_MAX, ring_bytes / (SW_W_BYTES + a_bytes)) : ring_bytes < SW_RING_BYTES_1 ? (nb > 64 ? 2 : 4) : nb > 128 ? 4 : nb > 64 ? 3 : nb > 32 ? 6 : SW_A_STAGES_MAX;
+  const int w_stages = PAIR ? a_stages : min(SW_W_STAGES_MAX, (ring_bytes - a_stages * a_bytes) / SW_W_BYTES);
   const uint32_t w_base = base + a_stages * a_bytes;        // a multiple of 2 KB from a 1 KB-aligned base ...
   static_assert(SW_W_BYTES % 1024 == 0, "swizzle atoms");   // ... since nb is a multiple of 16
-  const uint32_t tmem_cols = nb > 128 ? 256u : 128u;
+  const uint32_t tmem_cols = nb > 256 ? 512u : nb > 128 ? 256u : 128u;
   // what the epilogue needs of the descriptor and the bias (static), read here so that it is at hand when the
   // accumulator is; a lane owns four consecutive output columns
   const int N = g->N, epi = g->epi, ldc = g->ldc;
@@ -127,12 +148,19 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(tmem_cols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (PAIR) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(tmem_cols) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(tmem_cols) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   tc_fence_before();
   __syncthreads();
+  if constexpr (PAIR) cluster_sync_all();          // the pair's leader has its barriers before anything is counted on them
   tc_fence_after();
+  const uint32_t leader = (uint32_t)(2 * rank);    // PAIR: issues the MMAs of both
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
@@ -144,8 +172,13 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
     for (int kb = kb0; kb < kb1; ++kb) {
       // (a stage's first use has nothing to wait for)
       if (kb - kb0 >= w_stages && !mbar_wait(wempty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 41); break; }
-      mbar_expect_tx_elect(wfull_bar(stage), (uint32_t)SW_W_BYTES);
-      tma_load_2d_elect(w_base + stage * SW_W_BYTES, &g->tmW, kb * TC_BK, n0, wfull_bar(stage));
+      if constexpr (PAIR) {
+        if (half == 0) mbar_expect_tx_elect(wfull_bar(stage), 2u * (SW_W_BYTES + (uint32_t)a_bytes));   // (activations too)
+        tma_load_2d_pair_elect(w_base + stage * SW_W_BYTES, &g->tmW, kb * TC_BK, n0, mapa_shared(wfull_bar(stage), leader));
+      } else {
+        mbar_expect_tx_elect(wfull_bar(stage), (uint32_t)SW_W_BYTES);
+        tma_load_2d_elect(w_base + stage * SW_W_BYTES, &g->tmW, kb * TC_BK, n0, wfull_bar(stage));
+      }
       if (++stage == w_stages) { stage = 0; phase ^= 1u; }
     }
     pdl_begin(BESIDE);                                    // (every thread of the kernel waits once, see common.cuh)
@@ -156,41 +189,79 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
     // the first copy after the wait finds its map (1B decoder, 27 requests: 1226 -> 1210 us a step; the larger tiles of the
     // tile-pair kernel and attention gained nothing)
     tensormap_prefetch_elect(&g->tmA);
+    if (PAIR && nb2) { tensormap_acquire(&g->tmC); tensormap_prefetch_elect(&g->tmC); }
     pdl_begin(BESIDE);
     int stage = 0;
     uint32_t phase = 0;
     bool ok = true;
     for (int kb = kb0; kb < kb1; ++kb) {
-      if (kb - kb0 >= a_stages && !mbar_wait(aempty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 44); break; }
-      mbar_expect_tx_elect(afull_bar(stage), (uint32_t)a_bytes);
-      tma_load_2d_elect(base + stage * a_bytes, &g->tmA, kb * TC_BK, m0, afull_bar(stage));
+      if (kb - kb0 >= a_stages && !mbar_wait(PAIR ? wempty_bar(stage) : aempty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 44); break; }
+      if constexpr (PAIR) {
+        // (half of each MMA's rows; tmC holds the map for the second MMA's)
+        const uint32_t bar = mapa_shared(wfull_bar(stage), leader);
+        tma_load_2d_pair_elect(base + stage * a_bytes, &g->tmA, kb * TC_BK, m0 + half * (nb1 >> 1), bar);
+        if (nb2) tma_load_2d_pair_elect(base + stage * a_bytes + nb1 * TC_BK, &g->tmC, kb * TC_BK, m0 + nb1 + half * (nb2 >> 1), bar);
+      } else {
+        mbar_expect_tx_elect(afull_bar(stage), (uint32_t)a_bytes);
+        tma_load_2d_elect(base + stage * a_bytes, &g->tmA, kb * TC_BK, m0, afull_bar(stage));
+      }
       if (++stage == a_stages) { stage = 0; phase ^= 1u; }
     }
     if (!ok) { *abort_flag = 1; drain_sleep(200000ull); }
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
-    const uint32_t idesc = make_idesc(nb);
-    int ws = 0, as = 0;
-    uint32_t wphase = 0, aphase = 0;
-    bool ok = true;
-    for (int kb = kb0; kb < kb1; ++kb) {
-      if (!mbar_wait_both(afull_bar(as), aphase, wfull_bar(ws), wphase, abort_flag)) {
-        ok = false;
-        const int code = mbar_test(afull_bar(as), aphase) ? 42 : 45;
-        if (lane == 0) atomicExch(status, code);
-        break;
-      }
-      const uint64_t dw = make_smem_desc(w_base + ws * SW_W_BYTES), da = make_smem_desc(base + as * a_bytes);
+    // ------------------------------------------------------------ MMA issuer (PAIR: of the pair, in its first CTA)
+    if (half == 0) {
+      bool ok = true;
+      if constexpr (PAIR) {
+        // (one barrier a stage for both operands and a look ahead under the issue, as in the tile-pair kernel)
+        const uint32_t idesc = make_idesc_pair(nb1), idesc2 = make_idesc_pair(nb2);
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ready = false;
+        for (int kb = kb0; kb < kb1; ++kb) {
+          if (!ready && !mbar_wait<false>(wfull_bar(stage), phase, abort_flag)) { ok = false; if (lane == 0) atomicExch(status, 42); break; }
+          const uint64_t dw = make_smem_desc(w_base + stage * SW_W_BYTES), da = make_smem_desc(base + stage * a_bytes);
+          const uint64_t da2 = make_smem_desc(base + stage * a_bytes + nb1 * TC_BK);
+          const uint32_t used = wempty_bar(stage);
+          if (++stage == w_stages) { stage = 0; phase ^= 1u; }
+          ready = mbar_test(wfull_bar(stage), phase);
 #pragma unroll
-      for (int k = 0; k < TC_BK / 16; ++k)
-        mma_f16_elect(tmem_base, dw + (uint64_t)(k * 2), da + (uint64_t)(k * 2), idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-      mma_commit_elect(wempty_bar(ws));
-      mma_commit_elect(aempty_bar(as));
-      if (++ws == w_stages) { ws = 0; wphase ^= 1u; }
-      if (++as == a_stages) { as = 0; aphase ^= 1u; }
+          for (int k = 0; k < TC_BK / 16; ++k)
+            mma_f16_pair_elect(tmem_base, dw + (uint64_t)(k * 2), da + (uint64_t)(k * 2), idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+          if (nb2) {
+#pragma unroll
+            for (int k = 0; k < TC_BK / 16; ++k)
+              mma_f16_pair_elect(tmem_base + (uint32_t)nb1, dw + (uint64_t)(k * 2), da2 + (uint64_t)(k * 2), idesc2, (kb > kb0 || k > 0) ? 1u : 0u);
+          }
+          mma_commit_pair_elect(used, 3u << leader);
+        }
+      } else {
+        const uint32_t idesc = make_idesc(nb);
+        int ws = 0, as = 0;
+        uint32_t wphase = 0, aphase = 0;
+        for (int kb = kb0; kb < kb1; ++kb) {
+          if (!mbar_wait_both(afull_bar(as), aphase, wfull_bar(ws), wphase, abort_flag)) {
+            ok = false;
+            const int code = mbar_test(afull_bar(as), aphase) ? 42 : 45;
+            if (lane == 0) atomicExch(status, code);
+            break;
+          }
+          const uint64_t dw = make_smem_desc(w_base + ws * SW_W_BYTES), da = make_smem_desc(base + as * a_bytes);
+#pragma unroll
+          for (int k = 0; k < TC_BK / 16; ++k)
+            mma_f16_elect(tmem_base, dw + (uint64_t)(k * 2), da + (uint64_t)(k * 2), idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+          mma_commit_elect(wempty_bar(ws));
+          mma_commit_elect(aempty_bar(as));
+          if (++ws == w_stages) { ws = 0; wphase ^= 1u; }
+          if (++as == a_stages) { as = 0; aphase ^= 1u; }
+        }
+      }
+      if (!ok) *abort_flag = 1;
+      else if (!empty) {
+        if constexpr (PAIR) mma_commit_pair_elect(tfull_bar, 3u << leader);
+        else mma_commit_elect(tfull_bar);
+      }
     }
-    if (!ok) *abort_flag = 1;
-    else if (!empty) mma_commit_elect(tfull_bar);
   } else {
     // ------------------------------------------------------------ wait for this CTA's accumulator (warps 2..9)
     pdl_begin(BESIDE);
@@ -210,12 +281,12 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
     // Batch row m0 + c (TMEM column c) belongs to CTA c / rp of the cluster.  Its buffer, over the idle operand
     // ring, is [S sources][rp batch rows][128 columns] fp32; this CTA fills plane `rank` of every owner.  The two
     // warps of a lane quarter take alternate blocks of 16 rows.
-    const int quarter = warp & 3, half = (warp - 2) >> 2;
+    const int quarter = warp & 3, alt = (warp - 2) >> 2;
     const uint32_t col_off = (uint32_t)(quarter * 32 + lane) * 4u;
     tc_fence_after();
     const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16);
     const uint32_t plane = (uint32_t)(rank * rp) * (SW_BM * 4u) + col_off;
-    for (int c = half * 16; c < rows; c += 32) {
+    for (int c = alt * 16; c < rows; c += 32) {
       uint32_t r[16];
       if (empty || !acc_ok) {
 #pragma unroll
@@ -227,7 +298,7 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
 #pragma unroll
       for (int j4 = 0; j4 < 16; j4 += 4) {
         const int owner = S == 1 ? 0 : (c + j4) / rp;
-        const uint32_t dst = (S == 1 ? base : mapa_shared(base, (uint32_t)owner)) + plane + (uint32_t)(c + j4 - owner * rp) * (SW_BM * 4u);
+        const uint32_t dst = (S == 1 ? base : mapa_shared(base, (uint32_t)(PAIR ? 2 * owner + half : owner))) + plane + (uint32_t)(c + j4 - owner * rp) * (SW_BM * 4u);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           if (S == 1)
@@ -318,25 +389,29 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
     }
   }
   // (after the barrier above nobody touches another CTA's shared memory, so the CTAs may leave one by one)
+  // (a pair leaves together: its first CTA's MMAs have read the other's operands and report to its barriers)
   pdl_end(BESIDE);
   tc_fence_before();
   __syncthreads();
+  if constexpr (PAIR) cluster_sync_all();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
+    if constexpr (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
   }
 }
 
-template <int S>
+template <int S, bool PAIR>
 cudaError_t launch_swap(const GemmGroup* groups, int n_groups, int total_items, int max_nb, int* status, int sm_count, cudaStream_t st, int beside) {
-  const auto kernel = beside ? gemm_swap_kernel<S, true> : gemm_swap_kernel<S, false>;
+  const auto kernel = beside ? gemm_swap_kernel<S, true, PAIR> : gemm_swap_kernel<S, false, PAIR>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw_smem(SW_RING_BYTES_1));
   if (e != cudaSuccess) return e;
   // Tiles of more than 128 rows need the large ring (the reduction lands nb x 512 bytes in it).
   // (clusters of eight one-SM CTAs were slow to place: 25.8 us against 15.4 with two CTAs per SM, 2048 x 8192 at 128 rows)
-  const int ring_bytes = (max_nb <= 128 && (total_items * S > sm_count || S == 8)) ? SW_RING_BYTES_2 : SW_RING_BYTES_1;
+  const int ring_bytes = (!PAIR && max_nb <= 128 && (total_items * S > sm_count || S == 8)) ? SW_RING_BYTES_2 : SW_RING_BYTES_1;
+  constexpr int CTAS = PAIR ? 2 * S : S;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(total_items * S);
+  cfg.gridDim = dim3(total_items * CTAS);
   cfg.blockDim = dim3(SW_THREADS);
   cfg.dynamicSmemBytes = sw_smem(ring_bytes);
   cfg.stream = st;
@@ -344,7 +419,7 @@ cudaError_t launch_swap(const GemmGroup* groups, int n_groups, int total_items, 
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = S;
+  attr[1].val.clusterDim.x = CTAS;
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
@@ -360,8 +435,9 @@ cudaError_t launch_swap(const GemmGroup* groups, int n_groups, int total_items, 
 // 2048 x 8192 at 128 rows, nothing for 2048 x 2048).
 // Above, one CTA takes an SM and the clusters have to be resident together: 74 of two CTAs, 33 of four and 15 of eight
 // fit on 148 SMs (sizes between them fit no more CTAs; one cluster too many costs a second wave: 2048 x 2048 at 256
-// rows 27 us with 16 clusters of eight, 15 on tile pairs).  A k-block costs 0.23 us + 1.1 ns per row, the exchange of
-// the partial sums runs at 41.8 KB a microsecond per SM.
+// rows 27 us with 16 clusters of eight, 15 on tile pairs).  A k-block costs 0.13 us + 0.7 ns per row, a seventh more once
+// most SMs are at it (they share what L2 delivers), exchange and epilogue 20 ns per row; clusters
+// of eight start later.
 double gemm_swap_config(long long rows_cap, int N, int K, int sm_count, int* nb, int* ksplit) {
   const int tiles_n = (N + SW_BM - 1) / SW_BM, kblocks = (K + TC_BK - 1) / TC_BK;
   const int tiles_m = (int)((rows_cap + GEMM_SWAP_TILE_ROWS - 1) / GEMM_SWAP_TILE_ROWS);
@@ -379,16 +455,8 @@ double gemm_swap_config(long long rows_cap, int N, int K, int sm_count, int* nb,
     if (tiles <= fit[i] && kblocks >= 3 << i) s = 1 << i;
   *ksplit = s;
   const double rounds = (double)((tiles + fit[0] - 1) / fit[0]);
-  return 10.0 + rounds * ((kblocks + s - 1) / s) * (0.23 + 0.0011 * *nb) + (s > 1 ? *nb * 512.0 * (s - 1) / s / 41800.0 : 0.0);
-}
-
-// Up to 128 rows a tile of A would be mostly padding for the tile-pair kernel.  Above, the estimates decide: the split
-// wins where K is long and the output tiles are few (2048 x 8192 at 512 rows: 29 us against 37 to 47 on tile pairs;
-// 768 x 3072 at 197 rows 14.8 against 18.7), the tile pairs elsewhere (3072 x 2048 at 512 rows: 15.2 against 27).
-bool gemm_swap_eligible(long long rows_cap, int N, int K, int epi, int sm_count) {
-  if (rows_cap <= TC_BM) return true;
-  int nb = 0, s = 1, bn = 0;
-  return gemm_swap_config(rows_cap, N, K, sm_count, &nb, &s) < gemm_pair_config(rows_cap, N, K, epi, sm_count, &bn);
+  const bool full = tiles * s > 2 * sm_count / 3;
+  return 8.0 + 0.02 * *nb + (full ? 1.5 : 0.0) + (s == 8 ? 1.5 : 0.0) + rounds * ((kblocks + s - 1) / s) * (0.13 + 0.0007 * *nb) * (full ? 1.15 : 1.0);
 }
 
 int gemm_swap_tiles_n(int N) { return (N + SW_BM - 1) / SW_BM; }
@@ -397,11 +465,62 @@ cudaError_t launch_gemm_swap(const GemmGroup* groups, int n_groups, int total_it
                              int sm_count, cudaStream_t st, int beside) {
   if (n_groups == 0 || total_items == 0) return cudaSuccess;
   switch (ksplit) {
-    case 1: return launch_swap<1>(groups, n_groups, total_items, max_nb, status, sm_count, st, beside);
-    case 2: return launch_swap<2>(groups, n_groups, total_items, max_nb, status, sm_count, st, beside);
-    case 4: return launch_swap<4>(groups, n_groups, total_items, max_nb, status, sm_count, st, beside);
-    case 8: return launch_swap<8>(groups, n_groups, total_items, max_nb, status, sm_count, st, beside);
+    case 1: return launch_swap<1, false>(groups, n_groups, total_items, max_nb, status, sm_count, st, beside);
+    case 2: return launch_swap<2, false>(groups, n_groups, total_items, max_nb, status, sm_count, st, beside);
+    case 4: return launch_swap<4, false>(groups, n_groups, total_items, max_nb, status, sm_count, st, beside);
+    case 8: return launch_swap<8, false>(groups, n_groups, total_items, max_nb, status, sm_count, st, beside);
   }
+  return cudaErrorInvalidValue;
+}
+
+// ---- pairs of CTAs on 256 output columns
+int gemm_swap2_first(int nb) { return swap2_first(nb); }
+int gemm_swap2_tiles_n(int N) { return (N + 2 * SW_BM - 1) / (2 * SW_BM); }
+
+// The estimate, in microseconds: a k-block costs what its operands take to arrive (0.14 us + 0.3 ns a row) or its MMAs, a tile
+// 26 ns a row for exchange and epilogue; pairs of one launch: 74 clusters of two CTAs or 33 of four are resident.  Within 10 % of
+// measured launches: 2048 x 8192 at 536 rows 23.3 us with four row tiles of 160 and two k ranges (tile pairs, three row tiles of which
+// the last has 24 live rows: 32.6), at 509 rows 22.0 (one-CTA tiles 25.5), at 1000 32.9 (34.6); 16384 x 2048 at 280 rows 23.5 (tile
+// pairs 29.1), but at 536 rows, where the tiles take two rounds, 43.4 against 40.2.  With a short K most of a tile's W is requested
+// before the dependency wait, which a launch on its own does not show: one image through ViT-B (K 768) 578 us a step with its
+// projections on tile pairs, 549 here.
+double gemm_swap2_config(long long rows_cap, int N, int K, int sm_count, int* nb, int* ksplit) {
+  const int tiles_n = gemm_swap2_tiles_n(N), kblocks = (K + TC_BK - 1) / TC_BK;
+  const double start = kblocks <= 16 ? 7.0 : 8.5;
+  double best = 0;
+  *nb = 0;
+  *ksplit = 1;
+  for (int tiles_m = (int)((rows_cap + GEMM_SWAP2_TILE_ROWS - 1) / GEMM_SWAP2_TILE_ROWS); tiles_m <= 8; ++tiles_m) {
+    const int rows = (int)(((rows_cap + tiles_m - 1) / tiles_m + 31) / 32 * 32);
+    if (rows < 64) break;
+    const double k_block = std::max(0.14 + 0.00031 * rows, 0.00112 * rows), tile = 0.026 * rows;
+    for (int s = 1; s <= 2; ++s) {
+      const int tiles = tiles_n * tiles_m, fit = s == 1 ? sm_count / 2 : sm_count * 33 / 148;
+      if (s == 2 && (tiles > fit || kblocks < 8)) continue;
+      const int rounds = (tiles + fit - 1) / fit;
+      const double t = start + rounds * (tile + (kblocks + s - 1) / s * k_block) + (rounds - 1) * 3.0;
+      if (*nb == 0 || t < best) { best = t; *nb = rows; *ksplit = s; }
+    }
+  }
+  return best;
+}
+
+// Up to 128 rows a tile of A would be mostly padding for the tile-pair kernel.  Above, the estimates decide.
+int gemm_tc_choice(long long rows_cap, int N, int K, int epi, int sm_count, int* bn, int* ksplit) {
+  int nb = 0, s = 1, nb2 = 0, s2 = 1, w = 0;
+  const double t_swap = gemm_swap_config(rows_cap, N, K, sm_count, &nb, &s);
+  if (rows_cap <= TC_BM) { *bn = nb; *ksplit = s; return GEMM_SWAP; }
+  const double t_pair = gemm_pair_config(rows_cap, N, K, epi, sm_count, &w), t_swap2 = gemm_swap2_config(rows_cap, N, K, sm_count, &nb2, &s2);
+  if (nb2 > 0 && t_swap2 < t_pair && t_swap2 < t_swap) { *bn = nb2; *ksplit = s2; return GEMM_SWAP2; }
+  if (t_swap < t_pair) { *bn = nb; *ksplit = s; return GEMM_SWAP; }
+  *bn = w; *ksplit = 1;
+  return GEMM_PAIR;
+}
+
+cudaError_t launch_gemm_swap2(const GemmGroup* groups, int n_groups, int total_items, int ksplit, int* status, int sm_count, cudaStream_t st, int beside) {
+  if (n_groups == 0 || total_items == 0) return cudaSuccess;
+  if (ksplit == 1) return launch_swap<1, true>(groups, n_groups, total_items, 0, status, sm_count, st, beside);
+  if (ksplit == 2) return launch_swap<2, true>(groups, n_groups, total_items, 0, status, sm_count, st, beside);
   return cudaErrorInvalidValue;
 }
 

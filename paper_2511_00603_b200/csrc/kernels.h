@@ -39,10 +39,22 @@ cudaError_t launch_gemm_mlp_pair(const MlpGroup* groups, int n_groups, int total
 // max_nb: widest bn of the launch.
 constexpr int GEMM_SWAP_TILE_ROWS = 256;
 double gemm_swap_config(long long rows_cap, int N, int K, int sm_count, int* nb, int* ksplit);
-bool gemm_swap_eligible(long long rows_cap, int N, int K, int epi, int sm_count);
 int gemm_swap_tiles_n(int N);
 cudaError_t launch_gemm_swap(const GemmGroup* groups, int n_groups, int total_items, int ksplit, int max_nb, int* status,
                              int sm_count, cudaStream_t st, int beside = 0);
+
+// The same on pairs of CTAs (GemmGroup::stream == 5): tiles of 256 output columns and bn batch rows (a multiple of 32, at
+// most GEMM_SWAP2_TILE_ROWS), `ksplit` (1 or 2) pairs per tile; for some 200 to a thousand rows.  Maps: tmW box 128 rows,
+// tmA box half of gemm_swap2_first(bn) rows, tmC the activations again with a box of half the rest (when there is a rest).
+constexpr int GEMM_SWAP2_TILE_ROWS = 384;
+double gemm_swap2_config(long long rows_cap, int N, int K, int sm_count, int* nb, int* ksplit);
+int gemm_swap2_first(int nb);
+int gemm_swap2_tiles_n(int N);
+cudaError_t launch_gemm_swap2(const GemmGroup* groups, int n_groups, int total_items, int ksplit, int* status, int sm_count, cudaStream_t st,
+                              int beside = 0);
+enum : int { GEMM_PAIR = 2, GEMM_SWAP = 3, GEMM_SWAP2 = 5 };
+// The kernel for a GEMM that the weight-streaming kernel does not take, with its tile (GemmGroup::bn, ksplit).
+int gemm_tc_choice(long long rows_cap, int N, int K, int epi, int sm_count, int* bn, int* ksplit);
 
 // Weight-streaming GEMM (GemmGroup::stream == 1) for groups that never exceed 16 rows, and for small matrices: one block
 // per 16 rows of W over the whole K and 32 batch rows, mma.sync, no tensor maps.  total_items = sum of

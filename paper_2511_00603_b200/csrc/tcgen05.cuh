@@ -204,11 +204,12 @@ __device__ __forceinline__ void mma_commit_elect(uint32_t bar) {
       "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
       "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void mma_commit_pair_elect(uint32_t bar) {
+// (mask: the pair's two ranks in the cluster)
+__device__ __forceinline__ void mma_commit_pair_elect(uint32_t bar, uint32_t mask = 3u) {
   asm volatile(
       "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
       "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
-      ::"r"(bar), "h"((unsigned short)3) : "memory");
+      ::"r"(bar), "h"((unsigned short)mask) : "memory");
 }
 // Cluster barrier that orders no data: every CTA of the cluster has come this far.
 __device__ __forceinline__ void cluster_sync_relaxed() {
