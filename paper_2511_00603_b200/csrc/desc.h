@@ -74,7 +74,8 @@ struct alignas(TMAP_ALIGN) GemmGroup {
                    // tiles and tmW's box holds bn / 2 rows); 3: swapped operands (tmA's box holds bn rows, tmW's
                    // 128); 5: swapped operands on CTA pairs (see kernels.h); 0: plain CUDA-core comparator
   const ReqDesc* reqs;   // weight-streaming kernel: when set, row m of A is request m's input (an MLP's first layer)
-  int pad[4];
+  int m_base, n_base;    // tile pairs: first row and column of the group's first tile
+  int pad[2];
 };
 
 enum : int { NORM_LN = 0, NORM_RMS = 1 };

@@ -39,6 +39,8 @@ inline int gemm_pass(const GemmGroup& g) {
   return g.stream == GEMM_SWAP ? PASS_SWAP + swap_index(g.ksplit) : g.stream == GEMM_SWAP2 ? PASS_SWAP2 + swap_index(g.ksplit) : g.stream == 4 ? PASS_MLP : g.stream;
 }
 
+constexpr int FINE_BN[2] = {64, 128}, FINE_MIN_K = 2048;        // the tile-pair kernel's last round (see fine_tail in epara_step)
+
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 inline int round_up(int v, int a) { return (v + a - 1) / a * a; }
 
@@ -124,6 +126,7 @@ struct Op {
   int from_requests;  // GEMM: the rows of A are the requests' inputs
   AttnPrefillGroup apre;
   GemmGroup gemm;
+  CUtensorMap tmW_fine[2];   // tile pairs: W in the boxes of tiles FINE_BN[i] wide (see fine_tail())
   MlpGroup mlp;          // EPARA_K_GEMM with gemm.stream == 4: FC1, GELU, FC2 and the residual update in one kernel ...
   GemmGroup fc1, fc2;    // ... and the same as two GEMMs (same bits), for the tiles of a last round that few pairs would work
   NormGroup norm;
@@ -284,6 +287,8 @@ bool add_gemm(Builder& bl, Model* m, const void* A, int lda, long long rows_cap,
     g.stream = gemm_tc_choice(max_rows, N, K, g.epi, sm_count, &g.bn, &g.ksplit);
   }
   if (bl.c && !make_gemm_maps(g, rows_cap)) return false;
+  for (int i = 0; bl.c && g.stream == GEMM_PAIR && i < 2; ++i)
+    if (!make_tmap(&op.tmW_fine[i], W, N, K, K, FINE_BN[i] / 2)) return false;
   g.c_rows = (int)rows_cap;
   m->ops.push_back(op);
   return true;
@@ -1033,6 +1038,44 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
   // ---- plan (A1): sweep the kernel kinds until every model's op list is exhausted ----
   static const int sweep[] = {EPARA_K_GATHER, EPARA_K_TRACE, EPARA_K_ASSEMBLE, EPARA_K_NORM, EPARA_K_GEMM, EPARA_K_ROPE,
                               EPARA_K_ATTN_PREFILL, EPARA_K_ATTN_ENC, EPARA_K_ATTN_DEC, EPARA_K_OUTPUT};
+  // Tile pairs: a last round with few tiles takes as long as a full one.  The last row tiles of a group, or its last columns of
+  // tiles, that make up at least those tiles are cut finer, 64 or 128 columns wide (the narrowest that still fits the round: a k-block
+  // of such a tile takes some 0.65 and 0.8 of a 256-wide one's time), where the launch's groups have tiles of one kind.  An element's k
+  // order does not depend on the width: the same bits.  1B decoder, four prompts of 2048 tokens 16335 -> 16151 us a step, three of
+  // 1024 6193 -> 6144, one of 1300 3370 -> 3350; 8B, 1024 tokens 14496 -> 14379.  Not with K below 2048: there a round is 3 us and the
+  // fetch of the finer group's descriptor and map 1 (64 images of ViT-B, K 768, 2968 -> 2980; 203 of ViT-S 3176 -> 3193).
+  struct FineTail { Active* a; int tiles_m, tiles_n, width; };   // of the group's tiles: the last row tiles or the last column tiles
+  auto fine_tail = [&](const std::vector<Active*>& who) {
+    const FineTail no = {nullptr, 0, 0, 0};
+    const int pairs = c->sm_count / 2;
+    const GemmGroup* g0 = nullptr;
+    Active* most = nullptr;
+    int total = 0, tm = 0, tn = 0;
+    for (Active* a : who) {
+      const Op& op = a->m->ops[a->cursor];
+      const GemmGroup& g = op.gemm;
+      if (g.stream != GEMM_PAIR) continue;
+      if (!g0) g0 = &g;
+      if (g.bn != g0->bn || g.K != g0->K || g.epi != g0->epi || g.N != g0->N) return no;
+      const int rows = op.per_token ? a->rows : a->B * op.rows_per_req;
+      const int m = (rows + 2 * TC_BM - 1) / (2 * TC_BM);
+      tn = (g.N + g.bn - 1) / g.bn;
+      total += m * tn;
+      if (m > tm) { most = a; tm = m; }
+    }
+    const int rest = total > pairs ? total % pairs : 0;
+    if (rest == 0 || g0->K < FINE_MIN_K) return no;
+    const int cut_m = (rest + tn - 1) / tn, cut_n = (rest + tm - 1) / tm;
+    for (int i = 0; i < 2; ++i) {
+      if (FINE_BN[i] >= g0->bn) break;
+      const int fine_m = cut_m * ((g0->N + FINE_BN[i] - 1) / FINE_BN[i]), room_m = pairs + cut_m * tn - rest;
+      const int fine_n = tm * ((g0->N - (tn - cut_n) * g0->bn + FINE_BN[i] - 1) / FINE_BN[i]), room_n = pairs + cut_n * tm - rest;
+      const bool by_m = cut_m < tm && fine_m <= room_m, by_n = cut_n < tn && fine_n <= room_n;
+      if (by_m && (!by_n || fine_m <= fine_n)) return FineTail{most, cut_m, 0, i};
+      if (by_n) return FineTail{most, 0, cut_n, i};
+    }
+    return no;
+  };
   std::vector<Launch> launches;
   bool more = true;
   while (more && !overflow) {
@@ -1099,6 +1142,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
         cut_tiles = tiles > pairs ? tiles % pairs : 0;
         if (cut_tiles == 0 || cut_tiles > pairs / 2 || cut_tiles >= most) cut = nullptr;
       }
+      const FineTail fine = pass == GEMM_PAIR && kind == EPARA_K_GEMM && off < BLOB_BYTES / 2 ? fine_tail(who) : FineTail{nullptr, 0, 0, 0};
       Launch L;
       memset(&L, 0, sizeof(L));
       L.kind = kind;
@@ -1255,7 +1299,8 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
               g.tile_start = total;
               total += g.tiles_m * g.tiles_n;
             } else if (g.stream == 2) {
-              g.tiles_m = (rows + 2 * TC_BM - 1) / (2 * TC_BM); g.tiles_n = (g.N + g.bn - 1) / g.bn;
+              g.tiles_m = (rows + 2 * TC_BM - 1) / (2 * TC_BM) - (a == fine.a ? fine.tiles_m : 0);
+              g.tiles_n = (g.N + g.bn - 1) / g.bn - (a == fine.a ? fine.tiles_n : 0);
               g.tile_start = total;
               total += g.tiles_m * g.tiles_n;
             } else if (g.stream) {
@@ -1312,6 +1357,21 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
           }
         }
         if (pass == n_pass - 1) a->cursor++;
+      }
+      if (fine.a) {                                            // what its group above leaves out, in finer tiles
+        const Op& op = fine.a->m->ops[fine.a->cursor];
+        GemmGroup g = op.gemm;
+        g.M = op.per_token ? fine.a->rows : fine.a->B * op.rows_per_req;
+        const int tm = (g.M + 2 * TC_BM - 1) / (2 * TC_BM), tn = (g.N + g.bn - 1) / g.bn;
+        if (fine.tiles_m) g.m_base = (tm - fine.tiles_m) * 2 * TC_BM;
+        else g.n_base = (tn - fine.tiles_n) * g.bn;
+        g.tmW = op.tmW_fine[fine.width];
+        g.bn = FINE_BN[fine.width];
+        g.tiles_m = fine.tiles_m ? fine.tiles_m : tm; g.tiles_n = (g.N - g.n_base + g.bn - 1) / g.bn;
+        g.tile_start = total;
+        total += g.tiles_m * g.tiles_n;
+        ++n_put;
+        if (put(&g, sizeof(g), TMAP_ALIGN) == (size_t)-1) overflow = true;
       }
       L.p0 = total; L.p1 = mx;
       if (kind == EPARA_K_GATHER || kind == EPARA_K_GEMM || kind == EPARA_K_ATTN_ENC || kind == EPARA_K_ROPE) {

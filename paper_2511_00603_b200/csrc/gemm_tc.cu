@@ -50,13 +50,13 @@ __device__ __forceinline__ int find_group_tc(const GemmGroup* groups, int n, int
 struct GView {
   const bf16* bias;
   const CUtensorMap* tmC;
-  int N, epi, tile_start, tiles_m, tiles_n, bn, c_rows;
+  int N, epi, tile_start, tiles_m, tiles_n, bn, c_rows, m_base, n_base;
 };
 __device__ __forceinline__ GView load_view(const GemmGroup* g) {
   GView v;
   v.bias = g->bias; v.N = g->N; v.epi = g->epi; v.tile_start = g->tile_start;
   v.tiles_m = g->tiles_m; v.tiles_n = g->tiles_n; v.bn = g->bn;
-  v.tmC = &g->tmC; v.c_rows = g->c_rows;
+  v.tmC = &g->tmC; v.c_rows = g->c_rows; v.m_base = g->m_base; v.n_base = g->n_base;
   return v;
 }
 
@@ -64,7 +64,7 @@ __device__ __forceinline__ GView load_view(const GemmGroup* g) {
 // the current group (descriptor reads from global memory are latency the MMA issuer cannot hide).
 struct GroupCache {
   const GemmGroup* g;
-  int start, end, tiles_n, bn, kblocks;
+  int start, end, tiles_n, bn, kblocks, m_base, n_base;
 };
 __device__ __forceinline__ void group_cache(GroupCache& c, const GemmGroup* groups, int n_groups, int item) {
   if (c.g != nullptr && item >= c.start && item < c.end) return;
@@ -73,9 +73,14 @@ __device__ __forceinline__ void group_cache(GroupCache& c, const GemmGroup* grou
   c.start = g->tile_start;
   c.tiles_n = g->tiles_n;
   c.bn = g->bn;
+  c.m_base = g->m_base;
+  c.n_base = g->n_base;
   c.end = c.start + g->tiles_m * g->tiles_n;
   c.kblocks = (g->K + TC_BK - 1) / TC_BK;
 }
+
+// Columns of a tile that an epilogue warp works: a quarter, of 64-wide tiles half (two of the four then have none).
+__device__ __forceinline__ int part_cols(int bn) { return max(bn >> 2, 32); }
 
 // A work item of a group as the CTA of the given rank sees it: its first row and the tile's first column.
 struct Item {
@@ -84,8 +89,8 @@ struct Item {
 template <class G>
 __device__ __forceinline__ Item decode_item(const G& g, int local, int rank) {
   Item it;
-  it.m0 = (local / g.tiles_n) * (2 * TC_BM) + rank * TC_BM;
-  it.n0 = (local % g.tiles_n) * g.bn;
+  it.m0 = g.m_base + (local / g.tiles_n) * (2 * TC_BM) + rank * TC_BM;
+  it.n0 = g.n_base + (local % g.tiles_n) * g.bn;
   return it;
 }
 
@@ -106,8 +111,8 @@ __device__ __forceinline__ void epi_direct(const GView& g, const Item& it, uint3
   const uint32_t wst_u = smem_u32(wst);
   const int y0 = it.m0 + quarter * 32;
   const bool box_ok = y0 < g.c_rows;                         // some row of this warp's box is inside the tensor
-  const int c_begin = part * (g.bn >> 2);
-  const int c_end = min(c_begin + (g.bn >> 2), g.N - it.n0);
+  const int c_begin = part * part_cols(g.bn);
+  const int c_end = min(c_begin + part_cols(g.bn), min(g.bn, g.N - it.n0));
   if (c_begin >= c_end) {                                    // nothing to do for this warp: release at once
     tc_fence_before();
     __syncwarp();
@@ -358,8 +363,8 @@ gemm_tc_pair_kernel(const GemmGroup* __restrict__ groups, int n_groups, int tota
       const Item it = decode_item(g, item - g.tile_start, rank);
       uint2 bias_reg = make_uint2(0u, 0u);
       if (g.epi & EPI_BIAS) {
-        const int nb = it.n0 + part * (g.bn >> 2) + lane * 4;
-        if (lane * 4 >= (g.bn >> 2)) {
+        const int nb = it.n0 + part * part_cols(g.bn) + lane * 4;
+        if (lane * 4 >= part_cols(g.bn)) {
           // beyond this warp's columns
         } else if (nb + 4 <= g.N) {
           bias_reg = __ldg(reinterpret_cast<const uint2*>(g.bias + nb));
