@@ -40,7 +40,12 @@ PyObject* collect(PyObject* capsule, PyObject* const* args, Py_ssize_t n, PyObje
   if (!out) return nullptr;
   Py_buffer view;
   if (PyObject_GetBuffer(out, &view, PyBUF_WRITABLE) < 0) { Py_DECREF(out); return nullptr; }
-  const int status = c->fn(reinterpret_cast<void*>(static_cast<uintptr_t>(ctx)), ticket, view.buf);
+  // (without the interpreter lock, as ctypes calls it: the library may ask the CUDA driver whether the step's event is through,
+  // and the driver's own lock can be held by another thread's launches)
+  int status;
+  Py_BEGIN_ALLOW_THREADS
+  status = c->fn(reinterpret_cast<void*>(static_cast<uintptr_t>(ctx)), ticket, view.buf);
+  Py_END_ALLOW_THREADS
   PyBuffer_Release(&view);
   PyObject* s = PyLong_FromLong(status);
   PyObject* r = s ? PyTuple_New(2) : nullptr;

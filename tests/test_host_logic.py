@@ -5,6 +5,8 @@ import os
 import re
 import subprocess
 import sys
+import threading
+import time
 
 import numpy as np
 import pytest
@@ -127,3 +129,28 @@ def test_collect_method_without_ctypes_takes_what_the_general_one_takes(E):
         c.epara_collect("7")
     with pytest.raises(TypeError):
         c.epara_collect()
+
+
+def test_collect_method_lets_other_threads_run(E):
+    """The compiled method calls the library without the interpreter lock.  The C library's usleep stands in for epara_collect: it takes
+    its microseconds where the context's address goes."""
+    from paper_2511_00603_b200 import _fastcall
+
+    class Sleeper:
+        _handle = 300_000
+    usleep = ctypes.cast(ctypes.CDLL(None).usleep, ctypes.c_void_p).value
+    Sleeper.collect = _fastcall.collect_method(usleep, E.Output, None, "_handle")
+    inside = threading.Event()
+
+    def call():
+        inside.set()
+        Sleeper().collect(1)
+    t = threading.Thread(target=call)
+    t.start()
+    inside.wait()
+    turns = 0
+    while t.is_alive():
+        time.sleep(0.002)
+        turns += 1
+    t.join()
+    assert turns > 10
