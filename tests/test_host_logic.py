@@ -154,3 +154,17 @@ def test_collect_method_lets_other_threads_run(E):
         turns += 1
     t.join()
     assert turns > 10
+
+
+@pytest.mark.parametrize("cxx", ["/nowhere/c++", "false"])
+def test_build_goes_on_without_the_compiled_collect_method(monkeypatch, tmp_path, capfd, cxx):
+    """A compiler that is missing or fails leaves the extension out, one of an older source included, and the build goes on."""
+    from paper_2511_00603_b200 import build
+    old = tmp_path / "_fastcall.so"
+    old.write_bytes(b"of an older source")
+    monkeypatch.setattr(build, "FAST_LIB", str(old))
+    monkeypatch.setattr(build, "_stale", lambda: False)
+    os.utime(old, (0, 0))
+    monkeypatch.setenv("CXX", cxx)
+    assert build.build() == build.LIB
+    assert not old.exists() and "ctypes" in capfd.readouterr().err
