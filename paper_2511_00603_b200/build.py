@@ -48,10 +48,10 @@ def build_fastcall(force: bool = False) -> None:
     try:
         r = subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-I", include, FAST_SRC, "-o", FAST_LIB],
                            capture_output=True, text=True)
-        failed = r.stdout + r.stderr if r.returncode != 0 else ""
+        failed = f"{r.stdout}{r.stderr}exit status {r.returncode}" if r.returncode != 0 else None
     except OSError as e:
         failed = str(e)
-    if failed:
+    if failed is not None:
         sys.stderr.write("fastcall.cpp was not built, answers are collected through ctypes:\n" + failed + "\n")
 
 
