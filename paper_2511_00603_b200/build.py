@@ -16,7 +16,8 @@ OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libepara.so")
 SOURCES = ["epara_api.cu", "kernels_misc.cu", "gemm_simt.cu", "gemm_tc.cu", "gemm_stream.cu", "gemm_swap.cu", "attention.cu", "attention_flash.cu", "policy.cu",
            "selftest.cu"]
-FAST_SRC, FAST_LIB = os.path.join(CSRC, "fastcall.cpp"), os.path.join(HERE, "_fastcall.so")   # Python side of epara_collect
+# Python side of epara_collect; the file's name carries the interpreter's ABI, another interpreter does not load it
+FAST_SRC, FAST_LIB = os.path.join(CSRC, "fastcall.cpp"), os.path.join(HERE, "_fastcall" + sysconfig.get_config_var("EXT_SUFFIX"))
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC"]
 
 
@@ -43,12 +44,16 @@ def build_fastcall(force: bool = False) -> None:
     include = sysconfig.get_paths()["include"]
     if not os.path.exists(os.path.join(include, "Python.h")) or not (force or _newer(FAST_LIB, [FAST_SRC])):
         return
-    if os.path.exists(FAST_LIB):                # of an older source
-        os.remove(FAST_LIB)
+    for old in (FAST_LIB, os.path.join(os.path.dirname(FAST_LIB), "_fastcall.so")):   # of an older source; without an ABI in its name
+        if os.path.exists(old):
+            os.remove(old)
+    part = f"{FAST_LIB}.{os.getpid()}.part"      # renamed when complete: another process may import it meanwhile
     try:
-        r = subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-I", include, FAST_SRC, "-o", FAST_LIB],
+        r = subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-I", include, FAST_SRC, "-o", part],
                            capture_output=True, text=True)
         failed = f"{r.stdout}{r.stderr}exit status {r.returncode}" if r.returncode != 0 else None
+        if failed is None:
+            os.replace(part, FAST_LIB)
     except OSError as e:
         failed = str(e)
     if failed is not None:

@@ -3,10 +3,13 @@
 import ctypes
 import os
 import re
+import shutil
 import subprocess
 import sys
+import sysconfig
 import threading
 import time
+import types
 
 import numpy as np
 import pytest
@@ -117,7 +120,9 @@ def test_product_path_does_not_import_the_oracle():
 
 def test_collect_method_without_ctypes_takes_what_the_general_one_takes(E):
     """The binding's compiled epara_collect: positional, by keyword, ticket as a ctypes integer, wrong types; on a context without a
-    handle every form answers INVALID."""
+    handle every form answers INVALID.  (Where it can be built it is the one in use.)"""
+    if os.path.exists(os.path.join(sysconfig.get_paths()["include"], "Python.h")) and shutil.which(os.environ.get("CXX", "g++")):
+        assert not isinstance(E.Context.__dict__["epara_collect"], types.FunctionType)
     class NoContext(E.Context):
         def __init__(self):
             self.h, self._handle = E.C.c_void_p(), 0
@@ -160,7 +165,7 @@ def test_collect_method_lets_other_threads_run(E):
 def test_build_goes_on_without_the_compiled_collect_method(monkeypatch, tmp_path, capfd, cxx):
     """A compiler that is missing or fails leaves the extension out, one of an older source included, and the build goes on."""
     from paper_2511_00603_b200 import build
-    old = tmp_path / "_fastcall.so"
+    old = tmp_path / os.path.basename(build.FAST_LIB)
     old.write_bytes(b"of an older source")
     monkeypatch.setattr(build, "FAST_LIB", str(old))
     monkeypatch.setattr(build, "_stale", lambda: False)
@@ -168,3 +173,15 @@ def test_build_goes_on_without_the_compiled_collect_method(monkeypatch, tmp_path
     monkeypatch.setenv("CXX", cxx)
     assert build.build() == build.LIB
     assert not old.exists() and "ctypes" in capfd.readouterr().err
+
+
+def test_collect_extension_is_named_for_this_interpreter(E, monkeypatch, tmp_path):
+    """The extension is made for one interpreter's ABI: its file carries the tag, one without a tag is removed, nothing partial is left."""
+    from paper_2511_00603_b200 import _fastcall, build
+    suffix = sysconfig.get_config_var("EXT_SUFFIX")
+    assert suffix != ".so" and os.path.basename(_fastcall.__file__) == "_fastcall" + suffix
+    untagged, tagged = tmp_path / "_fastcall.so", tmp_path / os.path.basename(build.FAST_LIB)
+    untagged.write_bytes(b"of some other interpreter")
+    monkeypatch.setattr(build, "FAST_LIB", str(tagged))
+    build.build_fastcall()
+    assert os.listdir(tmp_path) == [tagged.name]
