@@ -329,6 +329,12 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
 size_t epara_gemm_scratch_bytes(int n_problems);
 size_t epara_gemm_scratch_bytes_for(int device, const epara_gemm_problem* problems, int n);
 
+/* The kernel that a GEMM runs on, on a GPU of sm_count SMs: `rows` is M for epara_grouped_gemm, the row capacity of the
+ * op for a placement.  Answers EPARA_GEMM_KERNEL_* (or EPARA_E_INVALID), its tile (swapped operands: batch rows; otherwise output
+ * columns) and how many ranges K is cut into.  Host only. */
+enum { EPARA_GEMM_KERNEL_STREAM = 1, EPARA_GEMM_KERNEL_TILE_PAIRS = 2, EPARA_GEMM_KERNEL_SWAPPED = 3, EPARA_GEMM_KERNEL_SWAPPED_PAIRS = 5 };
+int epara_gemm_plan(long long rows, int N, int K, int epilogue, int sm_count, int* tile, int* k_ranges);
+
 /* Split-KV paged decode attention with GQA (one layer).  q: bf16 [B, q_stride] (head h at
  * column h*hd); kv_layer: bf16 [kv_pages][2][Hkv][16][hd]; kv_lens int32 [B] = tokens to attend
  * (cached + appended; values outside [0, max_len] are clamped, a request of length 0 leaves its output

@@ -1546,6 +1546,16 @@ size_t epara_gemm_scratch_bytes_for(int device, const epara_gemm_problem* p, int
   return epara_gemm_scratch_bytes(n);
 }
 
+int epara_gemm_plan(long long rows, int N, int K, int epilogue, int sm_count, int* tile, int* k_ranges) {
+  static_assert(EPARA_GEMM_KERNEL_TILE_PAIRS == GEMM_PAIR && EPARA_GEMM_KERNEL_SWAPPED == GEMM_SWAP && EPARA_GEMM_KERNEL_SWAPPED_PAIRS == GEMM_SWAP2, "GemmGroup::stream");
+  if (rows <= 0 || N <= 0 || K <= 0 || sm_count < 2 || !tile || !k_ranges) return EPARA_E_INVALID;
+  if (gemm_stream_eligible(rows, N, K)) {
+    *tile = 16; *k_ranges = 1;
+    return EPARA_GEMM_KERNEL_STREAM;
+  }
+  return gemm_tc_choice(rows, N, K, epilogue, sm_count, tile, k_ranges);
+}
+
 int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm_problem* p, int n, void* scratch,
                        size_t scratch_bytes) {
   if (n < 0 || (n > 0 && !p) || !scratch || (reinterpret_cast<uintptr_t>(scratch) & 255)) return EPARA_E_INVALID;

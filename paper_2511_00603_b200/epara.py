@@ -73,7 +73,7 @@ EXPORTS = ["epara_init", "epara_register_model", "epara_submit", "epara_submit_m
            "epara_gemm_scratch_bytes", "epara_gemm_scratch_bytes_for", "epara_decode_attention", "epara_decode_attention_scratch_bytes",
            "epara_decode_attention_static", "epara_static_scratch_bytes", "epara_decode_attention_static_status",
            "epara_set_max_profile_launches", "epara_selftest_bounded_wait", "epara_offload_probabilities", "epara_simulate",
-           "epara_place_sssp"]
+           "epara_place_sssp", "epara_gemm_plan"]
 
 lib.epara_init.argtypes = [C.POINTER(Config), C.POINTER(C.c_void_p)]
 lib.epara_register_model.argtypes = [C.c_void_p, C.POINTER(ModelDesc), C.POINTER(C.c_int)]
@@ -100,6 +100,7 @@ lib.epara_gemm_scratch_bytes.argtypes = [C.c_int]
 lib.epara_gemm_scratch_bytes.restype = C.c_size_t
 lib.epara_gemm_scratch_bytes_for.argtypes = [C.c_int, C.POINTER(GemmProblem), C.c_int]
 lib.epara_gemm_scratch_bytes_for.restype = C.c_size_t
+lib.epara_gemm_plan.argtypes = [C.c_longlong, C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_int)]
 lib.epara_decode_attention.argtypes = [C.c_int, C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_longlong, C.c_void_p,
                                        C.c_void_p, C.c_int, C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int,
                                        C.c_int, C.c_void_p, C.c_size_t]
@@ -330,6 +331,16 @@ def gemm_problem_array(problems: Sequence[Dict]):
 
 def epara_gemm_scratch_bytes_for(problems: Sequence[Dict], device: int = 0) -> int:
     return lib.epara_gemm_scratch_bytes_for(device, gemm_problem_array(problems), len(problems))
+
+
+GEMM_KERNELS = {1: "stream", 2: "tile pairs", 3: "swapped", 5: "swapped pairs"}
+
+
+def epara_gemm_plan(rows: int, N: int, K: int, epilogue: int = 0, sm_count: int = 148):
+    """(kernel, tile, k ranges) of a GEMM with that row capacity; the kernel is one of GEMM_KERNELS' names."""
+    tile, k_ranges = C.c_int(0), C.c_int(0)
+    kernel = _check(lib.epara_gemm_plan(rows, N, K, epilogue, sm_count, C.byref(tile), C.byref(k_ranges)), "epara_gemm_plan")
+    return GEMM_KERNELS[kernel], tile.value, k_ranges.value
 
 
 def epara_grouped_gemm(problems: Sequence[Dict], stream_ptr: int, scratch, impl: int = GEMM_TCGEN05, device: int = 0):

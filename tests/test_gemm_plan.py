@@ -1,0 +1,24 @@
+"""Which kernel, tile and K split a GEMM gets (host only; 148 SMs)."""
+import pytest
+
+
+@pytest.fixture(scope="module")
+def E():
+    from paper_2511_00603_b200 import build
+    build.build()
+    from paper_2511_00603_b200 import epara
+    return epara
+
+
+def test_plan_names_the_kernel_by_rows(E):
+    """The 1B decoder's down projection from one row to thousands."""
+    kinds = [E.epara_gemm_plan(m, 2048, 8192, E.EPI_RESID_F32)[0] for m in (1, 16, 17, 128, 1100, 8192)]
+    assert kinds == ["stream", "stream", "swapped", "swapped", "swapped pairs", "tile pairs"]
+    assert E.epara_gemm_plan(100, 1024, 1024) == ("stream", 16, 1)        # a matrix of 2^20 elements
+
+
+@pytest.mark.parametrize("bad", [(0, 8, 8), (8, 0, 8), (8, 8, 0)])
+def test_plan_refuses_empty_problems(E, bad):
+    with pytest.raises(E.EparaError):
+        E.epara_gemm_plan(*bad)
+    assert E.lib.epara_gemm_plan(8, 8, 8, 0, 148, None, None) == E.E_INVALID
