@@ -437,7 +437,9 @@ cudaError_t launch_swap(const GemmGroup* groups, int n_groups, int total_items, 
 // fit on 148 SMs (sizes between them fit no more CTAs; one cluster too many costs a second wave: 2048 x 2048 at 256
 // rows 27 us with 16 clusters of eight, 15 on tile pairs).  A k-block costs 0.13 us + 0.7 ns per row, a seventh more once
 // most SMs are at it (they share what L2 delivers), exchange and epilogue 20 ns per row; clusters
-// of eight start later.
+// of eight start later.  (Calls on their own, W cold, against tile pairs: 2048 x 8192 at 160 / 224 / 400 rows 26.7 / 28.7 / 30.0 and
+// 41 / 41 / 42 us; 4096 x 4096 at 144 rows 25.0 and 29.7; 6144 x 4096 at 144 / 208 rows 27.8 / 29.9 and 31.8; 3072 x 2048 at 272 rows
+// 21.5 and 21.7; 768 x 3072 at 394 rows 21.7 and 23.7; 32000 x 2048 at 272 rows 66.6 and 68.6.)
 double gemm_swap_config(long long rows_cap, int N, int K, int sm_count, int* nb, int* ksplit) {
   const int tiles_n = (N + SW_BM - 1) / SW_BM, kblocks = (K + TC_BK - 1) / TC_BK;
   const int tiles_m = (int)((rows_cap + GEMM_SWAP_TILE_ROWS - 1) / GEMM_SWAP_TILE_ROWS);
@@ -477,13 +479,22 @@ cudaError_t launch_gemm_swap(const GemmGroup* groups, int n_groups, int total_it
 int gemm_swap2_first(int nb) { return swap2_first(nb); }
 int gemm_swap2_tiles_n(int N) { return (N + 2 * SW_BM - 1) / (2 * SW_BM); }
 
-// The estimate, in microseconds: a k-block costs what its operands take to arrive (0.14 us + 0.3 ns a row) or its MMAs, a tile
-// 26 ns a row for exchange and epilogue; pairs of one launch: 74 clusters of two CTAs or 33 of four are resident.  Within 10 % of
-// measured launches: 2048 x 8192 at 536 rows 23.3 us with four row tiles of 160 and two k ranges (tile pairs, three row tiles of which
-// the last has 24 live rows: 32.6), at 509 rows 22.0 (one-CTA tiles 25.5), at 1000 32.9 (34.6); 16384 x 2048 at 280 rows 23.5 (tile
-// pairs 29.1), but at 536 rows, where the tiles take two rounds, 43.4 against 40.2.  With a short K most of a tile's W is requested
-// before the dependency wait, which a launch on its own does not show: one image through ViT-B (K 768) 578 us a step with its
-// projections on tile pairs, 549 here.
+// The estimate, in microseconds: a k-block costs what its operands take to arrive (0.14 us + 0.3 ns a row; two ranges of a K of 4096
+// and more on all resident pairs 8 ns on top: W is then asked for twice as fast) or its MMAs, a tile
+// 26 ns a row for exchange and epilogue; pairs of one launch: 74 clusters of two CTAs or 33 of four are resident.  Chosen from 129 rows
+// (N and K decide) to some three thousand.  Calls on their own, W cold, the call's own 6 to 9 us included, against tile pairs:
+//   2048 x 8192    513 / 1100 / 1280 / 1536 / 1792 / 2500 / 3000 rows  33.7 / 46 / 44 / 50 / 54 / 73 / 83  and  44 / 54 / 54 / 56 / 56 / 93 / 95
+//   4096 x 14336   400 / 536 / 1100 / 1536 / 1792 rows                 59 / 66 / 101 / 130 / 155           and  71 / 87 / 153 / 155 / 159
+//   4096 x 4096    256 / 536 / 1100 / 1536 rows                        25.6 / 31.8 / 43 / 53               and  29.7 / 35.9 / 55 / 57
+//   3072 x 2048    192 / 1600 / 1900 rows                              20.5 / 32.8 / 33.8                  and  21.6 / 36.9 / 35.9
+//   16384 x 2048   288 rows                                            42                                  and  46
+// and against the form on one CTA, where the term for long K decides: 2048 x 8192 at 336 rows 30.6 and 29.1, at 512 31.8 and 34.8;
+// 4096 x 14336 at 192 rows 49.7 and 44.3, at 256 50.4 and 52.2; 4096 x 4096 at 129 rows 25.7 and 25.0, at 208 25.6 and 27.1.
+// Whole steps: 1B decoder, a prompt of 340 tokens 1484 us without that term and 1463 with it, 8B decoder, 144 tokens 4433 and 4392.
+// Products it still gets wrong by more than a twentieth: 768 x 768 at 577 to 768 rows (17.4 us, tile pairs 15.4; a step of three images
+// through ViT-B takes the same time with either).
+// With a short K most of a tile's W is requested before the dependency wait, which a launch on its own does not show: one image through
+// ViT-B (K 768) 578 us a step with its projections on tile pairs, 549 here.
 double gemm_swap2_config(long long rows_cap, int N, int K, int sm_count, int* nb, int* ksplit) {
   const int tiles_n = gemm_swap2_tiles_n(N), kblocks = (K + TC_BK - 1) / TC_BK;
   const double start = kblocks <= 16 ? 7.0 : 8.5;
@@ -493,12 +504,13 @@ double gemm_swap2_config(long long rows_cap, int N, int K, int sm_count, int* nb
   for (int tiles_m = (int)((rows_cap + GEMM_SWAP2_TILE_ROWS - 1) / GEMM_SWAP2_TILE_ROWS); tiles_m <= 8; ++tiles_m) {
     const int rows = (int)(((rows_cap + tiles_m - 1) / tiles_m + 31) / 32 * 32);
     if (rows < 64) break;
-    const double k_block = std::max(0.14 + 0.00031 * rows, 0.00112 * rows), tile = 0.026 * rows;
+    const double tile = 0.026 * rows;
     for (int s = 1; s <= 2; ++s) {
       const int tiles = tiles_n * tiles_m, fit = s == 1 ? sm_count / 2 : sm_count * 33 / 148;
       if (s == 2 && (tiles > fit || kblocks < 8)) continue;
       const int rounds = (tiles + fit - 1) / fit;
-      const double t = start + rounds * (tile + (kblocks + s - 1) / s * k_block) + (rounds - 1) * 3.0;
+      const double arrival = 0.14 + 0.00031 * rows + (s == 2 && kblocks >= 64 && tiles >= 0.95 * fit ? 0.008 : 0.0);
+      const double t = start + rounds * (tile + (kblocks + s - 1) / s * std::max(arrival, 0.00112 * rows)) + (rounds - 1) * 3.0;
       if (*nb == 0 || t < best) { best = t; *nb = rows; *ksplit = s; }
     }
   }

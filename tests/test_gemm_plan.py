@@ -22,3 +22,17 @@ def test_plan_refuses_empty_problems(E, bad):
     with pytest.raises(E.EparaError):
         E.epara_gemm_plan(*bad)
     assert E.lib.epara_gemm_plan(8, 8, 8, 0, 148, None, None) == E.E_INVALID
+
+
+# rows, N, K, epilogue flags, kernel and tile that measured faster
+MEASURED = [
+    (336, 2048, 8192, 8, "swapped", 176), (400, 2048, 8192, 8, "swapped", 208), (512, 2048, 8192, 8, "swapped pairs", 128),
+    (192, 4096, 14336, 8, "swapped", 192), (224, 4096, 14336, 8, "swapped", 224), (256, 4096, 14336, 8, "swapped pairs", 128),
+    (129, 4096, 4096, 8, "swapped", 144), (208, 4096, 4096, 8, "swapped pairs", 128), (256, 6144, 4096, 0, "swapped pairs", 96),
+    (1100, 2048, 8192, 8, "swapped pairs", 288), (3000, 2048, 8192, 8, "swapped pairs", 384), (8192, 2048, 8192, 8, "tile pairs", 256),
+]
+
+
+@pytest.mark.parametrize("rows,N,K,epi,kernel,tile", MEASURED)
+def test_plan_takes_the_kernel_that_measured_faster(E, rows, N, K, epi, kernel, tile):
+    assert E.epara_gemm_plan(rows, N, K, epi)[:2] == (kernel, tile)
