@@ -58,6 +58,8 @@ constexpr int SW_RING_BYTES_2 = 104 * 1024;      // two CTAs per SM: launches wi
                                                  // MMA-issuing thread per SM and no second wave pay (the LM head:
                                                  // 45 -> 31 us at 128 rows), while launches that fit one wave were a
                                                  // little faster with the deeper ring
+// (the exchange of a tile's partial sums, a row of 128 columns in fp32 for each of its rows, lies over the idle ring)
+static_assert(GEMM_SWAP2_TILE_ROWS * SW_BM * 4 <= SW_RING_BYTES_1 && GEMM_SWAP_TILE_ROWS * SW_BM * 4 <= SW_RING_BYTES_1, "exchange buffer");
 constexpr int SW_W_STAGES_MAX = 10;
 constexpr int SW_A_STAGES_MAX = 8;
 constexpr int SW_EPI_WARPS = 8;

@@ -36,3 +36,12 @@ MEASURED = [
 @pytest.mark.parametrize("rows,N,K,epi,kernel,tile", MEASURED)
 def test_plan_takes_the_kernel_that_measured_faster(E, rows, N, K, epi, kernel, tile):
     assert E.epara_gemm_plan(rows, N, K, epi)[:2] == (kernel, tile)
+
+
+def test_gpu_problems_get_the_kernels_they_are_written_for(E):
+    """The GPU tests of a kernel assert its plan before they run; the same here, where a changed estimate shows without a GPU."""
+    from tests import test_gpu_gemm_choice as choice, test_gpu_swap_pairs as pairs
+    flags = {"bias": E.EPI_BIAS, "gelu": E.EPI_GELU, "swiglu": E.EPI_SWIGLU, "resid": E.EPI_RESID_F32}
+    for want, (M, N, K, fl) in ([(("tile pairs", 128, 1), c) for c in choice.PAIRS] + [(("swapped", nb, s), c) for nb, s, c in choice.ONE_CTA] +
+                                [(("swapped pairs", nb, s), c) for nb, s, c in pairs.CASES]):
+        assert E.epara_gemm_plan(M, N, K, sum(flags[f] for f in fl)) == want, (M, N, K, fl)

@@ -116,3 +116,50 @@ def test_models_of_one_step_have_the_bits_of_steps_of_their_own(mods):
             assert torch.equal(a, b) and ia == ib
         assert all(torch.equal(p, q) for p, q in zip(pools, after))
     srv.close()
+
+
+def test_attention_launches_of_six_kinds_side_by_side(mods):
+    """One layer's attention as prompt chunks of both head sizes, encoders, and decode requests of three shapes (tensor cores with head
+    sizes 64 and 128 and a merge kernel behind each, CUDA cores with 32): every answer and cache has the bits of steps of one model."""
+    E, server = mods
+    srv = server.Server(workspace_bytes=2 << 30)
+    rng = np.random.default_rng(950)
+    reqs, pools = [], []
+    # (the encoder's second attention falls into the same sweep as the decoders' second)
+    v = synth.make_vit(d=128, n_layers=2, n_heads=2, mlp=256, n_cls=50, seed=951, device=DEV, std=0.05, perturb=0.2)
+    x = synth.make_images(7, seed=952, device=DEV)
+    reqs.append((srv.add_model(v, max_batch=7), [dict(x=x[i]) for i in range(7)]))
+    for k, (hd, Hq, Hkv, chunk, lens) in enumerate(((64, 16, 4, 200, [900, 17, 300]), (128, 8, 4, 130, [520, 33]), (64, 8, 8, 0, [1500, 256, 5]),
+                                                    (32, 8, 4, 0, [700, 40]))):
+        p = synth.make_decoder(d=256, n_layers=2, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=hd, ffn=512, vocab=300, seed=953 + k, device=DEV,
+                               std=0.05, perturb=0.2)
+        new, old = [1] * len(lens) + [chunk] * (chunk > 0), lens + [45] * (chunk > 0)
+        pages = [-(-(a + b) // synth.PAGE) for a, b in zip(old, new)]
+        order = rng.permutation(sum(pages)).astype(np.int32)
+        pool = synth.make_kv_pool(2, sum(pages), Hkv, hd, seed=960 + k, device=DEV)
+        m = srv.add_model(p, kv_pool=pool, max_kv_len=1500, max_batch=sum(new))
+        one, at = [], 0
+        for n, length, k_pages in zip(new, old, pages):
+            toks = [int(t) for t in rng.integers(0, 300, n)]
+            one.append(dict(kv_len=length, table=torch.as_tensor(order[at:at + k_pages], device=DEV), **(dict(tokens=toks) if n > 1 else dict(token=toks[0]))))
+            at += k_pages
+        reqs.append((m, one))
+        pools.append((pool, pool.clone()))
+
+    def run(groups):
+        t = [srv.submit(m, E.CAT_FS, **kw) for m, one in groups for kw in one]
+        srv.step()
+        torch.cuda.synchronize()
+        out = [srv.collect(i) for i in t]
+        assert all(s == E.OK for s, _, _ in out)
+        return [(l.clone(), int(a.item())) for _, l, a in out]
+
+    alone = [r for g in reqs for r in run([g])]
+    after = [pool.clone() for pool, _ in pools]
+    for _ in range(3):
+        for pool, before in pools:
+            pool.copy_(before)
+        for (a, ia), (b, ib) in zip(alone, run(reqs)):
+            assert torch.equal(a, b) and ia == ib
+        assert all(torch.equal(pool, q) for (pool, _), q in zip(pools, after))
+    srv.close()

@@ -74,3 +74,45 @@ def test_prompts_do_not_depend_on_the_last_round(mods, ffn, lens):
         assert torch.equal(part[0], whole[i][0]) and part[1] == whole[i][1]
     assert torch.equal(pool, pool_whole)
     srv.close()
+
+
+# d 2048 on 74 pairs, 256-wide tiles, K 2048: the last columns of tiles, with a bias
+@pytest.mark.parametrize("mlp,n", [
+    (2080, 23),     # FC1: one column, 64 wide, of which 32 exist
+    (4096, 20),     # QKV: one column in tiles 64 wide
+    (2176, 15),     # FC1: three columns in tiles 128 wide
+])
+def test_encoder_answers_do_not_depend_on_columns_of_the_last_round(mods, mlp, n):
+    E, server = mods
+    p = synth.make_vit(d=2048, n_layers=1, n_heads=32, mlp=mlp, n_cls=40, seed=962, device=DEV, std=0.03, perturb=0.2)
+    x = synth.make_images(n, seed=963, device=DEV)
+    srv = server.Server(workspace_bytes=1 << 30)
+    m = srv.add_model(p, max_batch=n)
+    whole = _answers(E, srv, [srv.submit(m, E.CAT_FS, x=x[i]) for i in range(n)])
+    for a in range(0, n, 3):                                   # three images: one round
+        part = _answers(E, srv, [srv.submit(m, E.CAT_FS, x=x[i]) for i in range(a, min(n, a + 3))])
+        for (u, iu), (v, iv) in zip(part, whole[a:a + 3]):
+            assert torch.equal(u, v) and iu == iv
+    srv.close()
+
+
+def test_a_last_round_of_several_models(mods):
+    """Two encoders of one shape in one launch, 50 and 14 images: the rows that are cut finer are those of the one with more tiles,
+    whichever it is."""
+    E, server = mods
+    srv = server.Server(workspace_bytes=1 << 30)
+    models = []
+    for k in range(2):
+        p = synth.make_vit(d=512, n_layers=2, n_heads=8, mlp=2048, n_cls=40, seed=964 + k, device=DEV, std=0.05, perturb=0.2)
+        models.append((srv.add_model(p, max_batch=50), synth.make_images(50, seed=966 + k, device=DEV)))
+
+    def submit(k, a, b):
+        m, x = models[k]
+        return [srv.submit(m, E.CAT_FS, x=x[i]) for i in range(a, b)]
+
+    alone = [[r for a in range(0, 50, 8) for r in _answers(E, srv, submit(k, a, min(50, a + 8)))] for k in range(2)]
+    for n0, n1 in ((50, 14), (14, 50)):
+        both = _answers(E, srv, submit(0, 0, n0) + submit(1, 0, n1))
+        for (u, iu), (v, iv) in zip(both, alone[0][:n0] + alone[1][:n1]):
+            assert torch.equal(u, v) and iu == iv
+    srv.close()
