@@ -23,15 +23,22 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
-# DRAM bytes (read + write) per tensor-core GEMM launch of the mixed step, from an ncu pass over the GEMM launches of
-# a step (80 tile-pair launches: 6.24 GB read + 3.60 GB written; 12 fused MLP-block launches: 2.70 GB read + 1.05 GB
-# written; 16 swapped-operand launches: 0.64 GB read; the 65 weight-streaming launches moved 2.08 GB).  Not measured by
-# this run: the profile it comes from is named beside it in the JSON line.  Set to None when the GEMM kernels change.
-GEMM_TC_TRAFFIC_PER_LAUNCH_MIXED = 14229706240 / 108
+# DRAM bytes (read + write) of the mixed step's tensor-core GEMM launches, from an ncu pass over the GEMM launches of a step (61
+# tile-pair launches: 5.84 GB read + 3.55 GB written; 12 fused MLP-block launches: 2.70 GB read + 1.00 GB written; 49 swapped-operand
+# launches on CTA pairs: 1.05 GB read; the 65 weight-streaming launches moved 2.08 GB), and their number.  Not measured by this run: the
+# profile it comes from is named beside it in the JSON line.  A step with another number of launches has other kernels: no figure then.
+GEMM_TC_TRAFFIC_MIXED, GEMM_TC_LAUNCHES_MIXED = 14137526272, 122
 GEMM_TRAFFIC_SOURCE = "profiles/gemm_kernels_mixed_step_dram_traffic.md (one ncu pass, dram__bytes_read.sum + dram__bytes_write.sum)"
 
 E2E_BUFS = 4          # device input buffers per instance in the end-to-end loop
 PROFILE_EVERY = 5     # one step in five of the timed region carries per-launch events
+
+
+
+def gemm_traffic(stress, launches):
+    """DRAM bytes of a tensor-core GEMM launch, where the profile is one of this step."""
+    return None if stress or launches != GEMM_TC_LAUNCHES_MIXED else GEMM_TC_TRAFFIC_MIXED / launches
+
 
 METRIC = "mixed-category requests/s"
 UNIT = "requests/s"
@@ -573,8 +580,8 @@ def run_gpu(args):
                 "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                 "frac_of_burst_peak": ach / peaks["bf16_tflops"], "frac_of_sustained_peak": ach / peaks["bf16_tflops_sustained"],
                 "sm_mhz_median": clocks.get("sm_mhz"), "launches_per_step": prof["gemm"][1], "ms_per_step": tc_ms,
-                "traffic": None if (stress or GEMM_TC_TRAFFIC_PER_LAUNCH_MIXED is None) else GEMM_TC_TRAFFIC_PER_LAUNCH_MIXED,
-                "traffic_source": None if stress else GEMM_TRAFFIC_SOURCE,
+                "traffic": gemm_traffic(stress, prof["gemm"][1]),
+                "traffic_source": None if gemm_traffic(stress, prof["gemm"][1]) is None else GEMM_TRAFFIC_SOURCE,
                 "peak_source": peaks["source"] + (" (burst: median SM clock within 10 % of max)" if near_max else " (sustained)")}
     elif dom == "attn_dec":
         ach = per_step(kvbytes) / (prof["attn_dec"][0] / 1e3) / 1e9

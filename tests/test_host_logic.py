@@ -185,3 +185,11 @@ def test_collect_extension_is_named_for_this_interpreter(E, monkeypatch, tmp_pat
     monkeypatch.setattr(build, "FAST_LIB", str(tagged))
     build.build_fastcall()
     assert os.listdir(tmp_path) == [tagged.name]
+
+
+def test_bench_gives_dram_traffic_only_for_the_profiled_step():
+    """The profile's figure belongs to a step of that many launches; other kernels, another number, no figure."""
+    import bench
+    n = bench.GEMM_TC_LAUNCHES_MIXED
+    assert bench.gemm_traffic(False, n) == bench.GEMM_TC_TRAFFIC_MIXED / n
+    assert bench.gemm_traffic(False, n - 14) is None and bench.gemm_traffic(True, n) is None
