@@ -212,6 +212,9 @@ int epara_step(epara_ctx*, void* cuda_stream, long long now_ns, epara_step_info*
  * step only.  INVALID for an unknown (or already collected) ticket.  A ticket still queued is PENDING.
  * An answer stays available until it is collected, however many steps run in between. */
 int epara_collect(epara_ctx*, uint64_t ticket, epara_output* out);
+/* The same for answers that an epara_collect or epara_step before has already found: PENDING for a request of a step that was still
+ * running then.  Never calls the CUDA driver. */
+int epara_collect_ready(epara_ctx*, uint64_t ticket, epara_output* out);
 
 /* With cfg.profile = 1: per kernel kind, total milliseconds and launch count of the most
  * recent finished step (arrays of EPARA_K_COUNT).  Synchronises that step.  */

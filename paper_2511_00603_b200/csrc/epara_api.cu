@@ -1480,24 +1480,11 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
   return slot.launch_status;
 }
 
-int epara_collect(epara_ctx* c, uint64_t ticket, epara_output* out) {
+int epara_collect_ready(epara_ctx* c, uint64_t ticket, epara_output* out) {
   if (!c) return EPARA_E_INVALID;
   auto it = c->tickets.find(ticket);
   if (it == c->tickets.end()) return EPARA_E_INVALID;
-  if (it->second.state == T_QUEUED) return EPARA_PENDING;
-  if (it->second.state == T_INFLIGHT) {
-    Slot& s = c->slots[it->second.step % N_SLOTS];
-    if (s.step_id == it->second.step && s.busy) {
-      cudaError_t e = cudaEventQuery(s.done);
-      if (e == cudaErrorNotReady) return EPARA_PENDING;
-      if (e != cudaSuccess) { s.launch_status = EPARA_E_CUDA; *s.status_host = 0; }
-      finalize_slot(c, s);            // answers every request of that step, this one included
-    }
-    if (it->second.state != T_DONE) {   // (cannot happen: an in-flight ticket's step is always in its slot)
-      it->second.state = T_DONE;
-      it->second.result = EPARA_E_CUDA;
-    }
-  }
+  if (it->second.state != T_DONE) return EPARA_PENDING;
   const Ticket t = it->second;
   if (out) {
     out->status = t.result;
@@ -1509,6 +1496,25 @@ int epara_collect(epara_ctx* c, uint64_t ticket, epara_output* out) {
   }
   c->tickets.erase(it);
   return t.result;
+}
+
+int epara_collect(epara_ctx* c, uint64_t ticket, epara_output* out) {
+  const int r = epara_collect_ready(c, ticket, out);
+  if (r != EPARA_PENDING) return r;
+  Ticket& t = c->tickets.find(ticket)->second;
+  if (t.state == T_QUEUED) return EPARA_PENDING;
+  Slot& s = c->slots[t.step % N_SLOTS];
+  if (s.step_id == t.step && s.busy) {
+    cudaError_t e = cudaEventQuery(s.done);
+    if (e == cudaErrorNotReady) return EPARA_PENDING;
+    if (e != cudaSuccess) { s.launch_status = EPARA_E_CUDA; *s.status_host = 0; }
+    finalize_slot(c, s);                // answers every request of that step, this one included
+  }
+  if (t.state != T_DONE) {              // (cannot happen: an in-flight ticket's step is always in its slot)
+    t.state = T_DONE;
+    t.result = EPARA_E_CUDA;
+  }
+  return epara_collect_ready(c, ticket, out);
 }
 
 int epara_set_max_profile_launches(epara_ctx* c, int n) {

@@ -73,7 +73,7 @@ EXPORTS = ["epara_init", "epara_register_model", "epara_submit", "epara_submit_m
            "epara_gemm_scratch_bytes", "epara_gemm_scratch_bytes_for", "epara_decode_attention", "epara_decode_attention_scratch_bytes",
            "epara_decode_attention_static", "epara_static_scratch_bytes", "epara_decode_attention_static_status",
            "epara_set_max_profile_launches", "epara_selftest_bounded_wait", "epara_offload_probabilities", "epara_simulate",
-           "epara_place_sssp", "epara_gemm_plan"]
+           "epara_place_sssp", "epara_gemm_plan", "epara_collect_ready"]
 
 lib.epara_init.argtypes = [C.POINTER(Config), C.POINTER(C.c_void_p)]
 lib.epara_register_model.argtypes = [C.c_void_p, C.POINTER(ModelDesc), C.POINTER(C.c_int)]
@@ -82,6 +82,7 @@ lib.epara_submit_many.argtypes = [C.c_void_p, C.c_int, C.c_int, C.POINTER(Inputs
                                   C.POINTER(C.c_int)]
 lib.epara_step.argtypes = [C.c_void_p, C.c_void_p, C.c_longlong, C.POINTER(StepInfo)]
 lib.epara_collect.argtypes = [C.c_void_p, C.c_uint64, C.POINTER(Output)]
+lib.epara_collect_ready.argtypes = [C.c_void_p, C.c_uint64, C.POINTER(Output)]
 lib.epara_step_profile.argtypes = [C.c_void_p, C.POINTER(C.c_float), C.POINTER(C.c_int)]
 lib.epara_set_profile.argtypes = [C.c_void_p, C.c_int]
 lib.epara_destroy.argtypes = [C.c_void_p]
@@ -312,7 +313,8 @@ class Context:
 # The same method without a foreign-function call per answer (csrc/fastcall.cpp).
 try:
     from . import _fastcall
-    Context.epara_collect = _fastcall.collect_method(C.cast(lib.epara_collect, C.c_void_p).value, Output, Context.epara_collect, "_handle")
+    Context.epara_collect = _fastcall.collect_method(C.cast(lib.epara_collect, C.c_void_p).value, C.cast(lib.epara_collect_ready, C.c_void_p).value, PENDING,
+                                                     Output, Context.epara_collect, "_handle")
 except ImportError:
     pass
 

@@ -137,14 +137,15 @@ def test_collect_method_without_ctypes_takes_what_the_general_one_takes(E):
 
 
 def test_collect_method_lets_other_threads_run(E):
-    """The compiled method calls the library without the interpreter lock.  The C library's usleep stands in for epara_collect: it takes
-    its microseconds where the context's address goes."""
+    """The compiled method asks for an answer that is not there yet without the interpreter lock.  The C library's usleep stands in for
+    epara_collect: it takes its microseconds where the context's address goes."""
     from paper_2511_00603_b200 import _fastcall
 
     class Sleeper:
         _handle = 300_000
     usleep = ctypes.cast(ctypes.CDLL(None).usleep, ctypes.c_void_p).value
-    Sleeper.collect = _fastcall.collect_method(usleep, E.Output, None, "_handle")
+    not_there = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.c_uint64, ctypes.c_void_p)(lambda ctx, ticket, out: E.PENDING)
+    Sleeper.collect = _fastcall.collect_method(usleep, ctypes.cast(not_there, ctypes.c_void_p).value, E.PENDING, E.Output, None, "_handle")
     inside = threading.Event()
 
     def call():
@@ -193,3 +194,18 @@ def test_bench_gives_dram_traffic_only_for_the_profiled_step():
     n = bench.GEMM_TC_LAUNCHES_MIXED
     assert bench.gemm_traffic(False, n) == bench.GEMM_TC_TRAFFIC_MIXED / n
     assert bench.gemm_traffic(False, n - 14) is None and bench.gemm_traffic(True, n) is None
+
+
+def test_collect_method_asks_once_for_an_answer_that_is_there(E):
+    from paper_2511_00603_b200 import _fastcall
+    calls = []
+    proto = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.c_uint64, ctypes.c_void_p)
+    fns = [proto(lambda ctx, ticket, out, k=k: calls.append((k, ctx, ticket)) or (E.PENDING if k == "ready" and ticket == 1 else E.E_TIMEOUT))
+           for k in ("collect", "ready")]
+
+    class Ctx:
+        _handle = 4096
+    Ctx.collect = _fastcall.collect_method(*(ctypes.cast(f, ctypes.c_void_p).value for f in fns), E.PENDING, E.Output, None, "_handle")
+    assert Ctx().collect(2)[0] == E.E_TIMEOUT and calls == [("ready", 4096, 2)]
+    assert Ctx().collect(1)[0] == E.E_TIMEOUT and calls[1:] == [("ready", 4096, 1), ("collect", 4096, 1)]
+    assert E.lib.epara_collect_ready(None, 1, None) == E.E_INVALID
