@@ -13,7 +13,7 @@ namespace epara {
 // Rule: a kernel touches nothing that an earlier kernel of the stream writes or reads
 // before its pdl_wait(); weights and the step's descriptors (uploaded by a copy that completes
 // before the first kernel) may be read earlier.  Every kernel waits at least once, so completion
-// is transitive along the stream.
+// is transitive along the stream.  (Launches `beside` another one wait at their end: see pdl_begin().)
 //
 // Why the trigger follows the wait: what a kernel does before its wait is mostly requests for weights.  With the trigger
 // at the top of each kernel these piled up several kernels deep, while the kernels they were early for -- norms,
@@ -31,7 +31,9 @@ __device__ __forceinline__ void pdl_wait() { pdl_wait_only(); pdl_trigger(); }
 // them waits as above; the others run `beside` it: they do not wait at their start -- they could only be launched once every block
 // of the kernel before had triggered, hence after all kernels before the wave were complete -- and one block of theirs waits
 // at its end, so that completion stays transitive.  Without a wait a kernel's L1 may hold old lines: what earlier kernels wrote
-// is read past L1 (TMA, cp.async.cg, ld.cg).  (512-token chunk beside 24 decode requests, 1B decoder: 2637 us a step with every
+// is read past L1 (TMA, cp.async.cg, ld.cg).  That such reads see it rests on the hardware, not on a written guarantee: the kernels
+// before the wave were complete, their writes in L2, when the wave's first launch passed its own wait, and CUDA promises visibility only
+// to a thread that has waited itself.  (512-token chunk beside 24 decode requests, 1B decoder: 2637 us a step with every
 // launch waiting, 2519 like this; the saturated mix 13100 and 13040.)
 __device__ __forceinline__ void pdl_begin(int beside) {
   if (!beside) pdl_wait_only();

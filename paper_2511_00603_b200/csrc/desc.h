@@ -55,7 +55,8 @@ constexpr int TMAP_ALIGN = 128;
 struct alignas(TMAP_ALIGN) GemmGroup {
   CUtensorMap tmA;
   CUtensorMap tmW;
-  CUtensorMap tmC;   // (swapped operands on pairs: the activations for a tile's second MMA)  output, written by TMA from the epilogue's staging rows: bf16 [rows, N] with a
+  CUtensorMap tmC;   // swapped operands on pairs: A again, in boxes for a tile's second MMA (their output leaves by plain stores).
+                     // Tile pairs: the output, written by TMA from the epilogue's staging rows: bf16 [rows, N] with a
                      // 32 x 32 box (SwiGLU: [rows, N/2], 16 x 32), or fp32 [rows, N] with a 16 x 32 box
                      // for the residual update (TMA reduce-add)
   const bf16* A;

@@ -36,7 +36,7 @@ constexpr int N_SWAP = PASS_SWAP2 - PASS_SWAP, N_SWAP2 = PASS_MLP - PASS_SWAP2; 
 inline int swap_index(int ksplit) { return ksplit >= 8 ? 3 : ksplit >= 4 ? 2 : ksplit >= 2 ? 1 : 0; }
 // The launch of a GEMM wave that takes a group.
 inline int gemm_pass(const GemmGroup& g) {
-  return g.stream == GEMM_SWAP ? PASS_SWAP + swap_index(g.ksplit) : g.stream == GEMM_SWAP2 ? PASS_SWAP2 + swap_index(g.ksplit) : g.stream == 4 ? PASS_MLP : g.stream;
+  return g.stream == GEMM_SWAP ? PASS_SWAP + swap_index(g.ksplit) : g.stream == GEMM_SWAP2 ? PASS_SWAP2 + swap_index(g.ksplit) : g.stream == GEMM_MLP ? PASS_MLP : g.stream;
 }
 
 constexpr int FINE_BN[2] = {64, 128}, FINE_MIN_K = 2048;        // the tile-pair kernel's last round (see fine_tail in epara_step)
@@ -127,7 +127,7 @@ struct Op {
   AttnPrefillGroup apre;
   GemmGroup gemm;
   CUtensorMap tmW_fine[2];   // tile pairs: W in the boxes of tiles FINE_BN[i] wide (see fine_tail())
-  MlpGroup mlp;          // EPARA_K_GEMM with gemm.stream == 4: FC1, GELU, FC2 and the residual update in one kernel ...
+  MlpGroup mlp;          // EPARA_K_GEMM with gemm.stream == GEMM_MLP: FC1, GELU, FC2 and the residual update in one kernel ...
   GemmGroup fc1, fc2;    // ... and the same as two GEMMs (same bits), for the tiles of a last round that few pairs would work
   NormGroup norm;
   GatherGroup gather;
@@ -277,9 +277,9 @@ bool add_gemm(Builder& bl, Model* m, const void* A, int lda, long long rows_cap,
   op.weight_bytes = 2.0 * N * K;
   g.ksplit = 1;
   if (bl.gemm_impl == EPARA_GEMM_SIMT) {
-    g.stream = 0;
+    g.stream = GEMM_SIMT;
   } else if (!one_sum && gemm_stream_eligible(max_rows, N, K)) {
-    g.stream = 1; g.bn = 16;
+    g.stream = GEMM_STREAM; g.bn = 16;
   } else if (one_sum) {
     g.stream = GEMM_PAIR;
     gemm_pair_config(max_rows, N, K, g.epi, sm_count, &g.bn);
@@ -295,7 +295,7 @@ bool add_gemm(Builder& bl, Model* m, const void* A, int lda, long long rows_cap,
 }
 
 // An encoder's MLP block as one fused op (see MlpGroup).  gemm.N / gemm.K carry the shapes for the step's
-// flop and byte accounting; gemm.stream == 4 routes the op to the fused kernel's launch.
+// flop and byte accounting; gemm.stream == GEMM_MLP routes the op to the fused kernel's launch.
 bool add_mlp(Builder& bl, Model* m, const void* X, long long rows_cap, const void* W1, const void* b1, const void* W2,
              const void* b2, float* Z, bf16* hidden, int d, int F, int rows_per_req) {
   Op op;
@@ -308,7 +308,7 @@ bool add_mlp(Builder& bl, Model* m, const void* X, long long rows_cap, const voi
   m->ops.pop_back();
   op.kind = EPARA_K_GEMM;
   op.rows_per_req = rows_per_req;
-  op.gemm.stream = 4; op.gemm.N = d; op.gemm.K = F; op.gemm.ksplit = 1; op.gemm.bn = d;
+  op.gemm.stream = GEMM_MLP; op.gemm.N = d; op.gemm.K = F; op.gemm.ksplit = 1; op.gemm.bn = d;
   op.weight_bytes = 2.0 * 2.0 * d * F;
   MlpGroup& g = op.mlp;
   g.b1 = (const bf16*)b1; g.b2 = (const bf16*)b2; g.d = d; g.F = F; g.c_rows = (int)rows_cap;
@@ -1041,9 +1041,12 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
   // Tile pairs: a last round with few tiles takes as long as a full one.  The last row tiles of a group, or its last columns of
   // tiles, that make up at least those tiles are cut finer, 64 or 128 columns wide (the narrowest that still fits the round: a k-block
   // of such a tile takes some 0.65 and 0.8 of a 256-wide one's time), where the launch's groups have tiles of one kind.  An element's k
-  // order does not depend on the width: the same bits.  1B decoder, four prompts of 2048 tokens 16335 -> 16151 us a step, three of
-  // 1024 6193 -> 6144, one of 1300 3370 -> 3350; 8B, 1024 tokens 14496 -> 14379.  Not with K below 2048: there a round is 3 us and the
-  // fetch of the finer group's descriptor and map 1 (64 images of ViT-B, K 768, 2968 -> 2980; 203 of ViT-S 3176 -> 3193).
+  // order does not depend on the width: the same bits. Step
+  // times without and with it (means of three contexts each, taken in turn; runs of one differ by 0.2 % in the mean): 1B decoder, four
+  // prompts of 2048 tokens 16680 and 16514 us, three of 1700 10828 and 10592, three of 1024 6308 and 6194, two of 1400 5988 and 5925, one of
+  // 1300 3420 and 3384, of 1000 2617 and 2564; 8B, 1024 tokens 14689 and 14630, 900 14366 and 14250, 600 no difference.  Not with K below
+  // 2048: there a round is 3 us and the fetch of the finer group's descriptor and map 1 (64 images of ViT-B, K 768, 2968 -> 2980; 203 of
+  // ViT-S 3176 -> 3193).
   struct FineTail { Active* a; int tiles_m, tiles_n, width; };   // of the group's tiles: the last row tiles or the last column tiles
   auto fine_tail = [&](const std::vector<Active*>& who) {
     const FineTail no = {nullptr, 0, 0, 0};
@@ -1270,7 +1273,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
           }
           case EPARA_K_GEMM: {
             if (gemm_pass(op.gemm) != pass) break;             // another pass takes it
-            if (op.gemm.stream == 4) {
+            if (op.gemm.stream == GEMM_MLP) {
               MlpGroup mg = op.mlp;
               mg.M = rows;
               mg.tiles_m = (rows + 2 * TC_BM - 1) / (2 * TC_BM);
@@ -1289,7 +1292,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
             }
             GemmGroup g = op.gemm;
             g.M = rows;
-            if (g.stream == 3) {
+            if (g.stream == GEMM_SWAP) {
               g.tiles_m = (rows + g.bn - 1) / g.bn; g.tiles_n = gemm_swap_tiles_n(g.N);
               g.tile_start = total;
               total += g.tiles_m * g.tiles_n;
@@ -1298,7 +1301,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
               g.tiles_m = (rows + g.bn - 1) / g.bn; g.tiles_n = gemm_swap2_tiles_n(g.N);
               g.tile_start = total;
               total += g.tiles_m * g.tiles_n;
-            } else if (g.stream == 2) {
+            } else if (g.stream == GEMM_PAIR) {
               g.tiles_m = (rows + 2 * TC_BM - 1) / (2 * TC_BM) - (a == fine.a ? fine.tiles_m : 0);
               g.tiles_n = (g.N + g.bn - 1) / g.bn - (a == fine.a ? fine.tiles_n : 0);
               g.tile_start = total;
@@ -1318,7 +1321,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
             inf.gemm_groups++;
             inf.gemm_flops += 2.0 * rows * g.N * g.K;
             inf.weight_bytes += op.weight_bytes;
-            if (g.stream == 1) {
+            if (g.stream == GEMM_STREAM) {
               inf.stream_gemm_flops += 2.0 * rows * g.N * g.K;
               inf.stream_weight_bytes += op.weight_bytes;
             }
@@ -1390,7 +1393,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
           g.tile_start = -(g.tiles_m - cut_tiles) * g.tiles_n;           // items 0 .. are the last tiles
           Launch R;
           memset(&R, 0, sizeof(R));
-          R.kind = kind; R.n_groups = 1; R.p0 = cut_tiles * g.tiles_n; R.p2 = 2;
+          R.kind = kind; R.n_groups = 1; R.p0 = cut_tiles * g.tiles_n; R.p2 = GEMM_PAIR;
           R.beside = part == &op.fc1;              // (other rows than the fused launch; the second GEMM needs the first)
           off = align_up(off, TMAP_ALIGN);
           R.off = off;
@@ -1430,7 +1433,7 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
     const unsigned char* gp = slot.dev + L.off;
     if (prof) {
       cudaEventRecord(slot.prof[2 * li], st);
-      slot.prof_kind.push_back(L.kind == EPARA_K_GEMM && L.p2 == 1 ? (int)EPARA_K_GEMM_STREAM : L.kind);
+      slot.prof_kind.push_back(L.kind == EPARA_K_GEMM && L.p2 == GEMM_STREAM ? (int)EPARA_K_GEMM_STREAM : L.kind);
     }
     switch (L.kind) {
       case EPARA_K_GATHER: launch_gather((const GatherGroup*)gp, L.n_groups, L.p1, st); break;
@@ -1440,8 +1443,8 @@ int epara_step(epara_ctx* c, void* cuda_stream, long long now_ns, epara_step_inf
         if (L.p2 == PASS_MLP) err = launch_gemm_mlp_pair((const MlpGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st, L.beside);
         else if (L.p2 >= PASS_SWAP2) err = launch_gemm_swap2((const GemmGroup*)gp, L.n_groups, L.p0, 1 << (L.p2 - PASS_SWAP2), dev_status, c->sm_count, st, L.beside);
         else if (L.p2 >= PASS_SWAP) err = launch_gemm_swap((const GemmGroup*)gp, L.n_groups, L.p0, 1 << (L.p2 - PASS_SWAP), L.p3, dev_status, c->sm_count, st, L.beside);
-        else if (L.p2 == 1) err = launch_gemm_stream((const GemmGroup*)gp, L.n_groups, L.p0, L.p1, st);
-        else if (L.p2 == 2) err = launch_gemm_tc_pair((const GemmGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st, L.beside);
+        else if (L.p2 == GEMM_STREAM) err = launch_gemm_stream((const GemmGroup*)gp, L.n_groups, L.p0, L.p1, st);
+        else if (L.p2 == GEMM_PAIR) err = launch_gemm_tc_pair((const GemmGroup*)gp, L.n_groups, L.p0, dev_status, c->sm_count, st, L.beside);
         else launch_gemm_simt((const GemmGroup*)gp, L.n_groups, L.p0, st);
         break;
       case EPARA_K_ROPE: launch_rope_append((const RopeGroup*)gp, L.n_groups, L.p1, st); break;
@@ -1602,7 +1605,7 @@ int epara_grouped_gemm(int device, void* cuda_stream, int impl, const epara_gemm
     g.bn = 128; g.ksplit = 1;
     g.c_rows = q.M;
     if (!simt && gemm_stream_eligible(q.M, q.N, q.K)) {
-      g.stream = 1; g.bn = 16;
+      g.stream = GEMM_STREAM; g.bn = 16;
       g.tiles_m = gemm_stream_tiles_m(q.M); g.tiles_n = gemm_stream_tiles_n(q.N);
       g.tile_start = total_stream;
       if (q.M > 0) total_stream += g.tiles_m * g.tiles_n;

@@ -1,5 +1,5 @@
-// Grouped bf16 GEMM for groups of 17 to about a thousand rows (decode batches, classification heads, single images,
-// prompts of some hundred tokens): C = epi(A W^T + bias) with the operands swapped on the tensor core.
+// Grouped bf16 GEMM for groups of 17 to about a thousand rows, of few wide shapes up to some three thousand (decode batches,
+// classification heads, single images, prompts of some hundred tokens): C = epi(A W^T + bias) with the operands swapped on the tensor core.
 //
 // With so few rows the work is streaming W once, or too few output tiles to fill the chip.  The MMA's 128-row
 // operand is a tile of W (128 output columns) and the batch is the MMA's N: one tile of up to 256 rows, several of
@@ -23,7 +23,7 @@
 // columns contiguous.  No partial ever travels through global memory and the reduction order is fixed, so a
 // request's bits do not depend on timing or on what else is in the launch.
 //
-// Pairs (PAIR; some 150 to a thousand rows).  With hundreds of rows what counts is what a CTA takes in: a tile of 128 columns and 256
+// Pairs (PAIR; from 129 rows on, see gemm_swap2_config()).  With hundreds of rows what counts is what a CTA takes in: a tile of 128 columns and 256
 // rows asks for 48 KB a k-block, as much as the MMAs of one SM can use in 512 cycles, and L2 delivers 61 bytes a cycle to an SM.
 // Here a tile has 256 columns and two CTAs (cta_group::2): each loads its own 128 rows of W and half of the batch rows, the first
 // one issues M = 256 MMAs for both (two per step when the tile has more than 256 rows), and each accumulates, exchanges and writes
@@ -183,7 +183,7 @@ gemm_swap_kernel(const GemmGroup* __restrict__ groups, int n_groups, int* __rest
       }
       if (++stage == w_stages) { stage = 0; phase ^= 1u; }
     }
-    pdl_begin(BESIDE);                                    // (every thread of the kernel waits once, see common.cuh)
+    pdl_begin(BESIDE);                                    // (not beside: every thread of the kernel waits once, see common.cuh)
     if (!ok) { *abort_flag = 1; drain_sleep(200000ull); }
   } else if (warp == SW_A_WARP) {
     // ------------------------------------------------------------ TMA producer of the activations (tmA: box of nb rows)

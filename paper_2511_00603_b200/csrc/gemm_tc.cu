@@ -1,7 +1,7 @@
 // Grouped bf16 GEMM on the sm_100a tensor cores: C_g = epi(A_g W_g^T + bias_g) for groups of more than 128 rows.
 //
 // One persistent launch covers every group (one group = one model's GEMM in this wave, with its own M, N, K and tile
-// width bn in {128, 192, 256}).  Work items -- tiles of 256 rows x bn columns, each worked by two CTAs of a cluster --
+// width bn in {128, 192, 256}; 64 in a finer last round, see fine_tail in epara_api.cu).  Work items -- tiles of 256 rows x bn columns, each worked by two CTAs of a cluster --
 // are numbered group after group; pair i takes items i, i + pairs, ...  Inside a CTA the roles run concurrently:
 //   warp 0            TMA producer of A: its own 128 rows x 64 columns of every k-block;
 //   warp 18           TMA producer of W: half of the tile's W rows (plain, non-multicast cp.async.bulk.tensor;
@@ -9,7 +9,7 @@
 //   warp 1 of rank 0  MMA issuer: tcgen05.mma cta_group::2 (M 256, N bn, K 16) into one of two TMEM accumulators (256
 //                     columns each), releasing stages with tcgen05.commit (warp 1 of rank 1 prefetches residual rows);
 //   warps 2..17       epilogue: tcgen05.ld of the finished accumulator (four warps per TMEM lane quarter, a quarter of
-//                     the tile's columns each), bias / GELU / SwiGLU / fp32 residual update, bf16 store -- while the
+//                     the tile's columns each; two of them half each of a tile 64 wide), bias / GELU / SwiGLU / fp32 residual update, bf16 store -- while the
 //                     MMA warp already fills the other accumulator.
 // The K reduction of an output element is the same sequence whatever else is in the launch.
 // Every mbarrier wait is bounded: when a wait runs out the kernel records a code in *status, all roles leave their
@@ -95,7 +95,7 @@ __device__ __forceinline__ Item decode_item(const G& g, int local, int rank) {
 }
 
 // Direct epilogue of one warp for one tile, with no block-level barrier.  Warp (quarter, part) owns
-// rows quarter*32..+31 and the part-th quarter of the tile's columns.  Per chunk (32 accumulator
+// rows quarter*32..+31 and the part-th part_cols() of the tile's columns (a quarter; none is left for parts 2 and 3 of a tile 64 wide).  Per chunk (32 accumulator
 // columns; 16 for an fp32 residual) each lane turns its row's values into outputs and parks them in
 // the warp's 2 KB staging area (64-byte rows, SwiGLU 32-byte rows, 16-byte pieces in the TMA swizzle
 // pattern, which also keeps the stores free of bank conflicts); one lane then hands the 32-row box to

@@ -44,7 +44,7 @@ cudaError_t launch_gemm_swap(const GemmGroup* groups, int n_groups, int total_it
                              int sm_count, cudaStream_t st, int beside = 0);
 
 // The same on pairs of CTAs (GemmGroup::stream == 5): tiles of 256 output columns and bn batch rows (a multiple of 32, at
-// most GEMM_SWAP2_TILE_ROWS), `ksplit` (1 or 2) pairs per tile; for some 200 to a thousand rows.  Maps: tmW box 128 rows,
+// most GEMM_SWAP2_TILE_ROWS), `ksplit` (1 or 2) pairs per tile; from 129 rows to some thousand, wide shapes three thousand, where its estimate is the smallest.  Maps: tmW box 128 rows,
 // tmA box half of gemm_swap2_first(bn) rows, tmC the activations again with a box of half the rest (when there is a rest).
 constexpr int GEMM_SWAP2_TILE_ROWS = 384;
 double gemm_swap2_config(long long rows_cap, int N, int K, int sm_count, int* nb, int* ksplit);
@@ -52,7 +52,7 @@ int gemm_swap2_first(int nb);
 int gemm_swap2_tiles_n(int N);
 cudaError_t launch_gemm_swap2(const GemmGroup* groups, int n_groups, int total_items, int ksplit, int* status, int sm_count, cudaStream_t st,
                               int beside = 0);
-enum : int { GEMM_PAIR = 2, GEMM_SWAP = 3, GEMM_SWAP2 = 5 };
+enum : int { GEMM_SIMT = 0, GEMM_STREAM = 1, GEMM_PAIR = 2, GEMM_SWAP = 3, GEMM_MLP = 4, GEMM_SWAP2 = 5 };   // GemmGroup::stream
 // The kernel for a GEMM that the weight-streaming kernel does not take, with its tile (GemmGroup::bn, ksplit).
 int gemm_tc_choice(long long rows_cap, int N, int K, int epi, int sm_count, int* bn, int* ksplit);
 
@@ -86,7 +86,10 @@ constexpr int FLASH_TILE = 128;
 // With decode attention beside it the launch also leaves SMs to that one's blocks: one tile keeps the launch short while they
 // are few, two tiles leave more SMs (1B decoder, a 512-token chunk, 128 tiles: with 4 / 12 / 24 / 60 decode requests, 14 / 42 /
 // 84 / 210 blocks per SM left over, 2306 / 2409 / 2560 / 2818 us a step with one tile and 2467 / 2485 / 2525 / 2779 with two; a
-// 256-token chunk with 24 / 60 requests, 20 / 50 blocks: 1822 / 2271 and 1955 / 2236).
+// 256-token chunk with 24 / 60 requests, 20 / 50 blocks: 1822 / 2271 and 1955 / 2236; 128 and 1024 tokens with 4 to 60 requests: the choice
+// within 1 % of the better one.  Head size 128, 8B decoder, 32 layers: 256 tokens with 4 / 12 / 24 / 60 requests 6689 / 7025 / 7541 / 9615
+// with one tile and 6932 / 7224 / 7723 / 9592 with two, 512 tokens with 24 / 60 12249 / 14171 and 12344 / 14102, where runs differ by 2 %).
+// All decode blocks of the step count, whichever model's: they share the SMs left over.
 constexpr int FLASH_DEC_BLOCKS = 48;
 inline int attn_flash_tiles(long long total_tiles, int sm_count, long long dec_blocks = 0) {
   return total_tiles <= sm_count && dec_blocks <= FLASH_DEC_BLOCKS * (sm_count - total_tiles) ? 1 : 2;

@@ -426,8 +426,8 @@ def test_fused_encoder_mlp_block_equals_the_unfused_kernels_and_the_oracle(mods,
     """The fused FC1 -> GELU -> FC2 -> residual kernel (default placement of encoder blocks with d <= 384 and more than
     128 rows) against the same model placed with every GEMM as its own launch: same rounding points, same
     reduction order, so the logits must be bit-identical; and against the oracle for the first and last image.
-    Shapes: ViT-S (two MMAs of N = 192 per k step), d 128 and 256 (one MMA), d 320 (two of 160; five k-blocks: a
-    partly filled second ring slot), with row counts that leave a ragged last pair."""
+    Shapes: ViT-S (two MMAs of N = 192 per k step), d 128 and 256 (one MMA), d 320 (two of 160; five k-blocks: the ring
+    of four W1 slots starts each chunk at another one), with row counts that leave a ragged last pair."""
     E, server = mods
     d, heads, mlp, layers, B, img = shape
     p = synth.make_vit(d=d, n_layers=layers, n_heads=heads, mlp=mlp, n_cls=100, seed=5, device=DEV, img=img, std=0.05,
