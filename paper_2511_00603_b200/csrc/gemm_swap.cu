@@ -30,9 +30,9 @@
 // out its own 128 columns as above, with the CTAs of the same half in the other k ranges.  Against tiles of 256 batch rows on
 // CTA pairs (the tile-pair kernel) the row tile is free: 536 rows are four of 160 and not two of 256 and a third that is nearly
 // empty, and K can be split where the tiles are few.  (One barrier a stage for both operands: with one each, as in the form on one
-// CTA, a k-block cost the issuer 650 cycles, now 360; 16 epilogue warps instead of eight gained nothing.)  512-token chunk beside
-// 24 decode requests, 1B decoder: 2498 -> 2367 us a step; a prompt of 509 tokens 1648 -> 1560, of 250 1419 -> 1271; two of 300, 8B,
-// 11310 -> 10600; one image through ViT-B 602 -> 548.
+// CTA, a k-block cost the issuer 650 cycles, now 360; 16 epilogue warps instead of eight gained nothing.)  Whole steps without
+// and with it (the builds before and after, in turn): 1B decoder, a prompt of 250 tokens 1408 and 1269 us, of 450 1632 and 1570, of 520 2074
+// and 1917, 512-token chunk beside 24 decode requests 2498 and 2367; 8B decoder, 300 tokens 7916 and 6236; one image through ViT-B 599 and 547.
 //
 // Roles per CTA (converged warps, an elected lane issues): warp 0 TMA producer of W -- it does not wait for the earlier
 // kernels of the stream, weights being static, so its ring is full when they finish; the last warp TMA producer of the
