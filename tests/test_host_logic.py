@@ -139,7 +139,7 @@ def test_collect_method_without_ctypes_takes_what_the_general_one_takes(E):
 def test_collect_method_lets_other_threads_run(E):
     """The compiled method asks for an answer that is not there yet without the interpreter lock.  The C library's usleep stands in for
     epara_collect: it takes its microseconds where the context's address goes."""
-    from paper_2511_00603_b200 import _fastcall
+    _fastcall = pytest.importorskip("paper_2511_00603_b200._fastcall")
 
     class Sleeper:
         _handle = 300_000
@@ -178,7 +178,8 @@ def test_build_goes_on_without_the_compiled_collect_method(monkeypatch, tmp_path
 
 def test_collect_extension_is_named_for_this_interpreter(E, monkeypatch, tmp_path):
     """The extension is made for one interpreter's ABI: its file carries the tag, one without a tag is removed, nothing partial is left."""
-    from paper_2511_00603_b200 import _fastcall, build
+    from paper_2511_00603_b200 import build
+    _fastcall = pytest.importorskip("paper_2511_00603_b200._fastcall")
     suffix = sysconfig.get_config_var("EXT_SUFFIX")
     assert suffix != ".so" and os.path.basename(_fastcall.__file__) == "_fastcall" + suffix
     untagged, tagged = tmp_path / "_fastcall.so", tmp_path / os.path.basename(build.FAST_LIB)
@@ -197,7 +198,7 @@ def test_bench_gives_dram_traffic_only_for_the_profiled_step():
 
 
 def test_collect_method_asks_once_for_an_answer_that_is_there(E):
-    from paper_2511_00603_b200 import _fastcall
+    _fastcall = pytest.importorskip("paper_2511_00603_b200._fastcall")
     calls = []
     proto = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.c_uint64, ctypes.c_void_p)
     fns = [proto(lambda ctx, ticket, out, k=k: calls.append((k, ctx, ticket)) or (E.PENDING if k == "ready" and ticket == 1 else E.E_TIMEOUT))
